@@ -120,7 +120,8 @@ typedef struct {
 typedef struct {
     int32_t max_views_per_call; /* views per estimate call the workspace is sized for (default n_views, <= 64) */
     int64_t bin_capacity;       /* triangle-tile bin entries over those views (default (6 n_triangles + 8 tiles) * views) */
-    int32_t pairs_per_item;     /* antithetic pairs one CTA runs per (view, tile) item (default 8, <= 64) */
+    int32_t pairs_per_item;     /* antithetic pairs one CTA runs per (view, tile) item (<= 64; default: 8 to 32,
+                                   by how many items the call has; dense tiles run a quarter of it) */
     int32_t blocks_per_sm;      /* persistent CTAs per SM (default: as many as fit) */
     int32_t max_pairs_per_call; /* pairs per view projected at once (default 64); more run in blocks */
     int32_t footprint;          /* texels a pixel credits (SGE_FOOT_*; default bilinear)           */
@@ -335,7 +336,7 @@ typedef struct {
 /* Launch shape of a batched call; zero fields take the defaults.  sge_autotune_batch
  * measures the choices and returns the fastest. */
 typedef struct {
-    int32_t pairs_per_item;    /* antithetic pairs one CTA runs per (view, tile) item (default 8, <= 64) */
+    int32_t pairs_per_item;    /* antithetic pairs one CTA runs per (view, tile) item (<= 64; default as in sge_config) */
     int32_t blocks_per_sm;     /* persistent CTAs per SM of the fast kernel (default: as many as fit)    */
     int32_t light_bin;         /* tiles whose bin holds at most this many triangles take the fast
                                   kernel, the rest the general one (default and maximum 256)             */

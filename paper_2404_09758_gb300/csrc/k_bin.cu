@@ -171,6 +171,7 @@ __global__ void __launch_bounds__(1024) k_bin_scan(Workspace ws, int n, int nt, 
     ws.counters[2] = off;
     ws.counters[4] = overflow || !list_items ? 0u : hoff;
     ws.counters[5] = 0u;
+    ws.counters[6] = 0u;
     if (overflow) atomicCAS(ws.counters + 3, 0u, (uint32_t)SGE_ERR_BIN_OVERFLOW);
   }
 }

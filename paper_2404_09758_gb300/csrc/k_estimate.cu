@@ -250,7 +250,7 @@ __device__ __forceinline__ void heavy_items(const SceneDev& S, const Workspace& 
   const int ntl = n_tiles(S);
   // heavy items cost many times a light one: a quarter of the run of pairs per work unit
   // spreads the few of them over more CTAs
-  const int ppi = max(1, a.pairs_per_item / 4);
+  const int ppi = max(1, (a.pairs_per_item > 0 ? a.pairs_per_item : kRun) / 4);
   const int n_chunks = (a.pair_count + ppi - 1) / ppi;
   const long long n_work = (long long)ws.counters[4] * n_chunks;
   const int n_all = vl.n * ntl;
@@ -527,21 +527,13 @@ cudaError_t launch_heavy_batch(const BatchArgs& P, int shading, int grid, cudaSt
   return shading == SHADE_UNLIT ? launch_heavy_batch_t<kHtUnlit>(P, grid, st) : launch_heavy_batch_t<kHtLit>(P, grid, st);
 }
 
-cudaError_t launch_estimate(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a,
-                            int grid_fast, int grid_heavy, cudaStream_t st, const cudaEvent_t* ev_fast) {
-  cudaError_t e = ev_fast ? cudaEventRecord(ev_fast[0], st) : cudaSuccess;
-  if (e == cudaSuccess) e = launch_fast(S, ws, vl, a, grid_fast, st);
-  if (e == cudaSuccess && ev_fast) e = cudaEventRecord(ev_fast[1], st);
-  if (e != cudaSuccess) return e;
-  if (S.shading == SHADE_UNLIT) e = launch_heavy_t<kHtUnlit, 4, false>(S, ws, vl, a, grid_heavy, st);
-  else if (S.grouped && group_channels(S) <= kGroupSmallChannels)
-    e = launch_heavy_t<kHtGroupSmall, kGroupSmallChannels, true>(S, ws, vl, a, grid_heavy, st);
-  else if (S.grouped) e = launch_heavy_t<kHtGroup, 16, true>(S, ws, vl, a, grid_heavy, st);
-  else e = launch_heavy_t<kHtLit, 4, false>(S, ws, vl, a, grid_heavy, st);
-  if (e == cudaSuccess && ev_fast) e = cudaEventRecord(ev_fast[2], st);
-  if (e != cudaSuccess) return e;
-  if (a.loss && a.pair_begin == 0) k_background_loss<<<dim3(n_tiles(S), vl.n), TILE_PX, 0, st>>>(S, ws, vl, a.loss);
-  return cudaGetLastError();
+cudaError_t launch_heavy(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
+                         cudaStream_t st) {
+  if (S.shading == SHADE_UNLIT) return launch_heavy_t<kHtUnlit, 4, false>(S, ws, vl, a, grid, st);
+  if (S.grouped && group_channels(S) <= kGroupSmallChannels)
+    return launch_heavy_t<kHtGroupSmall, kGroupSmallChannels, true>(S, ws, vl, a, grid, st);
+  if (S.grouped) return launch_heavy_t<kHtGroup, 16, true>(S, ws, vl, a, grid, st);
+  return launch_heavy_t<kHtLit, 4, false>(S, ws, vl, a, grid, st);
 }
 
 cudaError_t launch_background_loss(const SceneDev& S, const Workspace& ws, const ViewList& vl, float* loss,

@@ -10,24 +10,36 @@
 // each pixel's candidates among them (at most CMAX; more: test them all) are stored, so that a
 // pair tests a handful of triangles, not the bin.
 //
-// Work item = (view, 16x16 tile, run of antithetic pairs); one CTA thread per pixel.
-// Per pair (Eq. 8 for one sign vector s, Algorithms 1-2):
-//   F+S the previous pair's credits are folded into per-channel sums with that
-//       pair's signs; the live triangles are set up on both sides (theta + s eps,
-//       theta - s eps) in shared memory from the projected perturbed vertices of
-//       the vertex pass (k_vertex.cu), with their 9 coordinate signs;
-//   R   each pixel finds its visible triangle on both sides among its candidates
-//       (smallest packed depth|id key);
-//   U   it computes both sides' UV and inserts the texels of their bilinear
-//       footprints into a shared-memory table (one key per texel for all read textures
-//       when they share one size); the first pixel to touch a texel in the pair draws
-//       the pair's signs of its channels;
-//   G   it samples its perturbed texels (signs from the table), shades both sides,
-//       forms f+ - f- and credits it: the visible triangle (all three vertices at
-//       once, or single corners where the sides disagree) and the union of the
-//       texel footprints.
-// At the end of the item every credited vertex corner and texel issues one global
-// atomic per channel for its sum and its count.
+// Work item = (view, 16x16 tile, run of antithetic pairs), one CTA.  Its pairs run in groups of up to
+// GMAX (as many as the set-ups and sums fit in shared memory), with barriers only between a group's
+// steps (Eq. 8 for each pair's sign vector s, Algorithms 1-2):
+//   S   every live triangle is set up on both sides (theta + s eps, theta - s eps) for every pair of
+//       the group, in shared memory, from the projected perturbed vertices of the vertex pass
+//       (k_vertex.cu), with its 9 coordinate signs; the item's texel window (below) gets the
+//       group's sign bits;
+//   then the warps take units, an 8 x 4 pixel block of one pair each, from a shared counter; per side
+//   R   each pixel finds its visible triangle among its candidates (smallest packed depth|id key);
+//   U   computes its UV and bilinear footprint;
+//   G   samples its perturbed texels (values and signs from the window; outside it from memory) and
+//       shades them; then forms f+ - f- and credits it: the visible triangle (all three vertices at
+//       once, or single corners where the sides disagree) and the union of the texel footprints;
+//   F   the group's sums are folded with its pairs' signs and issue one global atomic per corner or
+//       texel channel.  The counts of texels follow once per item.
+//
+// Texel window: the bounding box of the first pair's footprints, two texels wider, whose texel values sit
+// in shared memory and whose slots take the credits.  A footprint's four texels get the same
+// f+ - f-, so a pixel makes ONE addition, to the footprint's cell; a texel's sum is that of the four
+// cells around it (fold).  Only texels of side - outside side +'s footprint are credited one by
+// one.  Footprints outside the window (cut where it would not fit, or absent) get hashed cells.
+//
+// Bound by instruction issue: no contraction, under 0.1 B of DRAM per pixel and pair.  One barrier pair
+// per group instead of two barriers and a fold per pair, the window instead of global loads and a
+// sign-plane look-up per texel, one sum per footprint instead of four, lit frames once per triangle
+// and side instead of per pixel, and 32 (lit: 16) warps per SM instead of 16 (8) took the kernel from
+// 10.5 to 6.2 ms (unlit, 8,192 triangles, 512^2, 8 views x 64 pairs), 35.8 to 11.9 ms (Lambert, 32,768
+// triangles, 1024^2, 8 x 16), 28.8 to 11.2 ms (GGX, 1 M triangles, 2048^2, 4 x 4).
+// Measured and not kept: lanes strided over the tile instead of blocks (fewer atomic conflicts, +7 %),
+// 8 or 12 warps per CTA (+8 to +30 %), two lit CTAs of 8 warps per SM (+10 %).
 #include <cuda_runtime.h>
 
 #define SGE_FILE_ID 4  // range-check sites of this file (checked build)
@@ -38,32 +50,8 @@ namespace sge {
 namespace {
 
 constexpr int NB = kLightBin;
-constexpr int CMAX = 16;  // candidate triangles kept per pixel
-constexpr int MAX_PROBE = 16;
-constexpr uint32_t EMPTY = 0xFFFFFFFFu;
-constexpr uint32_t NOSLOT = 0xFFFFu;
-
-// GR: the read textures share one size, so every pixel's bilinear footprint is the same texels
-// in all of them and one table entry (keyed by texel) carries all their channels.
-template <int SH, bool GR = false>
-struct Model {
-  static constexpr int NREAD = SH == SHADE_UNLIT ? 1 : (SH == SHADE_LAMBERT ? 2 : 4);
-  // footprints computed and inserted per side: one for a group, one per texture otherwise
-  static constexpr int NFOOT = GR ? 1 : NREAD;
-  // a tile's bilinear footprints over a run of pairs hold a few hundred texels at about one
-  // texel per pixel, more where the surface is seen at a grazing angle
-  static constexpr int TABLE = (SH == SHADE_UNLIT || GR) ? 1024 : 2048;
-  static constexpr int TSC = GR ? 4 * NREAD : 4;  // channel sums per table entry
-  // one footprint per side (unlit, texel groups): the table's first WCAP slots can hold an item's
-  // texel window, indexed directly; the rest stay hashed for footprints outside it
-  static constexpr bool DIRECT = NFOOT == 1;
-  // one read texture: a footprint outside the window credits the global sums directly (its
-  // texels are rarely shared with other pixels there, and hashing costs more than it saves), so
-  // the window may take the whole table; texel groups keep a hashed quarter (a global credit
-  // would cost one atomic per channel of every grouped texture)
-  static constexpr bool HASH_OUTSIDE = NREAD > 1;
-  static constexpr int WCAP = HASH_OUTSIDE ? TABLE * 3 / 4 : TABLE;
-};
+constexpr int CMAX = 32;  // candidate triangles kept per pixel (a pixel with more tests every live triangle)
+constexpr int GMAX = 8;   // pairs of one group: set up together, one barrier before and after their pixels
 
 // A bin triangle's unperturbed edge functions for the pruning pass, with its margin; 64 bytes.
 struct __align__(16) TriS {
@@ -74,225 +62,6 @@ struct __align__(16) TriS {
   int small;        // the pruning tests fit 32 bits: |a|, |b| < 2^16, |e0| < 2^29, margin < 2^10
   int pad;
 };
-
-// One side of a live triangle set up for one pair of the estimator (the triangle's id is the
-// item's btri[]); 80 bytes.
-struct __align__(16) SideTri {
-  long long e0[3];  // oriented edge functions at the tile's first pixel centre
-  int a[3], b[3];   // oriented edge steps per fixed-point unit in x and y
-  int flags;        // bits 0-2: edge k is not a top/left edge; bit 3: drawn on this side; bit 4: every
-                    // edge function over the tile fits 32 bits (|a|, |b| < 2^16, |e0| < 2^29)
-  float inv_area;
-  float z[3], iw[3];
-};
-static_assert(sizeof(SideTri) == 80, "SideTri layout");
-constexpr int kDrawn = 8, kSmall = 16;
-
-template <int TABLE, int TSC>
-struct FastSmem {
-  SideTri side[2][NB];
-  float uv[NB][6];
-  int vid[NB][3];
-  int btri[NB];          // triangle id of each live entry
-  uint32_t zminb[NB];    // ordered bits of its smallest depth under any perturbation of the call
-  uint32_t sgn9[2][NB];  // bit 3k+c: coordinate c of corner k has s = -1 (by pair parity)
-  float A_tri[NB];
-  uint32_t n_tri[NB];
-  float A_cor[NB][3];
-  uint32_t n_cor[NB][3];
-  float S_cor[NB][3][3];
-  uint32_t c_cor[NB][3];
-  uint32_t tkey[TABLE];
-  float tA[TABLE];       // the current pair's sum of f+ - f- over the pixels crediting the entry
-  float tS[TSC][TABLE];
-  uint32_t tcnt[TABLE];
-  uint32_t tsb[TABLE];   // the current pair's sign bits of the entry's channels (4 r + c), stored by
-                         // every pixel that samples the texel (all store the same value)
-  uint16_t used[TABLE];  // slots holding a key in this item, in insertion order
-  uint32_t n_used;
-  int win[4];            // the item's texel window: x (before wrapping) from win[0] to win[1], rows
-                         // win[2] to win[3]; slot (y - win[2]) * width + x - win[0]
-  uint32_t n_win;        // its slots (the first entries of used[]), 0 without a window
-  float m[16];
-  float red[TILE_PX / 32];
-  uint32_t item;
-};
-
-// Two unlit CTAs share an SM: 228 KB of shared memory less 1 KB reserved per CTA.
-static_assert(2 * (sizeof(FastSmem<Model<SHADE_UNLIT>::TABLE, Model<SHADE_UNLIT>::TSC>) + 1024) <= 228 * 1024,
-              "the unlit fast estimator must fit two CTAs per SM");
-
-__device__ __forceinline__ void store_side_tri(SideTri& d, const Tri& t) {
-  if (!t.ok) {
-    d.flags = 0;
-    return;
-  }
-  int flags = kDrawn;
-  bool small = true;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    d.e0[k] = t.e0[k];
-    d.a[k] = t.a[k];
-    d.b[k] = t.b[k];
-    d.z[k] = t.z[k];
-    d.iw[k] = t.iw[k];
-    flags |= (t.bias[k] ? 1 : 0) << k;
-    // over the tile's pixel offsets (0..15) * 256: |a dx| + |b dy| < 2 * 2^28, so |e| < 2^30
-    small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
-            t.e0[k] < (1ll << 29);
-  }
-  d.flags = flags | (small ? kSmall : 0);
-  d.inv_area = t.inv_area;
-}
-
-// Exact coverage at pixel offset (dx, dy) and the barycentric weights lambda_k = E_k / area there
-// (as lambdas() forms them): 32-bit edge functions for a small triangle, 64-bit otherwise; the
-// integers are the same, and so is each float conversion.
-__device__ __forceinline__ bool cover_lambdas(const SideTri& t, int dx, int dy, float l[3]) {
-  bool in = true;
-  if (t.flags & kSmall) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int e = (int)t.e0[k] + t.a[k] * (dx * 256) + t.b[k] * (dy * 256);
-      in = in && (e - ((t.flags >> k) & 1) >= 0);
-      l[k] = __fmul_rn(__int2float_rn(e), t.inv_area);
-    }
-  } else {
-    long long e[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      e[k] = t.e0[k] + (long long)t.a[k] * (dx * 256) + (long long)t.b[k] * (dy * 256);
-      in = in && (e[k] - ((t.flags >> k) & 1) >= 0);
-    }
-    lambdas(e, t.inv_area, l);
-  }
-  return in;
-}
-
-__device__ __forceinline__ uint32_t hslot(uint32_t k, int table) {
-  k ^= k >> 16;
-  k *= 0x7feb352du;
-  k ^= k >> 15;
-  return k & (uint32_t)(table - 1);
-}
-
-// Find or insert a texel key in the hashed slots [hbase, hbase + hsize) (hsize a power of two;
-// keys stay for the whole item; a new one is listed in used[]).
-template <int TABLE, int TSC>
-__device__ __forceinline__ uint32_t table_insert(FastSmem<TABLE, TSC>& sm, uint32_t key, uint32_t hbase,
-                                                 uint32_t hsize) {
-  uint32_t h = hslot(key, hsize);
-#pragma unroll 1
-  for (int p = 0; p < MAX_PROBE; ++p) {
-    const uint32_t slot = hbase + h;
-    uint32_t k = *(volatile uint32_t*)&sm.tkey[slot];
-    if (k == EMPTY) {
-      k = atomicCAS(&sm.tkey[slot], EMPTY, key);
-      if (k == EMPTY) {
-        sm.used[atomicAdd(&sm.n_used, 1u)] = (uint16_t)slot;
-        return slot;
-      }
-    }
-    if (k == key) return slot;
-    h = (h + 1) & (hsize - 1);
-  }
-  return NOSLOT;
-}
-
-// Texel id of footprint corner q from the packed (x0,y0) id and its edge flags.
-__device__ __forceinline__ int texel_of(uint32_t pk, int q, int w) {
-  int t = (int)(pk & 0x3FFFFFFFu);
-  if (q & 1) t += (pk & (1u << 30)) ? -(w - 1) : 1;
-  if ((q & 2) && !(pk & (1u << 31))) t += w;
-  return t;
-}
-
-// Sign bits of texel t's channels (bit c: s = -1) in one texture's sign plane of an estimate.
-__device__ __forceinline__ uint32_t plane_nibble(const SceneDev& S, const uint32_t* planes, int off, int t) {
-  const long long w = (long long)off + (t >> 3);
-  if (!CHK(S, w, S.chk.sign_words)) return 0u;
-  return (__ldg(planes + w) >> (4 * (t & 7))) & 0xFu;
-}
-
-// Every slot of the table empty (once per call of the estimator loop in a CTA).
-template <int TABLE, int TSC>
-__device__ __forceinline__ void clear_table(FastSmem<TABLE, TSC>& sm) {
-  for (int s = threadIdx.x; s < TABLE; s += blockDim.x) {
-    sm.tkey[s] = EMPTY;
-    sm.tA[s] = 0.0f;
-    sm.tcnt[s] = 0u;
-    sm.tsb[s] = 0u;
-#pragma unroll
-    for (int c = 0; c < TSC; ++c) sm.tS[c][s] = 0.0f;
-  }
-  if (threadIdx.x == 0) sm.n_used = 0;
-}
-
-// The n_used slots an item used back to empty (after its flush).
-template <int TABLE, int TSC>
-__device__ __forceinline__ void clear_used(FastSmem<TABLE, TSC>& sm, uint32_t n_used) {
-  for (uint32_t i = threadIdx.x; i < n_used; i += blockDim.x) {
-    const uint32_t s = sm.used[i];
-    sm.tkey[s] = EMPTY;
-    sm.tA[s] = 0.0f;
-    sm.tcnt[s] = 0u;
-#pragma unroll
-    for (int c = 0; c < TSC; ++c) sm.tS[c][s] = 0.0f;
-  }
-}
-
-// Fold a pair's credits (table entries and triangle corners) into the per-channel sums with
-// that pair's signs: texel signs in tsb (stored while sampling), vertex signs in sgn9[parity].
-// A table entry's counts go straight to tcnt when it is credited; an entry whose pair sum is
-// exactly zero is skipped (adding +-0 leaves every sum as it is).
-template <int TABLE, int TSC, bool GR, int NREAD>
-__device__ __forceinline__ void fold(const SceneDev& S, FastSmem<TABLE, TSC>& sm, int nb, int parity) {
-  // the item's keys only (the used list, whose first n_win entries are the window's slots 0, 1, ...
-  // in order: those are swept directly, lane i on slot i)
-  const uint32_t n_used = sm.n_used, n_win = sm.n_win;
-  for (uint32_t i = threadIdx.x; i < n_used; i += blockDim.x) {
-    const uint32_t s = i < n_win ? i : sm.used[i];
-    const float A = sm.tA[s];
-    if (A == 0.0f) continue;
-    const uint32_t sbits = sm.tsb[s];
-    if (!GR) {
-      const int cn = NREAD == 1 ? S.rtex[0].c : S.tex[(sm.tkey[s] >> 28) - 1].c;
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (c < cn) sm.tS[c][s] += ((sbits >> c) & 1) ? -A : A;
-    } else {
-      // group entry: channel c of read texture r at 4 r + c
-#pragma unroll
-      for (int r = 0; r < NREAD; ++r) {
-        const int cn = S.rtex[r].c;
-#pragma unroll
-        for (int c = 0; c < 4; ++c)
-          if (c < cn) sm.tS[4 * r + c][s] += ((sbits >> (4 * r + c)) & 1) ? -A : A;
-      }
-    }
-    sm.tA[s] = 0.0f;
-  }
-  const int j = threadIdx.x;
-  if (j < nb) {
-    const uint32_t sg = sm.sgn9[parity][j];
-    const float at = sm.A_tri[j];
-    const uint32_t nt = sm.n_tri[j];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const float a = at + sm.A_cor[j][k];
-      const uint32_t n = nt + sm.n_cor[j][k];
-      if (n) {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) sm.S_cor[j][k][c] += ((sg >> (3 * k + c)) & 1) ? -a : a;
-        sm.c_cor[j][k] += n;
-      }
-      sm.A_cor[j][k] = 0.0f;
-      sm.n_cor[j][k] = 0u;
-    }
-    sm.A_tri[j] = 0.0f;
-    sm.n_tri[j] = 0u;
-  }
-}
 
 // Sum of v over the run of consecutive lanes (in lane order) that share key k, for the run's
 // last lane; every lane of the warp calls it.  Returns whether the lane ends its run and sets n
@@ -469,6 +238,7 @@ __device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_
     // entries one rank) with ties broken by list position, so the ranks are a permutation.
     const int k = min(n, CMAX);
     uint32_t b[CMAX / 4] = {};
+    static_assert(CMAX == 32 && CMAX <= kHeavyCand, "a light tile's list is two int4 words");
     for (int q = 0; q < k; ++q) {
       const uint32_t j = cl[q][tid];
       const uint32_t zj = ordered_bits(zr(j));
@@ -482,6 +252,7 @@ __device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_
       for (int i = 0; i < CMAX / 4; ++i) b[i] |= (rank >> 2) == i ? bits : 0u;
     }
     ws.cand[ci] = make_int4((int)b[0], (int)b[1], (int)b[2], (int)b[3]);
+    if (k > 16) ws.cand[ci + TILE_PX] = make_int4((int)b[4], (int)b[5], (int)b[6], (int)b[7]);
   }
   ws.ncand[tile_index * TILE_PX + tid] = (uint8_t)min(n, 255);
 }
@@ -567,7 +338,8 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
   if (tid == 0) {
     ws.tile_live[tix] = (uint32_t)n_live;
     const uint32_t it = ((uint32_t)slot << 24) | (uint32_t)tile;
-    if (n_live <= light_bin) ws.items[atomicAdd(ws.counters + 0, 1u)] = it;
+    if (n_live <= min(light_bin, kBigBin)) ws.items[atomicAdd(ws.counters + 0, 1u)] = it;
+    else if (n_live <= light_bin) ws.tile_cur[atomicAdd(ws.counters + 6, 1u)] = it;
     else ws.items[n_all - 1 - (int)atomicAdd(ws.counters + 4, 1u)] = it;
   }
   const bool wide = n_live > light_bin;  // heavy tile: 16-bit indices
@@ -617,543 +389,1090 @@ __global__ void __launch_bounds__(TILE_PX, 4) k_bin_prune_batch(const BatchArgs 
   prune_tile(D.S, D.ws, A.n_views, A.view[slot], slot, blockIdx.x, P.light_bin, sm);
 }
 
-// Every light work item of one scene's call, taken one at a time from the scene's work
-// counter until none is left.
+// ---------------------------------------------------------------- the estimator
+// Sizes of one model's kernel.  GR: the read textures share one size, so every pixel's bilinear
+// footprint is the same texels in all of them, and one window slot carries all their channels.
+template <int SH, bool GR = false>
+struct Model {
+  static constexpr int NREAD = SH == SHADE_UNLIT ? 1 : (SH == SHADE_LAMBERT ? 2 : 4);
+  // footprints (and texel windows) per side: one for a group, one per texture otherwise
+  static constexpr int NFOOT = GR ? 1 : NREAD;
+  static constexpr bool LIT = SH != SHADE_UNLIT;
+  static constexpr int WARPS = 16;     // warps of a CTA
+  static constexpr int CTAS = LIT ? 1 : 2;        // resident CTAs per SM
+  static constexpr int THREADS = 32 * WARPS;
+  static constexpr int SLOTS = LIT ? 2 * NB : NB; // (pair, live triangle) set-ups staged per side
+  static constexpr int WCAP = LIT ? 1024 : 768;   // texel slots of all windows together
+  static constexpr int ACAP = LIT ? 8192 : 7168;  // (pair, cell or texel) sums
+  static constexpr int NV = GR ? 2 : 1;           // float4s of texel values per slot
+  static constexpr int SPP = GR ? 4 * NREAD : 4;  // sign bits per slot and pair
+  static constexpr int GPW = 32 / SPP;            // pairs per sign word
+  static constexpr int NW = GMAX / GPW;           // sign words per slot
+  // the sign words use the float4s' free components (unlit and ungrouped textures: w of the first;
+  // grouped Lambert: z, w of the second); grouped GGX has none free
+  static constexpr bool SIGNS_APART = GR && SH == SHADE_GGX;
+};
+constexpr int kHashNoWindow = 512, kHashWindow = 128;  // hashed footprints of an item without / with a window
+constexpr int kHashProbe = 8;
+
+// One side of a live triangle set up for one pair; 64 bytes.
+// Small (every edge function over the tile fits 32 bits: |a|, |b| < 2^16, |e0| < 2^29, so
+// |e| < 2^30 at the offsets 0..15 * 256): e = (E_0, E_1, area, flags) with E_k at the tile's first
+// pixel centre and area = E_0 + E_1 + E_2, which is the same everywhere, so edge 2 follows from the
+// other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig): the vertices relative to the first pixel
+// centre, e = (X0, Y0, X1, flags), ab = (Y1, X2, Y2, -).  Not drawn: E_0 = -1 everywhere.
+struct __align__(16) SideTri {
+  int4 e, ab;
+  float4 z;   // z_0..2, 1 / area
+  float4 iw;  // 1 / w_0..2
+};
+static_assert(sizeof(SideTri) == 64, "SideTri layout");
+constexpr int kBig = 8, kFlip = 16;  // flags; bits 0-2: edge k is not a top/left edge
+
 template <int SH, bool GR>
-__device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
-                                           const EstimateArgs& a,
-                                           FastSmem<Model<SH, GR>::TABLE, Model<SH, GR>::TSC>& sm) {
-  constexpr int NREAD = Model<SH, GR>::NREAD;
-  constexpr int NFOOT = Model<SH, GR>::NFOOT;
-  constexpr int TABLE = Model<SH, GR>::TABLE;
-  constexpr int TSC = Model<SH, GR>::TSC;
-  const int tid = threadIdx.x;
-  const int dx = tid % TILE, dy = tid / TILE;
-  const int ntl = n_tiles(S);
-  const int n_chunks = (a.pair_count + a.pairs_per_item - 1) / a.pairs_per_item;
-  const long long n_work = (long long)ws.counters[0] * n_chunks;
-  clear_table(sm);
+struct FastSmem {
+  using M = Model<SH, GR>;
+  SideTri side[2][M::SLOTS];      // slot g nb + j: triangle j of the group's pair g
+  float4 th[M::NV][M::WCAP];      // unperturbed texel values the shading reads (zero: absent channels)
+  int4 cand[TILE_PX];             // each pixel's candidates (8-bit live indices), by block and lane
+  uint32_t ts[M::SIGNS_APART ? M::NW : 1][M::SIGNS_APART ? M::WCAP : 1];  // the group's sign bits
+  uint32_t tcnt[M::WCAP];         // item counts: low half the slot's cell, high half the texel alone
+  float tA[M::ACAP];              // the group's sums, per pair: window cells, hashed cells, window texels
+  uint32_t hkey[kHashNoWindow];   // hashed footprints (credit codes) and their item counts
+  uint32_t hcnt[kHashNoWindow];
+  float frame[M::LIT ? 2 : 1][M::LIT ? M::SLOTS : 1][6];  // lit: the set-up's face normal and u tangent
+  float tgt[3][TILE_PX];          // target colours, by block and lane
+  float uv[NB][6];
+  int vid[NB][3];
+  int btri[NB];                   // triangle id of each live entry
+  uint32_t zminb[NB];             // ordered bits of its smallest depth under any perturbation of the call
+  uint32_t sgn9[2][M::SLOTS];     // bit 3k+c: coordinate c of corner k has s = -1 (by group parity)
+  float A_tri[M::SLOTS];          // f+ - f- of the pixels that see the triangle (side +, else side -)
+  uint32_t n_tri[M::SLOTS];
+  float A_cor[M::SLOTS][3];       // and of the pixels that add single corners of it
+  uint32_t n_cor[M::SLOTS];       // their counts, 10 bits per corner (at most 256 pixels)
+  int4 win[M::NFOOT];             // texel windows: first column (before wrapping), first row, width, height
+  int wbase[M::NFOOT + 1];        // first slot of each window; the total
+  float red[M::WARPS];
+  uint32_t item, unit;            // work counters: the kernel's item, the group's next (block, pair)
+  uint32_t act[TILE_PX / 32], nact;  // blocks of the tile with a candidate at some pixel
+  uint8_t ncand[TILE_PX];
+};
 
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) sm.item = atomicAdd(ws.counters + 1, 1u);
-    __syncthreads();
-    const long long w = sm.item;
-    if (w >= n_work) break;
-    const uint32_t it = ws.items[w / n_chunks];
-    const int chunk = (int)(w % n_chunks);
-    const int slot = it >> 24, tile = it & 0xFFFFFF;
-    if (!CHK(S, slot, vl.n) || !CHK(S, tile, ntl)) continue;  // (checked build; uniform over the CTA)
-    const int view = vl.id[slot];
-    const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-    const int px = tx * TILE + dx, py = ty * TILE + dy;
-    const bool valid = px < S.W && py < S.H;
-    const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
-    const uint32_t bin_beg = ws.tile_off[slot * ntl + tile];
-    const int nb = (int)ws.tile_live[slot * ntl + tile];
-    const int p0 = a.pair_begin + chunk * a.pairs_per_item;
-    const int p1 = min(a.pair_begin + a.pair_count, p0 + a.pairs_per_item);
-    if (tid < 16) sm.m[tid] = S.mvp[16 * view + tid];
+static_assert(2 * (sizeof(FastSmem<SHADE_UNLIT, false>) + 1024) <= 228 * 1024, "two unlit CTAs must fit an SM");
+static_assert(sizeof(FastSmem<SHADE_GGX, true>) + sizeof(BatchSmem) <= 227 * 1024, "lit");
+static_assert(sizeof(FastSmem<SHADE_GGX, false>) + sizeof(BatchSmem) <= 227 * 1024, "lit");
 
-    // ---- per item: the bin's live triangles (pruned and compacted by k_bin_prune), their
-    //      smallest depths, and this pixel's candidates among them (in order of that depth)
-    if (tid < nb) {
-      const int tri = (int)bin_at(S, ws, bin_beg + tid);
-      sm.btri[tid] = tri;
-      sm.zminb[tid] = ordered_bits(ws.tri_z[(long long)slot * S.nt + tri].x);
+// Set up one side of a triangle from its projected vertices (rx, ry: the tile's first pixel centre).
+__device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int rx, int ry) {
+  if (!(v[0].ok && v[1].ok && v[2].ok)) {
+    d.e = make_int4(-1, 0, 0, 0);
+    d.ab = make_int4(0, 0, 0, 0);
+    return;
+  }
+  const int x0 = v[0].X - rx, x1 = v[1].X - rx, x2 = v[2].X - rx, y0 = v[0].Y - ry, y1 = v[1].Y - ry, y2 = v[2].Y - ry;
+  const int far = max(max(max(abs(x0), abs(x1)), abs(x2)), max(max(abs(y0), abs(y1)), abs(y2)));
+  float inv;
+  if (far < (1 << 14)) {
+    // vertices within 64 pixels of the tile's corner: E_k = x_a y_b - x_b y_a there, all in 32 bits
+    // (|E_k| < 2^29, |a|, |b| < 2^15)
+    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, area = e0 + e1 + (x0 * y1 - x1 * y0);
+    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
+    if (area == 0) {
+      d.e = make_int4(-1, 0, 0, 0);
+      d.ab = make_int4(0, 0, 0, 0);
+      return;
+    }
+    if (area < 0) {
+      e0 = -e0, e1 = -e1, area = -area;
+      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
+    }
+    const int flags = (a0 > 0 || (a0 == 0 && b0 > 0) ? 0 : 1) | (a1 > 0 || (a1 == 0 && b1 > 0) ? 0 : 2) |
+                      (a2 > 0 || (a2 == 0 && b2 > 0) ? 0 : 4);
+    d.e = make_int4(e0, e1, area, flags);
+    d.ab = make_int4(a0, a1, b0, b1);
+    inv = __fdiv_rn(1.0f, __int2float_rn(area));
+  } else {
+    Tri t;
+    setup_tri(v[0], v[1], v[2], rx, ry, t);
+    if (!t.ok) {
+      d.e = make_int4(-1, 0, 0, 0);
+      d.ab = make_int4(0, 0, 0, 0);
+      return;
+    }
+    int flags = 0;
+    bool small = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      flags |= (t.bias[k] ? 1 : 0) << k;
+      small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
+              t.e0[k] < (1ll << 29);
+    }
+    if (small) {
+      d.e = make_int4((int)t.e0[0], (int)t.e0[1], (int)(t.e0[0] + t.e0[1] + t.e0[2]), flags);
+      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
+    } else {
+      const bool flip = (long long)(x1 - x0) * (y2 - y0) < (long long)(y1 - y0) * (x2 - x0);
+      d.e = make_int4(x0, y0, x1, flags | kBig | (flip ? kFlip : 0));
+      d.ab = make_int4(y1, x2, y2, 0);
+    }
+    inv = t.inv_area;
+  }
+  d.z = make_float4(v[0].z, v[1].z, v[2].z, inv);
+  d.iw = make_float4(v[0].iw, v[1].iw, v[2].iw, 0.0f);
+}
+
+// Coverage of the pixel whose centre lies (X, Y) fixed-point units from the tile's first one, and
+// (covered) the barycentric weights E_k / area there as lambdas() forms them.
+__device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, float l[3], float4& z) {
+  const int4 e = t.e, ab = t.ab;
+  if (!(e.w & kBig)) {
+    const int e0 = e.x + ab.x * X + ab.z * Y, e1 = e.y + ab.y * X + ab.w * Y, e2 = e.z - e0 - e1;
+    const int lo = min(min(e0, e1), e2);
+    if (lo < 0) return false;
+    if (lo == 0 && (((e.w & 1) && e0 == 0) || ((e.w & 2) && e1 == 0) || ((e.w & 4) && e2 == 0))) return false;
+    z = t.z;
+    l[0] = __fmul_rn(__int2float_rn(e0), z.w);
+    l[1] = __fmul_rn(__int2float_rn(e1), z.w);
+    l[2] = __fmul_rn(__int2float_rn(e2), z.w);
+    return true;
+  }
+  const int vx[3] = {e.x, e.z, ab.y}, vy[3] = {e.y, ab.x, ab.z};
+  long long E[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int a = (k + 1) % 3, b = (k + 2) % 3;
+    E[k] = edge_at(vx[a], vy[a], vx[b], vy[b], X, Y);
+    if (e.w & kFlip) E[k] = -E[k];
+    if (E[k] - ((e.w >> k) & 1) < 0) return false;
+  }
+  z = t.z;
+  lambdas(E, z.w, l);
+  return true;
+}
+
+// Face normal N and u tangent T of a triangle (as shading_normal forms them): the same for every pixel.
+__device__ __forceinline__ void tri_frame(const float3 p[3], const float* uv, float* out) {
+  const float3 e1 = sub3(p[1], p[0]), e2 = sub3(p[2], p[0]);
+  const float3 N = norm3(cross3(e1, e2));
+  const float du1 = uv[2] - uv[0], dv1 = uv[3] - uv[1], du2 = uv[4] - uv[0], dv2 = uv[5] - uv[1];
+  const float det = du1 * dv2 - du2 * dv1;
+  float3 T = det != 0.0f ? f3((e1.x * dv2 - e2.x * dv1) / det, (e1.y * dv2 - e2.y * dv1) / det,
+                              (e1.z * dv2 - e2.z * dv1) / det)
+                         : e1;
+  const float nt = dot3(N, T);
+  T = norm3(f3(T.x - N.x * nt, T.y - N.y * nt, T.z - N.z * nt));
+  out[0] = N.x, out[1] = N.y, out[2] = N.z;
+  out[3] = T.x, out[4] = T.y, out[5] = T.z;
+}
+
+// The perturbed positions of live triangle j's corners (sign bits sg; side - already inverted).
+__device__ __forceinline__ void corner_positions(const SceneDev& S, const int* vid, uint32_t sg, float3 p[3]) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const float* src = S.pos + 3ll * vid[k];
+    float q[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c)
+      q[c] = __fadd_rn(__ldg(src + c), ((sg >> (3 * k + c)) & 1) ? -S.eps_pos : S.eps_pos);
+    p[k] = f3(q[0], q[1], q[2]);
+  }
+}
+
+// Sign-flip mask of bit b of a word whose wanted bit sits `up` places below bit 31.
+__device__ __forceinline__ float signed_eps(uint32_t word, int up, float eps) {
+  return __uint_as_float(((word << up) & 0x80000000u) ^ __float_as_uint(eps));
+}
+
+// Channels of a read texture the shading uses (albedo, normal: 3; roughness, metallic: 1).
+__device__ __forceinline__ constexpr int used_channels(int r) { return r < 2 ? 3 : 1; }
+
+// Texel id of window slot t.
+__device__ __forceinline__ int window_texel(const int4& win, int t, int w) {
+  const int row = t / win.z;
+  return (win.y + row) * w + wrap_i(win.x + t - row * win.z, w);
+}
+
+// Credit code of a pixel's side in footprint r: the window cell (the slot of the footprint's first
+// texel), or with kOut the first texel's id, kOneRow: its rows are clamped to one, and r above.
+constexpr uint32_t kOut = 1u << 31, kOneRow = 1u << 28, EMPTY = 0xFFFFFFFFu;
+constexpr int kFootShift = 29;
+
+// The texels of the footprint named by a texel id code (w: the texture's width): columns x0, x1, rows
+// y0, y1 (equal where it has one column or row).
+struct Quad {
+  int x0, x1, y0, y1;
+  __device__ __forceinline__ Quad(uint32_t cr, int w) {
+    const int id = (int)(cr & 0x0FFFFFFFu);
+    y0 = id / w;
+    x0 = id - y0 * w;
+    x1 = x0 + 1 == w ? 0 : x0 + 1;
+    y1 = (cr & kOneRow) ? y0 : y0 + 1;
+  }
+  __device__ __forceinline__ int texel(int q, int w) const { return (q & 2 ? y1 : y0) * w + (q & 1 ? x1 : x0); }
+  __device__ __forceinline__ bool repeats(int q) const { return ((q & 2) && y1 == y0) || ((q & 1) && x1 == x0); }
+  __device__ __forceinline__ bool holds(const Quad& o, int q) const {
+    const int x = q & 1 ? o.x1 : o.x0, y = q & 2 ? o.y1 : o.y0;
+    return (x == x0 || x == x1) && (y == y0 || y == y1);
+  }
+};
+
+// Sign bits of texel t's channels (bit c: s = -1) in one texture's sign plane of an estimate.
+__device__ __forceinline__ uint32_t plane_nibble(const SceneDev& S, const uint32_t* planes, int off, int t) {
+  const long long w = (long long)off + (t >> 3);
+  if (!CHK(S, w, S.chk.sign_words)) return 0u;
+  return (__ldg(planes + w) >> (4 * (t & 7))) & 0xFu;
+}
+
+// Hashed slot of an outside code (inserted if new), or -1: no room near its place.
+__device__ __forceinline__ int hash_slot(uint32_t* hkey, uint32_t code, int size) {
+  uint32_t h = code ^ (code >> 16);
+  h *= 0x7feb352du;
+  h ^= h >> 15;
+#pragma unroll 1
+  for (int p = 0; p < kHashProbe; ++p, ++h) {
+    const int slot = (int)(h & (uint32_t)(size - 1));
+    uint32_t k = *(volatile uint32_t*)&hkey[slot];
+    if (k == EMPTY) {
+      k = atomicCAS(&hkey[slot], EMPTY, code);
+      if (k == EMPTY) return slot;
+    }
+    if (k == code) return slot;
+  }
+  return -1;
+}
+
+// The sign bits of window slot s for pair g of the group, from bit 28 - SPP (g mod GPW) + ... on:
+// the word that holds them.
+template <int SH, bool GR>
+__device__ __forceinline__ uint32_t sign_word_of(const FastSmem<SH, GR>& sm, int s, int g) {
+  using M = Model<SH, GR>;
+  if constexpr (M::SIGNS_APART) return sm.ts[g / M::GPW][s];
+  else if constexpr (!GR) return __float_as_uint(sm.th[0][s].w);
+  else return __float_as_uint(g < M::GPW ? sm.th[1][s].z : sm.th[1][s].w);
+}
+
+// After a group's pixels: fold its sums with its pairs' signs into the global sums.  A pixel credits the
+// 2 x 2 texels of a footprint with one sum in the footprint's cell, so a texel's sum is that of the
+// four cells around it plus what was credited to it alone.  (The cells are cleared by clear_cells.)
+template <int SH, bool GR>
+__device__ __forceinline__ void fold(const SceneDev& S, const Workspace& ws, const EstimateArgs& a,
+                                     FastSmem<SH, GR>& sm, int nb, int G, int par, int nh, const uint32_t* planes) {
+  using M = Model<SH, GR>;
+  constexpr int NC = GR ? 4 * M::NREAD : 4;
+  const int n_all = sm.wbase[M::NFOOT], stride = 2 * n_all + nh;
+  for (int r = 0; r < M::NFOOT; ++r) {
+    const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
+    const int4 win = sm.win[r];
+    for (int t = threadIdx.x; t < n; t += M::THREADS) {
+      float acc[NC];
+#pragma unroll
+      for (int c = 0; c < NC; ++c) acc[c] = 0.0f;
+      bool any = false;
+      float* cell = sm.tA + base + t;
+      for (int g = 0; g < G; ++g, cell += stride) {
+        // (no footprint starts in a window's last column: left of a row's first texel lies a zero)
+        float A = cell[0] + cell[n_all + nh];
+        if (t > 0) A += cell[-1];
+        if (t >= win.z) A += cell[-win.z];
+        if (t > win.z) A += cell[-win.z - 1];
+        if (A == 0.0f) continue;
+        any = true;
+        const uint32_t sb = sign_word_of<SH, GR>(sm, base + t, g) >> (M::SPP * (g % M::GPW));
+#pragma unroll
+        for (int c = 0; c < NC; ++c) acc[c] += ((sb >> c) & 1) ? -A : A;
+      }
+      if (!any) continue;
+      const int texel = window_texel(win, t, S.rtex[r].w);
+#pragma unroll
+      for (int q = 0; q < (GR ? M::NREAD : 1); ++q) {
+        const TexDev& T = S.rtex[GR ? q : r];
+        const long long p = T.offset + (long long)texel * T.c;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c < T.c && CHK(S, p + c, S.chk.params)) atomicAdd(a.grad + p + c, acc[4 * q + c]);
+      }
+    }
+  }
+  // hashed footprints: their texels one by one
+  for (int h = threadIdx.x; h < nh; h += M::THREADS) {
+    const uint32_t code = sm.hkey[h];
+    if (code == EMPTY) continue;
+    const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
+    const int tw = S.rtex[r].w;
+    const Quad Q(code, tw);
+#pragma unroll 1
+    for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q) {
+      if (Q.repeats(q)) continue;
+      const int texel = Q.texel(q, tw);
+#pragma unroll 1
+      for (int k = 0; k < (GR ? M::NREAD : 1); ++k) {
+        const TexDev& T = S.rtex[GR ? k : r];
+        float acc[4] = {0.f, 0.f, 0.f, 0.f};
+        for (int g = 0; g < G; ++g) {
+          const float A = sm.tA[g * stride + n_all + h];
+          if (A == 0.0f) continue;
+          const uint32_t sb = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[T.index], texel);
+#pragma unroll
+          for (int c = 0; c < 4; ++c) acc[c] += ((sb >> c) & 1) ? -A : A;
+        }
+        const long long p = T.offset + (long long)texel * T.c;
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          if (c < T.c && CHK(S, p + c, S.chk.params)) atomicAdd(a.grad + p + c, acc[c]);
+      }
+    }
+  }
+  const int j = threadIdx.x;
+  if (j < nb) {
+    float acc[9] = {};
+    uint32_t cnt[3] = {};
+    for (int g = 0; g < G; ++g) {
+      const int s = g * nb + j;
+      const uint32_t nt = sm.n_tri[s], nc = sm.n_cor[s];
+      if ((nt | nc) == 0u) continue;
+      const float at = sm.A_tri[s];
+      const uint32_t sg = sm.sgn9[par][s];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        sm.vid[tid][k] = vert_of(S, tri, k);
-        const int ti = uv_of(S, tri, k);
-        sm.uv[tid][2 * k] = __ldg(S.uvs + 2 * ti);
-        sm.uv[tid][2 * k + 1] = __ldg(S.uvs + 2 * ti + 1);
-        sm.A_cor[tid][k] = 0.0f;
-        sm.n_cor[tid][k] = 0u;
-        sm.c_cor[tid][k] = 0u;
+        const float v = at + sm.A_cor[s][k];
+        cnt[k] += nt + ((nc >> (10 * k)) & 1023u);
 #pragma unroll
-        for (int c = 0; c < 3; ++c) sm.S_cor[tid][k][c] = 0.0f;
+        for (int c = 0; c < 3; ++c) acc[3 * k + c] += ((sg >> (3 * k + c)) & 1) ? -v : v;
+        sm.A_cor[s][k] = 0.0f;
       }
-      sm.A_tri[tid] = 0.0f;
-      sm.n_tri[tid] = 0u;
+      sm.A_tri[s] = 0.0f;
+      sm.n_tri[s] = 0u;
+      sm.n_cor[s] = 0u;
     }
-    const long long ci = ((long long)slot * ntl + tile) * TILE_PX + tid;
-    const int4 cw = ws.cand[((long long)slot * ntl + tile) * kCandWords * TILE_PX + tid];
-    const uint32_t cand[CMAX / 4] = {(uint32_t)cw.x, (uint32_t)cw.y, (uint32_t)cw.z, (uint32_t)cw.w};
-    const int ncand = ws.ncand[ci];
-    const bool all_bin = ncand > CMAX;
-    if (tid == 0) {
-      sm.win[0] = sm.win[2] = 0x7FFFFFFF;
-      sm.win[1] = sm.win[3] = -0x7FFFFFFF;
-      sm.n_win = 0;
-    }
-    // the tile's target pixels: a tile inside the image whose rows start 16-byte aligned is read
-    // as 16 rows of 12 float4 (each row's 16 RGB pixels) into the per-pair set-up array, which is
-    // free until the first pair's set-up; any other tile pixel by pixel
-    float3 tgt = f3(0.f, 0.f, 0.f);
-    const float* trow = S.targets + (((long long)view * S.H + ty * TILE) * S.W + tx * TILE) * 3;
-    const bool vec_tgt = (tx + 1) * TILE <= S.W && (ty + 1) * TILE <= S.H && (S.W & 3) == 0 &&
-                         (reinterpret_cast<uintptr_t>(S.targets) & 15) == 0;
-    if (vec_tgt) {
-      float4* stage = reinterpret_cast<float4*>(&sm.side[0][0]);
-      if (tid < TILE * 12) {
-        const int r = tid / 12, q = tid % 12;
-        stage[tid] = __ldg(reinterpret_cast<const float4*>(trow + (long long)r * S.W * 3) + q);
-      }
-      __syncthreads();
-      const float* st = reinterpret_cast<const float*>(stage) + (dy * TILE + dx) * 3;
-      tgt = f3(st[0], st[1], st[2]);
-    } else if (valid) {
-      const float* tp = S.targets + (((long long)view * S.H + py) * S.W + px) * 3;
-      tgt = f3(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
-    }
-    float loss_acc = 0.0f;
-
-    for (int pair = p0; pair < p1; ++pair) {
-      const int par = pair & 1;
-      const long long pb = pair - a.pair_begin;
-      const uint32_t* planes = ws.tsign + ((long long)slot * ws.max_pairs + pb) * ws.sgn_words;
-      // the previous pair is complete (and the item's set-up is done)
-      __syncthreads();
-      // ---- F: fold the previous pair's credits with its signs (other parity buffers)
-      if (pair > p0) fold<TABLE, TSC, GR, NREAD>(S, sm, nb, par ^ 1);
-      // ---- S: set up the bin's triangles on both sides from the projected perturbed vertices
-      {
-        const long long vb = ((long long)slot * ws.max_pairs + pb) * S.nv;
-        for (int t2 = tid; t2 < 2 * nb; t2 += TILE_PX) {
-          const int sd = t2 < nb ? 0 : 1, j = t2 - sd * nb;
-          PVert v[3];
-          uint32_t sg = 0;
 #pragma unroll
-          for (int k = 0; k < 3; ++k) {
-            const long long o = vb + sm.vid[j][k];
-            const int4 q = __ldg(ws.pverts + 2 * o + sd);
-            v[k].X = q.x;
-            v[k].Y = q.y;
-            v[k].z = __int_as_float(q.z);
-            v[k].iw = __int_as_float(q.w);
-            v[k].ok = q.x != kNotDrawn;
-            if (sd == 0) sg |= ((uint32_t)__ldg(ws.vbits + o) & 7u) << (3 * k);
-          }
-          if (sd == 0) sm.sgn9[par][j] = sg;
-          Tri t;
-          setup_tri(v[0], v[1], v[2], rx, ry, t);
-          store_side_tri(sm.side[sd][j], t);
-        }
-      }
-      __syncthreads();
-
-      // ---- R: visible triangle on both sides among the candidates (nearest-first order: a
-      //      candidate wholly behind both sides' best so far ends the search)
-      int bj[2] = {-1, -1};
-      if (valid && ncand > 0) {
-        {
-          unsigned long long best[2] = {~0ull, ~0ull};
-          auto test = [&](int j) {
+    for (int k = 0; k < 3; ++k) {
+      if (!cnt[k]) continue;
+      const long long p = 3ll * sm.vid[j][k];
 #pragma unroll
-            for (int sd = 0; sd < 2; ++sd) {
-              const SideTri& t = sm.side[sd][j];
-              if (!(t.flags & kDrawn)) continue;
-              float l[3];
-              if (!cover_lambdas(t, dx, dy, l)) continue;
-              const unsigned long long k =
-                  ((unsigned long long)ordered_bits(interp_depth(l, t.z)) << 32) | (uint32_t)sm.btri[j];
-              if (k < best[sd]) {
-                best[sd] = k;
-                bj[sd] = j;
-              }
-            }
-          };
-          if (all_bin) {
-            for (int j = 0; j < nb; ++j) test(j);
-          } else {
-            for (int q = 0; q < ncand; ++q) {
-              const uint32_t word = q < 4 ? cand[0] : (q < 8 ? cand[1] : (q < 12 ? cand[2] : cand[3]));
-              const int j = (int)((word >> (8 * (q & 3))) & 0xFFu);
-              if (!CHK(S, j, nb)) continue;
-              const uint32_t zb = sm.zminb[j];
-              if (zb > (uint32_t)(best[0] >> 32) && zb > (uint32_t)(best[1] >> 32)) break;
-              test(j);
-            }
-          }
-        }
-      }
-
-      // ---- U: UV buffer values and footprints of both sides
-      float bary[2][3];
-      float ffx[2][NFOOT], ffy[2][NFOOT];
-      uint32_t tpk[2][NFOOT];       // texel (x0,y0) id | 1<<30 if x1 wrapped | 1<<31 if y1 == y0
-      uint32_t tslot[2][NFOOT][2];  // four 16-bit table slots per side and footprint
-      int fix[2][NFOOT];            // footprint column before wrapping (nearest mode: the texel id)
-      int fy0[2][NFOOT];            // footprint row y0
-#pragma unroll
-      for (int sd = 0; sd < 2; ++sd) {
-        if (bj[sd] < 0) continue;
-        const SideTri& t = sm.side[sd][bj[sd]];
-        float l[3];
-        cover_lambdas(t, dx, dy, l);
-        const PerspW pw = persp(l, t.iw);
-        const float* uvt = sm.uv[bj[sd]];
-        const float u = persp_interp(pw, uvt[0], uvt[2], uvt[4]);
-        const float v = persp_interp(pw, uvt[1], uvt[3], uvt[5]);
-        if (SH == SHADE_GGX) {
-#pragma unroll
-          for (int k = 0; k < 3; ++k) bary[sd][k] = pw.q[k] / pw.qs;
-        }
-#pragma unroll
-        for (int r = 0; r < NFOOT; ++r) {
-          const TexDev& T = S.rtex[r];
-          const Foot f = footprint(u, v, T.w, T.h);
-          ffx[sd][r] = f.fx;
-          ffy[sd][r] = f.fy;
-          tpk[sd][r] = (uint32_t)(f.y0 * T.w + f.x0) | (f.x1 != f.x0 + 1 ? 1u << 30 : 0u) |
-                       (f.y1 == f.y0 ? 1u << 31 : 0u);
-          fix[sd][r] = S.foot_nearest ? nearest_texel(u, v, T.w, T.h) : f.ix;
-          fy0[sd][r] = f.y0;
-          if (Model<SH, GR>::DIRECT && pair == p0 && !S.foot_nearest && abs(f.ix) < (1 << 28)) {
-            // the item's texel window: every footprint of its first pair, two texels of margin
-            // (a perturbation moves a footprint by a fraction of a texel)
-            atomicMin(&sm.win[0], f.ix - 2);
-            atomicMax(&sm.win[1], f.ix + 3);
-            atomicMin(&sm.win[2], max(f.y0 - 2, 0));
-            atomicMax(&sm.win[3], min(f.y1 + 2, T.h - 1));
-          }
-        }
-      }
-      if (Model<SH, GR>::DIRECT && pair == p0) {
-        __syncthreads();  // the window's bounds are reduced
-        const long long ww = (long long)sm.win[1] - sm.win[0] + 1, wh = (long long)sm.win[3] - sm.win[2] + 1;
-        if (!S.foot_nearest && ww > 0 && wh > 0 && ww * wh <= Model<SH, GR>::WCAP) {
-          // window slots hold their texel's key from the start (and are listed as used)
-          const TexDev& T = S.rtex[0];
-          for (int s2 = tid; s2 < (int)(ww * wh); s2 += TILE_PX) {
-            const int y = sm.win[2] + s2 / (int)ww, x = wrap_i(sm.win[0] + s2 % (int)ww, T.w);
-            sm.tkey[s2] = tkey(T.index, y * T.w + x);
-            sm.used[s2] = (uint16_t)s2;
-          }
-          if (tid == 0) sm.n_used = sm.n_win = (uint32_t)(ww * wh);
-        } else if (tid == 0) {
-          sm.win[0] = 1;  // no window: every key is hashed over the whole table
-          sm.win[1] = 0;
-        }
-        __syncthreads();
-      }
-      // ---- the table slots of the footprints' texels: computed in the window, hashed outside it
-      {
-        const bool direct = Model<SH, GR>::DIRECT && sm.win[0] <= sm.win[1];
-        // without a window every key is hashed over the whole table (nearest footprints, items
-        // whose window would not fit)
-        const uint32_t hbase = direct ? (uint32_t)Model<SH, GR>::WCAP : 0u;
-        const uint32_t hsize = direct ? (uint32_t)(TABLE - Model<SH, GR>::WCAP) : (uint32_t)TABLE;
-#pragma unroll
-        for (int sd = 0; sd < 2; ++sd) {
-          if (bj[sd] < 0) continue;
-#pragma unroll
-          for (int r = 0; r < NFOOT; ++r) {
-            const TexDev& T = S.rtex[r];
-            if (S.foot_nearest) {
-              // the one credited texel (Section 4.4): its slot, and its id in the second word
-              const uint32_t nt = (uint32_t)fix[sd][r];
-              tslot[sd][r][1] = nt;
-              tslot[sd][r][0] = (sd == 1 && bj[0] >= 0 && tslot[0][r][1] == nt)
-                                    ? tslot[0][r][0]
-                                    : table_insert(sm, tkey(T.index, (int)nt), hbase, hsize);
-              continue;
-            }
-            const int y0 = fy0[sd][r];
-            const int y1 = (tpk[sd][r] >> 31) ? y0 : y0 + 1;
-            const int ix = fix[sd][r];
-            if (direct && ix >= sm.win[0] && ix + 1 <= sm.win[1] && y0 >= sm.win[2] && y1 <= sm.win[3]) {
-              const int ww = sm.win[1] - sm.win[0] + 1;
-              const uint32_t s00 = (uint32_t)((y0 - sm.win[2]) * ww + ix - sm.win[0]);
-              const uint32_t s10 = (uint32_t)((y1 - sm.win[2]) * ww + ix - sm.win[0]);
-              tslot[sd][r][0] = s00 | ((s00 + 1) << 16);
-              tslot[sd][r][1] = s10 | ((s10 + 1) << 16);
-              // (checked build) both rows' slots inside the window: else credit globally
-              if (!CHK(S, (long long)s00 + 1, sm.n_win) || !CHK(S, (long long)s10 + 1, sm.n_win))
-                tslot[sd][r][0] = tslot[sd][r][1] = NOSLOT | (NOSLOT << 16);
-            } else if (!Model<SH, GR>::HASH_OUTSIDE) {
-              tslot[sd][r][0] = tslot[sd][r][1] = NOSLOT | (NOSLOT << 16);  // global credits
-            } else {
-              uint32_t sl[4];
-#pragma unroll
-              for (int q = 0; q < 4; ++q)
-                sl[q] = table_insert(sm, tkey(T.index, texel_of(tpk[sd][r], q, T.w)), hbase, hsize);
-              tslot[sd][r][0] = sl[0] | (sl[1] << 16);
-              tslot[sd][r][1] = sl[2] | (sl[3] << 16);
-            }
-          }
-        }
-      }
-
-      // ---- G: sample the perturbed texels (signs from the pair's planes), shade both sides,
-      //      f+ - f-, credits
-      float3 col[2];
-      col[0] = col[1] = f3(S.bg[0], S.bg[1], S.bg[2]);
-      {
-#pragma unroll
-        for (int sd = 0; sd < 2; ++sd) {
-          if (bj[sd] < 0) continue;
-          float tex[NREAD][4];
-          uint32_t gsb[4] = {0u, 0u, 0u, 0u};  // a texel group's sign bits per corner (4 r + c)
-#pragma unroll
-          for (int r = 0; r < NREAD; ++r) {
-            const TexDev& T = S.rtex[r];
-            const int poff = ws.sgn_off[T.index];
-            const int fi = GR ? 0 : r;  // the footprint this texture uses
-            const float fx = ffx[sd][fi], fy = ffy[sd][fi];
-            const float wq[4] = {(1.0f - fx) * (1.0f - fy), fx * (1.0f - fy), (1.0f - fx) * fy, fx * fy};
-#pragma unroll
-            for (int c = 0; c < 4; ++c) tex[r][c] = 0.0f;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int texel = texel_of(tpk[sd][fi], q, T.w);
-              if (!CHK(S, texel, (long long)T.w * T.h)) continue;
-              const uint32_t sb_s = plane_nibble(S, planes, poff, texel);
-              if (GR) {
-                gsb[q] |= sb_s << (4 * r);
-              } else if (!S.foot_nearest) {
-                const uint32_t sl = (tslot[sd][r][q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
-                if (sl != NOSLOT && CHK(S, sl, TABLE)) sm.tsb[sl] = sb_s;
-              } else if (texel == (int)tslot[sd][r][1] && (tslot[sd][r][0] & 0xFFFFu) != NOSLOT) {
-                sm.tsb[tslot[sd][r][0] & 0xFFFFu] = sb_s;
-              }
-              const uint32_t sb = sd == 1 ? ~sb_s : sb_s;  // side -: theta - s eps
-              const float* src = T.ptr + (long long)texel * T.c;
-#pragma unroll
-              for (int c = 0; c < 4; ++c)
-                if (c < T.c) tex[r][c] += wq[q] * __fadd_rn(__ldg(src + c), ((sb >> c) & 1) ? -T.eps : T.eps);
-            }
-            if (T.c == 1) tex[r][1] = tex[r][2] = tex[r][0];
-          }
-          if (GR) {
-            // the group entry of each corner carries every read texture's signs
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              uint32_t sl;
-              if (!S.foot_nearest) sl = (tslot[sd][0][q >> 1] >> (16 * (q & 1))) & 0xFFFFu;
-              else sl = texel_of(tpk[sd][0], q, S.rtex[0].w) == (int)tslot[sd][0][1] ? (tslot[sd][0][0] & 0xFFFFu)
-                                                                                     : NOSLOT;
-              if (sl != NOSLOT && CHK(S, sl, TABLE)) sm.tsb[sl] = gsb[q];
-            }
-          }
-          if (SH == SHADE_UNLIT) {
-            col[sd] = f3(tex[0][0], tex[0][1], tex[0][2]);
-          } else {
-            const int j = bj[sd];
-            const uint32_t sg = sm.sgn9[par][j] ^ (sd == 1 ? 0x1FFu : 0u);
-            float3 p[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              const float* src = S.pos + 3ll * sm.vid[j][k];
-              float q[3];
-#pragma unroll
-              for (int c = 0; c < 3; ++c)
-                q[c] = __fadd_rn(__ldg(src + c), ((sg >> (3 * k + c)) & 1) ? -S.eps_pos : S.eps_pos);
-              p[k] = f3(q[0], q[1], q[2]);
-            }
-            const float2 uvv[3] = {make_float2(sm.uv[j][0], sm.uv[j][1]), make_float2(sm.uv[j][2], sm.uv[j][3]),
-                                   make_float2(sm.uv[j][4], sm.uv[j][5])};
-            float alb[4] = {1.f, 1.f, 1.f, 1.f}, nm[4] = {0.5f, 0.5f, 1.f, 0.f}, rough[4] = {0.5f, 0.f, 0.f, 0.f},
-                  metal[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int r = 0; r < NREAD; ++r) {
-              const int role = S.rtex[r].role;
-              float* dst = role == ROLE_ALBEDO ? alb : role == ROLE_NORMAL ? nm : role == ROLE_ROUGHNESS ? rough : metal;
-#pragma unroll
-              for (int c = 0; c < 4; ++c) dst[c] = tex[r][c];
-            }
-            const float bz[3] = {SH == SHADE_GGX ? bary[sd][0] : 0.f, SH == SHADE_GGX ? bary[sd][1] : 0.f,
-                                 SH == SHADE_GGX ? bary[sd][2] : 0.f};
-            col[sd] = shade(S, view, alb, nm, rough, metal, p, uvv, bz);
-          }
-        }
-      }
-      float df = 0.0f;
-      if (valid) {
-        float fp, fm;
-        df = loss_diff(col[0], col[1], tgt, fp, fm);  // 0 where both sides show the background
-        loss_acc += 0.5f * (fp + fm);
-      }
-      if (valid && a.delta_f) a.delta_f[(((long long)slot * a.pairs + pair) * S.H + py) * S.W + px] = df;
-      // vertices: the visible triangle of side + (else side -), summed over each run of lanes that
-      // share it, one shared atomic per run
-      {
-        const int kt = !valid ? -1 : (bj[0] >= 0 ? bj[0] : bj[1]);
-        float v = df;
-        int n;
-        if (run_sum(kt, v, n) && kt >= 0) {
-          atomicAdd(&sm.A_tri[kt], v);
-          atomicAdd(&sm.n_tri[kt], (uint32_t)n);
-        }
-      }
-      if (valid && bj[0] >= 0 && bj[1] >= 0 && bj[1] != bj[0]) {
-        // side -'s corners that side +'s triangle does not share
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int v = sm.vid[bj[1]][k];
-          if (v != sm.vid[bj[0]][0] && v != sm.vid[bj[0]][1] && v != sm.vid[bj[0]][2]) {
-            atomicAdd(&sm.A_cor[bj[1]][k], df);
-            atomicAdd(&sm.n_cor[bj[1]][k], 1u);
-          }
-        }
-      }
-      // texels: union of both sides' footprints of every read texture (of the group)
-      if (valid) {
-        // credit texel id (table slot sl, or NOSLOT: straight to the global sums)
-        auto credit_texel = [&](int r, int id, uint32_t sl) {
-          if (sl != NOSLOT) {
-            if (!CHK(S, sl, TABLE)) return;
-            atomicAdd(&sm.tA[sl], df);
-            atomicAdd(&sm.tcnt[sl], 1u);
-            return;
-          }
-#pragma unroll
-          for (int g = 0; g < (GR ? NREAD : 1); ++g) {
-            const TexDev& U = S.rtex[GR ? g : r];
-            const uint32_t sb = plane_nibble(S, planes, ws.sgn_off[U.index], id);
-            const long long base = U.offset + (long long)id * U.c;
-            for (int c = 0; c < U.c; ++c) {
-              if (!CHK(S, base + c, S.chk.params)) continue;
-              atomicAdd(a.grad + base + c, ((sb >> c) & 1) ? -df : df);
-              atomicAdd(a.counts + base + c, 1u);
-            }
-          }
-        };
-#pragma unroll
-        for (int r = 0; r < NFOOT; ++r) {
-          const TexDev& T = S.rtex[r];
-          if (S.foot_nearest) {
-#pragma unroll
-            for (int sd = 0; sd < 2; ++sd) {
-              if (bj[sd] < 0) continue;
-              const int id = (int)tslot[sd][r][1];
-              if (sd == 1 && bj[0] >= 0 && (int)tslot[0][r][1] == id) continue;
-              credit_texel(r, id, tslot[sd][r][0] & 0xFFFFu);
-            }
-            continue;
-          }
-          int id0[4] = {-1, -1, -1, -1};
-          if (bj[0] >= 0) {
-#pragma unroll
-            for (int q = 0; q < 4; ++q) id0[q] = texel_of(tpk[0][r], q, T.w);
-          }
-          const bool same = bj[0] >= 0 && bj[1] >= 0 && tpk[0][r] == tpk[1][r];
-#pragma unroll
-          for (int sd = 0; sd < 2; ++sd) {
-            if (bj[sd] < 0 || (sd == 1 && same)) continue;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const int id = sd == 0 ? id0[q] : texel_of(tpk[1][r], q, T.w);
-              // the footprint's own repeats: its second row when the rows are clamped to one, its
-              // second column in a one-texel-wide texture (texel_of gives every other corner a
-              // different texel)
-              bool dup = ((q & 2) && (tpk[sd][r] >> 31)) || ((q & 1) && T.w == 1);
-              if (sd == 1) {
-#pragma unroll
-                for (int o = 0; o < 4; ++o) dup = dup || id0[o] == id;
-              }
-              if (dup) continue;
-              credit_texel(r, id, (tslot[sd][r][q >> 1] >> (16 * (q & 1))) & 0xFFFFu);
-            }
-          }
-        }
-      }
-    }
-    __syncthreads();
-    fold<TABLE, TSC, GR, NREAD>(S, sm, nb, (p1 - 1) & 1);
-    __syncthreads();
-    // ---- flush: one global atomic per credited vertex corner / texel and channel
-    const uint32_t n_used = sm.n_used;
-    for (uint32_t i = tid; i < n_used; i += blockDim.x) {
-      const uint32_t s = sm.used[i];
-      const uint32_t key = sm.tkey[s];
-      if (sm.tcnt[s] == 0) continue;
-      if (!GR) {
-        const TexDev& T = S.tex[(key >> 28) - 1];
-        const long long base = T.offset + (long long)(key & 0x0FFFFFFFu) * T.c;
-        for (int c = 0; c < T.c; ++c) {
-          if (!CHK(S, base + c, S.chk.params)) continue;
-          atomicAdd(a.grad + base + c, sm.tS[c][s]);
-          atomicAdd(a.counts + base + c, sm.tcnt[s]);
-        }
-      } else {
-        // a group entry: the texel of every read texture, channel c of texture r at 4 r + c
-#pragma unroll
-        for (int r = 0; r < NREAD; ++r) {
-          const TexDev& T = S.rtex[r];
-          const long long base = T.offset + (long long)(key & 0x0FFFFFFFu) * T.c;
-          for (int c = 0; c < T.c; ++c) {
-            if (!CHK(S, base + c, S.chk.params)) continue;
-            atomicAdd(a.grad + base + c, sm.tS[(4 * r + c) % TSC][s]);
-            atomicAdd(a.counts + base + c, sm.tcnt[s]);
-          }
-        }
-      }
-    }
-    if (tid < nb) {
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        const uint32_t cn = sm.c_cor[tid][k];
-        if (!cn) continue;
-        const long long base = 3ll * sm.vid[tid][k];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-          if (!CHK(S, base + c, S.chk.params)) continue;
-          atomicAdd(a.grad + base + c, sm.S_cor[tid][k][c]);
-          atomicAdd(a.counts + base + c, cn);
-        }
-      }
-    }
-    __syncthreads();
-    clear_used(sm, n_used);  // n_used as read before the flush: thread 0 resets the shared count
-    if (tid == 0) sm.n_used = 0;
-    if (a.loss) {
-      float v = loss_acc;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if ((tid & 31) == 0) sm.red[tid >> 5] = v;
-      __syncthreads();
-      if (tid == 0) {
-        float sum = 0.0f;
-        for (int i = 0; i < TILE_PX / 32; ++i) sum += sm.red[i];
-        atomicAdd(a.loss + slot, sum / (float)a.pairs);
+      for (int c = 0; c < 3; ++c) {
+        if (!CHK(S, p + c, S.chk.params)) continue;
+        atomicAdd(a.grad + p + c, acc[3 * k + c]);
+        atomicAdd(a.counts + p + c, cnt[k]);
       }
     }
   }
 }
 
+// The sums of G pairs back to zero (after every thread has folded).
 template <int SH, bool GR>
-__global__ void __launch_bounds__(TILE_PX, SH == SHADE_UNLIT ? 2 : 1)
+__device__ __forceinline__ void clear_sums(FastSmem<SH, GR>& sm, int G, int nh) {
+  using M = Model<SH, GR>;
+  const int n = G * (2 * sm.wbase[M::NFOOT] + nh);
+  for (int i = threadIdx.x; i < n; i += M::THREADS) sm.tA[i] = 0.0f;
+}
+
+// The item's texel counts into the global counts (its counters are cleared after a barrier).
+template <int SH, bool GR>
+__device__ __forceinline__ void flush_counts(const SceneDev& S, const EstimateArgs& a, FastSmem<SH, GR>& sm, int nh) {
+  using M = Model<SH, GR>;
+  for (int r = 0; r < M::NFOOT; ++r) {
+    const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
+    const int4 win = sm.win[r];
+    for (int t = threadIdx.x; t < n; t += M::THREADS) {
+      const uint32_t* cnt = sm.tcnt + base + t;
+      uint32_t c = (cnt[0] >> 16) + (cnt[0] & 0xFFFFu);
+      if (t > 0) c += cnt[-1] & 0xFFFFu;
+      if (t >= win.z) c += cnt[-win.z] & 0xFFFFu;
+      if (t > win.z) c += cnt[-win.z - 1] & 0xFFFFu;
+      if (c == 0u) continue;
+      const int texel = window_texel(win, t, S.rtex[r].w);
+#pragma unroll
+      for (int q = 0; q < (GR ? M::NREAD : 1); ++q) {
+        const TexDev& T = S.rtex[GR ? q : r];
+        const long long p = T.offset + (long long)texel * T.c;
+        for (int k = 0; k < T.c; ++k)
+          if (CHK(S, p + k, S.chk.params)) atomicAdd(a.counts + p + k, c);
+      }
+    }
+  }
+  for (int h = threadIdx.x; h < nh; h += M::THREADS) {
+    const uint32_t code = sm.hkey[h], c = sm.hcnt[h];
+    if (code == EMPTY) continue;
+    sm.hkey[h] = EMPTY;
+    sm.hcnt[h] = 0u;
+    const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
+    const int tw = S.rtex[r].w;
+    const Quad Q(code, tw);
+#pragma unroll 1
+    for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q) {
+      if (Q.repeats(q)) continue;
+      const int texel = Q.texel(q, tw);
+#pragma unroll 1
+      for (int k = 0; k < (GR ? M::NREAD : 1); ++k) {
+        const TexDev& T = S.rtex[GR ? k : r];
+        const long long p = T.offset + (long long)texel * T.c;
+        for (int i = 0; i < T.c; ++i)
+          if (CHK(S, p + i, S.chk.params)) atomicAdd(a.counts + p + i, c);
+      }
+    }
+  }
+}
+
+// The windows' sign bits of the group's G pairs (planes: the first one's).
+template <int SH, bool GR>
+__device__ __forceinline__ void load_signs(const SceneDev& S, const Workspace& ws, FastSmem<SH, GR>& sm,
+                                           const uint32_t* planes, int G) {
+  using M = Model<SH, GR>;
+  constexpr int NG = GR ? M::NREAD : 1;
+  for (int r = 0; r < M::NFOOT; ++r) {
+    const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
+    const int4 win = sm.win[r];
+    for (int t = threadIdx.x; t < n; t += M::THREADS) {
+      const int texel = window_texel(win, t, S.rtex[r].w), sh = 4 * (texel & 7);
+      uint32_t word[M::NW];
+#pragma unroll
+      for (int w = 0; w < M::NW; ++w) word[w] = 0u;
+#pragma unroll
+      for (int q = 0; q < NG; ++q) {
+        const TexDev& T = S.rtex[GR ? q : r];
+        const long long wi = (long long)ws.sgn_off[T.index] + (texel >> 3);
+        if (!CHK(S, wi, S.chk.sign_words)) continue;
+        const uint32_t* p = planes + wi;
+#pragma unroll
+        for (int g = 0; g < GMAX; ++g) {
+          uint32_t nib = 0;
+          if (g < G) nib = (__ldg(p) >> sh) & 0xFu;
+          if (T.c == 1) nib *= 7u;  // the shading reads the one channel as all three
+          word[g / M::GPW] |= nib << (M::SPP * (g % M::GPW) + 4 * q);
+          p += ws.sgn_words;
+        }
+      }
+      if constexpr (M::SIGNS_APART) {
+#pragma unroll
+        for (int w = 0; w < M::NW; ++w) sm.ts[w][base + t] = word[w];
+      } else if constexpr (!GR) {
+        sm.th[0][base + t].w = __uint_as_float(word[0]);
+      } else {
+        sm.th[1][base + t].z = __uint_as_float(word[0]);
+        sm.th[1][base + t].w = __uint_as_float(word[1]);
+      }
+    }
+  }
+}
+
+// The windows of an item from the bounds (columns, rows) of its first pair's footprints in
+// sm.win = (min column, min row, max column, max row): two texels of margin (a perturbation moves a
+// footprint by a fraction of a texel), cut around the middle where it does not fit.  One thread.
+template <int SH, bool GR>
+__device__ __forceinline__ void make_windows(const SceneDev& S, FastSmem<SH, GR>& sm) {
+  using M = Model<SH, GR>;
+  int base = 0;
+  for (int r = 0; r < M::NFOOT; ++r) {
+    const TexDev& T = S.rtex[r];
+    constexpr int cap = M::WCAP / M::NFOOT;
+    const int4 b = sm.win[r];  // (min > max where no pixel has a footprint)
+    int x0 = b.x - 2, y0 = max(b.y - 2, 0);
+    // no texel twice (at most the texture's width): one slot per texel
+    int w = b.z < b.x ? 0 : min(min(b.z - b.x, 1 << 28) + 6, T.w), h = b.z < b.x ? 0 : min(b.w + 3, T.h - 1) - y0 + 1;
+    if (w >= 2 && h >= 2 && (long long)w * h > cap) {
+      if (w >= h) {
+        const int keep = cap / h;
+        x0 += (w - keep) / 2;
+        w = keep;
+      } else {
+        const int keep = cap / w;
+        y0 += (h - keep) / 2;
+        h = keep;
+      }
+    }
+    if (w < 2 || h < 2) w = h = 0;
+    sm.win[r] = make_int4(x0, y0, w, h);
+    sm.wbase[r] = base;
+    base += w * h;
+  }
+  sm.wbase[M::NFOOT] = base;
+}
+
+// Pairs per item: `lo` doubled up to `hi` while every CTA still gets at least 16 items (a longer run
+// amortises the item's staging and texel windows, a shorter one balances the CTAs).
+__device__ __forceinline__ int run_of(const EstimateArgs& a, int n_items, int lo, int hi) {
+  int run = lo;
+  while (2 * run <= hi && (long long)n_items * (a.pair_count / (2 * run)) >= 16ll * gridDim.x) run *= 2;
+  return run;
+}
+
+// Every light work item of one scene's call, taken one at a time from the scene's work
+// counter until none is left.  own_first: a CTA's first item is its own index, without a round trip to
+// the counter (a launch's first asset, which every CTA starts at the same time).
+template <int SH, bool GR>
+__device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
+                                           const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
+  using M = Model<SH, GR>;
+  constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT, NG = GR ? NREAD : 1;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  // a warp's pixels: an 8 x 4 block, odd rows right to left, so that runs of lanes follow the surface
+  const int lx = (lane & 8) ? 7 - (lane & 7) : (lane & 7), ly = lane >> 3;
+  const int ntl = n_tiles(S);
+  // Tiles with more than kBigBin live triangles go first and, unless there are many, in runs a quarter as
+  // long: an item of such a tile costs up to ten times the average one, and as the last one taken it
+  // would leave the other CTAs idle (4 views x 16 pairs at 501 x 397: CTAs busy 0.55 of 1.06 ms without
+  // this, the kernel 0.63 ms with it; 8 views x 64 pairs at 512^2: 7.2 -> 5.9 ms with the longer runs).
+  const int n_small = (int)ws.counters[0], n_big = (int)ws.counters[6];
+  const int ppi = a.pairs_per_item > 0 ? a.pairs_per_item : kRun;
+  const int run = a.pairs_per_item > 0 ? ppi : run_of(a, n_small, ppi, 4 * kRun), run_big = run_of(a, n_big, max(1, ppi / 4), ppi);
+  const int chunks = (a.pair_count + run - 1) / run, chunks_big = (a.pair_count + run_big - 1) / run_big;
+  const long long work_big = (long long)n_big * chunks_big, n_work = work_big + (long long)n_small * chunks;
+  for (int s = tid; s < M::ACAP; s += M::THREADS) sm.tA[s] = 0.0f;
+  for (int s = tid; s < M::WCAP; s += M::THREADS) sm.tcnt[s] = 0u;
+  for (int s = tid; s < kHashNoWindow; s += M::THREADS) sm.hkey[s] = EMPTY, sm.hcnt[s] = 0u;
+  for (int s = tid; s < M::SLOTS; s += M::THREADS) {
+    sm.A_tri[s] = sm.A_cor[s][0] = sm.A_cor[s][1] = sm.A_cor[s][2] = 0.0f;
+    sm.n_tri[s] = sm.n_cor[s] = 0u;
+  }
+  if (tid == 0) sm.nact = 0u;
+  if (tid < NFOOT) sm.win[tid] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
+  if (tid <= NFOOT) sm.wbase[tid] = 0;
+  const uint32_t first_of = own_first ? gridDim.x : 0u;
+  if (tid == 0) sm.item = own_first ? blockIdx.x : atomicAdd(ws.counters + 1, 1u);
+  __syncthreads();
+
+  for (long long w = sm.item; w < n_work; w = sm.item) {
+    const bool big = w < work_big;
+    const int nch = big ? chunks_big : chunks, at = (int)((big ? w : w - work_big) / nch);
+    const int chunk = (int)((big ? w : w - work_big) - (long long)at * nch), len = big ? run_big : run;
+    const uint32_t it = big ? ws.tile_cur[at] : ws.items[at];
+    const int slot = it >> 24, tile = it & 0xFFFFFF;
+    uint32_t next = 0;
+    if (tid == 0) next = first_of + atomicAdd(ws.counters + 1, 1u);  // (in flight while this item is staged)
+    if (!CHK(S, slot, vl.n) || !CHK(S, tile, ntl)) {  // (checked build; uniform over the CTA)
+      __syncthreads();
+      if (tid == 0) sm.item = next;
+      __syncthreads();
+      continue;
+    }
+    const int view = vl.id[slot];
+    const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
+    const int rx = 256 * (tx * TILE) + 128, ry = 256 * (ty * TILE) + 128;
+    const uint32_t bin_beg = ws.tile_off[slot * ntl + tile];
+    const int nb = (int)ws.tile_live[slot * ntl + tile];
+    const int p0 = a.pair_begin + chunk * len;
+    const int p1 = min(a.pair_begin + a.pair_count, p0 + len);
+    float loss_acc = 0.0f;
+
+    // ---- per item: the bin's live triangles (pruned and compacted by k_bin_prune) and their smallest
+    //      depths; the pixels' targets and candidates (in order of that depth), block by block
+    for (int j = tid; j < nb; j += M::THREADS) {
+      const int tri = (int)bin_at(S, ws, bin_beg + j);
+      sm.btri[j] = tri;
+      sm.zminb[j] = ordered_bits(ws.tri_z[(long long)slot * S.nt + tri].x);
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        sm.vid[j][k] = vert_of(S, tri, k);
+        const int ti = uv_of(S, tri, k);
+        sm.uv[j][2 * k] = __ldg(S.uvs + 2 * ti);
+        sm.uv[j][2 * k + 1] = __ldg(S.uvs + 2 * ti + 1);
+      }
+    }
+    for (int b = warp; b < TILE_PX / 32; b += M::WARPS) {
+      const int dx = (b & 1) * 8 + lx, dy = (b >> 1) * 4 + ly, px = tx * TILE + dx, py = ty * TILE + dy;
+      const bool valid = px < S.W && py < S.H;
+      const long long tix = (long long)slot * ntl + tile;
+      const int n = valid ? ws.ncand[tix * TILE_PX + dy * TILE + dx] : 0;
+      float3 t = f3(0.f, 0.f, 0.f);
+      if (valid) {
+        const float* tp = S.targets + (((long long)view * S.H + py) * S.W + px) * 3;
+        t = f3(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
+      }
+      if (__any_sync(0xffffffffu, n > 0)) {
+        sm.cand[b * 32 + lane] = ws.cand[tix * kCandWords * TILE_PX + dy * TILE + dx];
+        sm.ncand[b * 32 + lane] = (uint8_t)n;
+        sm.tgt[0][b * 32 + lane] = t.x;
+        sm.tgt[1][b * 32 + lane] = t.y;
+        sm.tgt[2][b * 32 + lane] = t.z;
+        if (lane == 0) sm.act[atomicAdd(&sm.nact, 1u)] = (uint32_t)b;
+      } else if (valid) {
+        // a block no triangle can reach: the background on both sides of every pair
+        const float3 bg = f3(S.bg[0], S.bg[1], S.bg[2]);
+        float fp, fm;
+        loss_diff(bg, bg, t, fp, fm);
+        loss_acc += 0.5f * (fp + fm) * (float)(p1 - p0);
+      }
+    }
+    __syncthreads();
+    const int nact = (int)sm.nact;
+    // pairs of a group: as many as the set-ups, the sign words and (below) the sums hold
+    int Gcap = min(GMAX, M::SLOTS / max(nb, 1)), par = 0, G = 0, nh = 0;
+    bool first = true;
+    const uint32_t* planes0 =
+        ws.tsign + ((long long)slot * ws.max_pairs + (p0 - a.pair_begin)) * ws.sgn_words;  // the item's first pair's
+
+    for (int pg = p0; pg < p1 && nact > 0; pg += G) {
+      const uint32_t* planes = planes0 + (long long)(pg - p0) * ws.sgn_words;
+      // ---- F: fold the previous group's sums with its signs
+      if (!first) {
+        fold<SH, GR>(S, ws, a, sm, nb, G, par ^ 1, nh, planes - (long long)G * ws.sgn_words);
+        __syncthreads();
+        clear_sums(sm, G, nh);
+      }
+      G = min(Gcap, p1 - pg);
+      // ---- S: this group's triangles set up on both sides from the projected perturbed vertices
+      for (int t2 = tid; t2 < 2 * G * nb; t2 += M::THREADS) {
+        const int sd = t2 & 1, s = t2 >> 1, g = s / nb, j = s - g * nb;
+        const long long vb = ((long long)slot * ws.max_pairs + (pg - a.pair_begin) + g) * S.nv;
+        PVert v[3];
+        uint32_t sg = 0;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+          const long long o = vb + sm.vid[j][k];
+          const int4 q = __ldg(ws.pverts + 2 * o + sd);
+          v[k].X = q.x;
+          v[k].Y = q.y;
+          v[k].z = __int_as_float(q.z);
+          v[k].iw = __int_as_float(q.w);
+          v[k].ok = q.x != kNotDrawn;
+          if (M::LIT || sd == 0) sg |= ((uint32_t)__ldg(ws.vbits + o) & 7u) << (3 * k);
+        }
+        if (sd == 0) sm.sgn9[par][s] = sg;
+        set_up_side(sm.side[sd][s], v, rx, ry);
+        if (M::LIT) {
+          float3 p[3];
+          corner_positions(S, sm.vid[j], sd ? sg ^ 0x1FFu : sg, p);
+          tri_frame(p, sm.uv[j], sm.frame[sd][s]);
+        }
+      }
+      if (!first) load_signs<SH, GR>(S, ws, sm, planes, G);
+      if (tid == 0) sm.unit = 0u;
+      __syncthreads();
+
+      // ---- the group's units, a block of 32 pixels of one pair each, taken by the warps as they come
+      //      free; in the item's first group side + of the first pair comes first, up to its
+      //      footprints, whose bounds give the item's texel windows
+      bool bounds = first;
+      int g = 0, i = 0, u = 0;  // the warp's unit u = g nact + i: pair g of the group, block act[i]
+      for (;;) {
+        if (!bounds) {
+          int next = 0;
+          if (lane == 0) next = (int)atomicAdd(&sm.unit, 1u);
+          next = __shfl_sync(0xffffffffu, next, 0);
+          i += next - u;
+          u = next;
+          for (; i >= nact; i -= nact) ++g;
+          if (g >= G) break;
+        } else {
+          i = warp < nact ? warp : 0;
+        }
+        const int n_win = sm.wbase[NFOOT], stride = 2 * n_win + nh;
+        const int blk = (int)sm.act[i];
+        const int dx = (blk & 1) * 8 + lx, dy = (blk >> 1) * 4 + ly, X = dx * 256, Y = dy * 256;
+        const int px = tx * TILE + dx, py = ty * TILE + dy;
+        const bool valid = px < S.W && py < S.H;
+        const int4* cands = ws.cand + ((long long)slot * ntl + tile) * kCandWords * TILE_PX + dy * TILE + dx;
+        int ncand = sm.ncand[blk * 32 + lane];
+        if (bounds && (warp >= nact || ncand > CMAX)) ncand = 0;
+        const int sbase = g * nb;
+        int jA, jB = -1;                    // visible triangles: side +, side - (after the loop)
+        float3 cA, cB = f3(0.f, 0.f, 0.f);  // colours
+        uint32_t crA[NFOOT], crB[NFOOT];    // credit codes
+#pragma unroll
+        for (int r = 0; r < NFOOT; ++r) crB[r] = 0;
+        // one copy of the code serves both sides (the second pass moves the first's results on)
+#pragma unroll 1
+        for (int sd = 0; sd < 2; ++sd) {
+          jA = jB;
+          cA = cB;
+#pragma unroll
+          for (int r = 0; r < NFOOT; ++r) crA[r] = crB[r];
+          jB = -1;
+          cB = f3(S.bg[0], S.bg[1], S.bg[2]);
+          // -- R: the visible triangle among the candidates, nearest first (one wholly behind the
+          //    best so far ends the search)
+          uint32_t bz = 0xFFFFFFFFu;
+          float l[3] = {0.f, 0.f, 0.f};
+          const SideTri* sides = sm.side[sd] + sbase;
+          auto test = [&](int j) {
+            float q[3];
+            float4 z;
+            if (!cover_lambdas(sides[j], X, Y, q, z)) return;
+            const float zz[3] = {z.x, z.y, z.z};
+            const uint32_t zb = ordered_bits(interp_depth(q, zz));
+            if (zb < bz || (zb == bz && (jB < 0 || sm.btri[j] < sm.btri[jB]))) {
+              bz = zb;
+              jB = j;
+              l[0] = q[0], l[1] = q[1], l[2] = q[2];
+            }
+          };
+          if (ncand > CMAX) {
+            for (int j = 0; j < nb; ++j) test(j);
+          } else {
+            int4 list = sm.cand[blk * 32 + lane];
+            for (int q = 0; q < ncand; ++q) {
+              const int j = list.x & 0xFF;
+              list.x = (int)((uint32_t)list.x >> 8);
+              if ((q & 3) == 3) {
+                if (q == 15) list = __ldg(cands + TILE_PX);  // the list's second half (few pixels have one)
+                else list.x = list.y, list.y = list.z, list.z = list.w;
+              }
+              if (!CHK(S, j, nb)) continue;
+              if (sm.zminb[j] > bz) break;
+              test(j);
+            }
+          }
+          // -- U: the UV buffer value and footprints
+          float u0 = 0.f, v0 = 0.f;
+          PerspW pw;
+          if (jB >= 0) {
+            const float4 iw4 = sides[jB].iw;
+            const float iw[3] = {iw4.x, iw4.y, iw4.z};
+            pw = persp(l, iw);
+            const float* uvt = sm.uv[jB];
+            u0 = persp_interp(pw, uvt[0], uvt[2], uvt[4]);
+            v0 = persp_interp(pw, uvt[1], uvt[3], uvt[5]);
+          }
+          if (bounds) {
+#pragma unroll
+            for (int r = 0; r < NFOOT; ++r) {
+              const Foot f = footprint(u0, v0, S.rtex[r].w, S.rtex[r].h);
+              const bool in = jB >= 0 && abs(f.ix) < (1 << 28);
+              const int x0 = __reduce_min_sync(0xffffffffu, in ? f.ix : 0x3FFFFFFF);
+              const int x1 = __reduce_max_sync(0xffffffffu, in ? f.ix : -0x3FFFFFFF);
+              const int y0 = __reduce_min_sync(0xffffffffu, in ? f.y0 : 0x3FFFFFFF);
+              const int y1 = __reduce_max_sync(0xffffffffu, in ? f.y0 : -0x3FFFFFFF);
+              if (lane == 0 && x0 <= x1) {
+                atomicMin(&sm.win[r].x, x0);
+                atomicMin(&sm.win[r].y, y0);
+                atomicMax(&sm.win[r].z, x1);
+                atomicMax(&sm.win[r].w, y1);
+              }
+            }
+            break;
+          }
+          if (jB < 0) continue;
+          // -- G: sample the perturbed texels (values and signs from the window, else from memory)
+          float val[NREAD][3];
+#pragma unroll
+          for (int r = 0; r < NFOOT; ++r) {
+            const TexDev& T = S.rtex[r];
+            const int4 win = sm.win[r];
+            const float x = __fsub_rn(__fmul_rn(u0, (float)T.w), 0.5f), y = __fsub_rn(__fmul_rn(v0, (float)T.h), 0.5f);
+            const float xf = floorf(x), yf = floorf(y);
+            const float fx = __fsub_rn(x, xf), fy = __fsub_rn(y, yf);
+            const float wq[4] = {(1.0f - fx) * (1.0f - fy), fx * (1.0f - fy), (1.0f - fx) * fy, fx * fy};
+            const int wx = (int)xf - win.x, wy = (int)yf - win.y;
+#pragma unroll
+            for (int q = 0; q < NG; ++q) val[GR ? q : r][0] = val[GR ? q : r][1] = val[GR ? q : r][2] = 0.0f;
+            // (a column or row far from the window never passes, wrapped or not; no window: 0 < -1 fails)
+            bool inside = (uint32_t)wx < (uint32_t)max(win.z - 1, 0) && (uint32_t)wy < (uint32_t)max(win.w - 1, 0);
+            int nq = 0;  // nearest footprint: which of the four texels it is
+            if (S.foot_nearest && inside) {
+              const int nx = (int)floorf(__fmul_rn(u0, (float)T.w)) - (int)xf;
+              const int ny = (int)floorf(__fmul_rn(v0, (float)T.h)) - (int)yf;
+              inside = (uint32_t)nx < 2u && (uint32_t)ny < 2u;
+              nq = nx + ny * win.z;
+            }
+            if (inside) {
+              const int s00 = (NFOOT == 1 ? 0 : sm.wbase[r]) + wy * win.z + wx;
+              crB[r] = (uint32_t)(s00 + nq);
+              if (!CHK(S, s00 + win.z + 1, n_win)) continue;
+              const int up = 28 - M::SPP * (g % M::GPW);
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                const int sq = s00 + (q & 1) + (q & 2 ? win.z : 0);
+                const float4 t0 = sm.th[0][sq];
+                if constexpr (!GR) {
+                  const uint32_t sb = __float_as_uint(t0.w);
+                  const float e = sd ? -T.eps : T.eps;
+                  const float tv[3] = {t0.x, t0.y, t0.z};
+#pragma unroll
+                  for (int c = 0; c < (M::LIT && r >= 2 ? 1 : 3); ++c)
+                    val[r][c] += wq[q] * __fadd_rn(tv[c], (c < T.c || T.c == 1) ? signed_eps(sb, up + 3 - c, e) : 0.0f);
+                } else {
+                  const float4 t1 = sm.th[M::NV - 1][sq];
+                  const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+                  uint32_t sb;
+                  if constexpr (M::SIGNS_APART) sb = sm.ts[g / M::GPW][sq];
+                  else sb = __float_as_uint(g < M::GPW ? t1.z : t1.w);
+#pragma unroll
+                  for (int k = 0; k < NREAD; ++k) {
+                    const TexDev& U = S.rtex[k];
+                    const float e = sd ? -U.eps : U.eps;
+#pragma unroll
+                    for (int c = 0; c < used_channels(k); ++c)
+                      val[k][c] += wq[q] * __fadd_rn(tv[(k < 2 ? 3 * k : 4 + k) + c],
+                                                     (c < U.c || U.c == 1) ? signed_eps(sb, up + 3 - c - 4 * k, e) : 0.0f);
+                  }
+                }
+              }
+            } else {
+              const Foot f = footprint(u0, v0, T.w, T.h);
+              const uint32_t cr = kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | (f.y1 == f.y0 ? kOneRow : 0u) |
+                                  (uint32_t)(f.y0 * T.w + f.x0);
+              crB[r] = S.foot_nearest ? kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | kOneRow |
+                                            (uint32_t)nearest_texel(u0, v0, T.w, T.h)
+                                      : cr;
+              int texel[4];
+#pragma unroll
+              for (int q = 0; q < 4; ++q) {
+                texel[q] = (q & 2 ? f.y1 : f.y0) * T.w + (q & 1 ? f.x1 : f.x0);
+                if (!CHK(S, texel[q], (long long)T.w * T.h)) texel[q] = 0;
+              }
+              // (a texture at a time, its four texels' loads in flight together)
+#pragma unroll
+              for (int k = 0; k < NG; ++k) {
+                const TexDev& U = S.rtex[GR ? k : r];
+                uint32_t sb[4];
+                float tv[4][3];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  sb[q] = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], texel[q]);
+                  const float* src = U.ptr + (long long)texel[q] * U.c;
+#pragma unroll
+                  for (int c = 0; c < 3; ++c) tv[q][c] = c < U.c ? __ldg(src + c) : 0.0f;
+                }
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                  if (sd) sb[q] = ~sb[q];
+#pragma unroll
+                  for (int c = 0; c < 3; ++c)
+                    if (c < U.c) val[GR ? k : r][c] += wq[q] * __fadd_rn(tv[q][c], ((sb[q] >> c) & 1) ? -U.eps : U.eps);
+                }
+              }
+#pragma unroll
+              for (int k = 0; k < NG; ++k)
+                if (S.rtex[GR ? k : r].c == 1) val[GR ? k : r][1] = val[GR ? k : r][2] = val[GR ? k : r][0];
+            }
+          }
+          // -- shade
+          if constexpr (!M::LIT) {
+            cB = f3(val[0][0], val[0][1], val[0][2]);
+          } else {
+            const float* fr = sm.frame[sd][sbase + jB];
+            float3 P = f3(0.f, 0.f, 0.f);
+            float rough = 0.5f, metal = 0.0f;
+            if constexpr (SH == SHADE_GGX) {
+              float3 p[3];
+              corner_positions(S, sm.vid[jB], sm.sgn9[par][sbase + jB] ^ (sd ? 0x1FFu : 0u), p);
+              const float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
+              P = f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
+                     b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z);
+              rough = val[2][0];
+              metal = val[3][0];
+            }
+            cB = shade_lit<SH>(S, view, val[0], val[1], rough, metal, f3(fr[0], fr[1], fr[2]), f3(fr[3], fr[4], fr[5]),
+                               P);
+          }
+        }
+        if (bounds) {
+          bounds = false;
+          i = 0;
+          __syncthreads();
+          if (tid == 0) make_windows(S, sm);
+          __syncthreads();
+#pragma unroll 1
+          for (int r = 0; r < NFOOT; ++r) {
+            const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
+            const int4 win = sm.win[r];
+            for (int t = tid; t < n; t += M::THREADS) {
+              const int texel = window_texel(win, t, S.rtex[r].w);
+              float tv[8] = {};
+#pragma unroll
+              for (int k = 0; k < NG; ++k) {
+                const TexDev& T = S.rtex[GR ? k : r];
+                const float* src = T.ptr + (long long)texel * T.c;
+#pragma unroll
+                for (int c = 0; c < (GR ? used_channels(k) : 3); ++c)
+                  if (c < T.c || T.c == 1) tv[(GR ? (k < 2 ? 3 * k : 4 + k) : 0) + c] = __ldg(src + (T.c == 1 ? 0 : c));
+              }
+              sm.th[0][base + t] = make_float4(tv[0], tv[1], tv[2], tv[3]);
+              if constexpr (GR) sm.th[1][base + t] = make_float4(tv[4], tv[5], tv[6], tv[7]);
+            }
+          }
+          const int n = sm.wbase[NFOOT];
+          nh = n > 0 ? kHashWindow : kHashNoWindow;
+          Gcap = min(Gcap, M::ACAP / (2 * n + nh));
+          G = min(G, Gcap);
+          load_signs<SH, GR>(S, ws, sm, planes, G);
+          __syncthreads();
+          continue;
+        }
+
+        // -- f+ - f- and its credits
+        float df = 0.0f;
+        if (valid) {
+          const float3 tgt = f3(sm.tgt[0][blk * 32 + lane], sm.tgt[1][blk * 32 + lane], sm.tgt[2][blk * 32 + lane]);
+          float fp, fm;
+          df = loss_diff(cA, cB, tgt, fp, fm);  // 0 where both sides show the background
+          loss_acc += 0.5f * (fp + fm);
+          if (a.delta_f) a.delta_f[(((long long)slot * a.pairs + pg + g) * S.H + py) * S.W + px] = df;
+        }
+        // vertices: the visible triangle of side + (else side -), summed over each run of lanes that
+        // share it, one shared atomic per run
+        {
+          const int kt = jA >= 0 ? jA : jB;
+          float v = df;
+          int n;
+          if (run_sum(kt, v, n) && kt >= 0) {
+            atomicAdd(&sm.A_tri[sbase + kt], v);
+            atomicAdd(&sm.n_tri[sbase + kt], (uint32_t)n);
+          }
+        }
+        if (jA >= 0 && jB >= 0 && jB != jA) {
+          // side -'s corners that side +'s triangle does not share
+          uint32_t add = 0;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            const int v = sm.vid[jB][k];
+            if (v != sm.vid[jA][0] && v != sm.vid[jA][1] && v != sm.vid[jA][2]) {
+              atomicAdd(&sm.A_cor[sbase + jB][k], df);
+              add |= 1u << (10 * k);
+            }
+          }
+          if (add) atomicAdd(&sm.n_cor[sbase + jB], add);
+        }
+        // texels: union of both sides' footprints of every read texture (of the group)
+        if (jA < 0 && jB < 0) continue;
+        float* sums = sm.tA + g * stride;
+#pragma unroll
+        for (int r = 0; r < NFOOT; ++r) {
+          const TexDev& T = S.rtex[r];
+          const uint32_t A = jA >= 0 ? crA[r] : crB[r], B = jB >= 0 ? crB[r] : crA[r];
+          // one texel by its id, straight to the global sums
+          auto credit_id = [&](int id) {
+#pragma unroll 1
+            for (int k = 0; k < NG; ++k) {
+              const TexDev& U = S.rtex[GR ? k : r];
+              const uint32_t sb = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], id);
+              const long long base = U.offset + (long long)id * U.c;
+              for (int c = 0; c < U.c; ++c) {
+                if (!CHK(S, base + c, S.chk.params)) continue;
+                atomicAdd(a.grad + base + c, ((sb >> c) & 1) ? -df : df);
+                atomicAdd(a.counts + base + c, 1u);
+              }
+            }
+          };
+          // a footprint's texels by one sum in its cell (nearest: the one texel)
+          auto credit_cell = [&](uint32_t c) {
+            if (!(c & kOut)) {
+              if (!CHK(S, c, n_win)) return;
+              atomicAdd(sums + c + (S.foot_nearest ? n_win + nh : 0), df);
+              atomicAdd(sm.tcnt + c, S.foot_nearest ? 1u << 16 : 1u);
+              return;
+            }
+            const int h = hash_slot(sm.hkey, c, nh);
+            if (h >= 0) {
+              atomicAdd(sums + n_win + h, df);
+              atomicAdd(sm.hcnt + h, 1u);
+              return;
+            }
+            const Quad Q(c, T.w);
+#pragma unroll 1
+            for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q)
+              if (!Q.repeats(q)) credit_id(Q.texel(q, T.w));
+          };
+          credit_cell(A);
+          if (B == A) continue;
+          if (S.foot_nearest) {
+            // one texel each: a window slot and an outside id may be the same texel
+            bool dup = false;
+            if ((A ^ B) & kOut) {
+              const uint32_t in = (A & kOut) ? B : A, out = (A & kOut) ? A : B;
+              dup = window_texel(sm.win[r], (int)in - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w) == (int)(out & 0x0FFFFFFFu);
+            }
+            if (!dup) credit_cell(B);
+            continue;
+          }
+          if (!((A | B) & kOut)) {
+            // side -'s texels outside side +'s footprint
+            const uint32_t ww = (uint32_t)sm.win[r].z;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t s = B + (q & 1) + (q & 2 ? ww : 0u), d = s - A;
+              if (d <= 1u || d - ww <= 1u || !CHK(S, s, n_win)) continue;
+              atomicAdd(sums + n_win + nh + s, df);
+              atomicAdd(sm.tcnt + s, 1u << 16);
+            }
+            continue;
+          }
+          // some side outside the window: by texel id
+          auto as_id = [&](uint32_t c) {
+            if (c & kOut) return c;
+            return kOut | (uint32_t)window_texel(sm.win[r], (int)c - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w);
+          };
+          const Quad QA(as_id(A), T.w), QB(as_id(B), T.w);
+          uint32_t mine = 0, all = 0;  // side -'s texels (its footprint's own repeats left out), those not in side +'s
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (QB.repeats(q)) continue;
+            all |= 1u << q;
+            if (!QA.holds(QB, q)) mine |= 1u << q;
+          }
+          if (mine == all) {
+            credit_cell(B);
+          } else {
+#pragma unroll 1
+            for (; mine; mine &= mine - 1) credit_id(QB.texel(__ffs((int)mine) - 1, T.w));
+          }
+        }
+      }
+      __syncthreads();
+      first = false;
+      par ^= 1;
+    }
+    // ---- the last group's fold, the texel counts, the item's loss; then everything back to empty
+    if (nact > 0) {
+      fold<SH, GR>(S, ws, a, sm, nb, G, par ^ 1, nh, planes0 + (long long)((p1 - G) - p0) * ws.sgn_words);
+      __syncthreads();
+      flush_counts<SH, GR>(S, a, sm, nh);
+      clear_sums(sm, G, nh);
+    }
+    if (a.loss) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
+      if (lane == 0) sm.red[warp] = loss_acc;
+    }
+    __syncthreads();
+    for (int s = tid; s < sm.wbase[NFOOT]; s += M::THREADS) sm.tcnt[s] = 0u;
+    if (tid == 0) {
+      if (a.loss) {
+        float sum = 0.0f;
+        for (int i = 0; i < M::WARPS; ++i) sum += sm.red[i];
+        atomicAdd(a.loss + slot, sum / (float)a.pairs);
+      }
+      sm.item = next;
+      sm.nact = 0u;
+    }
+    __syncthreads();
+    if (tid < NFOOT) sm.win[tid] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
+    if (tid <= NFOOT) sm.wbase[tid] = 0;
+  }
+}
+
+template <int SH, bool GR>
+__global__ void __launch_bounds__(Model<SH, GR>::THREADS, Model<SH, GR>::CTAS)
     k_estimate_fast(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fast_items<SH, GR>(S, ws, vl, a,
-                     *reinterpret_cast<FastSmem<Model<SH, GR>::TABLE, Model<SH, GR>::TSC>*>(smem_raw));
+  fast_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true);
 }
 
 // The batched kernel keeps its asset after FastSmem, 16-byte aligned.  (Batched calls use the
-// per-texture table: their assets need not share texture sizes.)
+// per-texture windows: their assets need not share texture sizes.)
 template <int SH>
 __host__ __device__ constexpr size_t fast_batch_off() {
-  return (sizeof(FastSmem<Model<SH>::TABLE, Model<SH>::TSC>) + 15) & ~(size_t)15;
+  return (sizeof(FastSmem<SH, false>) + 15) & ~(size_t)15;
 }
 
 // Batched form: the assets of P in order, each until its light items run out.
 template <int SH>
-__global__ void __launch_bounds__(TILE_PX, SH == SHADE_UNLIT ? 2 : 1) k_estimate_fast_batch(const BatchArgs P) {
+__global__ void __launch_bounds__(Model<SH>::THREADS, Model<SH>::CTAS) k_estimate_fast_batch(const BatchArgs P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  auto& sm = *reinterpret_cast<FastSmem<Model<SH>::TABLE, Model<SH>::TSC>*>(smem_raw);
+  auto& sm = *reinterpret_cast<FastSmem<SH, false>*>(smem_raw);
   BatchSmem& b = *reinterpret_cast<BatchSmem*>(smem_raw + fast_batch_off<SH>());
   for (int ai = 0; ai < P.n; ++ai) {
     __syncthreads();
     load_asset(P, ai, b);
     __syncthreads();
-    fast_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm);
+    fast_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0);
   }
 }
 
 template <int SH, bool GR>
 size_t fast_smem() {
-  return sizeof(FastSmem<Model<SH, GR>::TABLE, Model<SH, GR>::TSC>);
+  return sizeof(FastSmem<SH, GR>);
 }
 
 template <int SH>
@@ -1166,7 +1485,7 @@ cudaError_t launch_fast_batch_t(const BatchArgs& P, int grid, cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(k_estimate_fast_batch<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)fast_batch_smem<SH>());
   if (e != cudaSuccess) return e;
-  k_estimate_fast_batch<SH><<<grid, TILE_PX, fast_batch_smem<SH>(), st>>>(P);
+  k_estimate_fast_batch<SH><<<grid, Model<SH>::THREADS, fast_batch_smem<SH>(), st>>>(P);
   return cudaGetLastError();
 }
 
@@ -1175,7 +1494,7 @@ int fast_batch_blocks_per_sm_t() {
   int n = 0;
   cudaFuncSetAttribute(k_estimate_fast_batch<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)fast_batch_smem<SH>());
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_estimate_fast_batch<SH>, TILE_PX, fast_batch_smem<SH>());
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_estimate_fast_batch<SH>, Model<SH>::THREADS, fast_batch_smem<SH>());
   return n > 0 ? n : 1;
 }
 
@@ -1185,7 +1504,7 @@ cudaError_t launch_fast_t(const SceneDev& S, const Workspace& ws, const ViewList
   cudaError_t e = cudaFuncSetAttribute(k_estimate_fast<SH, GR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        (int)fast_smem<SH, GR>());
   if (e != cudaSuccess) return e;
-  k_estimate_fast<SH, GR><<<grid, TILE_PX, fast_smem<SH, GR>(), st>>>(S, ws, vl, a);
+  k_estimate_fast<SH, GR><<<grid, Model<SH, GR>::THREADS, fast_smem<SH, GR>(), st>>>(S, ws, vl, a);
   return cudaGetLastError();
 }
 
@@ -1194,7 +1513,7 @@ int fast_blocks_per_sm_t() {
   int n = 0;
   cudaFuncSetAttribute(k_estimate_fast<SH, GR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                        (int)fast_smem<SH, GR>());
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_estimate_fast<SH, GR>, TILE_PX, fast_smem<SH, GR>());
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_estimate_fast<SH, GR>, Model<SH, GR>::THREADS, fast_smem<SH, GR>());
   return n > 0 ? n : 1;
 }
 

@@ -223,13 +223,14 @@ void make_dev(const sge_scene_desc* d, SceneDev& S) {
     if (first_of_role[t.role] < 0) first_of_role[t.role] = k;
   }
   S.n_params = off;
-  for (int k = 0; k < d->n_textures; ++k) {
-    const int role = d->textures[k].role;
-    bool read = first_of_role[role] == k &&
-                (d->shading == SGE_SHADE_GGX || role == SGE_ROLE_ALBEDO ||
-                 (d->shading == SGE_SHADE_LAMBERT && role == SGE_ROLE_NORMAL));
-    S.tex[k].read = read;
-    if (read) S.read_k[S.nread++] = k;
+  // read textures in role order (albedo, normal, roughness, metallic): kernels index them by role
+  for (int role = 0; role < 4; ++role) {
+    const int k = first_of_role[role];
+    const bool read = k >= 0 && (d->shading == SGE_SHADE_GGX || role == SGE_ROLE_ALBEDO ||
+                                 (d->shading == SGE_SHADE_LAMBERT && role == SGE_ROLE_NORMAL));
+    if (!read) continue;
+    S.tex[k].read = 1;
+    S.read_k[S.nread++] = k;
   }
   for (int r = 0; r < S.nread; ++r) S.rtex[r] = S.tex[S.read_k[r]];
   S.grouped = S.nread > 1;
@@ -378,7 +379,7 @@ int sge_create_scene(const sge_scene_desc* desc, const sge_config* cfg, void* wo
   int bps = (s->cfg.blocks_per_sm > 0) ? s->cfg.blocks_per_sm : fast_blocks_per_sm(desc->shading, s->dev.grouped);
   s->grid_fast = sms * bps;
   s->grid_heavy = sms * estimate_blocks_per_sm(desc->shading, s->dev.grouped, group_channels(s->dev));
-  if (s->cfg.pairs_per_item <= 0) s->cfg.pairs_per_item = 8;
+  if (s->cfg.pairs_per_item < 0) s->cfg.pairs_per_item = 0;  // 0: the kernels choose (k_fast.cu, run_of)
   if (s->cfg.pairs_per_item > kMaxPairsPerItem) s->cfg.pairs_per_item = kMaxPairsPerItem;
   *out = s;
   return SGE_OK;
@@ -474,7 +475,9 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
   }
   // pairs run in blocks of at most max_pairs_per_call (the projected-vertex buffer holds one
   // block); the first block's vertex pass and sign planes run on the side stream while the caller's
-  // stream bins and prunes
+  // stream bins and prunes.  The general estimator and the background's loss go to the side stream too,
+  // ahead of the fast estimator: their few long items overlap it instead of following it (while
+  // launches are timed, they follow it on the caller's stream, as the events need).
   EstimateArgs b0 = a;
   b0.pair_count = pairs_per_view < s->ws.max_pairs ? pairs_per_view : s->ws.max_pairs;
   if (e == cudaSuccess) e = cudaEventRecord(s->fork, st);
@@ -483,6 +486,7 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
   if (e == cudaSuccess) e = cudaEventRecord(s->join, s->side);
   if (e == cudaSuccess) e = launch_binning(s->dev, s->ws, vl, st, true);
   if (e == cudaSuccess) e = cudaStreamWaitEvent(st, s->join, 0);
+  const bool timed = s->n_tev > 0;
   for (int p0 = 0; p0 < pairs_per_view && e == cudaSuccess; p0 += s->ws.max_pairs) {
     EstimateArgs b = a;
     b.pair_begin = p0;
@@ -490,8 +494,25 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
     if (p0 > 0) e = rearm_work(s->ws, st);
     if (e == cudaSuccess && p0 > 0) e = launch_vertex_pass(s->dev, s->ws, vl, b, st);
     const cudaEvent_t* ev = nullptr;
-    if (s->n_tev && s->n_timed < sge_scene::kMaxTimed) ev = s->tev + 4 * s->n_timed++;
-    if (e == cudaSuccess) e = launch_estimate(s->dev, s->ws, vl, b, s->grid_fast, s->grid_heavy, st, ev);
+    if (timed && s->n_timed < sge_scene::kMaxTimed) ev = s->tev + 4 * s->n_timed++;
+    cudaStream_t hs = timed ? st : s->side;
+    if (!timed) {
+      if (e == cudaSuccess) e = cudaEventRecord(s->fork, st);
+      if (e == cudaSuccess) e = cudaStreamWaitEvent(hs, s->fork, 0);
+      if (e == cudaSuccess) e = launch_heavy(s->dev, s->ws, vl, b, s->grid_heavy, hs);
+      if (e == cudaSuccess && loss_out && p0 == 0) e = launch_background_loss(s->dev, s->ws, vl, loss_out, hs);
+      if (e == cudaSuccess) e = cudaEventRecord(s->join, hs);
+    }
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[0], st);
+    if (e == cudaSuccess) e = launch_fast(s->dev, s->ws, vl, b, s->grid_fast, st);
+    if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
+    if (timed) {
+      if (e == cudaSuccess) e = launch_heavy(s->dev, s->ws, vl, b, s->grid_heavy, hs);
+      if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], st);
+      if (e == cudaSuccess && loss_out && p0 == 0) e = launch_background_loss(s->dev, s->ws, vl, loss_out, hs);
+    } else if (e == cudaSuccess) {
+      e = cudaStreamWaitEvent(st, s->join, 0);
+    }
   }
   return e == cudaSuccess ? SGE_OK : cuda_fail(e, "sge_estimate_grad");
 }
@@ -704,7 +725,7 @@ int estimate_grad_batch(const sge_batch_entry* entries, int32_t n, uint64_t seed
   if (pairs_per_view < 1) return fail(SGE_ERR_INVALID_ARG, "pairs_per_view must be >= 1");
   sge_batch_tuning tu{};
   if (tuning) tu = *tuning;
-  if (tu.pairs_per_item <= 0) tu.pairs_per_item = 8;
+  if (tu.pairs_per_item < 0) tu.pairs_per_item = 0;  // 0: the kernels choose (k_fast.cu, run_of)
   if (tu.pairs_per_item > kMaxPairsPerItem) tu.pairs_per_item = kMaxPairsPerItem;
   if (tu.light_bin <= 0 || tu.light_bin > kLightBin) tu.light_bin = kLightBin;
   ViewList vls[SGE_MAX_BATCH];
@@ -953,12 +974,12 @@ int sge_kernel_time(sge_scene* s, float* total_ms, float* heavy_ms, int32_t* lau
 int sge_bin_stats(sge_scene* s, sge_stream_t stream, int64_t* light_items, int64_t* heavy_items,
                   int64_t* bin_entries) {
   if (!s || !light_items || !heavy_items || !bin_entries) return fail(SGE_ERR_INVALID_ARG, "NULL argument");
-  uint32_t c[6] = {0, 0, 0, 0, 0, 0};
+  uint32_t c[7] = {};
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(c, s->ws.counters, sizeof(c), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "sge_bin_stats");
-  *light_items = c[0];
+  *light_items = (int64_t)c[0] + c[6];
   *heavy_items = c[4];
   *bin_entries = c[2];
   return SGE_OK;

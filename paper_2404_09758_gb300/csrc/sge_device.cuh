@@ -308,6 +308,35 @@ __device__ __forceinline__ float3 shading_normal(const float3 p[3], const float2
   return norm3(n);
 }
 
+// GGX colour for the shading normal n, light direction L and surface point P.
+__device__ __forceinline__ float3 shade_ggx(const SceneDev& S, int view, float3 n, float3 L, const float* alb,
+                                            float rough, float metal, float3 P) {
+  // Cook-Torrance: GGX distribution, Smith-Schlick geometry (k = alpha/2), Schlick Fresnel.
+  const float ndl = fmaxf(dot3(n, L), 0.0f);
+  const float* cp = S.cam_pos + 3 * view;
+  float3 V = norm3(f3(__ldg(cp) - P.x, __ldg(cp + 1) - P.y, __ldg(cp + 2) - P.z));
+  float3 Hh = norm3(f3(L.x + V.x, L.y + V.y, L.z + V.z));
+  float ndv = fmaxf(dot3(n, V), 1e-4f), ndh = fmaxf(dot3(n, Hh), 0.0f), vdh = fmaxf(dot3(V, Hh), 0.0f);
+  float r = fminf(fmaxf(rough, 0.02f), 1.0f);
+  float a = r * r, a2 = a * a;
+  float dd = ndh * ndh * (a2 - 1.0f) + 1.0f;
+  float D = a2 / (3.14159265358979f * dd * dd);
+  float kk = 0.5f * a;
+  float G = (ndl / (ndl * (1.0f - kk) + kk)) * (ndv / (ndv * (1.0f - kk) + kk));
+  float mt = metal, om = 1.0f - vdh;
+  float om5 = om * om * om * om * om;
+  float out[3];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    float F0 = 0.04f * (1.0f - mt) + alb[c] * mt;
+    float F = F0 + (1.0f - F0) * om5;
+    float diff = (1.0f - F) * (1.0f - mt) * alb[c] * ndl * 0.318309886183791f;
+    float spec = D * G * F / (4.0f * ndv);
+    out[c] = S.light_rgb[c] * (diff + spec) + S.ambient * alb[c];
+  }
+  return f3(out[0], out[1], out[2]);
+}
+
 // Colour of a covered pixel.  p: perturbed world positions of the visible triangle,
 // uvs: its UVs, b: perspective-correct barycentrics, tex samples by role.
 __device__ __forceinline__ float3 shade(const SceneDev& S, int view, const float alb[4],
@@ -321,31 +350,28 @@ __device__ __forceinline__ float3 shade(const SceneDev& S, int view, const float
     return f3(alb[0] * (S.ambient + S.light_rgb[0] * ndl), alb[1] * (S.ambient + S.light_rgb[1] * ndl),
               alb[2] * (S.ambient + S.light_rgb[2] * ndl));
   }
-  // Cook-Torrance: GGX distribution, Smith-Schlick geometry (k = alpha/2), Schlick Fresnel.
-  const float* cp = S.cam_pos + 3 * view;
-  float3 P = f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
-                b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z);
-  float3 V = norm3(f3(__ldg(cp) - P.x, __ldg(cp + 1) - P.y, __ldg(cp + 2) - P.z));
-  float3 Hh = norm3(f3(L.x + V.x, L.y + V.y, L.z + V.z));
-  float ndv = fmaxf(dot3(n, V), 1e-4f), ndh = fmaxf(dot3(n, Hh), 0.0f), vdh = fmaxf(dot3(V, Hh), 0.0f);
-  float r = fminf(fmaxf(rough[0], 0.02f), 1.0f);
-  float a = r * r, a2 = a * a;
-  float dd = ndh * ndh * (a2 - 1.0f) + 1.0f;
-  float D = a2 / (3.14159265358979f * dd * dd);
-  float kk = 0.5f * a;
-  float G = (ndl / (ndl * (1.0f - kk) + kk)) * (ndv / (ndv * (1.0f - kk) + kk));
-  float mt = metal[0], om = 1.0f - vdh;
-  float om5 = om * om * om * om * om;
-  float out[3];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    float F0 = 0.04f * (1.0f - mt) + alb[c] * mt;
-    float F = F0 + (1.0f - F0) * om5;
-    float diff = (1.0f - F) * (1.0f - mt) * alb[c] * ndl * 0.318309886183791f;
-    float spec = D * G * F / (4.0f * ndv);
-    out[c] = S.light_rgb[c] * (diff + spec) + S.ambient * alb[c];
+  return shade_ggx(S, view, n, L, alb, rough[0], metal[0],
+                   f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
+                      b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z));
+}
+
+// shade() of a lit model for a triangle whose frame (face normal N, u tangent T) and surface point P
+// (GGX) are given; the same arithmetic, the frame formed once per triangle instead of per pixel.
+template <int SH>
+__device__ __forceinline__ float3 shade_lit(const SceneDev& S, int view, const float* alb, const float* nm, float rough,
+                                            float metal, float3 N, float3 T, float3 P) {
+  const float3 B = cross3(N, T);
+  const float mx = 2.0f * nm[0] - 1.0f, my = 2.0f * nm[1] - 1.0f, mz = 2.0f * nm[2] - 1.0f;
+  float3 n = f3(T.x * mx + B.x * my + N.x * mz, T.y * mx + B.y * my + N.y * mz, T.z * mx + B.z * my + N.z * mz);
+  if (dot3(n, n) == 0.0f) n = N;
+  n = norm3(n);
+  const float3 L = f3(S.light_dir[0], S.light_dir[1], S.light_dir[2]);
+  if (SH == SHADE_LAMBERT) {
+    const float ndl = fmaxf(dot3(n, L), 0.0f);
+    return f3(alb[0] * (S.ambient + S.light_rgb[0] * ndl), alb[1] * (S.ambient + S.light_rgb[1] * ndl),
+              alb[2] * (S.ambient + S.light_rgb[2] * ndl));
   }
-  return f3(out[0], out[1], out[2]);
+  return shade_ggx(S, view, n, L, alb, rough, metal, P);
 }
 
 // ---------------------------------------------------------------- one visible surface sample

@@ -14,6 +14,8 @@ constexpr int TILE = 16;                 // tile edge in pixels; one CTA thread 
 constexpr int TILE_PX = TILE * TILE;     // 256 threads
 constexpr int kLightBin = 256;           // bins up to this size use the fast path
 constexpr int kMaxPairsPerItem = 64;     // longest run of pairs one work item takes
+constexpr int kRun = 8;                  // its default where the kernels do not choose a longer one
+constexpr int kBigBin = 48;              // light tiles with more live triangles go first, in shorter runs
 constexpr int kHeavyCand = 32;           // candidate triangles kept per pixel of a heavy tile
 constexpr int kCandWords = kHeavyCand / 8;  // int4 words of a pixel's candidate list
 constexpr int kNotDrawn = (int)0x80000000;  // projected X of a vertex its triangles drop
@@ -96,11 +98,12 @@ struct Workspace {
   uint32_t* tile_cur;    // [max_views][n_tiles] fill cursors
   uint32_t* bins;        // [bin_capacity] triangle ids grouped by (view slot, tile)
   uint32_t* items;       // [max_views * n_tiles] (view slot << 24 | tile): light bins first, heavy from the end
+                         // (light ones above kBigBin: listed in tile_cur, whose cursors are spent by then)
   uint32_t* tile_live;   // [max_views][n_tiles] triangles left at the front of each bin by k_bin_prune
   int4* cand;            // [max_views][n_tiles][kCandWords][256] candidate triangles of each pixel: live
                          // indices, 8-bit in the first word of a light tile, 16-bit in all words of a heavy one
   uint8_t* ncand;        // [max_views][n_tiles][256] their number (> 16: test every live triangle)
-  uint32_t* counters;    // [0] light items, [1] their work counter, [2] total bin entries, [3] status,
+  uint32_t* counters;    // [0] light items of at most kBigBin live triangles, [6] of more, [1] their work counter, [2] total bin entries, [3] status,
                          // [4] heavy items, [5] their work counter
   unsigned long long* keys;  // [2][H*W] staged depth|ID buffers (both sides)
   float2* uvbuf;             // [2][H*W] staged UV buffers
@@ -170,7 +173,7 @@ struct EstimateArgs {
   uint64_t seed;
   uint32_t iter;
   int pairs;           // pairs per view of the whole call
-  int pairs_per_item;
+  int pairs_per_item;  // 0: the kernels choose
   int pair_begin;      // the block of pairs this launch covers: [pair_begin, pair_begin + pair_count)
   int pair_count;
   float* grad;
@@ -181,12 +184,10 @@ struct EstimateArgs {
 };
 // Iteration index of an estimate call: the device word when the call reads it at run time.
 __host__ __device__ inline uint32_t iter_of(const EstimateArgs& a) { return a.iter_dev ? *a.iter_dev : a.iter; }
-// Both estimator kernels: the fast path over light bins, the general one over heavy bins.
-// ev_fast (three events, or NULL) are recorded on st right before and after the fast kernel
-// and after the heavy one.
-cudaError_t launch_estimate(const SceneDev& S, const Workspace& ws, const ViewList& vl,
-                            const EstimateArgs& a, int grid_fast, int grid_heavy, cudaStream_t st,
-                            const cudaEvent_t* ev_fast = nullptr);
+// The estimator kernels: the fast path over light bins, the general one over heavy bins (independent
+// of each other: separate work counters, and the sums are atomics).
+cudaError_t launch_heavy(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
+                         cudaStream_t st);
 cudaError_t launch_fast(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a,
                         int grid, cudaStream_t st);
 // Perturbed, projected vertices of both sides for every (view slot, pair) of a block of pairs.
