@@ -443,9 +443,16 @@ __global__ void k_background_loss(SceneDev S, Workspace ws, ViewList vl, float* 
       v += d * d;
     }
   }
+  __shared__ float red[TILE_PX / 32];
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  if ((threadIdx.x & 31) == 0 && v != 0.0f) atomicAdd(loss + slot, v);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    float sum = 0.0f;
+    for (int i = 0; i < TILE_PX / 32; ++i) sum += red[i];
+    if (sum != 0.0f) atomicAdd(loss + slot, sum);
+  }
 }
 
 template <int HT, int TSC, bool GR>
