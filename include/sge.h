@@ -339,7 +339,7 @@ typedef struct {
     int32_t pairs_per_item;    /* antithetic pairs one CTA runs per (view, tile) item (<= 64; default as in sge_config) */
     int32_t blocks_per_sm;     /* persistent CTAs per SM of the fast kernel (default: as many as fit)    */
     int32_t light_bin;         /* tiles whose bin holds at most this many triangles take the fast
-                                  kernel, the rest the general one (default and maximum 256)             */
+                                  kernel, the rest the dense one (default and maximum 256)               */
 } sge_batch_tuning;
 
 /* sge_estimate_grad for several scenes (assets of different sizes, textures and

@@ -393,7 +393,7 @@ __global__ void __launch_bounds__(TILE_PX, 3) k_estimate_deep(SceneDev S, Worksp
         }
         continue;
       }
-      for_each_signed_channel<false>(S, ps, kq, [&](long long p, int, bool neg) {
+      for_each_signed_channel(S, ps, kq, [&](long long p, bool neg) {
         if (!CHK(S, p, S.chk.params)) return;
         atomicAdd(a.grad + p, neg ? -df : df);
       });

@@ -50,7 +50,7 @@ namespace sge {
 namespace {
 
 constexpr int NB = kLightBin;
-constexpr int CMAX = 32;  // candidate triangles kept per pixel (a pixel with more tests every live triangle)
+constexpr int CMAX = 16 * kCandWords;  // candidates kept per pixel (a pixel with more tests every live triangle)
 constexpr int GMAX = 8;   // pairs of one group: set up together, one barrier before and after their pixels
 
 // Sum of v over the run of consecutive lanes (in lane order) that share key k, for the run's
@@ -192,8 +192,8 @@ struct PruneSmem {
   uint32_t id[NB];
   uint32_t key[NB];    // ordered bits of the smallest depths, by bin position
   uint8_t live[NB];
-  uint16_t remap[NB];  // compacted position of each live entry of a single-chunk bin
-  uint16_t cl[kHeavyCand][TILE_PX];  // each pixel's first kHeavyCand candidates (column per thread)
+  uint8_t remap[NB];   // compacted position of each live entry of a single-chunk bin
+  uint8_t cl[CMAX][TILE_PX];  // each pixel's first CMAX candidates (column per thread)
   uint32_t span[NB][2];  // the pixels of the sure-cover and the maybe-visible tests
   float m[16];
   int wsum[TILE_PX / 32];
@@ -218,21 +218,22 @@ __device__ __forceinline__ int block_prefix(int flag, int* wsum, int* total) {
   return before + in_warp;
 }
 
-// Store a pixel's list (this thread's column of cl, n entries found): 8-bit indices (light tile, the
-// first CMAX) or 16-bit ones (the first kHeavyCand), in list order, and its length min(n, 255).
-__device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_index, int pixel, const uint16_t* col,
-                                            int n, bool wide) {
-  static_assert(CMAX == 32 && CMAX <= kHeavyCand, "a light tile's list is two int4 words");
+// Store a pixel's list (this thread's column of cl, n entries found): the first CMAX as 8-bit indices in
+// list order, and its length min(n, 255).
+__device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_index, int pixel, const uint8_t* col,
+                                            int n) {
+  static_assert(CMAX == 16 * kCandWords, "sixteen indices to an int4 word");
   const long long ci = tile_index * kCandWords * TILE_PX + pixel;
-  const int k = min(n, kHeavyCand), bits = wide ? 16 : 8, per = 128 / bits;
-  for (int w = 0; w * per < k; ++w) {
+  const int k = min(n, CMAX);
+  for (int w = 0; w * 16 < k; ++w) {
     uint32_t v[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
       v[i] = 0u;
-      for (int q = 0; q < per / 4; ++q) {
-        const int at = w * per + i * (per / 4) + q;
-        if (at < k) v[i] |= (uint32_t)col[at * TILE_PX] << (bits * q);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int at = w * 16 + i * 4 + q;
+        if (at < k) v[i] |= (uint32_t)col[at * TILE_PX] << (8 * q);
       }
     }
     ws.cand[ci + w * TILE_PX] = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
@@ -259,9 +260,8 @@ __device__ __forceinline__ void for_spans(const uint32_t (*span)[2], int which, 
 // make visible at any pixel of the tile (outside all margin-widened pixel tests, or behind a
 // triangle that surely covers the pixel), compact the rest to the front of the bin's range,
 // record their number in tile_live and list the tile as a light item (<= light_bin live
-// triangles) or a heavy one, and store each pixel's candidate triangles in cand/ncand (light:
-// up to CMAX 8-bit live indices; heavy: up to kHeavyCand 16-bit ones).  The pruned triangles
-// never change any render of the call in this tile.
+// triangles) or a heavy one, and store each pixel's candidate triangles of a light one in cand/ncand
+// (up to CMAX live indices).  The pruned triangles never change any render of the call in this tile.
 //
 // A light tile's live triangles are in ascending order of their smallest depth under any
 // perturbation (ordered bits, a total order with NaN; ties by bin position), so each pixel's list
@@ -327,8 +327,8 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
   }
   // pass 2: mark and compact the triangles some pixel may see (a single chunk is still staged;
   // its pixels' candidate lists are found on the way, by staged position, and renumbered below)
-  uint16_t* col = &sm.cl[0][tid];
-  int n_cl = 0;  // candidates found for this pixel (the first kHeavyCand kept in sm.cl)
+  uint8_t* col = &sm.cl[0][tid];
+  int n_cl = 0;  // candidates found for this pixel (the first CMAX kept in sm.cl)
   int n_live = 0;
   for (int c0 = 0; c0 < nb; c0 += NB) {
     const int cnt = min(NB, nb - c0);
@@ -344,7 +344,7 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
       if (!maybe_covers(sm.t[j], dx, dy) || (bounded && !(sm.zr[j].x <= zsure))) return;
       sm.live[j] = 1;
       if (single) {
-        if (n_cl < kHeavyCand) col[n_cl * TILE_PX] = (uint16_t)j;
+        if (n_cl < CMAX) col[n_cl * TILE_PX] = (uint8_t)j;
         ++n_cl;
       }
     });
@@ -355,7 +355,7 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
     // positions only move towards the front, past entries this CTA has already read
     if (f) {
       if (CHK(S, (long long)beg + n_live + pos, S.chk.bins)) ws.bins[beg + n_live + pos] = sm.id[tid];
-      if (single) sm.remap[tid] = (uint16_t)pos;
+      if (single) sm.remap[tid] = (uint8_t)pos;
     }
     n_live += total;
   }
@@ -366,32 +366,27 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
     else if (n_live <= light_bin) ws.tile_cur[atomicAdd(ws.counters + 6, 1u)] = it;
     else ws.items[n_all - 1 - (int)atomicAdd(ws.counters + 4, 1u)] = it;
   }
-  const bool wide = n_live > light_bin;  // heavy tile: 16-bit indices
+  if (n_live > light_bin) return;  // (the dense estimator takes no lists)
   if (single) {
     __syncthreads();
     // staged positions -> live indices (each pixel renumbers its own column)
-    const int k = min(n_cl, kHeavyCand);
+    const int k = min(n_cl, CMAX);
     for (int q = 0; q < k; ++q) col[q * TILE_PX] = sm.remap[col[q * TILE_PX]];
-    store_cands(ws, tix, pixel, col, n_cl, wide);
-    return;
-  }
-  // pass 3 (bins of more than one chunk): each pixel's candidates among the live triangles, in
-  // their compacted order, a chunk of live triangles at a time (ascending); a light tile's live
-  // triangles are one chunk, ranked by depth here and stored back in that order
-  for (int c0 = 0; c0 < n_live; c0 += NB) {
-    const int cnt = min(NB, n_live - c0);
+  } else if (n_live > 0) {
+    // pass 3 (bins of more than one chunk): the live triangles are one chunk, ranked by depth here and
+    // stored back in that order, and each pixel's candidates are found among them
     __syncthreads();
-    stage(c0, cnt, !wide);
-    if (!wide && tid < cnt && CHK(S, (long long)beg + tid, S.chk.bins)) ws.bins[beg + tid] = sm.id[tid];
-    for_spans(sm.span, 1, cnt, block, dx, dy, [&](int j) {
+    stage(0, n_live, true);
+    if (tid < n_live && CHK(S, (long long)beg + tid, S.chk.bins)) ws.bins[beg + tid] = sm.id[tid];
+    for_spans(sm.span, 1, n_live, block, dx, dy, [&](int j) {
       if (!valid) return;
       const bool bounded = sm.t[j].small || !(sm.t[j].tri == -2 || sm.t[j].margin == 0x7FFFFFFF);
       if (!maybe_covers(sm.t[j], dx, dy) || (bounded && !(sm.zr[j].x <= zsure))) return;
-      if (n_cl < kHeavyCand) col[n_cl * TILE_PX] = (uint16_t)(c0 + j);
+      if (n_cl < CMAX) col[n_cl * TILE_PX] = (uint8_t)j;
       ++n_cl;
     });
   }
-  store_cands(ws, tix, pixel, col, n_cl, wide);
+  store_cands(ws, tix, pixel, col, n_cl);
 }
 
 __global__ void __launch_bounds__(TILE_PX, 4) k_bin_prune(SceneDev S, Workspace ws, ViewList vl) {
@@ -436,6 +431,7 @@ struct Model {
 };
 constexpr int kHashNoWindow = 512, kHashWindow = 128;  // hashed footprints of an item without / with a window
 constexpr int kHashProbe = 8;
+constexpr int kDenseTri = NB * 11 / 4;
 
 // One side of a live triangle set up for one pair; 64 bytes.
 // Small (every edge function over the tile fits 32 bits: |a|, |b| < 2^16, |e0| < 2^29, so
@@ -464,10 +460,15 @@ struct FastSmem {
   uint32_t hcnt[kHashNoWindow];
   float frame[M::LIT ? 2 : 1][M::LIT ? M::SLOTS : 1][6];  // lit: the set-up's face normal and u tangent
   float tgt[3][TILE_PX];          // target colours, by block and lane
-  float uv[NB][6];
-  int vid[NB][3];
-  int btri[NB];                   // triangle id of each live entry
-  uint32_t zminb[NB];             // ordered bits of its smallest depth under any perturbation of the call
+  union {
+    struct {
+      float uv[NB][6];
+      int vid[NB][3];
+      int btri[NB];               // triangle id of each live entry
+      uint32_t zminb[NB];         // ordered bits of its smallest depth under any perturbation of the call
+    };
+    int4 dense[kDenseTri];        // (dense_items) vertices and id of the first live triangles
+  };
   uint32_t sgn9[2][M::SLOTS];     // bit 3k+c: coordinate c of corner k has s = -1 (by group parity)
   float A_tri[M::SLOTS];          // f+ - f- of the pixels that see the triangle (side +, else side -)
   uint32_t n_tri[M::SLOTS];
@@ -912,6 +913,325 @@ __device__ __forceinline__ void make_windows(const SceneDev& S, FastSmem<SH, GR>
   sm.wbase[M::NFOOT] = base;
 }
 
+// The windows' unperturbed texel values.
+template <int SH, bool GR>
+__device__ __forceinline__ void load_window(const SceneDev& S, FastSmem<SH, GR>& sm) {
+  using M = Model<SH, GR>;
+  constexpr int NG = GR ? M::NREAD : 1;
+#pragma unroll 1
+  for (int r = 0; r < M::NFOOT; ++r) {
+    const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
+    const int4 win = sm.win[r];
+    for (int t = threadIdx.x; t < n; t += M::THREADS) {
+      const int texel = window_texel(win, t, S.rtex[r].w);
+      float tv[8] = {};
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const TexDev& T = S.rtex[GR ? k : r];
+        const float* src = T.ptr + (long long)texel * T.c;
+#pragma unroll
+        for (int c = 0; c < (GR ? used_channels(k) : 3); ++c)
+          if (c < T.c || T.c == 1) tv[(GR ? (k < 2 ? 3 * k : 4 + k) : 0) + c] = __ldg(src + (T.c == 1 ? 0 : c));
+      }
+      sm.th[0][base + t] = make_float4(tv[0], tv[1], tv[2], tv[3]);
+      if constexpr (GR) sm.th[1][base + t] = make_float4(tv[4], tv[5], tv[6], tv[7]);
+    }
+  }
+}
+
+// A pixel's footprints (in: it sees a triangle, at UV (u0, v0)) into the windows' bounds; whole warps.
+template <int SH, bool GR>
+__device__ __forceinline__ void add_bounds(const SceneDev& S, FastSmem<SH, GR>& sm, bool seen, float u0, float v0) {
+#pragma unroll
+  for (int r = 0; r < Model<SH, GR>::NFOOT; ++r) {
+    const Foot f = footprint(u0, v0, S.rtex[r].w, S.rtex[r].h);
+    const bool in = seen && abs(f.ix) < (1 << 28);
+    const int x0 = __reduce_min_sync(0xffffffffu, in ? f.ix : 0x3FFFFFFF);
+    const int x1 = __reduce_max_sync(0xffffffffu, in ? f.ix : -0x3FFFFFFF);
+    const int y0 = __reduce_min_sync(0xffffffffu, in ? f.y0 : 0x3FFFFFFF);
+    const int y1 = __reduce_max_sync(0xffffffffu, in ? f.y0 : -0x3FFFFFFF);
+    if ((threadIdx.x & 31) == 0 && x0 <= x1) {
+      atomicMin(&sm.win[r].x, x0);
+      atomicMin(&sm.win[r].y, y0);
+      atomicMax(&sm.win[r].z, x1);
+      atomicMax(&sm.win[r].w, y1);
+    }
+  }
+}
+
+// One side of a pixel at UV (u0, v0), pair g of the group (planes: the group's first pair's): the perturbed
+// texels sampled (values and signs from the window, else from memory) into val, the channels of each
+// read texture the shading uses, and the side's credit codes into cr.
+template <int SH, bool GR>
+__device__ __forceinline__ void sample_side(const SceneDev& S, const Workspace& ws, const FastSmem<SH, GR>& sm,
+                                            const uint32_t* planes, int g, int sd, float u0, float v0, int n_win,
+                                            uint32_t (&cr)[Model<SH, GR>::NFOOT], float (&val)[Model<SH, GR>::NREAD][3]) {
+  using M = Model<SH, GR>;
+  constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT, NG = GR ? NREAD : 1;
+#pragma unroll
+  for (int r = 0; r < NFOOT; ++r) {
+    const TexDev& T = S.rtex[r];
+    const int4 win = sm.win[r];
+    const float x = __fsub_rn(__fmul_rn(u0, (float)T.w), 0.5f), y = __fsub_rn(__fmul_rn(v0, (float)T.h), 0.5f);
+    const float xf = floorf(x), yf = floorf(y);
+    const float fx = __fsub_rn(x, xf), fy = __fsub_rn(y, yf);
+    const float wq[4] = {(1.0f - fx) * (1.0f - fy), fx * (1.0f - fy), (1.0f - fx) * fy, fx * fy};
+    const int wx = (int)xf - win.x, wy = (int)yf - win.y;
+#pragma unroll
+    for (int q = 0; q < NG; ++q) val[GR ? q : r][0] = val[GR ? q : r][1] = val[GR ? q : r][2] = 0.0f;
+    // (a column or row far from the window never passes, wrapped or not; no window: 0 < -1 fails)
+    bool inside = (uint32_t)wx < (uint32_t)max(win.z - 1, 0) && (uint32_t)wy < (uint32_t)max(win.w - 1, 0);
+    int nq = 0;  // nearest footprint: which of the four texels it is
+    if (S.foot_nearest && inside) {
+      const int nx = (int)floorf(__fmul_rn(u0, (float)T.w)) - (int)xf;
+      const int ny = (int)floorf(__fmul_rn(v0, (float)T.h)) - (int)yf;
+      inside = (uint32_t)nx < 2u && (uint32_t)ny < 2u;
+      nq = nx + ny * win.z;
+    }
+    if (inside) {
+      const int s00 = (NFOOT == 1 ? 0 : sm.wbase[r]) + wy * win.z + wx;
+      cr[r] = (uint32_t)(s00 + nq);
+      if (!CHK(S, s00 + win.z + 1, n_win)) continue;
+      const int up = 28 - M::SPP * (g % M::GPW);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int sq = s00 + (q & 1) + (q & 2 ? win.z : 0);
+        const float4 t0 = sm.th[0][sq];
+        if constexpr (!GR) {
+          const uint32_t sb = __float_as_uint(t0.w);
+          const float e = sd ? -T.eps : T.eps;
+          const float tv[3] = {t0.x, t0.y, t0.z};
+#pragma unroll
+          for (int c = 0; c < (M::LIT && r >= 2 ? 1 : 3); ++c)
+            val[r][c] += wq[q] * __fadd_rn(tv[c], (c < T.c || T.c == 1) ? signed_eps(sb, up + 3 - c, e) : 0.0f);
+        } else {
+          const float4 t1 = sm.th[M::NV - 1][sq];
+          const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
+          uint32_t sb;
+          if constexpr (M::SIGNS_APART) sb = sm.ts[g / M::GPW][sq];
+          else sb = __float_as_uint(g < M::GPW ? t1.z : t1.w);
+#pragma unroll
+          for (int k = 0; k < NREAD; ++k) {
+            const TexDev& U = S.rtex[k];
+            const float e = sd ? -U.eps : U.eps;
+#pragma unroll
+            for (int c = 0; c < used_channels(k); ++c)
+              val[k][c] += wq[q] * __fadd_rn(tv[(k < 2 ? 3 * k : 4 + k) + c],
+                                             (c < U.c || U.c == 1) ? signed_eps(sb, up + 3 - c - 4 * k, e) : 0.0f);
+          }
+        }
+      }
+    } else {
+      const Foot f = footprint(u0, v0, T.w, T.h);
+      const uint32_t code = kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | (f.y1 == f.y0 ? kOneRow : 0u) |
+                          (uint32_t)(f.y0 * T.w + f.x0);
+      cr[r] = S.foot_nearest ? kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | kOneRow |
+                                    (uint32_t)nearest_texel(u0, v0, T.w, T.h)
+                              : code;
+      int texel[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        texel[q] = (q & 2 ? f.y1 : f.y0) * T.w + (q & 1 ? f.x1 : f.x0);
+        if (!CHK(S, texel[q], (long long)T.w * T.h)) texel[q] = 0;
+      }
+      // (a texture at a time, its four texels' loads in flight together)
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const TexDev& U = S.rtex[GR ? k : r];
+        uint32_t sb[4];
+        float tv[4][3];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          sb[q] = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], texel[q]);
+          const float* src = U.ptr + (long long)texel[q] * U.c;
+#pragma unroll
+          for (int c = 0; c < 3; ++c) tv[q][c] = c < U.c ? __ldg(src + c) : 0.0f;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (sd) sb[q] = ~sb[q];
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            if (c < U.c) val[GR ? k : r][c] += wq[q] * __fadd_rn(tv[q][c], ((sb[q] >> c) & 1) ? -U.eps : U.eps);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < NG; ++k)
+        if (S.rtex[GR ? k : r].c == 1) val[GR ? k : r][1] = val[GR ? k : r][2] = val[GR ? k : r][0];
+    }
+  }
+}
+
+// The colour of a sampled pixel: fr the triangle's frame (lit), vid its vertices, sg its 9 coordinate
+// signs on this side, pw the pixel's perspective-correct weights (GGX).
+template <int SH, bool GR>
+__device__ __forceinline__ float3 shade_side(const SceneDev& S, int view, const float (&val)[Model<SH, GR>::NREAD][3],
+                                             const float* fr, const int* vid, uint32_t sg, const PerspW& pw) {
+  if constexpr (SH == SHADE_UNLIT) {
+    return f3(val[0][0], val[0][1], val[0][2]);
+  } else {
+    float3 P = f3(0.f, 0.f, 0.f);
+    float rough = 0.5f, metal = 0.0f;
+    if constexpr (SH == SHADE_GGX) {
+      float3 p[3];
+      corner_positions(S, vid, sg, p);
+      const float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
+      P = f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
+             b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z);
+      rough = val[2][0];
+      metal = val[3][0];
+    }
+    return shade_lit<SH>(S, view, val[0], val[1], rough, metal, f3(fr[0], fr[1], fr[2]), f3(fr[3], fr[4], fr[5]), P);
+  }
+}
+
+// Credit f+ - f- of a pixel of pair g to the texels of the union of both sides' footprints of every read
+// texture (of the group); inA, inB: the sides that see a triangle (at least one).
+template <int SH, bool GR>
+__device__ __forceinline__ void credit_texels(const SceneDev& S, const Workspace& ws, const EstimateArgs& a,
+                                              FastSmem<SH, GR>& sm, const uint32_t* planes, int g, int stride, int n_win,
+                                              int nh, float df, bool inA, bool inB,
+                                              const uint32_t (&crA)[Model<SH, GR>::NFOOT],
+                                              const uint32_t (&crB)[Model<SH, GR>::NFOOT]) {
+  using M = Model<SH, GR>;
+  constexpr int NFOOT = M::NFOOT, NG = GR ? M::NREAD : 1;
+  float* sums = sm.tA + g * stride;
+#pragma unroll
+  for (int r = 0; r < NFOOT; ++r) {
+    const TexDev& T = S.rtex[r];
+    const uint32_t A = inA ? crA[r] : crB[r], B = inB ? crB[r] : crA[r];
+    // one texel by its id, straight to the global sums
+    auto credit_id = [&](int id) {
+#pragma unroll 1
+      for (int k = 0; k < NG; ++k) {
+        const TexDev& U = S.rtex[GR ? k : r];
+        const uint32_t sb = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], id);
+        const long long base = U.offset + (long long)id * U.c;
+        for (int c = 0; c < U.c; ++c) {
+          if (!CHK(S, base + c, S.chk.params)) continue;
+          atomicAdd(a.grad + base + c, ((sb >> c) & 1) ? -df : df);
+          atomicAdd(a.counts + base + c, 1u);
+        }
+      }
+    };
+    // a footprint's texels by one sum in its cell (nearest: the one texel)
+    auto credit_cell = [&](uint32_t c) {
+      if (!(c & kOut)) {
+        if (!CHK(S, c, n_win)) return;
+        atomicAdd(sums + c + (S.foot_nearest ? n_win + nh : 0), df);
+        atomicAdd(sm.tcnt + c, S.foot_nearest ? 1u << 16 : 1u);
+        return;
+      }
+      const int h = hash_slot(sm.hkey, c, nh);
+      if (h >= 0) {
+        atomicAdd(sums + n_win + h, df);
+        atomicAdd(sm.hcnt + h, 1u);
+        return;
+      }
+      const Quad Q(c, T.w);
+#pragma unroll 1
+      for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q)
+        if (!Q.repeats(q)) credit_id(Q.texel(q, T.w));
+    };
+    credit_cell(A);
+    if (B == A) continue;
+    if (S.foot_nearest) {
+      // one texel each: a window slot and an outside id may be the same texel
+      bool dup = false;
+      if ((A ^ B) & kOut) {
+        const uint32_t in = (A & kOut) ? B : A, out = (A & kOut) ? A : B;
+        dup = window_texel(sm.win[r], (int)in - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w) == (int)(out & 0x0FFFFFFFu);
+      }
+      if (!dup) credit_cell(B);
+      continue;
+    }
+    if (!((A | B) & kOut)) {
+      // side -'s texels outside side +'s footprint
+      const uint32_t ww = (uint32_t)sm.win[r].z;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t s = B + (q & 1) + (q & 2 ? ww : 0u), d = s - A;
+        if (d <= 1u || d - ww <= 1u || !CHK(S, s, n_win)) continue;
+        atomicAdd(sums + n_win + nh + s, df);
+        atomicAdd(sm.tcnt + s, 1u << 16);
+      }
+      continue;
+    }
+    // some side outside the window: by texel id
+    auto as_id = [&](uint32_t c) {
+      if (c & kOut) return c;
+      return kOut | (uint32_t)window_texel(sm.win[r], (int)c - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w);
+    };
+    const Quad QA(as_id(A), T.w), QB(as_id(B), T.w);
+    uint32_t mine = 0, all = 0;  // side -'s texels (its footprint's own repeats left out), those not in side +'s
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (QB.repeats(q)) continue;
+      all |= 1u << q;
+      if (!QA.holds(QB, q)) mine |= 1u << q;
+    }
+    if (mine == all) {
+      credit_cell(B);
+    } else {
+#pragma unroll 1
+      for (; mine; mine &= mine - 1) credit_id(QB.texel(__ffs((int)mine) - 1, T.w));
+    }
+  }
+}
+
+// An empty start of a CTA's loop over items.
+template <int SH, bool GR>
+__device__ __forceinline__ void reset_smem(FastSmem<SH, GR>& sm) {
+  using M = Model<SH, GR>;
+  for (int s = threadIdx.x; s < M::ACAP; s += M::THREADS) sm.tA[s] = 0.0f;
+  for (int s = threadIdx.x; s < M::WCAP; s += M::THREADS) sm.tcnt[s] = 0u;
+  for (int s = threadIdx.x; s < kHashNoWindow; s += M::THREADS) sm.hkey[s] = EMPTY, sm.hcnt[s] = 0u;
+  for (int s = threadIdx.x; s < M::SLOTS; s += M::THREADS) {
+    sm.A_tri[s] = sm.A_cor[s][0] = sm.A_cor[s][1] = sm.A_cor[s][2] = 0.0f;
+    sm.n_tri[s] = sm.n_cor[s] = 0u;
+  }
+  for (int s = threadIdx.x; s < SGE_MAX_VIEWS_PER_CALL; s += M::THREADS) sm.loss[s] = 0.0;
+  if (threadIdx.x == 0) sm.nact = 0u;
+  if (threadIdx.x < M::NFOOT) sm.win[threadIdx.x] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
+  if (threadIdx.x <= M::NFOOT) sm.wbase[threadIdx.x] = 0;
+}
+
+// The end of an item: its loss to the CTA's sum of the view slot, its counters back to empty, the next item.
+template <int SH, bool GR>
+__device__ __forceinline__ void end_item(const EstimateArgs& a, FastSmem<SH, GR>& sm, int slot, float loss_acc,
+                                         uint32_t next) {
+  using M = Model<SH, GR>;
+  const int tid = threadIdx.x;
+  if (a.loss) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
+    if ((tid & 31) == 0) sm.red[tid >> 5] = loss_acc;
+  }
+  __syncthreads();
+  for (int s = tid; s < sm.wbase[M::NFOOT]; s += M::THREADS) sm.tcnt[s] = 0u;
+  if (tid == 0) {
+    if (a.loss) {
+      double sum = 0.0;
+      for (int i = 0; i < M::WARPS; ++i) sum += sm.red[i];
+      sm.loss[slot] += sum;
+    }
+    sm.item = next;
+    sm.nact = 0u;
+  }
+  __syncthreads();
+  if (tid < M::NFOOT) sm.win[tid] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
+  if (tid <= M::NFOOT) sm.wbase[tid] = 0;
+}
+
+template <int SH, bool GR>
+__device__ __forceinline__ void add_losses(const EstimateArgs& a, FastSmem<SH, GR>& sm, int n_slots) {
+  // one addition per CTA and view, however many items the call is cut into: their rounding stays below that
+  // of the pixels' own sums
+  if (a.loss)
+    for (int s = threadIdx.x; s < n_slots; s += Model<SH, GR>::THREADS)
+      if (sm.loss[s] != 0.0) atomicAdd(a.loss + s, (float)(sm.loss[s] / (double)a.pairs));
+}
+
 // Pairs per item: `lo` doubled up to `hi` while every CTA still gets at least 16 items (a longer run
 // amortises the item's staging and texel windows, a shorter one balances the CTAs).
 __device__ __forceinline__ int run_of(const EstimateArgs& a, int n_items, int lo, int hi) {
@@ -927,7 +1247,7 @@ template <int SH, bool GR>
 __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
                                            const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
   using M = Model<SH, GR>;
-  constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT, NG = GR ? NREAD : 1;
+  constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   // a warp's pixels: an 8 x 4 block, odd rows right to left, so that runs of lanes follow the surface
   const int lx = (lane & 8) ? 7 - (lane & 7) : (lane & 7), ly = lane >> 3;
@@ -941,17 +1261,7 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
   const int run = a.pairs_per_item > 0 ? ppi : run_of(a, n_small, ppi, 4 * kRun), run_big = run_of(a, n_big, max(1, ppi / 4), ppi);
   const int chunks = (a.pair_count + run - 1) / run, chunks_big = (a.pair_count + run_big - 1) / run_big;
   const long long work_big = (long long)n_big * chunks_big, n_work = work_big + (long long)n_small * chunks;
-  for (int s = tid; s < M::ACAP; s += M::THREADS) sm.tA[s] = 0.0f;
-  for (int s = tid; s < M::WCAP; s += M::THREADS) sm.tcnt[s] = 0u;
-  for (int s = tid; s < kHashNoWindow; s += M::THREADS) sm.hkey[s] = EMPTY, sm.hcnt[s] = 0u;
-  for (int s = tid; s < M::SLOTS; s += M::THREADS) {
-    sm.A_tri[s] = sm.A_cor[s][0] = sm.A_cor[s][1] = sm.A_cor[s][2] = 0.0f;
-    sm.n_tri[s] = sm.n_cor[s] = 0u;
-  }
-  for (int s = tid; s < SGE_MAX_VIEWS_PER_CALL; s += M::THREADS) sm.loss[s] = 0.0;
-  if (tid == 0) sm.nact = 0u;
-  if (tid < NFOOT) sm.win[tid] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
-  if (tid <= NFOOT) sm.wbase[tid] = 0;
+  reset_smem<SH, GR>(sm);
   const uint32_t first_of = own_first ? gridDim.x : 0u;
   if (tid == 0) sm.item = own_first ? blockIdx.x : atomicAdd(ws.counters + 1, 1u);
   __syncthreads();
@@ -1022,10 +1332,10 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
     const int nact = (int)sm.nact;
     // pairs of a group: as many as the set-ups, the sign words and (below) the sums hold
     int Gcap = min(GMAX, M::SLOTS / max(nb, 1)), par = 0, G = 0, nh = 0;
-    // an unlit item of one or two pairs takes no window: finding its bounds costs half a pair, and its
-    // footprints all go through hashed cells (one 256^2 estimate: the kernel 37.0 -> 29.5 us; 4 views x 16
-    // pairs with runs of 2 on dense tiles 640 -> 610 us; lit items lose, 11.2 -> 20.1 ms)
-    const bool windowed = M::LIT || p1 - p0 > 2;
+    // unlit calls of one or two pairs take no window: finding its bounds costs half a pair, and the
+    // footprints all go through hashed cells (one 256^2 estimate: the kernel 37.0 -> 29.5 us; lit items
+    // lose, 11.2 -> 20.1 ms)
+    const bool windowed = M::LIT || a.pair_count > 2;
     if (!windowed) {
       nh = kHashNoWindow;
       Gcap = min(Gcap, M::ACAP / nh);
@@ -1157,137 +1467,15 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
             v0 = persp_interp(pw, uvt[1], uvt[3], uvt[5]);
           }
           if (bounds) {
-#pragma unroll
-            for (int r = 0; r < NFOOT; ++r) {
-              const Foot f = footprint(u0, v0, S.rtex[r].w, S.rtex[r].h);
-              const bool in = jB >= 0 && abs(f.ix) < (1 << 28);
-              const int x0 = __reduce_min_sync(0xffffffffu, in ? f.ix : 0x3FFFFFFF);
-              const int x1 = __reduce_max_sync(0xffffffffu, in ? f.ix : -0x3FFFFFFF);
-              const int y0 = __reduce_min_sync(0xffffffffu, in ? f.y0 : 0x3FFFFFFF);
-              const int y1 = __reduce_max_sync(0xffffffffu, in ? f.y0 : -0x3FFFFFFF);
-              if (lane == 0 && x0 <= x1) {
-                atomicMin(&sm.win[r].x, x0);
-                atomicMin(&sm.win[r].y, y0);
-                atomicMax(&sm.win[r].z, x1);
-                atomicMax(&sm.win[r].w, y1);
-              }
-            }
+            add_bounds<SH, GR>(S, sm, jB >= 0, u0, v0);
             break;
           }
           if (jB < 0) continue;
-          // -- G: sample the perturbed texels (values and signs from the window, else from memory)
+          // -- G: sample the perturbed texels and shade
           float val[NREAD][3];
-#pragma unroll
-          for (int r = 0; r < NFOOT; ++r) {
-            const TexDev& T = S.rtex[r];
-            const int4 win = sm.win[r];
-            const float x = __fsub_rn(__fmul_rn(u0, (float)T.w), 0.5f), y = __fsub_rn(__fmul_rn(v0, (float)T.h), 0.5f);
-            const float xf = floorf(x), yf = floorf(y);
-            const float fx = __fsub_rn(x, xf), fy = __fsub_rn(y, yf);
-            const float wq[4] = {(1.0f - fx) * (1.0f - fy), fx * (1.0f - fy), (1.0f - fx) * fy, fx * fy};
-            const int wx = (int)xf - win.x, wy = (int)yf - win.y;
-#pragma unroll
-            for (int q = 0; q < NG; ++q) val[GR ? q : r][0] = val[GR ? q : r][1] = val[GR ? q : r][2] = 0.0f;
-            // (a column or row far from the window never passes, wrapped or not; no window: 0 < -1 fails)
-            bool inside = (uint32_t)wx < (uint32_t)max(win.z - 1, 0) && (uint32_t)wy < (uint32_t)max(win.w - 1, 0);
-            int nq = 0;  // nearest footprint: which of the four texels it is
-            if (S.foot_nearest && inside) {
-              const int nx = (int)floorf(__fmul_rn(u0, (float)T.w)) - (int)xf;
-              const int ny = (int)floorf(__fmul_rn(v0, (float)T.h)) - (int)yf;
-              inside = (uint32_t)nx < 2u && (uint32_t)ny < 2u;
-              nq = nx + ny * win.z;
-            }
-            if (inside) {
-              const int s00 = (NFOOT == 1 ? 0 : sm.wbase[r]) + wy * win.z + wx;
-              crB[r] = (uint32_t)(s00 + nq);
-              if (!CHK(S, s00 + win.z + 1, n_win)) continue;
-              const int up = 28 - M::SPP * (g % M::GPW);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const int sq = s00 + (q & 1) + (q & 2 ? win.z : 0);
-                const float4 t0 = sm.th[0][sq];
-                if constexpr (!GR) {
-                  const uint32_t sb = __float_as_uint(t0.w);
-                  const float e = sd ? -T.eps : T.eps;
-                  const float tv[3] = {t0.x, t0.y, t0.z};
-#pragma unroll
-                  for (int c = 0; c < (M::LIT && r >= 2 ? 1 : 3); ++c)
-                    val[r][c] += wq[q] * __fadd_rn(tv[c], (c < T.c || T.c == 1) ? signed_eps(sb, up + 3 - c, e) : 0.0f);
-                } else {
-                  const float4 t1 = sm.th[M::NV - 1][sq];
-                  const float tv[8] = {t0.x, t0.y, t0.z, t0.w, t1.x, t1.y, t1.z, t1.w};
-                  uint32_t sb;
-                  if constexpr (M::SIGNS_APART) sb = sm.ts[g / M::GPW][sq];
-                  else sb = __float_as_uint(g < M::GPW ? t1.z : t1.w);
-#pragma unroll
-                  for (int k = 0; k < NREAD; ++k) {
-                    const TexDev& U = S.rtex[k];
-                    const float e = sd ? -U.eps : U.eps;
-#pragma unroll
-                    for (int c = 0; c < used_channels(k); ++c)
-                      val[k][c] += wq[q] * __fadd_rn(tv[(k < 2 ? 3 * k : 4 + k) + c],
-                                                     (c < U.c || U.c == 1) ? signed_eps(sb, up + 3 - c - 4 * k, e) : 0.0f);
-                  }
-                }
-              }
-            } else {
-              const Foot f = footprint(u0, v0, T.w, T.h);
-              const uint32_t cr = kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | (f.y1 == f.y0 ? kOneRow : 0u) |
-                                  (uint32_t)(f.y0 * T.w + f.x0);
-              crB[r] = S.foot_nearest ? kOut | ((uint32_t)(GR ? 0 : r) << kFootShift) | kOneRow |
-                                            (uint32_t)nearest_texel(u0, v0, T.w, T.h)
-                                      : cr;
-              int texel[4];
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                texel[q] = (q & 2 ? f.y1 : f.y0) * T.w + (q & 1 ? f.x1 : f.x0);
-                if (!CHK(S, texel[q], (long long)T.w * T.h)) texel[q] = 0;
-              }
-              // (a texture at a time, its four texels' loads in flight together)
-#pragma unroll
-              for (int k = 0; k < NG; ++k) {
-                const TexDev& U = S.rtex[GR ? k : r];
-                uint32_t sb[4];
-                float tv[4][3];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                  sb[q] = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], texel[q]);
-                  const float* src = U.ptr + (long long)texel[q] * U.c;
-#pragma unroll
-                  for (int c = 0; c < 3; ++c) tv[q][c] = c < U.c ? __ldg(src + c) : 0.0f;
-                }
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                  if (sd) sb[q] = ~sb[q];
-#pragma unroll
-                  for (int c = 0; c < 3; ++c)
-                    if (c < U.c) val[GR ? k : r][c] += wq[q] * __fadd_rn(tv[q][c], ((sb[q] >> c) & 1) ? -U.eps : U.eps);
-                }
-              }
-#pragma unroll
-              for (int k = 0; k < NG; ++k)
-                if (S.rtex[GR ? k : r].c == 1) val[GR ? k : r][1] = val[GR ? k : r][2] = val[GR ? k : r][0];
-            }
-          }
-          // -- shade
-          if constexpr (!M::LIT) {
-            cB = f3(val[0][0], val[0][1], val[0][2]);
-          } else {
-            const float* fr = sm.frame[sd][sbase + jB];
-            float3 P = f3(0.f, 0.f, 0.f);
-            float rough = 0.5f, metal = 0.0f;
-            if constexpr (SH == SHADE_GGX) {
-              float3 p[3];
-              corner_positions(S, sm.vid[jB], sm.sgn9[par][sbase + jB] ^ (sd ? 0x1FFu : 0u), p);
-              const float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
-              P = f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
-                     b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z);
-              rough = val[2][0];
-              metal = val[3][0];
-            }
-            cB = shade_lit<SH>(S, view, val[0], val[1], rough, metal, f3(fr[0], fr[1], fr[2]), f3(fr[3], fr[4], fr[5]),
-                               P);
-          }
+          sample_side<SH, GR>(S, ws, sm, planes, g, sd, u0, v0, n_win, crB, val);
+          cB = shade_side<SH, GR>(S, view, val, sm.frame[M::LIT ? sd : 0][M::LIT ? sbase + jB : 0], sm.vid[jB],
+                                  sm.sgn9[par][sbase + jB] ^ (sd ? 0x1FFu : 0u), pw);
         }
         if (bounds) {
           bounds = false;
@@ -1295,25 +1483,7 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
           __syncthreads();
           if (tid == 0) make_windows(S, sm);
           __syncthreads();
-#pragma unroll 1
-          for (int r = 0; r < NFOOT; ++r) {
-            const int base = sm.wbase[r], n = sm.wbase[r + 1] - base;
-            const int4 win = sm.win[r];
-            for (int t = tid; t < n; t += M::THREADS) {
-              const int texel = window_texel(win, t, S.rtex[r].w);
-              float tv[8] = {};
-#pragma unroll
-              for (int k = 0; k < NG; ++k) {
-                const TexDev& T = S.rtex[GR ? k : r];
-                const float* src = T.ptr + (long long)texel * T.c;
-#pragma unroll
-                for (int c = 0; c < (GR ? used_channels(k) : 3); ++c)
-                  if (c < T.c || T.c == 1) tv[(GR ? (k < 2 ? 3 * k : 4 + k) : 0) + c] = __ldg(src + (T.c == 1 ? 0 : c));
-              }
-              sm.th[0][base + t] = make_float4(tv[0], tv[1], tv[2], tv[3]);
-              if constexpr (GR) sm.th[1][base + t] = make_float4(tv[4], tv[5], tv[6], tv[7]);
-            }
-          }
+          load_window<SH, GR>(S, sm);
           const int n = sm.wbase[NFOOT];
           nh = n > 0 ? kHashWindow : kHashNoWindow;
           Gcap = min(Gcap, M::ACAP / (2 * n + nh));
@@ -1356,90 +1526,8 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
           }
           if (add) atomicAdd(&sm.n_cor[sbase + jB], add);
         }
-        // texels: union of both sides' footprints of every read texture (of the group)
-        if (jA < 0 && jB < 0) continue;
-        float* sums = sm.tA + g * stride;
-#pragma unroll
-        for (int r = 0; r < NFOOT; ++r) {
-          const TexDev& T = S.rtex[r];
-          const uint32_t A = jA >= 0 ? crA[r] : crB[r], B = jB >= 0 ? crB[r] : crA[r];
-          // one texel by its id, straight to the global sums
-          auto credit_id = [&](int id) {
-#pragma unroll 1
-            for (int k = 0; k < NG; ++k) {
-              const TexDev& U = S.rtex[GR ? k : r];
-              const uint32_t sb = plane_nibble(S, planes + g * ws.sgn_words, ws.sgn_off[U.index], id);
-              const long long base = U.offset + (long long)id * U.c;
-              for (int c = 0; c < U.c; ++c) {
-                if (!CHK(S, base + c, S.chk.params)) continue;
-                atomicAdd(a.grad + base + c, ((sb >> c) & 1) ? -df : df);
-                atomicAdd(a.counts + base + c, 1u);
-              }
-            }
-          };
-          // a footprint's texels by one sum in its cell (nearest: the one texel)
-          auto credit_cell = [&](uint32_t c) {
-            if (!(c & kOut)) {
-              if (!CHK(S, c, n_win)) return;
-              atomicAdd(sums + c + (S.foot_nearest ? n_win + nh : 0), df);
-              atomicAdd(sm.tcnt + c, S.foot_nearest ? 1u << 16 : 1u);
-              return;
-            }
-            const int h = hash_slot(sm.hkey, c, nh);
-            if (h >= 0) {
-              atomicAdd(sums + n_win + h, df);
-              atomicAdd(sm.hcnt + h, 1u);
-              return;
-            }
-            const Quad Q(c, T.w);
-#pragma unroll 1
-            for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q)
-              if (!Q.repeats(q)) credit_id(Q.texel(q, T.w));
-          };
-          credit_cell(A);
-          if (B == A) continue;
-          if (S.foot_nearest) {
-            // one texel each: a window slot and an outside id may be the same texel
-            bool dup = false;
-            if ((A ^ B) & kOut) {
-              const uint32_t in = (A & kOut) ? B : A, out = (A & kOut) ? A : B;
-              dup = window_texel(sm.win[r], (int)in - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w) == (int)(out & 0x0FFFFFFFu);
-            }
-            if (!dup) credit_cell(B);
-            continue;
-          }
-          if (!((A | B) & kOut)) {
-            // side -'s texels outside side +'s footprint
-            const uint32_t ww = (uint32_t)sm.win[r].z;
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-              const uint32_t s = B + (q & 1) + (q & 2 ? ww : 0u), d = s - A;
-              if (d <= 1u || d - ww <= 1u || !CHK(S, s, n_win)) continue;
-              atomicAdd(sums + n_win + nh + s, df);
-              atomicAdd(sm.tcnt + s, 1u << 16);
-            }
-            continue;
-          }
-          // some side outside the window: by texel id
-          auto as_id = [&](uint32_t c) {
-            if (c & kOut) return c;
-            return kOut | (uint32_t)window_texel(sm.win[r], (int)c - (NFOOT == 1 ? 0 : sm.wbase[r]), T.w);
-          };
-          const Quad QA(as_id(A), T.w), QB(as_id(B), T.w);
-          uint32_t mine = 0, all = 0;  // side -'s texels (its footprint's own repeats left out), those not in side +'s
-#pragma unroll
-          for (int q = 0; q < 4; ++q) {
-            if (QB.repeats(q)) continue;
-            all |= 1u << q;
-            if (!QA.holds(QB, q)) mine |= 1u << q;
-          }
-          if (mine == all) {
-            credit_cell(B);
-          } else {
-#pragma unroll 1
-            for (; mine; mine &= mine - 1) credit_id(QB.texel(__ffs((int)mine) - 1, T.w));
-          }
-        }
+        if (jA >= 0 || jB >= 0)
+          credit_texels<SH, GR>(S, ws, a, sm, planes, g, stride, n_win, nh, df, jA >= 0, jB >= 0, crA, crB);
       }
       __syncthreads();
       first = false;
@@ -1452,31 +1540,315 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
       flush_counts<SH, GR>(S, a, sm, nh);
       clear_sums(sm, G, nh);
     }
-    if (a.loss) {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) loss_acc += __shfl_xor_sync(0xffffffffu, loss_acc, o);
-      if (lane == 0) sm.red[warp] = loss_acc;
-    }
-    __syncthreads();
-    for (int s = tid; s < sm.wbase[NFOOT]; s += M::THREADS) sm.tcnt[s] = 0u;
-    if (tid == 0) {
-      if (a.loss) {
-        double sum = 0.0;
-        for (int i = 0; i < M::WARPS; ++i) sum += sm.red[i];
-        sm.loss[slot] += sum;
-      }
-      sm.item = next;
-      sm.nact = 0u;
-    }
-    __syncthreads();
-    if (tid < NFOOT) sm.win[tid] = make_int4(0x3FFFFFFF, 0x3FFFFFFF, -0x3FFFFFFF, -0x3FFFFFFF);
-    if (tid <= NFOOT) sm.wbase[tid] = 0;
+    end_item<SH, GR>(a, sm, slot, loss_acc, next);
   }
-  // one addition per CTA and view, however many items the call is cut into: their rounding stays below that
-  // of the pixels' own sums
-  if (a.loss)
-    for (int s = tid; s < vl.n; s += M::THREADS)
-      if (sm.loss[s] != 0.0) atomicAdd(a.loss + s, (float)(sm.loss[s] / (double)a.pairs));
+  add_losses<SH, GR>(a, sm, vl.n);
+}
+
+// A projected triangle (records of the vertex pass) into the tile's keys: the nearest (depth bits << 32 |
+// id) of each pixel centre it covers.  The arithmetic of set_up_side, cover_lambdas and
+// interp_depth, with the division left until a pixel is covered (most triangles of a dense tile cover
+// none or one).
+__device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const int4& q2, int id, int rx, int ry,
+                                           unsigned long long* keys) {
+  if (q0.x == kNotDrawn || q1.x == kNotDrawn || q2.x == kNotDrawn) return;
+  const int x0 = q0.x - rx, x1 = q1.x - rx, x2 = q2.x - rx, y0 = q0.y - ry, y1 = q1.y - ry, y2 = q2.y - ry;
+  // pixel centres in the vertex box
+  const int xl = min(x0, min(x1, x2)), xh = max(x0, max(x1, x2)), yl = min(y0, min(y1, y2)), yh = max(y0, max(y1, y2));
+  const int c0 = max((xl + 255) >> 8, 0), c1 = min(xh >> 8, TILE - 1), r0 = max((yl + 255) >> 8, 0), r1 = min(yh >> 8, TILE - 1);
+  if (c0 > c1 || r0 > r1) return;
+  auto put = [&](int x, int y, const float (&l)[3]) {
+    const float z[3] = {__int_as_float(q0.z), __int_as_float(q1.z), __int_as_float(q2.z)};
+    const unsigned long long key = ((unsigned long long)ordered_bits(interp_depth(l, z)) << 32) | (uint32_t)id;
+    unsigned long long* out = keys + y * TILE + x;
+    if (key < *(volatile unsigned long long*)out) atomicMin(out, key);
+  };
+  if (max(max(xh, yh), -min(xl, yl)) < (1 << 14)) {
+    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, e2 = x0 * y1 - x1 * y0, area = e0 + e1 + e2;
+    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
+    if (area == 0) return;
+    if (area < 0) {
+      e0 = -e0, e1 = -e1, e2 = -e2, area = -area;
+      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
+    }
+    float inv = 0.0f;
+    for (int y = r0; y <= r1; ++y) {
+      int E0 = e0 + a0 * (c0 * 256) + b0 * (y * 256), E1 = e1 + a1 * (c0 * 256) + b1 * (y * 256);
+      for (int x = c0; x <= c1; ++x, E0 += a0 * 256, E1 += a1 * 256) {
+        const int E2 = area - E0 - E1, lo = min(min(E0, E1), E2);
+        if (lo < 0) continue;
+        if (lo == 0 && ((E0 == 0 && !(a0 > 0 || (a0 == 0 && b0 > 0))) || (E1 == 0 && !(a1 > 0 || (a1 == 0 && b1 > 0))) ||
+                        (E2 == 0 && !(a2 > 0 || (a2 == 0 && b2 > 0)))))
+          continue;
+        if (inv == 0.0f) inv = __fdiv_rn(1.0f, __int2float_rn(area));
+        const float l[3] = {__fmul_rn(__int2float_rn(E0), inv), __fmul_rn(__int2float_rn(E1), inv),
+                            __fmul_rn(__int2float_rn(E2), inv)};
+        put(x, y, l);
+      }
+    }
+    return;
+  }
+  PVert v[3];
+  const int4 q[3] = {q0, q1, q2};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = PVert{q[k].x, q[k].y, __int_as_float(q[k].z), __int_as_float(q[k].w), true};
+  SideTri d;
+  set_up_side(d, v, rx, ry);
+  for (int y = r0; y <= r1; ++y)
+    for (int x = c0; x <= c1; ++x) {
+      float l[3];
+      float4 z;
+      if (cover_lambdas(d, x * 256, y * 256, l, z)) put(x, y, l);
+    }
+}
+
+// Every heavy work item of one scene's call: tiles with more live triangles than the fast path's set-ups
+// hold (dense meshes, poles, silhouettes seen edge-on).  The same steps with another split:
+// the triangles are many and small (a pixel may have a hundred candidates), so R goes by triangle: each
+// is set up and tested at the pixel centres of its box, and the nearest key wins by an atomic minimum; then
+// a warp keeps one block of the tile and one of P pairs, and each pixel sets its visible triangles up
+// again by itself (one is seen by a pixel or two, so there is nothing to share) and shades.  Vertex
+// credits go to the global sums directly, texel credits through the windows and cells as in the fast path.
+// Bound by instruction issue (R is 70 % of it).  Against the general kernel it replaces, which set every
+// live triangle up in shared memory per pair, tested up to all of them at each pixel and hashed vertices and
+// texels: 24.6 -> 9.6 ms (GGX, 1 M triangles, 6,175 dense tiles x 4 pairs), 4.82 -> 2.11 ms (a batch of 8 unlit
+// assets), 1.32 -> 0.28 ms (Lambert, 41 tiles x 16 pairs).
+template <int SH, bool GR>
+__device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
+                                            const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
+  using M = Model<SH, GR>;
+  constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT, BLOCKS = TILE_PX / 32;
+  constexpr int P = M::WARPS / BLOCKS;  // pairs at a time
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, stream = warp / BLOCKS, blk = warp % BLOCKS;
+  const int dx = (blk & 1) * 8 + (lane & 7), dy = (blk >> 1) * 4 + (lane >> 3), X = dx * 256, Y = dy * 256;
+  // the visible triangle's (depth bits << 32 | id) per pair, side and pixel, in the fast path's set-ups' place
+  unsigned long long* keys = reinterpret_cast<unsigned long long*>(&sm.side[0][0]);
+  static_assert(sizeof(sm.side) >= 2 * P * TILE_PX * sizeof(unsigned long long), "keys");
+  const int ntl = n_tiles(S), n_heavy = (int)ws.counters[4];
+  const int run = a.pairs_per_item > 0 ? max(1, a.pairs_per_item / 4) : run_of(a, n_heavy, P, kRun);
+  const int chunks = (a.pair_count + run - 1) / run;
+  const long long n_work = (long long)n_heavy * chunks;
+  if (n_work == 0 || (own_first && blockIdx.x >= n_work)) return;  // (uniform over the CTA)
+  reset_smem<SH, GR>(sm);
+  const uint32_t first_of = own_first ? gridDim.x : 0u;
+  if (tid == 0) sm.item = own_first ? blockIdx.x : atomicAdd(ws.counters + 5, 1u);
+  __syncthreads();
+
+  for (long long w = sm.item; w < n_work; w = sm.item) {
+    const int at = (int)(w / chunks), chunk = (int)(w - (long long)at * chunks);
+    const uint32_t it = ws.items[vl.n * ntl - 1 - at];
+    const int slot = it >> 24, tile = it & 0xFFFFFF;
+    uint32_t next = 0;
+    if (tid == 0) next = first_of + atomicAdd(ws.counters + 5, 1u);
+    if (!CHK(S, slot, vl.n) || !CHK(S, tile, ntl)) {  // (checked build; uniform over the CTA)
+      __syncthreads();
+      if (tid == 0) sm.item = next;
+      __syncthreads();
+      continue;
+    }
+    const int view = vl.id[slot];
+    const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
+    const int rx = 256 * (tx * TILE) + 128, ry = 256 * (ty * TILE) + 128;
+    const uint32_t bin_beg = ws.tile_off[slot * ntl + tile];
+    const int nb = (int)ws.tile_live[slot * ntl + tile];  // pruned and compacted by k_bin_prune
+    const int p0 = a.pair_begin + chunk * run, p1 = min(a.pair_begin + a.pair_count, p0 + run);
+    const int px = tx * TILE + dx, py = ty * TILE + dy;
+    const bool valid = px < S.W && py < S.H;
+    // ---- per item: the first live triangles' vertices and this pixel's target
+    for (int j = tid; j < min(nb, kDenseTri); j += M::THREADS) {
+      const int tri = (int)bin_at(S, ws, bin_beg + j);
+      sm.dense[j] = make_int4(vert_of(S, tri, 0), vert_of(S, tri, 1), vert_of(S, tri, 2), tri);
+    }
+    // live triangle j: its vertices and id
+    auto triangle = [&](int j) {
+      if (j < kDenseTri) return sm.dense[j];
+      const int tri = (int)bin_at(S, ws, bin_beg + j);
+      return make_int4(vert_of(S, tri, 0), vert_of(S, tri, 1), vert_of(S, tri, 2), tri);
+    };
+    // its projected vertices for one side of a pair (vb: the pair's first vertex record)
+    auto vertices = [&](const int4& t, long long vb, int sd, PVert (&v)[3]) {
+      const int id[3] = {t.x, t.y, t.z};
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int4 q = __ldg(ws.pverts + 2 * (vb + id[k]) + sd);
+        v[k].X = q.x;
+        v[k].Y = q.y;
+        v[k].z = __int_as_float(q.z);
+        v[k].iw = __int_as_float(q.w);
+        v[k].ok = q.x != kNotDrawn;
+      }
+    };
+    float3 tgt = f3(0.f, 0.f, 0.f);
+    if (valid) {
+      const float* tp = S.targets + (((long long)view * S.H + py) * S.W + px) * 3;
+      tgt = f3(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2));
+    }
+    float loss_acc = 0.0f;
+    int Gcap = GMAX, G = 0, nh = 0;
+    const bool windowed = M::LIT || a.pair_count > 2;  // as in fast_items
+    if (!windowed) {
+      nh = kHashNoWindow;
+      Gcap = min(Gcap, M::ACAP / nh);
+    }
+    bool first = true;
+    const uint32_t* planes0 = ws.tsign + ((long long)slot * ws.max_pairs + (p0 - a.pair_begin)) * ws.sgn_words;
+
+    for (int pg = p0; pg < p1; pg += G) {
+      const uint32_t* planes = planes0 + (long long)(pg - p0) * ws.sgn_words;
+      if (!first) {
+        fold<SH, GR>(S, ws, a, sm, 0, G, 0, nh, planes - (long long)G * ws.sgn_words);
+        __syncthreads();
+        clear_sums(sm, G, nh);
+      }
+      G = min(Gcap, p1 - pg);
+      if (!first && windowed) load_signs<SH, GR>(S, ws, sm, planes, G);
+      bool bounds = first && windowed;
+      for (int s0 = 0; s0 < G; s0 += P) {
+        const int g = s0 + stream;  // this warp's pair of the group, if there is one
+        const long long vb0 = ((long long)slot * ws.max_pairs + (pg - a.pair_begin) + s0) * S.nv;
+        // ---- R: every live triangle into the pixels of its box, both sides of the step's pairs
+        __syncthreads();  // the previous step's keys (or the item's set-up) are done with
+        for (int i = tid; i < 2 * P * TILE_PX; i += M::THREADS) keys[i] = ~0ull;
+        __syncthreads();
+        for (int st = 0; st < P && s0 + st < G; ++st) {
+          // (the next triangle's vertices are in flight while one is rasterized)
+          const long long vb1 = vb0 + (long long)st * S.nv;
+          int4 t, q[3];
+          auto fetch = [&](int t2) {
+            t = triangle(t2 >> 1);
+            const int4* p = ws.pverts + 2 * vb1 + (t2 & 1);
+            q[0] = __ldg(p + 2ll * t.x);
+            q[1] = __ldg(p + 2ll * t.y);
+            q[2] = __ldg(p + 2ll * t.z);
+          };
+          if (tid < 2 * nb) fetch(tid);
+          for (int t2 = tid; t2 < 2 * nb; t2 += M::THREADS) {
+            const int4 v0 = q[0], v1 = q[1], v2 = q[2];
+            const int id = t.w;
+            if (t2 + M::THREADS < 2 * nb) fetch(t2 + M::THREADS);
+            raster_tri(v0, v1, v2, id, rx, ry, keys + (st * 2 + (t2 & 1)) * TILE_PX);
+          }
+        }
+        __syncthreads();
+        int tri[2] = {-1, -1};
+        if (valid && g < G) {
+#pragma unroll
+          for (int sd = 0; sd < 2; ++sd) {
+            const unsigned long long k = keys[(stream * 2 + sd) * TILE_PX + dy * TILE + dx];
+            if (k != ~0ull) tri[sd] = (int)(uint32_t)k;
+          }
+        }
+        // ---- U, G: both sides' winners, set up, sampled and shaded by their pixel
+        const long long vb = vb0 + (long long)stream * S.nv;
+        int n_win = sm.wbase[NFOOT];
+        int vidA[3], vidB[3] = {-1, -1, -1};  // the visible triangles' vertices and signs: side +, side -
+        uint32_t sgA = 0, sgB = 0;
+        float3 cA, cB = f3(0.f, 0.f, 0.f);
+        uint32_t crA[NFOOT], crB[NFOOT];
+#pragma unroll
+        for (int r = 0; r < NFOOT; ++r) crB[r] = 0;
+#pragma unroll 1
+        for (int sd = 0; sd < 2; ++sd) {
+          const int vis = sd == 0 ? tri[0] : tri[1];
+          cA = cB;
+          sgA = sgB;
+#pragma unroll
+          for (int k = 0; k < 3; ++k) vidA[k] = vidB[k];
+#pragma unroll
+          for (int r = 0; r < NFOOT; ++r) crA[r] = crB[r];
+          vidB[0] = vidB[1] = vidB[2] = -1;
+          cB = f3(S.bg[0], S.bg[1], S.bg[2]);
+          float u0 = 0.f, v0 = 0.f;
+          PerspW pw;
+          float uvt[6];
+          if (vis >= 0) {
+            const int4 t = make_int4(vert_of(S, vis, 0), vert_of(S, vis, 1), vert_of(S, vis, 2), vis);
+            vidB[0] = t.x, vidB[1] = t.y, vidB[2] = t.z;
+            PVert v[3];
+            vertices(t, vb, sd, v);
+            sgB = 0;
+#pragma unroll
+            for (int k = 0; k < 3; ++k) {
+              sgB |= ((uint32_t)__ldg(ws.vbits + vb + vidB[k]) & 7u) << (3 * k);
+              const int ti = uv_of(S, t.w, k);
+              uvt[2 * k] = __ldg(S.uvs + 2 * ti);
+              uvt[2 * k + 1] = __ldg(S.uvs + 2 * ti + 1);
+            }
+            SideTri d;
+            set_up_side(d, v, rx, ry);
+            float l[3] = {0.f, 0.f, 0.f};
+            float4 z;
+            cover_lambdas(d, X, Y, l, z);
+            const float iw[3] = {v[0].iw, v[1].iw, v[2].iw};
+            pw = persp(l, iw);
+            u0 = persp_interp(pw, uvt[0], uvt[2], uvt[4]);
+            v0 = persp_interp(pw, uvt[1], uvt[3], uvt[5]);
+          }
+          if (bounds) {
+            // the item's first pairs: their side + footprints bound the windows
+            bounds = false;
+            add_bounds<SH, GR>(S, sm, vis >= 0, u0, v0);
+            __syncthreads();
+            if (tid == 0) make_windows(S, sm);
+            __syncthreads();
+            load_window<SH, GR>(S, sm);
+            n_win = sm.wbase[NFOOT];
+            nh = n_win > 0 ? kHashWindow : kHashNoWindow;
+            Gcap = min(Gcap, M::ACAP / (2 * n_win + nh));
+            G = min(G, Gcap);
+            load_signs<SH, GR>(S, ws, sm, planes, G);
+            __syncthreads();
+          }
+          if (vis < 0) continue;
+          float val[NREAD][3];
+          sample_side<SH, GR>(S, ws, sm, planes, g, sd, u0, v0, n_win, crB, val);
+          const uint32_t sg = sgB ^ (sd ? 0x1FFu : 0u);
+          float fr[6];
+          if constexpr (M::LIT) {
+            float3 p[3];
+            corner_positions(S, vidB, sg, p);
+            tri_frame(p, uvt, fr);
+          }
+          cB = shade_side<SH, GR>(S, view, val, fr, vidB, sg, pw);
+        }
+        // ---- f+ - f- and its credits
+        if (g >= G) continue;
+        const int stride = 2 * n_win + nh;
+        float df = 0.0f;
+        if (valid) {
+          float fp, fm;
+          df = loss_diff(cA, cB, tgt, fp, fm);
+          loss_acc += 0.5f * (fp + fm);
+          if (a.delta_f) a.delta_f[(((long long)slot * a.pairs + pg + g) * S.H + py) * S.W + px] = df;
+        }
+        const bool inA = vidA[0] >= 0, inB = vidB[0] >= 0;
+        if (!inA && !inB) continue;
+#pragma unroll 1
+        for (int i = 0; i < 6; ++i) {
+          const int k = i % 3;
+          const int v = i < 3 ? (k == 0 ? vidA[0] : (k == 1 ? vidA[1] : vidA[2])) : (k == 0 ? vidB[0] : (k == 1 ? vidB[1] : vidB[2]));
+          if (v < 0 || (i >= 3 && inA && (v == vidA[0] || v == vidA[1] || v == vidA[2]))) continue;
+          const uint32_t sb = (i < 3 ? sgA : sgB) >> (3 * k);
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const long long p = 3ll * v + c;
+            if (!CHK(S, p, S.chk.params)) continue;
+            atomicAdd(a.grad + p, ((sb >> c) & 1) ? -df : df);
+            atomicAdd(a.counts + p, 1u);
+          }
+        }
+        credit_texels<SH, GR>(S, ws, a, sm, planes, g, stride, n_win, nh, df, inA, inB, crA, crB);
+      }
+      __syncthreads();
+      first = false;
+    }
+    fold<SH, GR>(S, ws, a, sm, 0, G, 0, nh, planes0 + (long long)((p1 - G) - p0) * ws.sgn_words);
+    __syncthreads();
+    flush_counts<SH, GR>(S, a, sm, nh);
+    clear_sums(sm, G, nh);
+    end_item<SH, GR>(a, sm, slot, loss_acc, next);
+  }
+  add_losses<SH, GR>(a, sm, vl.n);
 }
 
 template <int SH, bool GR>
@@ -1484,6 +1856,13 @@ __global__ void __launch_bounds__(Model<SH, GR>::THREADS, Model<SH, GR>::CTAS)
     k_estimate_fast(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   fast_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true);
+}
+
+template <int SH, bool GR>
+__global__ void __launch_bounds__(Model<SH, GR>::THREADS, 1)
+    k_estimate_dense(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  dense_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true);
 }
 
 // The batched kernel keeps its asset after FastSmem, 16-byte aligned.  (Batched calls use the
@@ -1507,6 +1886,20 @@ __global__ void __launch_bounds__(Model<SH>::THREADS, Model<SH>::CTAS) k_estimat
   }
 }
 
+// and each until its heavy items run out.
+template <int SH>
+__global__ void __launch_bounds__(Model<SH>::THREADS, 1) k_estimate_dense_batch(const BatchArgs P) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  auto& sm = *reinterpret_cast<FastSmem<SH, false>*>(smem_raw);
+  BatchSmem& b = *reinterpret_cast<BatchSmem*>(smem_raw + fast_batch_off<SH>());
+  for (int ai = 0; ai < P.n; ++ai) {
+    __syncthreads();
+    load_asset(P, ai, b);
+    __syncthreads();
+    dense_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0);
+  }
+}
+
 template <int SH, bool GR>
 size_t fast_smem() {
   return sizeof(FastSmem<SH, GR>);
@@ -1523,6 +1916,25 @@ cudaError_t launch_fast_batch_t(const BatchArgs& P, int grid, cudaStream_t st) {
                                        (int)fast_batch_smem<SH>());
   if (e != cudaSuccess) return e;
   k_estimate_fast_batch<SH><<<grid, Model<SH>::THREADS, fast_batch_smem<SH>(), st>>>(P);
+  return cudaGetLastError();
+}
+
+template <int SH>
+cudaError_t launch_dense_batch_t(const BatchArgs& P, int grid, cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_estimate_dense_batch<SH>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)fast_batch_smem<SH>());
+  if (e != cudaSuccess) return e;
+  k_estimate_dense_batch<SH><<<grid, Model<SH>::THREADS, fast_batch_smem<SH>(), st>>>(P);
+  return cudaGetLastError();
+}
+
+template <int SH, bool GR>
+cudaError_t launch_dense_t(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
+                           cudaStream_t st) {
+  cudaError_t e = cudaFuncSetAttribute(k_estimate_dense<SH, GR>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)fast_smem<SH, GR>());
+  if (e != cudaSuccess) return e;
+  k_estimate_dense<SH, GR><<<grid, Model<SH, GR>::THREADS, fast_smem<SH, GR>(), st>>>(S, ws, vl, a);
   return cudaGetLastError();
 }
 
@@ -1566,6 +1978,16 @@ cudaError_t launch_fast(const SceneDev& S, const Workspace& ws, const ViewList& 
                    : launch_fast_t<SHADE_GGX, false>(S, ws, vl, a, grid, st);
 }
 
+cudaError_t launch_dense(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
+                         cudaStream_t st) {
+  if (S.shading == SHADE_UNLIT) return launch_dense_t<SHADE_UNLIT, false>(S, ws, vl, a, grid, st);
+  if (S.shading == SHADE_LAMBERT)
+    return S.grouped ? launch_dense_t<SHADE_LAMBERT, true>(S, ws, vl, a, grid, st)
+                     : launch_dense_t<SHADE_LAMBERT, false>(S, ws, vl, a, grid, st);
+  return S.grouped ? launch_dense_t<SHADE_GGX, true>(S, ws, vl, a, grid, st)
+                   : launch_dense_t<SHADE_GGX, false>(S, ws, vl, a, grid, st);
+}
+
 cudaError_t launch_prune(const SceneDev& S, const Workspace& ws, const ViewList& vl, cudaStream_t st) {
   k_bin_prune<<<dim3(n_tiles(S), vl.n), TILE_PX, 0, st>>>(S, ws, vl);
   return cudaGetLastError();
@@ -1580,6 +2002,12 @@ cudaError_t launch_fast_batch(const BatchArgs& P, int shading, int grid, cudaStr
   if (shading == SHADE_UNLIT) return launch_fast_batch_t<SHADE_UNLIT>(P, grid, st);
   if (shading == SHADE_LAMBERT) return launch_fast_batch_t<SHADE_LAMBERT>(P, grid, st);
   return launch_fast_batch_t<SHADE_GGX>(P, grid, st);
+}
+
+cudaError_t launch_dense_batch(const BatchArgs& P, int shading, int grid, cudaStream_t st) {
+  if (shading == SHADE_UNLIT) return launch_dense_batch_t<SHADE_UNLIT>(P, grid, st);
+  if (shading == SHADE_LAMBERT) return launch_dense_batch_t<SHADE_LAMBERT>(P, grid, st);
+  return launch_dense_batch_t<SHADE_GGX>(P, grid, st);
 }
 
 int fast_batch_blocks_per_sm(int shading) {

@@ -378,7 +378,7 @@ int sge_create_scene(const sge_scene_desc* desc, const sge_config* cfg, void* wo
   }
   int bps = (s->cfg.blocks_per_sm > 0) ? s->cfg.blocks_per_sm : fast_blocks_per_sm(desc->shading, s->dev.grouped);
   s->grid_fast = sms * bps;
-  s->grid_heavy = sms * estimate_blocks_per_sm(desc->shading, s->dev.grouped, group_channels(s->dev));
+  s->grid_heavy = sms;
   if (s->cfg.pairs_per_item < 0) s->cfg.pairs_per_item = 0;  // 0: the kernels choose (k_fast.cu, run_of)
   if (s->cfg.pairs_per_item > kMaxPairsPerItem) s->cfg.pairs_per_item = kMaxPairsPerItem;
   *out = s;
@@ -475,7 +475,7 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
   }
   // pairs run in blocks of at most max_pairs_per_call (the projected-vertex buffer holds one
   // block); the first block's vertex pass and sign planes run on the side stream while the caller's
-  // stream bins and prunes.  The general estimator and the background's loss go to the side stream too,
+  // stream bins and prunes.  The dense tiles' estimator and the background's loss go to the side stream too,
   // ahead of the fast estimator: their few long items overlap it instead of following it (while
   // launches are timed, they follow it on the caller's stream, as the events need).
   EstimateArgs b0 = a;
@@ -499,7 +499,7 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
     if (!timed) {
       if (e == cudaSuccess) e = cudaEventRecord(s->fork, st);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(hs, s->fork, 0);
-      if (e == cudaSuccess) e = launch_heavy(s->dev, s->ws, vl, b, s->grid_heavy, hs);
+      if (e == cudaSuccess) e = launch_dense(s->dev, s->ws, vl, b, s->grid_heavy, hs);
       if (e == cudaSuccess && loss_out && p0 == 0) e = launch_background_loss(s->dev, s->ws, vl, loss_out, hs);
       if (e == cudaSuccess) e = cudaEventRecord(s->join, hs);
     }
@@ -507,7 +507,7 @@ int estimate_grad(sge_scene* s, uint64_t seed, uint32_t iter, const uint32_t* it
     if (e == cudaSuccess) e = launch_fast(s->dev, s->ws, vl, b, s->grid_fast, st);
     if (e == cudaSuccess && ev) e = cudaEventRecord(ev[1], st);
     if (timed) {
-      if (e == cudaSuccess) e = launch_heavy(s->dev, s->ws, vl, b, s->grid_heavy, hs);
+      if (e == cudaSuccess) e = launch_dense(s->dev, s->ws, vl, b, s->grid_heavy, hs);
       if (e == cudaSuccess && ev) e = cudaEventRecord(ev[2], st);
       if (e == cudaSuccess && loss_out && p0 == 0) e = launch_background_loss(s->dev, s->ws, vl, loss_out, hs);
     } else if (e == cudaSuccess) {
@@ -825,7 +825,7 @@ int estimate_grad_batch(const sge_batch_entry* entries, int32_t n, uint64_t seed
       if (P.n == 0) continue;
       const int bps = tu.blocks_per_sm > 0 ? tu.blocks_per_sm : fast_batch_blocks_per_sm(sh);
       e = launch_fast_batch(P, sh, sms * bps, st);
-      if (e == cudaSuccess) e = launch_heavy_batch(P, sh, sms * heavy_batch_blocks_per_sm(sh), st);
+      if (e == cudaSuccess) e = launch_dense_batch(P, sh, sms, st);
     }
   }
   return e == cudaSuccess ? SGE_OK : cuda_fail(e, "sge_estimate_grad_batch");

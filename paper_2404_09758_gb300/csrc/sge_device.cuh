@@ -479,48 +479,6 @@ __device__ __forceinline__ void sample_tex_ps(const TexDev& T, const Foot& f, co
   if (T.c == 1) out[1] = out[2] = out[0];
 }
 
-// surface() with the signs of ps (side +1 or -1).
-__device__ __forceinline__ void surface_ps(const SceneDev& S, int view, int tri, const Tri& t, const long long e[3],
-                                           const PairSigns& ps, int side, Surf& out) {
-  float l[3];
-  lambdas(e, t.inv_area, l);
-  PerspW pw = persp(l, t.iw);
-  int t0 = uv_of(S, tri, 0), t1 = uv_of(S, tri, 1), t2 = uv_of(S, tri, 2);
-  float2 uv[3] = {make_float2(__ldg(S.uvs + 2 * t0), __ldg(S.uvs + 2 * t0 + 1)),
-                  make_float2(__ldg(S.uvs + 2 * t1), __ldg(S.uvs + 2 * t1 + 1)),
-                  make_float2(__ldg(S.uvs + 2 * t2), __ldg(S.uvs + 2 * t2 + 1))};
-  out.u = persp_interp(pw, uv[0].x, uv[1].x, uv[2].x);
-  out.v = persp_interp(pw, uv[0].y, uv[1].y, uv[2].y);
-  float alb[4] = {1.f, 1.f, 1.f, 1.f}, nm[4] = {0.5f, 0.5f, 1.f, 0.f}, rough[4] = {0.5f, 0.f, 0.f, 0.f},
-        metal[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-  for (int r = 0; r < MAX_READ; ++r) {
-    if (r >= S.nread) break;
-    const TexDev& T = S.rtex[r];
-    out.foot[r] = footprint(out.u, out.v, T.w, T.h);
-    if (S.foot_nearest) out.foot[r].nearest = nearest_texel(out.u, out.v, T.w, T.h);
-    float* dst = T.role == ROLE_ALBEDO ? alb : T.role == ROLE_NORMAL ? nm : T.role == ROLE_ROUGHNESS ? rough : metal;
-    sample_tex_ps(T, out.foot[r], ps, side, dst);
-  }
-  if (S.shading == SHADE_UNLIT) {
-    out.rgb = f3(alb[0], alb[1], alb[2]);
-    return;
-  }
-  float3 p[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int vi = vert_of(S, tri, k);
-    uint32_t sb = vertex_signs(ps, vi);
-    if (side < 0) sb = ~sb;
-    const float* src = S.pos + 3ll * vi;
-    p[k] = f3(__fadd_rn(__ldg(src), (sb & 1) ? -S.eps_pos : S.eps_pos),
-              __fadd_rn(__ldg(src + 1), (sb & 2) ? -S.eps_pos : S.eps_pos),
-              __fadd_rn(__ldg(src + 2), (sb & 4) ? -S.eps_pos : S.eps_pos));
-  }
-  float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
-  out.rgb = shade(S, view, alb, nm, rough, metal, p, uv, b);
-}
-
 // Project the three perturbed vertices of `tri` and set it up at reference point (rx, ry).
 __device__ __forceinline__ void setup_from_scene(const SceneDev& S, const float* m, int tri, uint64_t key,
                                                  int side, long long rx, long long ry, Tri& t) {
@@ -574,62 +532,20 @@ __device__ __forceinline__ bool cover(const Tri& t, int dx, int dy, long long e[
 __device__ __forceinline__ uint32_t vkey(int v) { return (uint32_t)v; }
 __device__ __forceinline__ uint32_t tkey(int k, int texel) { return ((uint32_t)(k + 1) << 28) | (uint32_t)texel; }
 
-// Every parameter channel of a contributor key: f(parameter index, its channel slot in a table
-// entry).  Vertex keys: x, y, z; texel keys: the texture's channels, or with GR (a group key of
-// for_each_contrib<true>) channel c of every read texture r, at slot (channels of the read
-// textures before r) + c.
-template <bool GR, typename F>
-__device__ __forceinline__ void for_each_channel(const SceneDev& S, uint32_t key, F&& f) {
-  const uint32_t kind = key >> 28, idx = key & 0x0FFFFFFFu;
-  if (kind == 0) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) f(3ll * idx + c, c);
-    return;
-  }
-  if constexpr (GR) {
-    int co = 0;
-#pragma unroll
-    for (int r = 0; r < MAX_READ; ++r) {
-      if (r >= S.nread) break;
-      const TexDev& T = S.rtex[r];
-      const long long base = T.offset + (long long)idx * T.c;
-      for (int c = 0; c < T.c; ++c) f(base + c, co + c);
-      co += T.c;
-    }
-  } else {
-    const TexDev& T = S.tex[kind - 1];
-    const long long base = T.offset + (long long)idx * T.c;
-    for (int c = 0; c < T.c; ++c) f(base + c, c);
-  }
-}
-
-// Sign of every parameter channel of a contributor key under ps: f(parameter index, slot, s = -1).
-template <bool GR, typename F>
+// Sign of every parameter channel of a contributor key under ps: f(parameter index, s = -1).
+template <typename F>
 __device__ __forceinline__ void for_each_signed_channel(const SceneDev& S, const PairSigns& ps, uint32_t key, F&& f) {
   const uint32_t kind = key >> 28, idx = key & 0x0FFFFFFFu;
   if (kind == 0) {
     const uint32_t sb = vertex_signs(ps, (int)idx);
 #pragma unroll
-    for (int c = 0; c < 3; ++c) f(3ll * idx + c, c, ((sb >> c) & 1) != 0);
+    for (int c = 0; c < 3; ++c) f(3ll * idx + c, ((sb >> c) & 1) != 0);
     return;
   }
-  if constexpr (GR) {
-    int co = 0;
-#pragma unroll
-    for (int r = 0; r < MAX_READ; ++r) {
-      if (r >= S.nread) break;
-      const TexDev& T = S.rtex[r];
-      const long long base = T.offset + (long long)idx * T.c;
-      const uint32_t sb = texel_signs(ps, T.index, idx);
-      for (int c = 0; c < T.c; ++c) f(base + c, co + c, ((sb >> c) & 1) != 0);
-      co += T.c;
-    }
-  } else {
-    const TexDev& T = S.tex[kind - 1];
-    const long long base = T.offset + (long long)idx * T.c;
-    const uint32_t sb = texel_signs(ps, T.index, idx);
-    for (int c = 0; c < T.c; ++c) f(base + c, c, ((sb >> c) & 1) != 0);
-  }
+  const TexDev& T = S.tex[kind - 1];
+  const long long base = T.offset + (long long)idx * T.c;
+  const uint32_t sb = texel_signs(ps, T.index, idx);
+  for (int c = 0; c < T.c; ++c) f(base + c, ((sb >> c) & 1) != 0);
 }
 
 __device__ __forceinline__ void key_params(const SceneDev& S, uint32_t key, long long& base, int& nch) {
@@ -648,7 +564,7 @@ __device__ __forceinline__ void key_params(const SceneDev& S, uint32_t key, long
 // both sides (tris[0] = side +, tris[1] = side -, -1 = background) of the visible
 // triangle's three welded vertices and the bilinear 2x2 footprint of each read
 // texture.  foot[sd][r] is side sd's footprint of the r-th read texture.
-template <bool GR = false, typename F>
+template <typename F>
 __device__ __forceinline__ void for_each_contrib(const SceneDev& S, const int tris[2],
                                                  const Foot (&foot)[2][MAX_READ], F&& f) {
   int vid[2][3];
@@ -665,7 +581,7 @@ __device__ __forceinline__ void for_each_contrib(const SceneDev& S, const int tr
     }
   }
 #pragma unroll
-  for (int r = 0; r < (GR ? 1 : MAX_READ); ++r) {
+  for (int r = 0; r < MAX_READ; ++r) {
     if (r >= S.nread) break;
     const int k = S.read_k[r];
     const int tw = S.tex[k].w;

@@ -16,8 +16,7 @@ constexpr int kLightBin = 256;           // bins up to this size use the fast pa
 constexpr int kMaxPairsPerItem = 64;     // longest run of pairs one work item takes
 constexpr int kRun = 8;                  // its default where the kernels do not choose a longer one
 constexpr int kBigBin = 48;              // light tiles with more live triangles go first, in shorter runs
-constexpr int kHeavyCand = 32;           // candidate triangles kept per pixel of a heavy tile
-constexpr int kCandWords = kHeavyCand / 8;  // int4 words of a pixel's candidate list
+constexpr int kCandWords = 2;            // int4 words of a pixel's candidate list, 16 8-bit indices each
 constexpr int kNotDrawn = (int)0x80000000;  // projected X of a vertex its triangles drop
 constexpr int ROLE_ALBEDO = SGE_ROLE_ALBEDO, ROLE_NORMAL = SGE_ROLE_NORMAL;
 constexpr int ROLE_ROUGHNESS = SGE_ROLE_ROUGHNESS, ROLE_METALLIC = SGE_ROLE_METALLIC;
@@ -100,9 +99,9 @@ struct Workspace {
   uint32_t* items;       // [max_views * n_tiles] (view slot << 24 | tile): light bins first, heavy from the end
                          // (light ones above kBigBin: listed in tile_cur, whose cursors are spent by then)
   uint32_t* tile_live;   // [max_views][n_tiles] triangles left at the front of each bin by k_bin_prune
-  int4* cand;            // [max_views][n_tiles][kCandWords][256] candidate triangles of each pixel: live
-                         // indices, 8-bit in the first word of a light tile, 16-bit in all words of a heavy one
-  uint8_t* ncand;        // [max_views][n_tiles][256] their number (> 16: test every live triangle)
+  int4* cand;            // [max_views][n_tiles][kCandWords][256] candidate triangles of each pixel of a light
+                         // tile: 8-bit live indices in ascending order of their smallest depth
+  uint8_t* ncand;        // [max_views][n_tiles][256] their number (more than fit: test every live triangle)
   uint32_t* counters;    // [0] light items of at most kBigBin live triangles, [6] of more, [1] their work counter, [2] total bin entries, [3] status,
                          // [4] heavy items, [5] their work counter
   unsigned long long* keys;  // [2][H*W] staged depth|ID buffers (both sides)
@@ -184,18 +183,15 @@ struct EstimateArgs {
 };
 // Iteration index of an estimate call: the device word when the call reads it at run time.
 __host__ __device__ inline uint32_t iter_of(const EstimateArgs& a) { return a.iter_dev ? *a.iter_dev : a.iter; }
-// The estimator kernels: the fast path over light bins, the general one over heavy bins (independent
+// The estimator kernels: the fast path over light bins, the dense one over heavy bins (independent
 // of each other: separate work counters, and the sums are atomics).
-cudaError_t launch_heavy(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
+cudaError_t launch_dense(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a, int grid,
                          cudaStream_t st);
 cudaError_t launch_fast(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a,
                         int grid, cudaStream_t st);
 // Perturbed, projected vertices of both sides for every (view slot, pair) of a block of pairs.
 cudaError_t launch_vertex_pass(const SceneDev& S, const Workspace& ws, const ViewList& vl, const EstimateArgs& a,
                                cudaStream_t st);
-int estimate_blocks_per_sm(int shading, int grouped, int group_channels);
-// channels of every read texture together (the channel sums of a texel-group table entry)
-int group_channels(const SceneDev& S);
 int fast_blocks_per_sm(int shading, int grouped);
 
 // Batched form of the two estimator kernels over BatchArgs' assets.
@@ -204,9 +200,8 @@ cudaError_t launch_background_loss(const SceneDev& S, const Workspace& ws, const
                                    cudaStream_t st);
 cudaError_t launch_put_desc(const AssetDesc& d, AssetDesc* dst, cudaStream_t st);
 cudaError_t launch_fast_batch(const BatchArgs& P, int shading, int grid, cudaStream_t st);
-cudaError_t launch_heavy_batch(const BatchArgs& P, int shading, int grid, cudaStream_t st);
+cudaError_t launch_dense_batch(const BatchArgs& P, int shading, int grid, cudaStream_t st);
 int fast_batch_blocks_per_sm(int shading);
-int heavy_batch_blocks_per_sm(int shading);
 
 // Staged path: render one side of one estimate into keys/uv/rgb.
 cudaError_t launch_render(const SceneDev& S, const Workspace& ws, int slot, int view, uint64_t key,
