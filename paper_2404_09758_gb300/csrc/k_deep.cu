@@ -99,7 +99,7 @@ __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& w
                                             long long ry, int dx, int dy, const int4* pv = nullptr) {
   const int ntl = n_tiles(S);
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
-  int nb = (int)(ws.tile_off[slot * ntl + tile + 1] - beg);
+  int nb = (int)ws.tile_count[slot * ntl + tile];
   // after a bin overflow (reported in the status word) the tile's list was not stored
   if ((long long)beg + nb > ws.bin_capacity) nb = 0;
 #pragma unroll

@@ -241,21 +241,6 @@ __device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_
   ws.ncand[tile_index * TILE_PX + pixel] = (uint8_t)min(n, 255);
 }
 
-// f(j) for every triangle j < cnt, in order, whose pixel span `which` reaches the warp's block of the
-// tile (columns bits 0-15, rows bits 16-31 of block) and holds this thread's pixel.
-template <typename F>
-__device__ __forceinline__ void for_spans(const uint32_t (*span)[2], int which, int cnt, uint32_t block, int dx, int dy,
-                                          F&& f) {
-  const int lane = threadIdx.x & 31;
-  for (int j0 = 0; j0 < cnt; j0 += 32) {
-    const uint32_t s = j0 + lane < cnt ? span[j0 + lane][which] & block : 0u;
-    for (uint32_t hit = __ballot_sync(0xffffffffu, (s & 0xFFFFu) && (s >> 16)); hit; hit &= hit - 1) {
-      const int j = j0 + __ffs((int)hit) - 1;
-      if (in_span(span[j][which], dx, dy)) f(j);
-    }
-  }
-}
-
 // Per (view slot, tile): drop from the bin every triangle that no perturbation of the call can
 // make visible at any pixel of the tile (outside all margin-widened pixel tests, or behind a
 // triangle that surely covers the pixel), compact the rest to the front of the bin's range,
@@ -275,9 +260,9 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
                                            int tile, int light_bin, PruneSmem& sm) {
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int ntl = n_tiles(S), n_all = n_views * ntl;
-  if ((long long)ws.tile_off[n_all] > ws.bin_capacity) return;  // overflow: the bins were not stored
+  if ((long long)ws.counters[2] > ws.bin_capacity) return;  // overflow: the bins were not stored
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
-  const int nb = (int)(ws.tile_off[slot * ntl + tile + 1] - beg);
+  const int nb = (int)ws.tile_count[slot * ntl + tile];
   if (nb == 0) return;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
   const int bx = (warp & 1) * 8, by = (warp >> 1) * 4, dx = bx + (lane & 7), dy = by + (lane >> 3);
@@ -433,20 +418,6 @@ constexpr int kHashNoWindow = 512, kHashWindow = 128;  // hashed footprints of a
 constexpr int kHashProbe = 8;
 constexpr int kDenseTri = NB * 11 / 4;
 
-// One side of a live triangle set up for one pair; 64 bytes.
-// Small (every edge function over the tile fits 32 bits: |a|, |b| < 2^16, |e0| < 2^29, so
-// |e| < 2^30 at the offsets 0..15 * 256): e = (E_0, E_1, area, flags) with E_k at the tile's first
-// pixel centre and area = E_0 + E_1 + E_2, which is the same everywhere, so edge 2 follows from the
-// other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig): the vertices relative to the first pixel
-// centre, e = (X0, Y0, X1, flags), ab = (Y1, X2, Y2, -).  Not drawn: E_0 = -1 everywhere.
-struct __align__(16) SideTri {
-  int4 e, ab;
-  float4 z;   // z_0..2, 1 / area
-  float4 iw;  // 1 / w_0..2
-};
-static_assert(sizeof(SideTri) == 64, "SideTri layout");
-constexpr int kBig = 8, kFlip = 16;  // flags; bits 0-2: edge k is not a top/left edge
-
 template <int SH, bool GR>
 struct FastSmem {
   using M = Model<SH, GR>;
@@ -486,109 +457,6 @@ struct FastSmem {
 static_assert(2 * (sizeof(FastSmem<SHADE_UNLIT, false>) + 1024) <= 228 * 1024, "two unlit CTAs must fit an SM");
 static_assert(sizeof(FastSmem<SHADE_GGX, true>) + sizeof(BatchSmem) <= 227 * 1024, "lit");
 static_assert(sizeof(FastSmem<SHADE_GGX, false>) + sizeof(BatchSmem) <= 227 * 1024, "lit");
-
-// Set up one side of a triangle from its projected vertices (rx, ry: the tile's first pixel centre).
-__device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int rx, int ry) {
-  if (!(v[0].ok && v[1].ok && v[2].ok)) {
-    d.e = make_int4(-1, 0, 0, 0);
-    d.ab = make_int4(0, 0, 0, 0);
-    return;
-  }
-  const int x0 = v[0].X - rx, x1 = v[1].X - rx, x2 = v[2].X - rx, y0 = v[0].Y - ry, y1 = v[1].Y - ry, y2 = v[2].Y - ry;
-  const int far = max(max(max(abs(x0), abs(x1)), abs(x2)), max(max(abs(y0), abs(y1)), abs(y2)));
-  float inv;
-  if (far < (1 << 14)) {
-    // vertices within 64 pixels of the tile's corner: E_k = x_a y_b - x_b y_a there, all in 32 bits
-    // (|E_k| < 2^29, |a|, |b| < 2^15)
-    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, area = e0 + e1 + (x0 * y1 - x1 * y0);
-    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
-    if (area == 0) {
-      d.e = make_int4(-1, 0, 0, 0);
-      d.ab = make_int4(0, 0, 0, 0);
-      return;
-    }
-    if (area < 0) {
-      e0 = -e0, e1 = -e1, area = -area;
-      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
-    }
-    const int flags = (a0 > 0 || (a0 == 0 && b0 > 0) ? 0 : 1) | (a1 > 0 || (a1 == 0 && b1 > 0) ? 0 : 2) |
-                      (a2 > 0 || (a2 == 0 && b2 > 0) ? 0 : 4);
-    d.e = make_int4(e0, e1, area, flags);
-    d.ab = make_int4(a0, a1, b0, b1);
-    inv = __fdiv_rn(1.0f, __int2float_rn(area));
-  } else {
-    Tri t;
-    setup_tri(v[0], v[1], v[2], rx, ry, t);
-    if (!t.ok) {
-      d.e = make_int4(-1, 0, 0, 0);
-      d.ab = make_int4(0, 0, 0, 0);
-      return;
-    }
-    int flags = 0;
-    bool small = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      flags |= (t.bias[k] ? 1 : 0) << k;
-      small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
-              t.e0[k] < (1ll << 29);
-    }
-    if (small) {
-      d.e = make_int4((int)t.e0[0], (int)t.e0[1], (int)(t.e0[0] + t.e0[1] + t.e0[2]), flags);
-      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
-    } else {
-      const bool flip = (long long)(x1 - x0) * (y2 - y0) < (long long)(y1 - y0) * (x2 - x0);
-      d.e = make_int4(x0, y0, x1, flags | kBig | (flip ? kFlip : 0));
-      d.ab = make_int4(y1, x2, y2, 0);
-    }
-    inv = t.inv_area;
-  }
-  d.z = make_float4(v[0].z, v[1].z, v[2].z, inv);
-  d.iw = make_float4(v[0].iw, v[1].iw, v[2].iw, 0.0f);
-}
-
-// Coverage of the pixel whose centre lies (X, Y) fixed-point units from the tile's first one, and
-// (covered) the barycentric weights E_k / area there as lambdas() forms them.
-__device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, float l[3], float4& z) {
-  const int4 e = t.e, ab = t.ab;
-  if (!(e.w & kBig)) {
-    const int e0 = e.x + ab.x * X + ab.z * Y, e1 = e.y + ab.y * X + ab.w * Y, e2 = e.z - e0 - e1;
-    const int lo = min(min(e0, e1), e2);
-    if (lo < 0) return false;
-    if (lo == 0 && (((e.w & 1) && e0 == 0) || ((e.w & 2) && e1 == 0) || ((e.w & 4) && e2 == 0))) return false;
-    z = t.z;
-    l[0] = __fmul_rn(__int2float_rn(e0), z.w);
-    l[1] = __fmul_rn(__int2float_rn(e1), z.w);
-    l[2] = __fmul_rn(__int2float_rn(e2), z.w);
-    return true;
-  }
-  const int vx[3] = {e.x, e.z, ab.y}, vy[3] = {e.y, ab.x, ab.z};
-  long long E[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int a = (k + 1) % 3, b = (k + 2) % 3;
-    E[k] = edge_at(vx[a], vy[a], vx[b], vy[b], X, Y);
-    if (e.w & kFlip) E[k] = -E[k];
-    if (E[k] - ((e.w >> k) & 1) < 0) return false;
-  }
-  z = t.z;
-  lambdas(E, z.w, l);
-  return true;
-}
-
-// Face normal N and u tangent T of a triangle (as shading_normal forms them): the same for every pixel.
-__device__ __forceinline__ void tri_frame(const float3 p[3], const float* uv, float* out) {
-  const float3 e1 = sub3(p[1], p[0]), e2 = sub3(p[2], p[0]);
-  const float3 N = norm3(cross3(e1, e2));
-  const float du1 = uv[2] - uv[0], dv1 = uv[3] - uv[1], du2 = uv[4] - uv[0], dv2 = uv[5] - uv[1];
-  const float det = du1 * dv2 - du2 * dv1;
-  float3 T = det != 0.0f ? f3((e1.x * dv2 - e2.x * dv1) / det, (e1.y * dv2 - e2.y * dv1) / det,
-                              (e1.z * dv2 - e2.z * dv1) / det)
-                         : e1;
-  const float nt = dot3(N, T);
-  T = norm3(f3(T.x - N.x * nt, T.y - N.y * nt, T.z - N.z * nt));
-  out[0] = N.x, out[1] = N.y, out[2] = N.z;
-  out[3] = T.x, out[4] = T.y, out[5] = T.z;
-}
 
 // The perturbed positions of live triangle j's corners (sign bits sg; side - already inverted).
 __device__ __forceinline__ void corner_positions(const SceneDev& S, const int* vid, uint32_t sg, float3 p[3]) {
@@ -1296,12 +1164,8 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
       sm.btri[j] = tri;
       sm.zminb[j] = ordered_bits(ws.tri_z[(long long)slot * S.nt + tri].x);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        sm.vid[j][k] = vert_of(S, tri, k);
-        const int ti = uv_of(S, tri, k);
-        sm.uv[j][2 * k] = __ldg(S.uvs + 2 * ti);
-        sm.uv[j][2 * k + 1] = __ldg(S.uvs + 2 * ti + 1);
-      }
+      for (int k = 0; k < 3; ++k) sm.vid[j][k] = vert_of(S, tri, k);
+      load_uvs(S, tri, sm.uv[j]);
     }
     for (int b = warp; b < TILE_PX / 32; b += M::WARPS) {
       const int dx = (b & 1) * 8 + lx, dy = (b >> 1) * 4 + ly, px = tx * TILE + dx, py = ty * TILE + dy;
@@ -1545,63 +1409,6 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
   add_losses<SH, GR>(a, sm, vl.n);
 }
 
-// A projected triangle (records of the vertex pass) into the tile's keys: the nearest (depth bits << 32 |
-// id) of each pixel centre it covers.  The arithmetic of set_up_side, cover_lambdas and
-// interp_depth, with the division left until a pixel is covered (most triangles of a dense tile cover
-// none or one).
-__device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const int4& q2, int id, int rx, int ry,
-                                           unsigned long long* keys) {
-  if (q0.x == kNotDrawn || q1.x == kNotDrawn || q2.x == kNotDrawn) return;
-  const int x0 = q0.x - rx, x1 = q1.x - rx, x2 = q2.x - rx, y0 = q0.y - ry, y1 = q1.y - ry, y2 = q2.y - ry;
-  // pixel centres in the vertex box
-  const int xl = min(x0, min(x1, x2)), xh = max(x0, max(x1, x2)), yl = min(y0, min(y1, y2)), yh = max(y0, max(y1, y2));
-  const int c0 = max((xl + 255) >> 8, 0), c1 = min(xh >> 8, TILE - 1), r0 = max((yl + 255) >> 8, 0), r1 = min(yh >> 8, TILE - 1);
-  if (c0 > c1 || r0 > r1) return;
-  auto put = [&](int x, int y, const float (&l)[3]) {
-    const float z[3] = {__int_as_float(q0.z), __int_as_float(q1.z), __int_as_float(q2.z)};
-    const unsigned long long key = ((unsigned long long)ordered_bits(interp_depth(l, z)) << 32) | (uint32_t)id;
-    unsigned long long* out = keys + y * TILE + x;
-    if (key < *(volatile unsigned long long*)out) atomicMin(out, key);
-  };
-  if (max(max(xh, yh), -min(xl, yl)) < (1 << 14)) {
-    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, e2 = x0 * y1 - x1 * y0, area = e0 + e1 + e2;
-    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
-    if (area == 0) return;
-    if (area < 0) {
-      e0 = -e0, e1 = -e1, e2 = -e2, area = -area;
-      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
-    }
-    float inv = 0.0f;
-    for (int y = r0; y <= r1; ++y) {
-      int E0 = e0 + a0 * (c0 * 256) + b0 * (y * 256), E1 = e1 + a1 * (c0 * 256) + b1 * (y * 256);
-      for (int x = c0; x <= c1; ++x, E0 += a0 * 256, E1 += a1 * 256) {
-        const int E2 = area - E0 - E1, lo = min(min(E0, E1), E2);
-        if (lo < 0) continue;
-        if (lo == 0 && ((E0 == 0 && !(a0 > 0 || (a0 == 0 && b0 > 0))) || (E1 == 0 && !(a1 > 0 || (a1 == 0 && b1 > 0))) ||
-                        (E2 == 0 && !(a2 > 0 || (a2 == 0 && b2 > 0)))))
-          continue;
-        if (inv == 0.0f) inv = __fdiv_rn(1.0f, __int2float_rn(area));
-        const float l[3] = {__fmul_rn(__int2float_rn(E0), inv), __fmul_rn(__int2float_rn(E1), inv),
-                            __fmul_rn(__int2float_rn(E2), inv)};
-        put(x, y, l);
-      }
-    }
-    return;
-  }
-  PVert v[3];
-  const int4 q[3] = {q0, q1, q2};
-#pragma unroll
-  for (int k = 0; k < 3; ++k) v[k] = PVert{q[k].x, q[k].y, __int_as_float(q[k].z), __int_as_float(q[k].w), true};
-  SideTri d;
-  set_up_side(d, v, rx, ry);
-  for (int y = r0; y <= r1; ++y)
-    for (int x = c0; x <= c1; ++x) {
-      float l[3];
-      float4 z;
-      if (cover_lambdas(d, x * 256, y * 256, l, z)) put(x, y, l);
-    }
-}
-
 // Every heavy work item of one scene's call: tiles with more live triangles than the fast path's set-ups
 // hold (dense meshes, poles, silhouettes seen edge-on).  The same steps with another split:
 // the triangles are many and small (a pixel may have a hundred candidates), so R goes by triangle: each
@@ -1770,10 +1577,8 @@ __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& 
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
               sgB |= ((uint32_t)__ldg(ws.vbits + vb + vidB[k]) & 7u) << (3 * k);
-              const int ti = uv_of(S, t.w, k);
-              uvt[2 * k] = __ldg(S.uvs + 2 * ti);
-              uvt[2 * k + 1] = __ldg(S.uvs + 2 * ti + 1);
             }
+            load_uvs(S, t.w, uvt);
             SideTri d;
             set_up_side(d, v, rx, ry);
             float l[3] = {0.f, 0.f, 0.f};

@@ -11,114 +11,181 @@ namespace sge {
 
 namespace {
 
-constexpr int RCHUNK = 128;  // triangles staged per pass (two sides fit the 48 KB static limit)
+constexpr int RCHUNK = TILE_PX;  // binned triangles staged per pass, one per thread
 
+template <int NS>
 struct RSmem {
-  Tri t[RCHUNK];
+  SideTri t[NS][RCHUNK];
+  unsigned long long keys[NS][TILE_PX];
+  uint32_t span[RCHUNK][2];  // pixels each staged triangle may cover, per side
   int tri[RCHUNK];
+  // (one side) each staged triangle's UVs and frame, where the kernel shades
+  float uv[NS == 1 ? RCHUNK : 1][6], fr[NS == 1 ? RCHUNK : 1][6];
   float m[16];
 };
 
-// Visible triangle of every pixel of a tile for `nsides` sides (side0, -side0):
-// binned triangles are set up in shared memory a chunk at a time.
+// What one side of a pixel sees: the nearest (depth bits << 32 | id), ~0 where nothing, and the barycentric
+// weights and 1 / w of that triangle there.
+struct Hit {
+  unsigned long long key;
+  float l[3], iw[3];
+  int slot;  // its place in the staged chunk, or -1
+};
+
+// This thread's pixel of the tile: 8 x 4 blocks per warp.
+__device__ __forceinline__ int pixel_dx() { return ((threadIdx.x >> 5) & 1) * 8 + (threadIdx.x & 7); }
+__device__ __forceinline__ int pixel_dy() { return (threadIdx.x >> 6) * 4 + ((threadIdx.x >> 3) & 3); }
+
+// Visible triangle of every pixel of a tile for NS sides.  A bin of one chunk is set up in shared memory
+// and each pixel tests the triangles whose box holds it (warps skip those that miss their block); a larger
+// one (dense meshes) goes triangle by triangle into the pixels of its box.  Bound by instruction issue;
+// 64-bit tests of every binned triangle at every pixel, and a second set-up per pixel, took 190 us for a view
+// of 32,768 triangles at 1024^2 (Lambert) where this takes 101 us.
 template <int NS>
-__device__ __forceinline__ void raster_tile(const SceneDev& S, const Workspace& ws, RSmem (&sm)[NS], int slot,
-                                            int tile, uint64_t key, const int (&sides)[NS],
-                                            unsigned long long (&best)[NS], long long rx, long long ry, int dx,
-                                            int dy) {
-  const int ntl = n_tiles(S);
+__device__ __forceinline__ void raster_tile(const SceneDev& S, const Workspace& ws, RSmem<NS>& sm, int slot, int tile,
+                                            uint64_t key, const int (&sides)[NS], Hit (&hit)[NS], int rx, int ry,
+                                            bool surfaces = false) {
+  const int ntl = n_tiles(S), tid = threadIdx.x, dx = pixel_dx(), dy = pixel_dy();
+  const uint32_t block = (0xFFu << (dx & 8)) | (0xF0000u << (dy & 12));
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
-  int nb = (int)(ws.tile_off[slot * ntl + tile + 1] - beg);
+  int nb = (int)ws.tile_count[slot * ntl + tile];
   // after a bin overflow (reported in the status word) the tile's list was not stored
   if ((long long)beg + nb > ws.bin_capacity) nb = 0;
 #pragma unroll
-  for (int s = 0; s < NS; ++s) best[s] = ~0ull;
-  for (int c0 = 0; c0 < nb; c0 += RCHUNK) {
-    const int cnt = min(RCHUNK, nb - c0);
-    __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-      const int tri = (int)bin_at(S, ws, beg + c0 + threadIdx.x);
+  for (int s = 0; s < NS; ++s) hit[s].key = ~0ull, hit[s].slot = -1;
+  if (nb == 0) return;
+  auto project_side = [&](int tri, int s, PVert (&v)[3]) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float3 q = perturbed_pos(S, vert_of(S, tri, k), key, sides[s]);
+      v[k] = project(sm.m, q.x, q.y, q.z, S.W, S.H, S.near_w);
+    }
+  };
+  if (nb <= RCHUNK) {
+    if (tid < nb) {
+      const int tri = (int)bin_at(S, ws, beg + tid);
+      sm.tri[tid] = tri;
 #pragma unroll
       for (int s = 0; s < NS; ++s) {
-        setup_from_scene(S, sm[0].m, tri, key, sides[s], rx, ry, sm[s].t[threadIdx.x]);
-        sm[s].tri[threadIdx.x] = sm[s].t[threadIdx.x].ok ? tri : -1;
+        PVert v[3];
+        project_side(tri, s, v);
+        set_up_side(sm.t[s][tid], v, rx, ry);
+        sm.span[tid][s] = v[0].ok && v[1].ok && v[2].ok ? box_span(v, rx, ry, 0) : 0u;
       }
+      if constexpr (NS == 1)
+        if (surfaces) load_surface(S, tri, key, sides[0], sm.uv[tid], sm.fr[tid]);
     }
     __syncthreads();
-    for (int j = 0; j < cnt; ++j) {
 #pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        const int tri = sm[s].tri[j];
-        if (tri < 0) continue;
-        long long e[3];
-        if (!cover(sm[s].t[j], dx, dy, e)) continue;
+    for (int s = 0; s < NS; ++s) {
+      int& best = hit[s].slot;
+      for_spans(sm.span, s, nb, block, dx, dy, [&](int j) {
         float l[3];
-        lambdas(e, sm[s].t[j].inv_area, l);
-        unsigned long long k = ((unsigned long long)ordered_bits(interp_depth(l, sm[s].t[j].z)) << 32) | (uint32_t)tri;
-        if (k < best[s]) best[s] = k;
+        float4 z;
+        if (!cover_lambdas(sm.t[s][j], dx * 256, dy * 256, l, z)) return;
+        const float zz[3] = {z.x, z.y, z.z};
+        const unsigned long long k = ((unsigned long long)ordered_bits(interp_depth(l, zz)) << 32) | (uint32_t)sm.tri[j];
+        if (k >= hit[s].key) return;
+        hit[s].key = k;
+        hit[s].l[0] = l[0], hit[s].l[1] = l[1], hit[s].l[2] = l[2];
+        best = j;
+      });
+      if (best >= 0) {
+        const float4 iw = sm.t[s][best].iw;
+        hit[s].iw[0] = iw.x, hit[s].iw[1] = iw.y, hit[s].iw[2] = iw.z;
       }
     }
+    return;
+  }
+#pragma unroll
+  for (int s = 0; s < NS; ++s) sm.keys[s][tid] = ~0ull;
+  __syncthreads();
+  for (int j = tid; j < nb; j += TILE_PX) {
+    const int tri = (int)bin_at(S, ws, beg + j);
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+      PVert v[3];
+      project_side(tri, s, v);
+      int4 q[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) q[k] = make_int4(v[k].ok ? v[k].X : kNotDrawn, v[k].Y, __float_as_int(v[k].z), 0);
+      raster_tri(q[0], q[1], q[2], tri, rx, ry, sm.keys[s]);
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int s = 0; s < NS; ++s) {
+    hit[s].key = sm.keys[s][dy * TILE + dx];
+    if (hit[s].key == ~0ull) continue;
+    PVert v[3];
+    project_side((int)(uint32_t)hit[s].key, s, v);
+    SideTri d;
+    set_up_side(d, v, rx, ry);
+    float4 z;
+    cover_lambdas(d, dx * 256, dy * 256, hit[s].l, z);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) hit[s].iw[k] = v[k].iw;
   }
 }
 
-__global__ void __launch_bounds__(TILE_PX) k_render(SceneDev S, Workspace ws, int slot, int view, uint64_t key,
+// Shade what a pixel sees; the triangle's UVs and frame come from the staged chunk where it is one.
+__device__ __forceinline__ void surface_hit(const SceneDev& S, int view, const RSmem<1>& sm, const Hit& hit, uint64_t key,
+                                            int side, Surf& sf) {
+  const int tri = (int)(uint32_t)hit.key;
+  if (hit.slot >= 0) {
+    surface(S, view, tri, hit.l, hit.iw, sm.uv[hit.slot], sm.fr[hit.slot], key, side, sf);
+    return;
+  }
+  float uv[6], fr[6];
+  load_surface(S, tri, key, side, uv, fr);
+  surface(S, view, tri, hit.l, hit.iw, uv, fr, key, side, sf);
+}
+
+__global__ void __launch_bounds__(TILE_PX, 4) k_render(SceneDev S, Workspace ws, int slot, int view, uint64_t key,
                                                     int side, unsigned long long* keys, float2* uv, float* rgb) {
-  __shared__ RSmem sm[1];
+  __shared__ RSmem<1> sm;
   const int tile = blockIdx.x;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int dx = threadIdx.x % TILE, dy = threadIdx.x / TILE;
-  const int px = tx * TILE + dx, py = ty * TILE + dy;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
-  if (threadIdx.x < 16) sm[0].m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
+  const int px = tx * TILE + pixel_dx(), py = ty * TILE + pixel_dy();
+  if (threadIdx.x < 16) sm.m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
-  unsigned long long best[1];
+  Hit hit[1];
   const int sides[1] = {side};
-  raster_tile<1>(S, ws, sm, slot, tile, key, sides, best, rx, ry, dx, dy);
+  raster_tile<1>(S, ws, sm, slot, tile, key, sides, hit, 256 * (tx * TILE) + 128, 256 * (ty * TILE) + 128, rgb != nullptr || uv != nullptr);
   if (px >= S.W || py >= S.H) return;
   const long long p = (long long)py * S.W + px;
-  if (keys) keys[p] = best[0];
-  if (best[0] == ~0ull) {
+  if (keys) keys[p] = hit[0].key;
+  if (hit[0].key == ~0ull) {
     if (uv) uv[p] = make_float2(0.f, 0.f);
     if (rgb) rgb[3 * p] = S.bg[0], rgb[3 * p + 1] = S.bg[1], rgb[3 * p + 2] = S.bg[2];
     return;
   }
-  const int tri = (int)(best[0] & 0xFFFFFFFFu);
-  Tri t;
-  setup_from_scene(S, sm[0].m, tri, key, side, rx, ry, t);
-  long long e[3];
-  cover(t, dx, dy, e);
+  if (!uv && !rgb) return;
   Surf sf;
-  surface(S, view, tri, t, e, key, side, sf);
+  surface_hit(S, view, sm, hit[0], key, side, sf);
   if (uv) uv[p] = make_float2(sf.u, sf.v);
   if (rgb) rgb[3 * p] = sf.rgb.x, rgb[3 * p + 1] = sf.rgb.y, rgb[3 * p + 2] = sf.rgb.z;
 }
 
 // Unperturbed render of one view reduced to its image error f = sum_p || I_p(theta) - I_p ||^2
 // (Table 1): the forward value of the autograd form.  Adds the view's sum to loss[slot].
-__global__ void __launch_bounds__(TILE_PX) k_render_loss(SceneDev S, Workspace ws, int slot, int view, float* loss) {
-  __shared__ RSmem sm[1];
+__global__ void __launch_bounds__(TILE_PX, 4) k_render_loss(SceneDev S, Workspace ws, int slot, int view, float* loss) {
+  __shared__ RSmem<1> sm;
   __shared__ float red[TILE_PX / 32];
   const int tile = blockIdx.x;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int dx = threadIdx.x % TILE, dy = threadIdx.x / TILE;
-  const int px = tx * TILE + dx, py = ty * TILE + dy;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
-  if (threadIdx.x < 16) sm[0].m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
+  const int px = tx * TILE + pixel_dx(), py = ty * TILE + pixel_dy();
+  if (threadIdx.x < 16) sm.m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
-  unsigned long long best[1];
+  Hit hit[1];
   const int sides[1] = {0};
-  raster_tile<1>(S, ws, sm, slot, tile, 0, sides, best, rx, ry, dx, dy);
+  raster_tile<1>(S, ws, sm, slot, tile, 0, sides, hit, 256 * (tx * TILE) + 128, 256 * (ty * TILE) + 128, true);
   float f = 0.0f;
   if (px < S.W && py < S.H) {
     float3 c = f3(S.bg[0], S.bg[1], S.bg[2]);
-    if (best[0] != ~0ull) {
-      const int tri = (int)(best[0] & 0xFFFFFFFFu);
-      Tri t;
-      setup_from_scene(S, sm[0].m, tri, 0, 0, rx, ry, t);
-      long long e[3];
-      cover(t, dx, dy, e);
+    if (hit[0].key != ~0ull) {
       Surf sf;
-      surface(S, view, tri, t, e, 0, 0, sf);
+      surface_hit(S, view, sm, hit[0], 0, 0, sf);
       c = sf.rgb;
     }
     const float* tp = S.targets + (((long long)view * S.H + py) * S.W + px) * 3;
@@ -137,33 +204,25 @@ __global__ void __launch_bounds__(TILE_PX) k_render_loss(SceneDev S, Workspace w
 }
 
 // Plain path, step R: both sides' depth|ID and UV buffers of one estimate.
-__global__ void __launch_bounds__(TILE_PX) k_raster_pair(SceneDev S, Workspace ws, int slot, int view, uint64_t key) {
-  __shared__ RSmem sm[2];
+__global__ void __launch_bounds__(TILE_PX, 3) k_raster_pair(SceneDev S, Workspace ws, int slot, int view, uint64_t key) {
+  __shared__ RSmem<2> sm;
   const int tile = blockIdx.x;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int dx = threadIdx.x % TILE, dy = threadIdx.x / TILE;
-  const int px = tx * TILE + dx, py = ty * TILE + dy;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
-  if (threadIdx.x < 16) sm[0].m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
+  const int px = tx * TILE + pixel_dx(), py = ty * TILE + pixel_dy();
+  if (threadIdx.x < 16) sm.m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
-  unsigned long long best[2];
+  Hit hit[2];
   const int sides[2] = {1, -1};
-  raster_tile<2>(S, ws, sm, slot, tile, key, sides, best, rx, ry, dx, dy);
+  raster_tile<2>(S, ws, sm, slot, tile, key, sides, hit, 256 * (tx * TILE) + 128, 256 * (ty * TILE) + 128);
   if (px >= S.W || py >= S.H) return;
   const long long npx = (long long)S.W * S.H, p = (long long)py * S.W + px;
 #pragma unroll
   for (int s = 0; s < 2; ++s) {
-    ws.keys[s * npx + p] = best[s];
+    ws.keys[s * npx + p] = hit[s].key;
     float2 uvv = make_float2(0.f, 0.f);
-    if (best[s] != ~0ull) {
-      const int tri = (int)(best[s] & 0xFFFFFFFFu);
-      Tri t;
-      setup_from_scene(S, sm[0].m, tri, key, sides[s], rx, ry, t);
-      long long e[3];
-      cover(t, dx, dy, e);
-      float l[3];
-      lambdas(e, t.inv_area, l);
-      PerspW pw = persp(l, t.iw);
+    if (hit[s].key != ~0ull) {
+      const int tri = (int)(uint32_t)hit[s].key;
+      PerspW pw = persp(hit[s].l, hit[s].iw);
       int t0 = uv_of(S, tri, 0), t1 = uv_of(S, tri, 1), t2 = uv_of(S, tri, 2);
       uvv.x = persp_interp(pw, __ldg(S.uvs + 2 * t0), __ldg(S.uvs + 2 * t1), __ldg(S.uvs + 2 * t2));
       uvv.y = persp_interp(pw, __ldg(S.uvs + 2 * t0 + 1), __ldg(S.uvs + 2 * t1 + 1), __ldg(S.uvs + 2 * t2 + 1));
@@ -194,8 +253,12 @@ __global__ void k_shade_delta(SceneDev S, Workspace ws, int view, uint64_t key, 
       setup_from_scene(S, m, tri, key, side, rx, ry, t);
       long long e[3];
       cover(t, px - tx * TILE, py - ty * TILE, e);
+      float l[3];
+      lambdas(e, t.inv_area, l);
+      float uv[6], fr[6];
+      load_surface(S, tri, key, side, uv, fr);
       Surf sf;
-      surface(S, view, tri, t, e, key, side, sf);
+      surface(S, view, tri, l, t.iw, uv, fr, key, side, sf);
       col[s] = sf.rgb;
     }
     const float* tp = S.targets + ((long long)view * npx + p) * 3;
@@ -236,9 +299,10 @@ __global__ void k_scatter(SceneDev S, Workspace ws, uint64_t key, float* grad, u
     long long base;
     int nch;
     key_params(S, ck, base, nch);
+    const uint32_t sb = sign_bits(key, (uint64_t)base, nch);
     for (int c = 0; c < nch; ++c) {
       if (!CHK(S, base + c, S.chk.params)) continue;
-      atomicAdd(grad + base + c, sign_neg(key, (uint64_t)(base + c)) ? -df : df);
+      atomicAdd(grad + base + c, ((sb >> c) & 1) ? -df : df);
       atomicAdd(counts + base + c, 1u);
     }
   });

@@ -24,11 +24,10 @@ __global__ void k_vertex_pass(SceneDev S, Workspace ws, ViewList vl, EstimateArg
   const uint64_t pkey = pair_key(a.seed, iter_of(a), (uint32_t)view, (uint32_t)(a.pair_begin + pb));
   const float* p = S.pos + 3ll * v;
   float qp[3], qm[3];
-  uint32_t bits = 0;
+  uint32_t bits = sign_bits(pkey, 3ull * (uint64_t)v, 3) & 7u;
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
-    const bool neg = sign_neg(pkey, 3ull * (uint64_t)v + c);
-    bits |= (uint32_t)neg << c;
+    const bool neg = (bits >> c) & 1u;
     const float th = __ldg(p + c), d = neg ? -S.eps_pos : S.eps_pos;
     qp[c] = __fadd_rn(th, d);
     qm[c] = __fadd_rn(th, -d);
@@ -51,11 +50,7 @@ __global__ void k_vertex_pass(SceneDev S, Workspace ws, ViewList vl, EstimateArg
 // one nibble per texel.
 template <int C>
 __device__ __forceinline__ uint32_t sign_word(uint64_t pkey, long long first_param, int n_texels) {
-  const uint64_t i0 = (uint64_t)first_param, blk0 = i0 >> 6;
-  const int sh = (int)(i0 & 63);
-  uint64_t x = mix64(pkey + (blk0 + 1) * kGamma) >> sh;
-  if (sh + 8 * C > 64) x |= mix64(pkey + (blk0 + 2) * kGamma) << (64 - sh);
-  const uint32_t b = (uint32_t)x;
+  const uint32_t b = sign_bits(pkey, (uint64_t)first_param, 8 * C);
   uint32_t bits;
   if (C == 4) {
     bits = b;

@@ -83,11 +83,13 @@ __device__ __forceinline__ bool sign_neg(uint64_t key, uint64_t i) {
   return ((mix64(key + ((i >> 6) + 1) * kGamma) >> (i & 63)) & 1) != 0;
 }
 
-// theta_i + side * s_i * eps_i, rounded to float (the perturbed parameter Algorithm 1 stores).
-__device__ __forceinline__ float perturb(float theta, float eps, uint64_t key, uint64_t i, int side) {
-  if (side == 0) return theta;
-  bool neg = sign_neg(key, i) != (side < 0);
-  return __fadd_rn(theta, neg ? -eps : eps);
+// Bits 0..n-1 (n <= 32): s_{i0 + j} = -1, from the one or two generator outputs they lie in.
+__device__ __forceinline__ uint32_t sign_bits(uint64_t key, uint64_t i0, int n) {
+  const uint64_t blk = i0 >> 6;
+  const int sh = (int)(i0 & 63);
+  uint64_t x = mix64(key + (blk + 1) * kGamma) >> sh;
+  if (sh + n > 64) x |= mix64(key + (blk + 2) * kGamma) << (64 - sh);
+  return (uint32_t)x;
 }
 
 // ---------------------------------------------------------------- projection
@@ -254,7 +256,7 @@ __device__ __forceinline__ int nearest_texel(float u, float v, int W, int H) {
 }
 
 // ---------------------------------------------------------------- device scene view
-// Sample all channels of perturbed texture k at footprint f (bilinear), float32.
+// Sample all channels of perturbed texture T at footprint f (bilinear), float32.
 __device__ __forceinline__ void sample_tex(const TexDev& T, const Foot& f, uint64_t key, int side,
                                            float out[4]) {
   float w[4] = {(1.0f - f.fx) * (1.0f - f.fy), f.fx * (1.0f - f.fy), (1.0f - f.fx) * f.fy,
@@ -267,10 +269,18 @@ __device__ __forceinline__ void sample_tex(const TexDev& T, const Foot& f, uint6
   for (int j = 0; j < 4; ++j) {
     long long t = (long long)ty[j] * T.w + tx[j];
     const float* src = T.ptr + t * T.c;
-    long long pi = T.offset + t * T.c;
+    uint32_t sb = 0;
+    float eps = 0.0f;
+    if (side != 0) {
+      sb = sign_bits(key, (uint64_t)(T.offset + t * T.c), T.c);
+      eps = side < 0 ? -T.eps : T.eps;
+    }
 #pragma unroll
     for (int c = 0; c < 4; ++c)
-      if (c < T.c) out[c] += w[j] * perturb(__ldg(src + c), T.eps, key, (uint64_t)(pi + c), side);
+      if (c < T.c) {
+        const float th = __ldg(src + c);
+        out[c] += w[j] * (side == 0 ? th : __fadd_rn(th, ((sb >> c) & 1) ? -eps : eps));
+      }
   }
   if (T.c == 1) out[1] = out[2] = out[0];
 }
@@ -284,28 +294,6 @@ __device__ __forceinline__ float3 cross3(float3 a, float3 b) {
 __device__ __forceinline__ float3 norm3(float3 a) {
   float n = sqrtf(dot3(a, a));
   return n > 0.0f ? f3(a.x / n, a.y / n, a.z / n) : a;
-}
-
-// Shading normal: tangent-space normal-map vector (2 t - 1) in the frame of the
-// triangle's own perturbed geometry and UVs: N face normal, T along +u
-// (Gram-Schmidt against N), B = N x T.
-__device__ __forceinline__ float3 shading_normal(const float3 p[3], const float2 uv[3], const float nm[4]) {
-  float3 e1 = sub3(p[1], p[0]), e2 = sub3(p[2], p[0]);
-  float3 N = norm3(cross3(e1, e2));
-  float du1 = uv[1].x - uv[0].x, dv1 = uv[1].y - uv[0].y;
-  float du2 = uv[2].x - uv[0].x, dv2 = uv[2].y - uv[0].y;
-  float det = du1 * dv2 - du2 * dv1;
-  float3 T = det != 0.0f ? f3((e1.x * dv2 - e2.x * dv1) / det, (e1.y * dv2 - e2.y * dv1) / det,
-                              (e1.z * dv2 - e2.z * dv1) / det)
-                         : e1;
-  float nt = dot3(N, T);
-  T = norm3(f3(T.x - N.x * nt, T.y - N.y * nt, T.z - N.z * nt));
-  float3 B = cross3(N, T);
-  float mx = 2.0f * nm[0] - 1.0f, my = 2.0f * nm[1] - 1.0f, mz = 2.0f * nm[2] - 1.0f;
-  float3 n = f3(T.x * mx + B.x * my + N.x * mz, T.y * mx + B.y * my + N.y * mz,
-                T.z * mx + B.z * my + N.z * mz);
-  if (dot3(n, n) == 0.0f) n = N;
-  return norm3(n);
 }
 
 // GGX colour for the shading normal n, light direction L and surface point P.
@@ -337,26 +325,9 @@ __device__ __forceinline__ float3 shade_ggx(const SceneDev& S, int view, float3 
   return f3(out[0], out[1], out[2]);
 }
 
-// Colour of a covered pixel.  p: perturbed world positions of the visible triangle,
-// uvs: its UVs, b: perspective-correct barycentrics, tex samples by role.
-__device__ __forceinline__ float3 shade(const SceneDev& S, int view, const float alb[4],
-                                        const float nm[4], const float rough[4], const float metal[4],
-                                        const float3 p[3], const float2 uv[3], const float b[3]) {
-  if (S.shading == SHADE_UNLIT) return f3(alb[0], alb[1], alb[2]);
-  float3 n = shading_normal(p, uv, nm);
-  float3 L = f3(S.light_dir[0], S.light_dir[1], S.light_dir[2]);
-  float ndl = fmaxf(dot3(n, L), 0.0f);
-  if (S.shading == SHADE_LAMBERT) {
-    return f3(alb[0] * (S.ambient + S.light_rgb[0] * ndl), alb[1] * (S.ambient + S.light_rgb[1] * ndl),
-              alb[2] * (S.ambient + S.light_rgb[2] * ndl));
-  }
-  return shade_ggx(S, view, n, L, alb, rough[0], metal[0],
-                   f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
-                      b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z));
-}
-
-// shade() of a lit model for a triangle whose frame (face normal N, u tangent T) and surface point P
-// (GGX) are given; the same arithmetic, the frame formed once per triangle instead of per pixel.
+// Colour of a covered pixel of a lit model.  The shading normal is the tangent-space normal-map vector
+// (2 t - 1) in the frame of the triangle's own perturbed geometry and UVs: N face normal, T along +u
+// (Gram-Schmidt against N), B = N x T (tri_frame).  P: the surface point (GGX).
 template <int SH>
 __device__ __forceinline__ float3 shade_lit(const SceneDev& S, int view, const float* alb, const float* nm, float rough,
                                             float metal, float3 N, float3 T, float3 P) {
@@ -386,43 +357,81 @@ struct Surf {
 // Perturbed world position of welded vertex vi.
 __device__ __forceinline__ float3 perturbed_pos(const SceneDev& S, int vi, uint64_t key, int side) {
   const float* p = S.pos + 3ll * vi;
-  uint64_t i0 = 3ull * (uint64_t)vi;
-  return f3(perturb(__ldg(p), S.eps_pos, key, i0, side), perturb(__ldg(p + 1), S.eps_pos, key, i0 + 1, side),
-            perturb(__ldg(p + 2), S.eps_pos, key, i0 + 2, side));
+  const float x = __ldg(p), y = __ldg(p + 1), z = __ldg(p + 2);
+  if (side == 0) return f3(x, y, z);
+  const uint32_t sb = sign_bits(key, 3ull * (uint64_t)vi, 3);
+  const float e = side < 0 ? -S.eps_pos : S.eps_pos;
+  return f3(__fadd_rn(x, (sb & 1) ? -e : e), __fadd_rn(y, (sb & 2) ? -e : e), __fadd_rn(z, (sb & 4) ? -e : e));
 }
 
-// Shade triangle `tri` at a pixel whose oriented edge functions are e[3] (set up as t).
-__device__ __forceinline__ void surface(const SceneDev& S, int view, int tri, const Tri& t,
-                                        const long long e[3], uint64_t key, int side, Surf& out) {
-  float l[3];
-  lambdas(e, t.inv_area, l);
-  PerspW pw = persp(l, t.iw);
-  int t0 = uv_of(S, tri, 0), t1 = uv_of(S, tri, 1), t2 = uv_of(S, tri, 2);
-  float2 uv[3] = {make_float2(__ldg(S.uvs + 2 * t0), __ldg(S.uvs + 2 * t0 + 1)),
-                  make_float2(__ldg(S.uvs + 2 * t1), __ldg(S.uvs + 2 * t1 + 1)),
-                  make_float2(__ldg(S.uvs + 2 * t2), __ldg(S.uvs + 2 * t2 + 1))};
-  out.u = persp_interp(pw, uv[0].x, uv[1].x, uv[2].x);
-  out.v = persp_interp(pw, uv[0].y, uv[1].y, uv[2].y);
-  float alb[4] = {1.f, 1.f, 1.f, 1.f}, nm[4] = {0.5f, 0.5f, 1.f, 0.f}, rough[4] = {0.5f, 0.f, 0.f, 0.f},
-        metal[4] = {0.f, 0.f, 0.f, 0.f};
+// Face normal N and u tangent T of a triangle : the same for every pixel.
+__device__ __forceinline__ void tri_frame(const float3 p[3], const float* uv, float* out) {
+  const float3 e1 = sub3(p[1], p[0]), e2 = sub3(p[2], p[0]);
+  const float3 N = norm3(cross3(e1, e2));
+  const float du1 = uv[2] - uv[0], dv1 = uv[3] - uv[1], du2 = uv[4] - uv[0], dv2 = uv[5] - uv[1];
+  const float det = du1 * dv2 - du2 * dv1;
+  float3 T = det != 0.0f ? f3((e1.x * dv2 - e2.x * dv1) / det, (e1.y * dv2 - e2.y * dv1) / det,
+                              (e1.z * dv2 - e2.z * dv1) / det)
+                         : e1;
+  const float nt = dot3(N, T);
+  T = norm3(f3(T.x - N.x * nt, T.y - N.y * nt, T.z - N.z * nt));
+  out[0] = N.x, out[1] = N.y, out[2] = N.z;
+  out[3] = T.x, out[4] = T.y, out[5] = T.z;
+}
+
+// The three UVs of triangle tri.
+__device__ __forceinline__ void load_uvs(const SceneDev& S, int tri, float* uv) {
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int t = uv_of(S, tri, k);
+    uv[2 * k] = __ldg(S.uvs + 2 * t);
+    uv[2 * k + 1] = __ldg(S.uvs + 2 * t + 1);
+  }
+}
+
+// Shade triangle `tri` at a pixel with barycentric weights l (iw: 1 / w of its vertices, uv: its UVs, fr:
+// its frame for the lit models).
+__device__ __forceinline__ void surface(const SceneDev& S, int view, int tri, const float l[3], const float iw[3],
+                                        const float* uv, const float* fr, uint64_t key, int side, Surf& out) {
+  PerspW pw = persp(l, iw);
+  out.u = persp_interp(pw, uv[0], uv[2], uv[4]);
+  out.v = persp_interp(pw, uv[1], uv[3], uv[5]);
+  // (read textures come in role order: albedo, normal, roughness, metallic)
+  float val[MAX_READ][4];
 #pragma unroll
   for (int r = 0; r < MAX_READ; ++r) {
     if (r >= S.nread) break;
-    const TexDev& T = S.tex[S.read_k[r]];
+    const TexDev& T = S.rtex[r];
     out.foot[r] = footprint(out.u, out.v, T.w, T.h);
     if (S.foot_nearest) out.foot[r].nearest = nearest_texel(out.u, out.v, T.w, T.h);
-    float* dst = T.role == ROLE_ALBEDO ? alb : T.role == ROLE_NORMAL ? nm : T.role == ROLE_ROUGHNESS ? rough : metal;
-    sample_tex(T, out.foot[r], key, side, dst);
+    sample_tex(T, out.foot[r], key, side, val[r]);
   }
   if (S.shading == SHADE_UNLIT) {
-    out.rgb = f3(alb[0], alb[1], alb[2]);
+    out.rgb = f3(val[0][0], val[0][1], val[0][2]);
     return;
   }
-  int v0 = vert_of(S, tri, 0), v1 = vert_of(S, tri, 1), v2 = vert_of(S, tri, 2);
-  float3 p[3] = {perturbed_pos(S, v0, key, side), perturbed_pos(S, v1, key, side),
-                 perturbed_pos(S, v2, key, side)};
-  float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
-  out.rgb = shade(S, view, alb, nm, rough, metal, p, uv, b);
+  const float3 N = f3(fr[0], fr[1], fr[2]), T = f3(fr[3], fr[4], fr[5]);
+  if (S.shading == SHADE_LAMBERT) {
+    out.rgb = shade_lit<SHADE_LAMBERT>(S, view, val[0], val[1], 0.5f, 0.0f, N, T, f3(0.f, 0.f, 0.f));
+    return;
+  }
+  float3 p[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = perturbed_pos(S, vert_of(S, tri, k), key, side);
+  const float b[3] = {pw.q[0] / pw.qs, pw.q[1] / pw.qs, pw.q[2] / pw.qs};
+  const float3 P = f3(b[0] * p[0].x + b[1] * p[1].x + b[2] * p[2].x, b[0] * p[0].y + b[1] * p[1].y + b[2] * p[2].y,
+                      b[0] * p[0].z + b[1] * p[1].z + b[2] * p[2].z);
+  out.rgb = shade_lit<SHADE_GGX>(S, view, val[0], val[1], val[2][0], val[3][0], N, T, P);
+}
+
+// The UVs and (lit models) the frame that surface() takes, for one side of an estimate.
+__device__ __forceinline__ void load_surface(const SceneDev& S, int tri, uint64_t key, int side, float* uv, float* fr) {
+  load_uvs(S, tri, uv);
+  if (S.shading == SHADE_UNLIT) return;
+  float3 p[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) p[k] = perturbed_pos(S, vert_of(S, tri, k), key, side);
+  tri_frame(p, uv, fr);
 }
 
 // ---------------------------------------------------------------- signs of one estimate, precomputed
@@ -513,6 +522,181 @@ __device__ __forceinline__ uint32_t box_span(const PVert (&v)[3], long long rx, 
 
 __device__ __forceinline__ bool in_span(uint32_t span, int dx, int dy) {
   return ((span >> dx) & (span >> (16 + dy)) & 1u) != 0;
+}
+
+// ---------------------------------------------------------------- a triangle set up for one tile
+// 64 bytes in shared memory.
+// Small (every edge function over the tile fits 32 bits: |a|, |b| < 2^16, |e0| < 2^29, so
+// |e| < 2^30 at the offsets 0..15 * 256): e = (E_0, E_1, area, flags) with E_k at the tile's first
+// pixel centre and area = E_0 + E_1 + E_2, which is the same everywhere, so edge 2 follows from the
+// other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig): the vertices relative to the first pixel
+// centre, e = (X0, Y0, X1, flags), ab = (Y1, X2, Y2, -).  Not drawn: E_0 = -1 everywhere.
+struct __align__(16) SideTri {
+  int4 e, ab;
+  float4 z;   // z_0..2, 1 / area
+  float4 iw;  // 1 / w_0..2
+};
+static_assert(sizeof(SideTri) == 64, "SideTri layout");
+constexpr int kBig = 8, kFlip = 16;  // flags; bits 0-2: edge k is not a top/left edge
+
+// Set up one side of a triangle from its projected vertices (rx, ry: the tile's first pixel centre).
+__device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int rx, int ry) {
+  if (!(v[0].ok && v[1].ok && v[2].ok)) {
+    d.e = make_int4(-1, 0, 0, 0);
+    d.ab = make_int4(0, 0, 0, 0);
+    return;
+  }
+  const int x0 = v[0].X - rx, x1 = v[1].X - rx, x2 = v[2].X - rx, y0 = v[0].Y - ry, y1 = v[1].Y - ry, y2 = v[2].Y - ry;
+  const int far = max(max(max(abs(x0), abs(x1)), abs(x2)), max(max(abs(y0), abs(y1)), abs(y2)));
+  float inv;
+  if (far < (1 << 14)) {
+    // vertices within 64 pixels of the tile's corner: E_k = x_a y_b - x_b y_a there, all in 32 bits
+    // (|E_k| < 2^29, |a|, |b| < 2^15)
+    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, area = e0 + e1 + (x0 * y1 - x1 * y0);
+    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
+    if (area == 0) {
+      d.e = make_int4(-1, 0, 0, 0);
+      d.ab = make_int4(0, 0, 0, 0);
+      return;
+    }
+    if (area < 0) {
+      e0 = -e0, e1 = -e1, area = -area;
+      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
+    }
+    const int flags = (a0 > 0 || (a0 == 0 && b0 > 0) ? 0 : 1) | (a1 > 0 || (a1 == 0 && b1 > 0) ? 0 : 2) |
+                      (a2 > 0 || (a2 == 0 && b2 > 0) ? 0 : 4);
+    d.e = make_int4(e0, e1, area, flags);
+    d.ab = make_int4(a0, a1, b0, b1);
+    inv = __fdiv_rn(1.0f, __int2float_rn(area));
+  } else {
+    Tri t;
+    setup_tri(v[0], v[1], v[2], rx, ry, t);
+    if (!t.ok) {
+      d.e = make_int4(-1, 0, 0, 0);
+      d.ab = make_int4(0, 0, 0, 0);
+      return;
+    }
+    int flags = 0;
+    bool small = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      flags |= (t.bias[k] ? 1 : 0) << k;
+      small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
+              t.e0[k] < (1ll << 29);
+    }
+    if (small) {
+      d.e = make_int4((int)t.e0[0], (int)t.e0[1], (int)(t.e0[0] + t.e0[1] + t.e0[2]), flags);
+      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
+    } else {
+      const bool flip = (long long)(x1 - x0) * (y2 - y0) < (long long)(y1 - y0) * (x2 - x0);
+      d.e = make_int4(x0, y0, x1, flags | kBig | (flip ? kFlip : 0));
+      d.ab = make_int4(y1, x2, y2, 0);
+    }
+    inv = t.inv_area;
+  }
+  d.z = make_float4(v[0].z, v[1].z, v[2].z, inv);
+  d.iw = make_float4(v[0].iw, v[1].iw, v[2].iw, 0.0f);
+}
+
+// Coverage of the pixel whose centre lies (X, Y) fixed-point units from the tile's first one, and
+// (covered) the barycentric weights E_k / area there as lambdas() forms them.
+__device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, float l[3], float4& z) {
+  const int4 e = t.e, ab = t.ab;
+  if (!(e.w & kBig)) {
+    const int e0 = e.x + ab.x * X + ab.z * Y, e1 = e.y + ab.y * X + ab.w * Y, e2 = e.z - e0 - e1;
+    const int lo = min(min(e0, e1), e2);
+    if (lo < 0) return false;
+    if (lo == 0 && (((e.w & 1) && e0 == 0) || ((e.w & 2) && e1 == 0) || ((e.w & 4) && e2 == 0))) return false;
+    z = t.z;
+    l[0] = __fmul_rn(__int2float_rn(e0), z.w);
+    l[1] = __fmul_rn(__int2float_rn(e1), z.w);
+    l[2] = __fmul_rn(__int2float_rn(e2), z.w);
+    return true;
+  }
+  const int vx[3] = {e.x, e.z, ab.y}, vy[3] = {e.y, ab.x, ab.z};
+  long long E[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    const int a = (k + 1) % 3, b = (k + 2) % 3;
+    E[k] = edge_at(vx[a], vy[a], vx[b], vy[b], X, Y);
+    if (e.w & kFlip) E[k] = -E[k];
+    if (E[k] - ((e.w >> k) & 1) < 0) return false;
+  }
+  z = t.z;
+  lambdas(E, z.w, l);
+  return true;
+}
+
+// A projected triangle (records as the vertex pass writes them) into the tile's keys: the nearest (depth bits << 32 |
+// id) of each pixel centre it covers.  The arithmetic of set_up_side, cover_lambdas and
+// interp_depth, with the division left until a pixel is covered (most triangles of a dense tile cover
+// none or one).
+__device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const int4& q2, int id, int rx, int ry,
+                                           unsigned long long* keys) {
+  if (q0.x == kNotDrawn || q1.x == kNotDrawn || q2.x == kNotDrawn) return;
+  const int x0 = q0.x - rx, x1 = q1.x - rx, x2 = q2.x - rx, y0 = q0.y - ry, y1 = q1.y - ry, y2 = q2.y - ry;
+  // pixel centres in the vertex box
+  const int xl = min(x0, min(x1, x2)), xh = max(x0, max(x1, x2)), yl = min(y0, min(y1, y2)), yh = max(y0, max(y1, y2));
+  const int c0 = max((xl + 255) >> 8, 0), c1 = min(xh >> 8, TILE - 1), r0 = max((yl + 255) >> 8, 0), r1 = min(yh >> 8, TILE - 1);
+  if (c0 > c1 || r0 > r1) return;
+  auto put = [&](int x, int y, const float (&l)[3]) {
+    const float z[3] = {__int_as_float(q0.z), __int_as_float(q1.z), __int_as_float(q2.z)};
+    const unsigned long long key = ((unsigned long long)ordered_bits(interp_depth(l, z)) << 32) | (uint32_t)id;
+    unsigned long long* out = keys + y * TILE + x;
+    if (key < *(volatile unsigned long long*)out) atomicMin(out, key);
+  };
+  if (max(max(xh, yh), -min(xl, yl)) < (1 << 14)) {
+    int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, e2 = x0 * y1 - x1 * y0, area = e0 + e1 + e2;
+    int a0 = y1 - y2, a1 = y2 - y0, a2 = y0 - y1, b0 = x2 - x1, b1 = x0 - x2, b2 = x1 - x0;
+    if (area == 0) return;
+    if (area < 0) {
+      e0 = -e0, e1 = -e1, e2 = -e2, area = -area;
+      a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
+    }
+    float inv = 0.0f;
+    for (int y = r0; y <= r1; ++y) {
+      int E0 = e0 + a0 * (c0 * 256) + b0 * (y * 256), E1 = e1 + a1 * (c0 * 256) + b1 * (y * 256);
+      for (int x = c0; x <= c1; ++x, E0 += a0 * 256, E1 += a1 * 256) {
+        const int E2 = area - E0 - E1, lo = min(min(E0, E1), E2);
+        if (lo < 0) continue;
+        if (lo == 0 && ((E0 == 0 && !(a0 > 0 || (a0 == 0 && b0 > 0))) || (E1 == 0 && !(a1 > 0 || (a1 == 0 && b1 > 0))) ||
+                        (E2 == 0 && !(a2 > 0 || (a2 == 0 && b2 > 0)))))
+          continue;
+        if (inv == 0.0f) inv = __fdiv_rn(1.0f, __int2float_rn(area));
+        const float l[3] = {__fmul_rn(__int2float_rn(E0), inv), __fmul_rn(__int2float_rn(E1), inv),
+                            __fmul_rn(__int2float_rn(E2), inv)};
+        put(x, y, l);
+      }
+    }
+    return;
+  }
+  PVert v[3];
+  const int4 q[3] = {q0, q1, q2};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) v[k] = PVert{q[k].x, q[k].y, __int_as_float(q[k].z), __int_as_float(q[k].w), true};
+  SideTri d;
+  set_up_side(d, v, rx, ry);
+  for (int y = r0; y <= r1; ++y)
+    for (int x = c0; x <= c1; ++x) {
+      float l[3];
+      float4 z;
+      if (cover_lambdas(d, x * 256, y * 256, l, z)) put(x, y, l);
+    }
+}
+
+// f(j) for every triangle j < cnt, in order, whose pixel span `which` reaches the warp's block of the
+// tile (columns bits 0-15, rows bits 16-31 of block) and holds this thread's pixel.
+template <typename F>
+__device__ __forceinline__ void for_spans(const uint32_t (*span)[2], int which, int cnt, uint32_t block, int dx, int dy,
+                                          F&& f) {
+  const int lane = threadIdx.x & 31;
+  for (int j0 = 0; j0 < cnt; j0 += 32) {
+    const uint32_t s = j0 + lane < cnt ? span[j0 + lane][which] & block : 0u;
+    for (uint32_t hit = __ballot_sync(0xffffffffu, (s & 0xFFFFu) && (s >> 16)); hit; hit &= hit - 1) {
+      const int j = j0 + __ffs((int)hit) - 1;
+      if (in_span(span[j][which], dx, dy)) f(j);
+    }
+  }
 }
 
 // Evaluate the oriented edge functions of t at offset (dx, dy) pixels from its reference point.

@@ -93,7 +93,7 @@ struct Workspace {
   int4* pverts;          // [max_views][max_pairs][nv][2] projected perturbed vertices (X, Y, z, iw), sides +/-
   uint8_t* vbits;        // [max_views][max_pairs][nv] bits 0-2: s = -1 for x,y,z; 3: side + drawable; 4: side -
   uint32_t* tile_count;  // [max_views][n_tiles]
-  uint32_t* tile_off;    // [max_views][n_tiles + 1] exclusive scan of counts
+  uint32_t* tile_off;    // [max_views][n_tiles] where each tile's bin starts
   uint32_t* tile_cur;    // [max_views][n_tiles] fill cursors
   uint32_t* bins;        // [bin_capacity] triangle ids grouped by (view slot, tile)
   uint32_t* items;       // [max_views * n_tiles] (view slot << 24 | tile): light bins first, heavy from the end
