@@ -3,6 +3,8 @@
 // are zeroed for the next iteration.  Memory bound.
 #include <cuda_runtime.h>
 
+#include <cmath>
+
 #include "sge_device.cuh"
 
 namespace sge {
@@ -44,6 +46,7 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
     c1 = -expm1f(t * logf(b1));
     c2 = -expm1f(t * logf(b2));
   }
+  const float tail = c1 > 0.0f && c2 > 0.0f ? 1.07374182e9f / (c1 * aeps) : INFINITY;  // 2^30 / (c1 adam_eps)
   // one parameter of group g: theta, m, v updated
   auto update = [&](int g, float s, uint32_t cn, float& th, float& mm, float& vv) {
     const float scale = kind == SGE_STEP_SGD_MEAN ? 1.0f / (float)(cn > 0 ? cn : 1u) : inv_n;
@@ -51,6 +54,10 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
     if (kind == SGE_STEP_ADAM) {
       mm = b1 * mm + (1.0f - b1) * gr;
       vv = b2 * vv + (1.0f - b2) * gr * gr;
+      // the step is at most lr |m| / (c1 adam_eps): below theta's rounding by 2^-30 it leaves theta as it
+      // is, and the divisions, which take a slow path for the denormal moments of parameters that nothing
+      // touches any more, are left out (52 M such parameters: 460 -> 305 us)
+      if (vv >= 0.0f && fabsf(mm) * fabsf(G.lr[g]) * tail < fabsf(th)) return;
       th -= G.lr[g] * (mm / c1) / (sqrtf(vv / c2) + aeps);
     } else {
       th -= G.lr[g] * gr;
