@@ -8,10 +8,17 @@
 // in shared memory a chunk at a time; each pixel keeps both sides' lists in registers (with each
 // entry's chunk slot, so that a bin of one chunk is not set up again to shade), then shades,
 // forms f+ - f- and credits the union of its fragments' parameters.  When the bin fits one chunk
-// the vertex credits are summed per staged triangle corner in shared memory and reach the global
+// the vertex credits are summed per staged triangle in shared memory and reach the global
 // sums once per corner at the end of the CTA; texel credits (and every credit of a larger bin) go
 // to global atomics per pixel.  Bins come from the conservative binning without pruning: a
 // fragment behind another is still listed.
+//
+// Bound by instruction issue.  The set-up uses every thread and 32-bit edge functions, warps visit only the
+// triangles whose box reaches their 8 x 4 block, a triangle whose corners are all new credits them with
+// one sum, and the union over the two lists compares footprints by the difference of their first
+// texels' ids and triangles by a 32-bit signature instead of searching lists of keys in local memory.
+// 9.3 -> 5.3 ms per call (6,144 triangles, 512^2, 8 views x 16 pairs); 3 CTAs per SM instead of 4 take 5.9 ms,
+// 5 no less, with 0.8 GB of spilled registers reaching DRAM.
 #include <cuda_runtime.h>
 
 #define SGE_FILE_ID 2  // range-check sites of this file (checked build)
@@ -27,49 +34,22 @@ constexpr int kDeepEstimates = 16384;    // estimates (grid rows) of one launch
 
 template <int NS>
 struct DeepSmem {
-  Tri t[NS][DCHUNK];
-  uint32_t span[NS][DCHUNK];  // box_span of each staged side-triangle: the pixels it may cover
-  uint8_t small[NS][DCHUNK];  // its edge functions over the tile fit 32 bits
+  SideTri t[NS][DCHUNK];
+  uint32_t span[DCHUNK][2];  // box_span of each staged side-triangle: the pixels it may cover
   int tri[DCHUNK];
-  // estimator (two sides) with a bin of one chunk: each staged triangle's welded vertices, and
-  // per corner the sum of f+ - f- and the count of the pixels that credit it through this triangle
+  float uv[DCHUNK][6];
+  // estimator (two sides) with a bin of one chunk: each staged triangle's welded vertices, and the
+  // sums of f+ - f- and the counts of the pixels that credit them through this triangle
   static constexpr int NV = NS == 2 ? DCHUNK : 1;
   int vid[NV][3];
-  float vA[NV][3];
-  uint32_t vn[NV][3];
+  uint32_t sig[NV];  // bit v mod 32 of each vertex v: triangles without a common bit share no vertex
+  float A_tri[NV];   // credited through all three corners at once
+  uint32_t n_tri[NV];
+  float A_cor[NV][3];  // and through single corners (counts: 10 bits each, at most 256 pixels)
+  uint32_t n_cor[NV];
   float m[16];
   float red[TILE_PX / 32];
 };
-
-// Every edge function of t over the tile fits 32 bits: |a|, |b| < 2^16 and |e0| < 2^29, so
-// |e0 + a 256 dx + b 256 dy| < 2^30 for the pixel offsets 0..15.
-__device__ __forceinline__ bool small_tri(const Tri& t) {
-  bool small = true;
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
-            t.e0[k] < (1ll << 29);
-  return small;
-}
-
-// cover() and lambdas() at pixel offset (dx, dy): the same integers and the same float
-// conversions, in 32-bit arithmetic for a small triangle.
-__device__ __forceinline__ bool cover_lambdas(const Tri& t, bool small, int dx, int dy, float l[3]) {
-  if (small) {
-    bool in = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const int e = (int)t.e0[k] + t.a[k] * (dx * 256) + t.b[k] * (dy * 256);
-      in = in && (e + t.bias[k] >= 0);
-      l[k] = __fmul_rn(__int2float_rn(e), t.inv_area);
-    }
-    return in;
-  }
-  long long e[3];
-  const bool in = cover(t, dx, dy, e);
-  lambdas(e, t.inv_area, l);
-  return in;
-}
 
 // Insert key k (staged at shared-memory slot q) into the ascending list L (slots P); the
 // largest key falls off the end.
@@ -95,9 +75,10 @@ __device__ __forceinline__ void deep_insert(unsigned long long (&L)[K], int (&P)
 template <int NS>
 __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& ws, DeepSmem<NS>& sm, int slot,
                                             int tile, uint64_t key, const int (&sides)[NS],
-                                            unsigned long long (&L)[NS][K], int (&P)[NS][K], long long rx,
-                                            long long ry, int dx, int dy, const int4* pv = nullptr) {
+                                            unsigned long long (&L)[NS][K], int (&P)[NS][K], int rx, int ry,
+                                            int dx, int dy, const int4* pv = nullptr) {
   const int ntl = n_tiles(S);
+  const uint32_t block = (0xFFu << (dx & 8)) | (0xF0000u << (dy & 12));  // the warp's 8 x 4 pixels
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
   int nb = (int)ws.tile_count[slot * ntl + tile];
   // after a bin overflow (reported in the status word) the tile's list was not stored
@@ -109,53 +90,68 @@ __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& w
   for (int c0 = 0; c0 < nb; c0 += DCHUNK) {
     const int cnt = min(DCHUNK, nb - c0);
     __syncthreads();
-    if ((int)threadIdx.x < cnt) {
-      const int tri = (int)bin_at(S, ws, beg + c0 + threadIdx.x);
-      sm.tri[threadIdx.x] = tri;
-      if constexpr (NS == 2) {
+    for (int t2 = threadIdx.x; t2 < NS * cnt; t2 += TILE_PX) {
+      // (two sides: neighbouring threads, whose projected vertices lie next to each other)
+      const int s = NS == 2 ? t2 & 1 : 0, j = NS == 2 ? t2 >> 1 : t2;
+      const int tri = (int)bin_at(S, ws, beg + c0 + j);
+      uint32_t sig = 0u;
+      PVert v[3];
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          sm.vid[threadIdx.x][k] = vert_of(S, tri, k);
-          sm.vA[threadIdx.x][k] = 0.0f;
-          sm.vn[threadIdx.x][k] = 0u;
+      for (int k = 0; k < 3; ++k) {
+        const int vi = vert_of(S, tri, k);
+        if (pv) {
+          const int4 q = __ldg(pv + 2 * vi + s);
+          v[k].X = q.x;
+          v[k].Y = q.y;
+          v[k].z = __int_as_float(q.z);
+          v[k].iw = __int_as_float(q.w);
+          v[k].ok = q.x != kNotDrawn;
+        } else {
+          const float3 p = perturbed_pos(S, vi, key, s == 0 ? sides[0] : sides[NS - 1]);
+          v[k] = project(sm.m, p.x, p.y, p.z, S.W, S.H, S.near_w);
         }
-      }
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        PVert v[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int vi = vert_of(S, tri, k);
-          if (pv) {
-            const int4 q = __ldg(pv + 2 * vi + s);
-            v[k].X = q.x;
-            v[k].Y = q.y;
-            v[k].z = __int_as_float(q.z);
-            v[k].iw = __int_as_float(q.w);
-            v[k].ok = q.x != kNotDrawn;
-          } else {
-            const float3 p = perturbed_pos(S, vi, key, sides[s]);
-            v[k] = project(sm.m, p.x, p.y, p.z, S.W, S.H, S.near_w);
+        if constexpr (NS == 2) {
+          if (s == 0) {
+            sm.vid[j][k] = vi;
+            sm.A_cor[j][k] = 0.0f;
+            sig |= 1u << (vi & 31);
           }
         }
-        Tri& t = sm.t[s][threadIdx.x];
-        setup_tri(v[0], v[1], v[2], rx, ry, t);
-        // a covered pixel centre lies in the triangle's vertex box
-        sm.span[s][threadIdx.x] = t.ok ? box_span(v, rx, ry, 0) : 0u;
-        sm.small[s][threadIdx.x] = t.ok && small_tri(t);
       }
+      if (s == 0) {
+        if constexpr (NS == 2) {
+          sm.sig[j] = sig;
+          sm.A_tri[j] = 0.0f;
+          sm.n_tri[j] = sm.n_cor[j] = 0u;
+        }
+        sm.tri[j] = tri;
+        load_uvs(S, tri, sm.uv[j]);
+      }
+      set_up_side(sm.t[s][j], v, rx, ry);
+      // a covered pixel centre lies in the triangle's vertex box
+      sm.span[j][s] = v[0].ok && v[1].ok && v[2].ok ? box_span(v, rx, ry, 0) : 0u;
     }
     __syncthreads();
-    for (int j = 0; j < cnt; ++j) {
-#pragma unroll
-      for (int s = 0; s < NS; ++s) {
-        if (!in_span(sm.span[s][j], dx, dy)) continue;
-        const Tri& t = sm.t[s][j];
-        if (!t.ok) continue;
+#pragma unroll 1
+    for (int s = 0; s < NS; ++s) {
+      // (one copy of the insertion for both sides: the lists change places)
+      unsigned long long (&M)[K] = L[0];
+      int (&Q)[K] = P[0];
+      for_spans(sm.span, s, cnt, block, dx, dy, [&](int j) {
         float l[3];
-        if (!cover_lambdas(t, sm.small[s][j] != 0, dx, dy, l)) continue;
-        deep_insert(L[s], P[s], ((unsigned long long)ordered_bits(interp_depth(l, t.z)) << 32) | (uint32_t)sm.tri[j],
-                    j);
+        float4 z;
+        if (!cover_lambdas(sm.t[s][j], dx * 256, dy * 256, l, z)) return;
+        const float zz[3] = {z.x, z.y, z.z};
+        deep_insert(M, Q, ((unsigned long long)ordered_bits(interp_depth(l, zz)) << 32) | (uint32_t)sm.tri[j], j);
+      });
+      if constexpr (NS == 2) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) {
+          const unsigned long long x = L[0][k];
+          L[0][k] = L[1][k], L[1][k] = x;
+          const int y = P[0][k];
+          P[0][k] = P[1][k], P[1][k] = y;
+        }
       }
     }
   }
@@ -172,7 +168,7 @@ __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& w
 template <typename F>
 __device__ __forceinline__ float3 deep_composite(const SceneDev& S, const float* m, uint64_t key, int side,
                                                  const unsigned long long (&L)[K], const int (&P)[K],
-                                                 const Tri* staged, long long rx, long long ry, int dx, int dy,
+                                                 const SideTri* staged, const float (*uvs)[6], int rx, int ry, int dx, int dy,
                                                  F&& on_fragment, const PairSigns* ps = nullptr,
                                                  const int4* pv = nullptr) {
   const TexDev& A = S.rtex[0];  // the RGBA albedo, the one texture this model reads
@@ -181,35 +177,41 @@ __device__ __forceinline__ float3 deep_composite(const SceneDev& S, const float*
   // kernel's code within the instruction cache (the lists are read from local memory instead)
 #pragma unroll 1
   for (int j = 0; j < K; ++j) {
-    if (L[j] == ~0ull) continue;
+    if (L[j] == ~0ull) break;  // (ascending: nothing follows)
     const int tri = (int)(L[j] & 0xFFFFFFFFu);
-    Tri own;
-    if (!staged) {
-      if (pv) {
-        PVert v[3];
+    float l[3] = {0.f, 0.f, 0.f}, iw[3], uv[6];
+    float4 z;
+    if (staged) {
+      const SideTri& t = staged[P[j]];
+      cover_lambdas(t, dx * 256, dy * 256, l, z);
+      iw[0] = t.iw.x, iw[1] = t.iw.y, iw[2] = t.iw.z;
 #pragma unroll
-        for (int k = 0; k < 3; ++k) {
-          const int4 q = __ldg(pv + 2 * vert_of(S, tri, k) + (side < 0 ? 1 : 0));
+      for (int k = 0; k < 6; ++k) uv[k] = uvs[P[j]][k];
+    } else {
+      PVert v[3];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        const int vi = vert_of(S, tri, k);
+        if (pv) {
+          const int4 q = __ldg(pv + 2 * vi + (side < 0 ? 1 : 0));
           v[k].X = q.x;
           v[k].Y = q.y;
           v[k].z = __int_as_float(q.z);
           v[k].iw = __int_as_float(q.w);
           v[k].ok = q.x != kNotDrawn;
+        } else {
+          const float3 p = perturbed_pos(S, vi, key, side);
+          v[k] = project(m, p.x, p.y, p.z, S.W, S.H, S.near_w);
         }
-        setup_tri(v[0], v[1], v[2], rx, ry, own);
-      } else {
-        setup_from_scene(S, m, tri, key, side, rx, ry, own);
+        iw[k] = v[k].iw;
       }
+      SideTri own;
+      set_up_side(own, v, rx, ry);
+      cover_lambdas(own, dx * 256, dy * 256, l, z);
+      load_uvs(S, tri, uv);
     }
-    const Tri& t = staged ? staged[P[j]] : own;
-    long long e[3];
-    cover(t, dx, dy, e);
-    float l[3];
-    lambdas(e, t.inv_area, l);
-    PerspW pw = persp(l, t.iw);
-    const int t0 = uv_of(S, tri, 0), t1 = uv_of(S, tri, 1), t2 = uv_of(S, tri, 2);
-    const float u = persp_interp(pw, __ldg(S.uvs + 2 * t0), __ldg(S.uvs + 2 * t1), __ldg(S.uvs + 2 * t2));
-    const float v = persp_interp(pw, __ldg(S.uvs + 2 * t0 + 1), __ldg(S.uvs + 2 * t1 + 1), __ldg(S.uvs + 2 * t2 + 1));
+    const PerspW pw = persp(l, iw);
+    const float u = persp_interp(pw, uv[0], uv[2], uv[4]), v = persp_interp(pw, uv[1], uv[3], uv[5]);
     Foot f = footprint(u, v, A.w, A.h);
     if (S.foot_nearest) f.nearest = nearest_texel(u, v, A.w, A.h);
     float a[4];
@@ -261,7 +263,7 @@ __device__ __forceinline__ void cta_add(float v, float* red, float* out) {
 }
 
 // One estimate per grid row: blockIdx.y = slot * pair_count + (pair - pair_begin).
-__global__ void __launch_bounds__(TILE_PX, 3) k_estimate_deep(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a,
+__global__ void __launch_bounds__(TILE_PX, 4) k_estimate_deep(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a,
                                                            int row0) {
   __shared__ DeepSmem<2> sm;
   const int tile = blockIdx.x;
@@ -270,9 +272,10 @@ __global__ void __launch_bounds__(TILE_PX, 3) k_estimate_deep(SceneDev S, Worksp
   const int view = vl.id[slot];
   const uint64_t key = pair_key(a.seed, iter_of(a), (uint32_t)view, (uint32_t)pair);
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int dx = threadIdx.x % TILE, dy = threadIdx.x / TILE;
+  // warps own 8 x 4 blocks
+  const int dx = ((threadIdx.x >> 5) & 1) * 8 + (threadIdx.x & 7), dy = (threadIdx.x >> 6) * 4 + ((threadIdx.x >> 3) & 3);
   const int px = tx * TILE + dx, py = ty * TILE + dy;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
+  const int rx = 256 * (tx * TILE) + 128, ry = 256 * (ty * TILE) + 128;
   if (threadIdx.x < 16) sm.m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
   unsigned long long L[2][K];
@@ -287,116 +290,129 @@ __global__ void __launch_bounds__(TILE_PX, 3) k_estimate_deep(SceneDev S, Worksp
   float lv = 0.0f;
   if (px < S.W && py < S.H) {
     const long long npx = (long long)S.W * S.H, p = (long long)py * S.W + px;
-    // the contributor set, gathered while compositing: every listed fragment's welded vertices
-    // and footprint texels, both sides, each key once
+    // every listed fragment of both sides, gathered while compositing: its triangle (chunk slot where the
+    // bin is one chunk, else id) and its footprint's code (nearest footprint: the texel)
     const TexDev& A = S.rtex[0];
-    // vertex keys and texel keys in separate lists (a key of one kind never equals one of the other)
-    uint32_t vk[2 * K * 3], tk[2 * K * 4];
-    int nvk = 0, ntk = 0;
-    auto addv = [&](uint32_t k) {
-      for (int q = 0; q < nvk; ++q)
-        if (vk[q] == k) return;
-      vk[nvk++] = k;
-    };
-    auto addt = [&](uint32_t k) {
-      for (int q = 0; q < ntk; ++q)
-        if (tk[q] == k) return;
-      tk[ntk++] = k;
-    };
-    // side +'s fragments (layer j: triangle and footprint); a side - fragment on a triangle listed
-    // there brings no new vertex, one with a footprint listed there no new texel
-    int g_tri[K], g_fp[K];
-#pragma unroll
-    for (int j = 0; j < K; ++j) g_tri[j] = -1, g_fp[j] = -1;
-    bool minus = false;
-    // a bin of one chunk: the pixel's distinct triangles by chunk slot, each with the corners whose
-    // vertex no earlier one of them has; their credits go to the shared per-corner sums
-    int ds[2 * K];
-    uint32_t dm[2 * K];
-    int nds = 0;
-    auto credit_keys = [&](int tri, const Foot& f, int j, int q) {
-      // a footprint: its first texel and whether its rows were clamped to one (x1 follows from x0)
-      const int fp = S.foot_nearest ? f.nearest : 2 * (f.y0 * A.w + f.x0) + (f.y1 != f.y0 ? 1 : 0);
-      bool tri_seen = false, fp_seen = false;
-      if (!minus) {
-        g_tri[j] = tri;
-        g_fp[j] = fp;
-      } else {
-#pragma unroll
-        for (int i = 0; i < K; ++i) {
-          tri_seen = tri_seen || g_tri[i] == tri;
-          fp_seen = fp_seen || (g_tri[i] >= 0 && g_fp[i] == fp);
-        }
-      }
-      if (!tri_seen && resident) {
-        uint32_t mask = 7u;
-        for (int i = 0; i < nds; ++i) {
-          const int o = ds[i];
-#pragma unroll
-          for (int k = 0; k < 3; ++k)
-#pragma unroll
-            for (int kk = 0; kk < 3; ++kk)
-              if (sm.vid[q][k] == sm.vid[o][kk]) mask &= ~(1u << k);
-        }
-        ds[nds] = q;
-        dm[nds++] = mask;
-      } else if (!tri_seen) {
-#pragma unroll
-        for (int v = 0; v < 3; ++v) addv(vkey(vert_of(S, tri, v)));
-      }
-      if (fp_seen) return;
+    uint32_t code[2 * K];
+    int who[2 * K], n = 0;
+    bool odd = false;  // some footprint wraps, is clamped to a row or is one texel wide
+    auto fragment = [&](int tri, const Foot& f, int, int q) {
       if (S.foot_nearest) {
-        addt(tkey(A.index, f.nearest));
-        return;
+        code[n] = (uint32_t)f.nearest;
+      } else {
+        code[n] = (uint32_t)(f.y0 * A.w + f.x0) | (f.y1 == f.y0 ? kOneRow : 0u);
+        odd = odd || f.y1 == f.y0 || f.x1 != f.x0 + 1;
       }
-      addt(tkey(A.index, f.y0 * A.w + f.x0));
-      addt(tkey(A.index, f.y0 * A.w + f.x1));
-      addt(tkey(A.index, f.y1 * A.w + f.x0));
-      addt(tkey(A.index, f.y1 * A.w + f.x1));
+      who[n++] = resident ? q : tri;
     };
-    const float3 cp = deep_composite(S, sm.m, key, 1, L[0], P[0], resident ? sm.t[0] : nullptr, rx, ry, dx, dy,
-                                     credit_keys, &ps, pv);
-    minus = true;
-    const float3 cm = deep_composite(S, sm.m, key, -1, L[1], P[1], resident ? sm.t[1] : nullptr, rx, ry, dx, dy,
-                                     credit_keys, &ps, pv);
+    const float3 cp = deep_composite(S, sm.m, key, 1, L[0], P[0], resident ? sm.t[0] : nullptr, sm.uv, rx, ry, dx, dy,
+                                     fragment, &ps, pv);
+    const float3 cm = deep_composite(S, sm.m, key, -1, L[1], P[1], resident ? sm.t[1] : nullptr, sm.uv, rx, ry, dx, dy,
+                                     fragment, &ps, pv);
     const float* tp = S.targets + ((long long)view * npx + p) * 3;
     float fp, fm;
     const float df = loss_diff(cp, cm, f3(__ldg(tp), __ldg(tp + 1), __ldg(tp + 2)), fp, fm);
     lv = 0.5f * (fp + fm);
     if (a.delta_f) a.delta_f[((long long)slot * a.pairs + pair) * npx + p] = df;
-    for (int i = 0; i < nds; ++i) {
-      const int q = ds[i];
+    // vertices of the distinct listed triangles, each vertex once
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const int q = who[i];
+      uint32_t mask = 7u;
+#pragma unroll 1
+      for (int j = 0; j < i && mask; ++j) {
+        const int o = who[j];
+        if (o == q) mask = 0u;
+        else if (!resident || (sm.sig[q] & sm.sig[o])) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        if (!((dm[i] >> k) & 1u)) continue;
-        atomicAdd(&sm.vA[q][k], df);
-        atomicAdd(&sm.vn[q][k], 1u);
+          for (int k = 0; k < 3; ++k)
+#pragma unroll
+            for (int kk = 0; kk < 3; ++kk)
+              if ((resident ? sm.vid[q][k] : vert_of(S, q, k)) == (resident ? sm.vid[o][kk] : vert_of(S, o, kk)))
+                mask &= ~(1u << k);
+        }
       }
-    }
-    // one count per key (k_expand_counts gives it to every channel after the call), a signed
-    // sum per channel (RGBA texels of an 8-byte aligned gradient: two vector reductions)
-    const bool pairs4 = A.c == 4 && ((reinterpret_cast<uintptr_t>(a.grad + A.offset) & 7) == 0);
-    for (int q = 0; q < nvk + ntk; ++q) {
-      const uint32_t kq = q < nvk ? vk[q] : tk[q - nvk];
-      const uint32_t kind = kq >> 28, idx = kq & 0x0FFFFFFFu;
-      const long long kc = kind == 0 ? (long long)idx : ws.kc_off[kind - 1] + idx;
-      if (CHK(S, kc, ws.n_kcount)) atomicAdd(ws.kcount + kc, 1u);
-      if (kind != 0 && pairs4) {
-        // an RGBA texel: two 2-channel reductions
-        const long long base = A.offset + (long long)idx * 4;
-        const uint32_t sb = texel_signs(ps, A.index, idx);
-        if (CHK(S, base + 3, S.chk.params)) {
-          atomicAdd(reinterpret_cast<float2*>(a.grad + base),
-                    make_float2((sb & 1) ? -df : df, (sb & 2) ? -df : df));
-          atomicAdd(reinterpret_cast<float2*>(a.grad + base + 2),
-                    make_float2((sb & 4) ? -df : df, (sb & 8) ? -df : df));
+      if (resident) {
+        if (mask == 7u) {
+          atomicAdd(&sm.A_tri[q], df);
+          atomicAdd(&sm.n_tri[q], 1u);
+        } else if (mask) {
+          uint32_t add = 0u;
+#pragma unroll
+          for (int k = 0; k < 3; ++k)
+            if ((mask >> k) & 1u) {
+              atomicAdd(&sm.A_cor[q][k], df);
+              add |= 1u << (10 * k);
+            }
+          atomicAdd(&sm.n_cor[q], add);
         }
         continue;
       }
-      for_each_signed_channel(S, ps, kq, [&](long long p, bool neg) {
-        if (!CHK(S, p, S.chk.params)) return;
-        atomicAdd(a.grad + p, neg ? -df : df);
-      });
+      for (; mask; mask &= mask - 1) {
+        const int v = vert_of(S, q, __ffs((int)mask) - 1);
+        if (CHK(S, v, ws.n_kcount)) atomicAdd(ws.kcount + v, 1u);
+        const uint32_t sb = vertex_signs(ps, v);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const long long p = 3ll * v + c;
+          if (CHK(S, p, S.chk.params)) atomicAdd(a.grad + p, ((sb >> c) & 1) ? -df : df);
+        }
+      }
+    }
+    // texels of the distinct footprints, each texel once: one count per key (k_expand_counts gives it to
+    // every channel after the call), a signed sum per channel (RGBA texels of an 8-byte aligned gradient:
+    // two vector reductions)
+    const bool pairs4 = A.c == 4 && ((reinterpret_cast<uintptr_t>(a.grad + A.offset) & 7) == 0);
+    auto credit_texel = [&](int id) {
+      const long long kc = ws.kc_off[A.index] + id;
+      if (CHK(S, kc, ws.n_kcount)) atomicAdd(ws.kcount + kc, 1u);
+      const long long base = A.offset + (long long)id * A.c;
+      const uint32_t sb = texel_signs(ps, A.index, id);
+      if (pairs4) {
+        if (!CHK(S, base + 3, S.chk.params)) return;
+        atomicAdd(reinterpret_cast<float2*>(a.grad + base), make_float2((sb & 1) ? -df : df, (sb & 2) ? -df : df));
+        atomicAdd(reinterpret_cast<float2*>(a.grad + base + 2), make_float2((sb & 4) ? -df : df, (sb & 8) ? -df : df));
+        return;
+      }
+      for (int c = 0; c < A.c; ++c)
+        if (CHK(S, base + c, S.chk.params)) atomicAdd(a.grad + base + c, ((sb >> c) & 1) ? -df : df);
+    };
+    const uint32_t w = (uint32_t)A.w;
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      uint32_t mask = S.foot_nearest ? 1u : 15u;
+      if (!odd || S.foot_nearest) {
+        // ids c, c + 1, c + w, c + w + 1: membership in an earlier footprint by id differences
+#pragma unroll 1
+        for (int j = 0; j < i && mask; ++j) {
+          const uint32_t d = code[i] - code[j];
+          if (d == 0u) mask = 0u;
+          else if (!S.foot_nearest && d + w + 1u <= 2u * w + 2u) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+              const uint32_t s = d + (q & 1) + (q & 2 ? w : 0u);
+              if (s <= 1u || s - w <= 1u) mask &= ~(1u << q);
+            }
+          }
+        }
+        for (; mask; mask &= mask - 1) {
+          const int q = __ffs((int)mask) - 1;
+          credit_texel((int)(code[i] + (q & 1) + (q & 2 ? w : 0u)));
+        }
+        continue;
+      }
+      const Quad Q(code[i], A.w);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (Q.repeats(q)) mask &= ~(1u << q);
+#pragma unroll 1
+      for (int j = 0; j < i && mask; ++j) {
+        const Quad E(code[j], A.w);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (E.holds(Q, q)) mask &= ~(1u << q);
+      }
+      for (; mask; mask &= mask - 1) credit_texel(Q.texel(__ffs((int)mask) - 1, A.w));
     }
   }
   if (resident) {
@@ -406,11 +422,11 @@ __global__ void __launch_bounds__(TILE_PX, 3) k_estimate_deep(SceneDev S, Worksp
     if (t < nb) {
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        const uint32_t n = sm.vn[t][k];
+        const uint32_t n = sm.n_tri[t] + ((sm.n_cor[t] >> (10 * k)) & 1023u);
         if (!n) continue;
         const int v = sm.vid[t][k];
         if (CHK(S, v, ws.n_kcount)) atomicAdd(ws.kcount + v, n);
-        const float A = sm.vA[t][k];
+        const float A = sm.A_tri[t] + sm.A_cor[t][k];
         if (A == 0.0f) continue;
         const uint32_t sb = vertex_signs(ps, v);
 #pragma unroll
@@ -431,9 +447,10 @@ __global__ void __launch_bounds__(TILE_PX) k_render_deep(SceneDev S, Workspace w
   __shared__ DeepSmem<1> sm;
   const int tile = blockIdx.x;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int dx = threadIdx.x % TILE, dy = threadIdx.x / TILE;
+  // warps own 8 x 4 blocks
+  const int dx = ((threadIdx.x >> 5) & 1) * 8 + (threadIdx.x & 7), dy = (threadIdx.x >> 6) * 4 + ((threadIdx.x >> 3) & 3);
   const int px = tx * TILE + dx, py = ty * TILE + dy;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
+  const int rx = 256 * (tx * TILE) + 128, ry = 256 * (ty * TILE) + 128;
   if (threadIdx.x < 16) sm.m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
   unsigned long long L[1][K];
@@ -448,7 +465,7 @@ __global__ void __launch_bounds__(TILE_PX) k_render_deep(SceneDev S, Workspace w
       for (int j = 0; j < K; ++j) deep[j * npx + p] = L[0][j];
     }
     if (rgb || loss) {
-      const float3 c = deep_composite(S, sm.m, key, side, L[0], P[0], resident ? sm.t[0] : nullptr, rx, ry, dx, dy,
+      const float3 c = deep_composite(S, sm.m, key, side, L[0], P[0], resident ? sm.t[0] : nullptr, sm.uv, rx, ry, dx, dy,
                                       [](int, const Foot&, int, int) {});
       if (rgb) rgb[3 * p] = c.x, rgb[3 * p + 1] = c.y, rgb[3 * p + 2] = c.z;
       if (loss) {

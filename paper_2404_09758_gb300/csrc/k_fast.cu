@@ -486,28 +486,9 @@ __device__ __forceinline__ int window_texel(const int4& win, int t, int w) {
 }
 
 // Credit code of a pixel's side in footprint r: the window cell (the slot of the footprint's first
-// texel), or with kOut the first texel's id, kOneRow: its rows are clamped to one, and r above.
-constexpr uint32_t kOut = 1u << 31, kOneRow = 1u << 28, EMPTY = 0xFFFFFFFFu;
+// texel), or with kOut a footprint code (Quad) and r above it.
+constexpr uint32_t kOut = 1u << 31, EMPTY = 0xFFFFFFFFu;
 constexpr int kFootShift = 29;
-
-// The texels of the footprint named by a texel id code (w: the texture's width): columns x0, x1, rows
-// y0, y1 (equal where it has one column or row).
-struct Quad {
-  int x0, x1, y0, y1;
-  __device__ __forceinline__ Quad(uint32_t cr, int w) {
-    const int id = (int)(cr & 0x0FFFFFFFu);
-    y0 = id / w;
-    x0 = id - y0 * w;
-    x1 = x0 + 1 == w ? 0 : x0 + 1;
-    y1 = (cr & kOneRow) ? y0 : y0 + 1;
-  }
-  __device__ __forceinline__ int texel(int q, int w) const { return (q & 2 ? y1 : y0) * w + (q & 1 ? x1 : x0); }
-  __device__ __forceinline__ bool repeats(int q) const { return ((q & 2) && y1 == y0) || ((q & 1) && x1 == x0); }
-  __device__ __forceinline__ bool holds(const Quad& o, int q) const {
-    const int x = q & 1 ? o.x1 : o.x0, y = q & 2 ? o.y1 : o.y0;
-    return (x == x0 || x == x1) && (y == y0 || y == y1);
-  }
-};
 
 // Sign bits of texel t's channels (bit c: s = -1) in one texture's sign plane of an estimate.
 __device__ __forceinline__ uint32_t plane_nibble(const SceneDev& S, const uint32_t* planes, int off, int t) {

@@ -247,6 +247,26 @@ __device__ __forceinline__ Foot footprint(float u, float v, int W, int H) {
   return f;
 }
 
+// The texels of the footprint named by a code, its first texel's id and kOneRow where its rows are clamped to
+// one (w: the texture's width): columns x0, x1, rows y0, y1 (equal where it has one column or row).
+constexpr uint32_t kOneRow = 1u << 28;
+struct Quad {
+  int x0, x1, y0, y1;
+  __device__ __forceinline__ Quad(uint32_t cr, int w) {
+    const int id = (int)(cr & 0x0FFFFFFFu);
+    y0 = id / w;
+    x0 = id - y0 * w;
+    x1 = x0 + 1 == w ? 0 : x0 + 1;
+    y1 = (cr & kOneRow) ? y0 : y0 + 1;
+  }
+  __device__ __forceinline__ int texel(int q, int w) const { return (q & 2 ? y1 : y0) * w + (q & 1 ? x1 : x0); }
+  __device__ __forceinline__ bool repeats(int q) const { return ((q & 2) && y1 == y0) || ((q & 1) && x1 == x0); }
+  __device__ __forceinline__ bool holds(const Quad& o, int q) const {
+    const int x = q & 1 ? o.x1 : o.x0, y = q & 2 ? o.y1 : o.y0;
+    return (x == x0 || x == x1) && (y == y0 || y == y1);
+  }
+};
+
 // The texel whose square holds the sample point, (floor(u W) wrapped, floor(v H) clamped): the one
 // texel Section 4.4 credits ("nearest" footprint); its id y W + x.
 __device__ __forceinline__ int nearest_texel(float u, float v, int W, int H) {
@@ -715,22 +735,6 @@ __device__ __forceinline__ bool cover(const Tri& t, int dx, int dy, long long e[
 // (its x, y, z), kind k+1 = texel of texture k (all its channels).
 __device__ __forceinline__ uint32_t vkey(int v) { return (uint32_t)v; }
 __device__ __forceinline__ uint32_t tkey(int k, int texel) { return ((uint32_t)(k + 1) << 28) | (uint32_t)texel; }
-
-// Sign of every parameter channel of a contributor key under ps: f(parameter index, s = -1).
-template <typename F>
-__device__ __forceinline__ void for_each_signed_channel(const SceneDev& S, const PairSigns& ps, uint32_t key, F&& f) {
-  const uint32_t kind = key >> 28, idx = key & 0x0FFFFFFFu;
-  if (kind == 0) {
-    const uint32_t sb = vertex_signs(ps, (int)idx);
-#pragma unroll
-    for (int c = 0; c < 3; ++c) f(3ll * idx + c, ((sb >> c) & 1) != 0);
-    return;
-  }
-  const TexDev& T = S.tex[kind - 1];
-  const long long base = T.offset + (long long)idx * T.c;
-  const uint32_t sb = texel_signs(ps, T.index, idx);
-  for (int c = 0; c < T.c; ++c) f(base + c, ((sb >> c) & 1) != 0);
-}
 
 __device__ __forceinline__ void key_params(const SceneDev& S, uint32_t key, long long& base, int& nch) {
   uint32_t kind = key >> 28, idx = key & 0x0FFFFFFFu;
