@@ -83,7 +83,17 @@ __global__ void k_bin_rect_count(SceneDev S, Workspace ws, ViewList vl) {
   // unit for the two snaps and slack for float rounding; "full" = unbounded.
   int margin = 0x7FFFFFFF;
   if (!full && !skip && disp < 1.0e4f) margin = (int)ceilf(disp * 256.0f * 1.002f) + 4;
-  ws.tri_margin[(long long)slot * S.nt + tri] = margin;
+  if (ws.tri_rec && !skip) {
+    PVert v[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float* p = S.pos + 3ll * vi[k];
+      v[k] = project(m, p[0], p[1], p[2], S.W, S.H, S.near_w);
+    }
+    int4* rec = ws.tri_rec + 2 * ((long long)slot * S.nt + tri);
+    rec[0] = make_int4(v[0].X, v[0].Y, v[1].X, v[1].Y);
+    rec[1] = make_int4(v[2].X, v[2].Y, margin, v[0].ok && v[1].ok && v[2].ok ? 1 : 0);
+  }
   // interpolated depth of a covered pixel lies between the vertex depths; slack for float rounding
   ws.tri_z[(long long)slot * S.nt + tri] =
       make_float2(zlo - (1e-6f + 1e-5f * fabsf(zlo)), zhi + (1e-6f + 1e-5f * fabsf(zhi)));

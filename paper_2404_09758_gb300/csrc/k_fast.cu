@@ -97,68 +97,60 @@ __device__ __forceinline__ long long sure_reach(int a, int b, int margin) {
 }
 
 // ---------------------------------------------------------------- bin pruning
-// Unperturbed set-up of a bin triangle with its perturbation margin; a triangle not drawable
-// unperturbed (zero area, a vertex behind the near limit) gets tri = -2: a perturbed version may still
-// be drawable, so it is a candidate everywhere.  span: the pixels that may pass surely_covers (inside
-// the triangle) and maybe_visible (inside its edges pushed out by the margin terms); a triangle those
-// tests always fail / pass: none / all.
-__device__ __forceinline__ void stage_unperturbed(const SceneDev& S, const Workspace& ws, const float* m, int slot,
-                                                  int tri, long long rx, long long ry, TriS& d, uint32_t (&span)[2]) {
-  PVert v[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const float3 q = perturbed_pos(S, vert_of(S, tri, k), 0, 0);
-    v[k] = project(m, q.x, q.y, q.z, S.W, S.H, S.near_w);
-  }
-  Tri t;
-  setup_tri(v[0], v[1], v[2], rx, ry, t);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    d.a[k] = t.a[k];
-    d.b[k] = t.b[k];
-  }
-  d.tri = t.ok ? tri : -2;
-  d.margin = ws.tri_margin[(long long)slot * S.nt + tri];
-  const bool can = d.tri >= 0 && d.margin != 0x7FFFFFFF;
-  bool small = can && d.margin < (1 << 10);
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    small = small && abs(t.a[k]) < (1 << 16) && abs(t.b[k]) < (1 << 16) && t.e0[k] > -(1ll << 29) &&
-            t.e0[k] < (1ll << 29);
-  d.small = small;
+// Unperturbed set-up of a bin triangle from its record (k_bin.cu) with its perturbation margin; a triangle
+// not drawable unperturbed (zero area, a vertex behind the near limit) gets tri = -2: a perturbed version
+// may still be drawable, so it is a candidate everywhere.  span: the pixels that may pass surely_covers
+// (inside the triangle) and maybe_covers (inside its edges pushed out by the margin terms); a triangle
+// those tests always fail / pass: none / all.
+__device__ __forceinline__ void stage_unperturbed(const int4& r0, const int4& r1, int tri, int rx, int ry, TriS& d,
+                                                  uint32_t (&span)[2]) {
+  const bool ok = r1.w != 0;
+  const PVert v[3] = {PVert{r0.x, r0.y, 0.f, 0.f, ok}, PVert{r0.z, r0.w, 0.f, 0.f, ok}, PVert{r1.x, r1.y, 0.f, 0.f, ok}};
+  SideTri t;
+  set_up_side(t, v, rx, ry);
+  const bool drawable = !(t.e.x == -1 && t.e.z == 0 && t.e.w == 0);
+  d.tri = drawable ? tri : -2;
+  d.margin = r1.z;
+  const bool can = drawable && d.margin != 0x7FFFFFFF;
   span[0] = 0u;
   span[1] = 0xFFFFFFFFu;
-  if (can) {
-    span[1] = box_span(v, rx, ry, d.margin);
-    // a pixel inside all three edges by their reach has E_0 + E_1 + E_2 = area above the reaches' sum:
-    // triangles no wider than the perturbation moves them surely cover nothing
-    long long need = 0;
+  d.small = 0;
+  if (!can) return;
+  span[1] = box_span(v, rx, ry, d.margin);
+  long long e[3];
+  if (!(t.e.w & kBig)) {
+    e[0] = t.e.x, e[1] = t.e.y, e[2] = t.e.z - t.e.x - t.e.y;
+    d.a[0] = t.ab.x, d.a[1] = t.ab.y, d.a[2] = -t.ab.x - t.ab.y;
+    d.b[0] = t.ab.z, d.b[1] = t.ab.w, d.b[2] = -t.ab.z - t.ab.w;
+    d.small = d.margin < (1 << 10);
+  } else {
+    Tri g;
+    setup_tri(v[0], v[1], v[2], rx, ry, g);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) need += sure_reach(t.a[k], t.b[k], d.margin);
-    if (t.e0[0] + t.e0[1] + t.e0[2] > need) span[0] = box_span(v, rx, ry, 0);
+    for (int k = 0; k < 3; ++k) e[k] = g.e0[k], d.a[k] = g.a[k], d.b[k] = g.b[k];
   }
+  // a pixel inside all three edges by their reach has E_0 + E_1 + E_2 = area above the reaches' sum:
+  // triangles no wider than the perturbation moves them surely cover nothing
+  long long reach[3];
+#pragma unroll
+  for (int k = 0; k < 3; ++k) reach[k] = sure_reach(d.a[k], d.b[k], d.margin);
+  if (e[0] + e[1] + e[2] > reach[0] + reach[1] + reach[2]) span[0] = box_span(v, rx, ry, 0);
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    if (small) {
-      // (|reach| < 2^28 and |margin terms| < 2^28 here, so both fit)
-      d.es[k] = (int)(t.e0[k] - sure_reach(t.a[k], t.b[k], d.margin) - 1);
-      d.em[k] = (int)t.e0[k] + d.margin * (abs(t.a[k]) + abs(t.b[k]));
+    if (d.small) {
+      // (reach and the margin terms stay below 2^28 here, so both fit)
+      d.es[k] = (int)(e[k] - reach[k] - 1);
+      d.em[k] = (int)e[k] + d.margin * (abs(d.a[k]) + abs(d.b[k]));
     }
   }
-  if (!small) {
+  if (!d.small) {
 #pragma unroll
-    for (int k = 0; k < 3; ++k) d.e0[k] = t.e0[k];
+    for (int k = 0; k < 3; ++k) d.e0[k] = e[k];
   }
 }
 
-// Does every perturbed version of t cover pixel (dx, dy)?  (Inside its span[0], so t is drawable and its
-// margin bounded.)
+// Not small: does every perturbed version of t cover pixel (dx, dy)?  (t drawable, its margin bounded.)
 __device__ __forceinline__ bool surely_covers(const TriS& t, int dx, int dy) {
-  if (t.small) {
-    const int X = dx * 256, Y = dy * 256;
-    return min(min(t.es[0] + t.a[0] * X + t.b[0] * Y, t.es[1] + t.a[1] * X + t.b[1] * Y),
-               t.es[2] + t.a[2] * X + t.b[2] * Y) >= 0;
-  }
   bool sure = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
@@ -168,20 +160,13 @@ __device__ __forceinline__ bool surely_covers(const TriS& t, int dx, int dy) {
   return sure;
 }
 
-// May some perturbed version of t cover pixel (dx, dy)?  No if its margin-widened edge functions miss it.
+// Not small: may some perturbed version of t cover pixel (dx, dy)?  (t drawable, its margin bounded.)
 __device__ __forceinline__ bool maybe_covers(const TriS& t, int dx, int dy) {
-  if (t.small) {
-    const int X = dx * 256, Y = dy * 256;
-    return min(min(t.em[0] + t.a[0] * X + t.b[0] * Y, t.em[1] + t.a[1] * X + t.b[1] * Y),
-               t.em[2] + t.a[2] * X + t.b[2] * Y) >= 0;
-  }
-  if (t.tri == -2 || t.margin == 0x7FFFFFFF) return true;
   bool maybe = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     const long long e = t.e0[k] + (long long)t.a[k] * (dx * 256) + (long long)t.b[k] * (dy * 256);
-    const long long reach = (long long)t.margin * (long long)(abs(t.a[k]) + abs(t.b[k]));
-    maybe = maybe && (e + reach >= 0);
+    maybe = maybe && (e + (long long)t.margin * (long long)(abs(t.a[k]) + abs(t.b[k])) >= 0);
   }
   return maybe;
 }
@@ -190,12 +175,12 @@ struct PruneSmem {
   TriS t[NB];
   float2 zr[NB];
   uint32_t id[NB];
-  uint32_t key[NB];    // ordered bits of the smallest depths, by bin position
-  uint8_t live[NB];
-  uint8_t remap[NB];   // compacted position of each live entry of a single-chunk bin
-  uint8_t cl[CMAX][TILE_PX];  // each pixel's first CMAX candidates (column per thread)
+  uint32_t key[NB];      // ordered bits of the smallest depths, by bin position
   uint32_t span[NB][2];  // the pixels of the sure-cover and the maybe-visible tests
-  float m[16];
+  uint32_t zsure[TILE_PX];         // ordered bits of the nearest far end of a surely covering triangle
+  uint32_t mask[NB / 32][TILE_PX]; // each pixel's candidates among the staged triangles
+  uint8_t live[NB];
+  uint8_t remap[NB];     // compacted position of each live entry of a single-chunk bin
   int wsum[TILE_PX / 32];
 };
 
@@ -218,27 +203,58 @@ __device__ __forceinline__ int block_prefix(int flag, int* wsum, int* total) {
   return before + in_warp;
 }
 
-// Store a pixel's list (this thread's column of cl, n entries found): the first CMAX as 8-bit indices in
-// list order, and its length min(n, 255).
-__device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_index, int pixel, const uint8_t* col,
-                                            int n) {
-  static_assert(CMAX == 16 * kCandWords, "sixteen indices to an int4 word");
-  const long long ci = tile_index * kCandWords * TILE_PX + pixel;
-  const int k = min(n, CMAX);
-  for (int w = 0; w * 16 < k; ++w) {
-    uint32_t v[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      v[i] = 0u;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int at = w * 16 + i * 4 + q;
-        if (at < k) v[i] |= (uint32_t)col[at * TILE_PX] << (8 * q);
+// The staged triangles j < cnt go into the pixels they reach, inside columns <= cmax and rows <= rmax.
+// kMark = 0: the nearest far end of a triangle that surely covers each pixel; 1: the candidates that may be
+// visible, not wholly behind that (a triangle whose perturbed versions are not bounded is one everywhere).
+// kStep threads take the rows of one triangle's box in turn; a warp's lanes meet again after each triangle (left
+// to themselves they ran its loops one after another: 2.0 G instead of 1.3 G warp instructions at 1 M triangles).
+template <int kMark, int kStep>
+__device__ __forceinline__ void for_rows(PruneSmem& sm, int cnt, int cmax, int rmax) {
+  for (int u0 = threadIdx.x & ~31; u0 < cnt * kStep; u0 += TILE_PX) {
+    const int u = u0 + (threadIdx.x & 31), j = u / kStep;
+    const uint32_t s = u < cnt * kStep ? sm.span[j][kMark] : 0u;
+    // (columns and rows are both empty or both not)
+    const int r0 = __ffs((int)(s >> 16)) - 1 + u % kStep, r1 = min(15 - __clz((int)s), rmax);
+    if (s && r0 <= r1) {
+      const int c0 = __ffs((int)s) - 1, c1 = min(31 - __clz((int)(s & 0xFFFFu)), cmax);
+      const TriS& t = sm.t[j];
+      const float z = kMark ? sm.zr[j].x : sm.zr[j].y;
+      const uint32_t bit = 1u << (j & 31);
+      uint32_t* mask = sm.mask[j >> 5];
+      if (t.small) {
+        const uint32_t zb = kMark || z == z ? ordered_bits(z) : 0xFFFFFFFFu;
+        const int* e = kMark ? t.em : t.es;
+        const int a0 = t.a[0] * 256, a1 = t.a[1] * 256, a2 = t.a[2] * 256, b0 = t.b[0] * 256, b1 = t.b[1] * 256, b2 = t.b[2] * 256;
+        bool live = false;
+        for (int row = r0; row <= r1; row += kStep) {
+          int e0 = e[0] + a0 * c0 + b0 * row, e1 = e[1] + a1 * c0 + b1 * row, e2 = e[2] + a2 * c0 + b2 * row;
+          for (int p = row * TILE + c0; p <= row * TILE + c1; ++p, e0 += a0, e1 += a1, e2 += a2) {
+            if (min(min(e0, e1), e2) < 0) continue;
+            if (!kMark) {
+              atomicMin(&sm.zsure[p], zb);
+            } else if (zb <= sm.zsure[p]) {
+              live = true;
+              atomicOr(mask + p, bit);
+            }
+          }
+        }
+        if (live) sm.live[j] = 1;
+      } else {
+        const bool all = t.tri == -2 || t.margin == 0x7FFFFFFF;
+        for (int row = r0; row <= r1; row += kStep)
+          for (int c = c0; c <= c1; ++c) {
+            const int p = row * TILE + c;
+            if (!kMark) {
+              if (z == z && surely_covers(t, c, row)) atomicMin(&sm.zsure[p], ordered_bits(z));
+            } else if (all || (maybe_covers(t, c, row) && ordered_bits(z) <= sm.zsure[p])) {
+              sm.live[j] = 1;
+              atomicOr(mask + p, bit);
+            }
+          }
       }
     }
-    ws.cand[ci + w * TILE_PX] = make_int4((int)v[0], (int)v[1], (int)v[2], (int)v[3]);
+    __syncwarp();
   }
-  ws.ncand[tile_index * TILE_PX + pixel] = (uint8_t)min(n, 255);
 }
 
 // Per (view slot, tile): drop from the bin every triangle that no perturbation of the call can
@@ -252,88 +268,81 @@ __device__ __forceinline__ void store_cands(const Workspace& ws, long long tile_
 // perturbation (ordered bits, a total order with NaN; ties by bin position), so each pixel's list
 // is: the estimator stops at the first candidate wholly behind the nearest covering one found.
 // Bound by instruction issue.  The bin is ranked once per tile (a comparison per pair of triangles)
-// instead of every pixel sorting its list; warps own 8 x 4 blocks and visit only the triangles whose
-// box reaches the block (a ballot over 32 boxes at a time).  Before / after on GB300: 29.4 / 22.7 us
-// (2,048 triangles, 256^2, one view), 260 / 180 us (8,192 triangles, 512^2, 8 views), 9,955 / 5,650 us (1 M
+// instead of every pixel sorting its list; the triangles go by rows into the pixels of their boxes instead of
+// every pixel testing every triangle, a pixel's candidates are the bits of a mask, which come out in
+// rank order, and the projected vertices come from the binning.  Before any of this / now: 29.4 / 21.1 us (2,048
+// triangles, 256^2, one view), 260 / 135 us (8,192 triangles, 512^2, 8 views), 9,955 / 1,965 us (1 M
 // triangles, 2048^2, 4 views).
-__device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& ws, int n_views, int view, int slot,
-                                           int tile, int light_bin, PruneSmem& sm) {
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+template <int kStep>
+__device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& ws, int n_views, int slot, int tile,
+                                           int light_bin, PruneSmem& sm) {
+  const int tid = threadIdx.x;
   const int ntl = n_tiles(S), n_all = n_views * ntl;
   if ((long long)ws.counters[2] > ws.bin_capacity) return;  // overflow: the bins were not stored
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
   const int nb = (int)ws.tile_count[slot * ntl + tile];
   if (nb == 0) return;
   const int tx = tile % S.tiles_x, ty = tile / S.tiles_x;
-  const int bx = (warp & 1) * 8, by = (warp >> 1) * 4, dx = bx + (lane & 7), dy = by + (lane >> 3);
-  const uint32_t block = (0xFFu << bx) | (0xF0000u << by);
-  const int pixel = dy * TILE + dx;
-  const bool valid = tx * TILE + dx < S.W && ty * TILE + dy < S.H;
-  const long long rx = 256ll * (tx * TILE) + 128, ry = 256ll * (ty * TILE) + 128;
+  const int cmax = min(TILE, S.W - tx * TILE) - 1, rmax = min(TILE, S.H - ty * TILE) - 1;
+  const int rx = 256 * (tx * TILE) + 128, ry = 256 * (ty * TILE) + 128;
   const long long tix = (long long)slot * ntl + tile;
-  if (tid < 16) sm.m[tid] = S.mvp[16 * view + tid];
+  sm.zsure[tid] = ordered_bits(3.4e38f);
   // a chunk of the bin set up; ranked: in ascending order of the smallest depths
   auto stage = [&](int c0, int cnt, bool ranked) {
     int tri = 0, at = tid;
     float2 zr = make_float2(0.f, 0.f);
+    int4 r0, r1;
     if (tid < cnt) {
       tri = (int)bin_at(S, ws, beg + c0 + tid);
-      zr = ws.tri_z[(long long)slot * S.nt + tri];
+      const long long i = (long long)slot * S.nt + tri;
+      zr = ws.tri_z[i];
+      r0 = ws.tri_rec[2 * i];
+      r1 = ws.tri_rec[2 * i + 1];
       sm.key[tid] = ordered_bits(zr.x);
     }
+#pragma unroll
+    for (int w = 0; w < NB / 32; ++w) sm.mask[w][tid] = 0u;
     __syncthreads();
     if (tid < cnt) {
       if (ranked) {
+        // ties by bin position: entries of the warps before count when equal too, of the warps behind not
         const uint32_t k = sm.key[tid];
+        const int w0 = tid & ~31, w1 = min(w0 + 32, cnt);
         at = 0;
-#pragma unroll 4
-        for (int j = 0; j < cnt; ++j) {
-          const uint32_t o = sm.key[j];
-          at += o < k || (o == k && j < tid) ? 1 : 0;
-        }
+#pragma unroll 8
+        for (int j = 0; j < w0; ++j) at += sm.key[j] <= k ? 1 : 0;
+#pragma unroll 8
+        for (int j = w0; j < w1; ++j) at += sm.key[j] < k || (sm.key[j] == k && j < tid) ? 1 : 0;
+#pragma unroll 8
+        for (int j = w1; j < cnt; ++j) at += sm.key[j] < k ? 1 : 0;
       }
       sm.id[at] = (uint32_t)tri;
       sm.zr[at] = zr;
       sm.live[at] = 0;
-      stage_unperturbed(S, ws, sm.m, slot, tri, rx, ry, sm.t[at], sm.span[at]);
+      stage_unperturbed(r0, r1, tri, rx, ry, sm.t[at], sm.span[at]);
     }
     __syncthreads();
   };
+  // mark the staged triangles some pixel may see, and each pixel's
+  auto mark = [&](int cnt) {
+    for_rows<1, kStep>(sm, cnt, cmax, rmax);
+    __syncthreads();
+  };
   const bool single = nb <= NB;
-  // pass 1: nearest far end of the triangles that surely cover this pixel
-  float zsure = 3.4e38f;
+  // pass 1: nearest far end of the triangles that surely cover each pixel
   for (int c0 = 0; c0 < nb; c0 += NB) {
     const int cnt = min(NB, nb - c0);
     __syncthreads();
     stage(c0, cnt, single);
-    for_spans(sm.span, 0, cnt, block, dx, dy, [&](int j) {
-      if (surely_covers(sm.t[j], dx, dy)) zsure = fminf(zsure, sm.zr[j].y);
-    });
+    for_rows<0, kStep>(sm, cnt, cmax, rmax);
   }
-  // pass 2: mark and compact the triangles some pixel may see (a single chunk is still staged;
-  // its pixels' candidate lists are found on the way, by staged position, and renumbered below)
-  uint8_t* col = &sm.cl[0][tid];
-  int n_cl = 0;  // candidates found for this pixel (the first CMAX kept in sm.cl)
+  // pass 2: mark and compact the triangles some pixel may see (a single chunk is still staged)
   int n_live = 0;
   for (int c0 = 0; c0 < nb; c0 += NB) {
     const int cnt = min(NB, nb - c0);
-    if (!single) {
-      __syncthreads();
-      stage(c0, cnt, false);
-    }
-    for_spans(sm.span, 1, cnt, block, dx, dy, [&](int j) {
-      if (!valid || !(single || !sm.live[j])) return;
-      // wholly behind the far end of a triangle that surely covers the pixel: not visible (a triangle whose
-      // perturbed versions are not bounded is a candidate everywhere)
-      const bool bounded = sm.t[j].small || !(sm.t[j].tri == -2 || sm.t[j].margin == 0x7FFFFFFF);
-      if (!maybe_covers(sm.t[j], dx, dy) || (bounded && !(sm.zr[j].x <= zsure))) return;
-      sm.live[j] = 1;
-      if (single) {
-        if (n_cl < CMAX) col[n_cl * TILE_PX] = (uint8_t)j;
-        ++n_cl;
-      }
-    });
     __syncthreads();
+    if (!single) stage(c0, cnt, false);
+    mark(cnt);
     const int f = tid < cnt ? sm.live[tid] : 0;
     int total;
     const int pos = block_prefix(f, sm.wsum, &total);
@@ -352,43 +361,59 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
     else ws.items[n_all - 1 - (int)atomicAdd(ws.counters + 4, 1u)] = it;
   }
   if (n_live > light_bin) return;  // (the dense estimator takes no lists)
-  if (single) {
-    __syncthreads();
-    // staged positions -> live indices (each pixel renumbers its own column)
-    const int k = min(n_cl, CMAX);
-    for (int q = 0; q < k; ++q) col[q * TILE_PX] = sm.remap[col[q * TILE_PX]];
-  } else if (n_live > 0) {
+  if (!single && n_live > 0) {
     // pass 3 (bins of more than one chunk): the live triangles are one chunk, ranked by depth here and
     // stored back in that order, and each pixel's candidates are found among them
     __syncthreads();
     stage(0, n_live, true);
-    if (tid < n_live && CHK(S, (long long)beg + tid, S.chk.bins)) ws.bins[beg + tid] = sm.id[tid];
-    for_spans(sm.span, 1, n_live, block, dx, dy, [&](int j) {
-      if (!valid) return;
-      const bool bounded = sm.t[j].small || !(sm.t[j].tri == -2 || sm.t[j].margin == 0x7FFFFFFF);
-      if (!maybe_covers(sm.t[j], dx, dy) || (bounded && !(sm.zr[j].x <= zsure))) return;
-      if (n_cl < CMAX) col[n_cl * TILE_PX] = (uint8_t)j;
-      ++n_cl;
-    });
+    if (tid < n_live) {
+      sm.remap[tid] = (uint8_t)tid;
+      if (CHK(S, (long long)beg + tid, S.chk.bins)) ws.bins[beg + tid] = sm.id[tid];
+    }
+    mark(n_live);
+  } else {
+    __syncthreads();
   }
-  store_cands(ws, tix, pixel, col, n_cl);
+  // this pixel's list: the live indices of its mask's bits, in rank order, the first CMAX of them
+  static_assert(CMAX == 16 * kCandWords, "sixteen indices to an int4 word");
+  int n = 0;
+  uint32_t word[4] = {0u, 0u, 0u, 0u};
+  int4* out = ws.cand + tix * kCandWords * TILE_PX + tid;
+#pragma unroll 1
+  for (int w = 0; w < NB / 32 && w * 32 < nb; ++w)
+    for (uint32_t m = sm.mask[w][tid]; m; m &= m - 1) {
+      if (n < CMAX) {
+        const uint32_t bits = (uint32_t)sm.remap[w * 32 + __ffs((int)m) - 1] << (8 * (n & 3));
+        const int i = (n >> 2) & 3;
+#pragma unroll
+        for (int x = 0; x < 4; ++x) word[x] |= x == i ? bits : 0u;
+        if ((n & 15) == 15) {
+          out[(n >> 4) * TILE_PX] = make_int4((int)word[0], (int)word[1], (int)word[2], (int)word[3]);
+          word[0] = word[1] = word[2] = word[3] = 0u;
+        }
+      }
+      ++n;
+    }
+  if (n < CMAX && (n & 15)) out[(n >> 4) * TILE_PX] = make_int4((int)word[0], (int)word[1], (int)word[2], (int)word[3]);
+  ws.ncand[tix * TILE_PX + tid] = (uint8_t)min(n, 255);
 }
 
-__global__ void __launch_bounds__(TILE_PX, 4) k_bin_prune(SceneDev S, Workspace ws, ViewList vl) {
+template <int kStep, int kCtas>
+__global__ void __launch_bounds__(TILE_PX, kCtas) k_bin_prune(SceneDev S, Workspace ws, ViewList vl) {
   __shared__ PruneSmem sm;
-  prune_tile(S, ws, vl.n, vl.id[blockIdx.y], blockIdx.y, blockIdx.x, ws.light_bin, sm);
+  prune_tile<kStep>(S, ws, vl.n, blockIdx.y, blockIdx.x, ws.light_bin, sm);
 }
 
 // Batched form: every (tile, view slot, asset) of a batched call in one launch; each CTA reads
 // its asset's scene and workspace from the asset's launch descriptor in device memory.
-__global__ void __launch_bounds__(TILE_PX, 4) k_bin_prune_batch(const BatchArgs P) {
+__global__ void __launch_bounds__(TILE_PX, 7) k_bin_prune_batch(const BatchArgs P) {
   __shared__ PruneSmem sm;
   const BatchAsset& A = P.as[blockIdx.z];
   const int slot = blockIdx.y;
   if (slot >= A.n_views) return;
   const AssetDesc& D = *A.desc;
   if ((int)blockIdx.x >= D.S.tiles_x * D.S.tiles_y) return;
-  prune_tile(D.S, D.ws, A.n_views, A.view[slot], slot, blockIdx.x, P.light_bin, sm);
+  prune_tile<4>(D.S, D.ws, A.n_views, slot, blockIdx.x, P.light_bin, sm);
 }
 
 // ---------------------------------------------------------------- the estimator
@@ -1774,8 +1799,19 @@ cudaError_t launch_dense(const SceneDev& S, const Workspace& ws, const ViewList&
                    : launch_dense_t<SHADE_GGX, false>(S, ws, vl, a, grid, st);
 }
 
+// Grids of up to two CTAs per SM run at once and take as long as their fullest tile: a row per thread and
+// registers without spills.  Larger grids are bound by issue: 7 resident CTAs in 32 registers, whose barriers
+// hide behind one another, and 4 threads to a triangle, so small boxes leave few lanes idle (8,192 triangles,
+// 512^2, 8 views / 1 M triangles, 2048^2, 4 views: 7 CTAs 135 us / 1.96 ms, 5 CTAs 169 us / 2.29 ms; 8 threads
+// to a triangle 127 us / 2.16 ms; one wave of 256 tiles: 21.1 us with 16 threads, 24.1 us with 4).
+constexpr int kPruneOneWave = 2 * 152;
+
 cudaError_t launch_prune(const SceneDev& S, const Workspace& ws, const ViewList& vl, cudaStream_t st) {
-  k_bin_prune<<<dim3(n_tiles(S), vl.n), TILE_PX, 0, st>>>(S, ws, vl);
+  const dim3 grid(n_tiles(S), vl.n);
+  if ((long long)grid.x * grid.y <= kPruneOneWave)
+    k_bin_prune<16, 2><<<grid, TILE_PX, 0, st>>>(S, ws, vl);
+  else
+    k_bin_prune<4, 7><<<grid, TILE_PX, 0, st>>>(S, ws, vl);
   return cudaGetLastError();
 }
 

@@ -60,7 +60,7 @@ namespace {
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
 struct Layout {
-  size_t tri_rect, tri_margin, tri_z, pverts, vbits, tile_count, tile_off, tile_cur, bins, items, counters, keys, uvbuf, dfbuf,
+  size_t tri_rect, tri_rec, tri_z, pverts, vbits, tile_count, tile_off, tile_cur, bins, items, counters, keys, uvbuf, dfbuf,
       desc, tile_live, cand, ncand, tsign, kcount, total;
   int max_views, max_pairs;
   long long bin_capacity;
@@ -147,13 +147,13 @@ int make_layout(const sge_scene_desc* d, const sge_config* c, Layout& L) {
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o = align256(o + bytes); return at; };
   L.tri_rect = take(sizeof(int4) * (size_t)L.max_views * d->n_triangles);
-  L.tri_margin = take(sizeof(int) * (size_t)L.max_views * d->n_triangles);
+  L.tri_rec = take(sizeof(int4) * 2 * (size_t)L.max_views * d->n_triangles);
   L.tri_z = take(sizeof(float2) * (size_t)L.max_views * d->n_triangles);
   L.max_pairs = (c && c->max_pairs_per_call > 0) ? c->max_pairs_per_call : 64;
   L.pverts = take(sizeof(int4) * 2 * (size_t)L.max_views * L.max_pairs * d->n_vertices);
   L.vbits = take((size_t)L.max_views * L.max_pairs * d->n_vertices);
   L.tile_count = take(sizeof(uint32_t) * (size_t)(L.max_views * ntl));
-  L.tile_off = take(sizeof(uint32_t) * (size_t)(L.max_views * ntl + 1));
+  L.tile_off = take(sizeof(uint32_t) * (size_t)(L.max_views * ntl));
   L.tile_cur = take(sizeof(uint32_t) * (size_t)(L.max_views * ntl));
   L.bins = take(sizeof(uint32_t) * (size_t)L.bin_capacity);
   L.items = take(sizeof(uint32_t) * (size_t)(L.max_views * ntl));
@@ -324,7 +324,7 @@ int sge_create_scene(const sge_scene_desc* desc, const sge_config* cfg, void* wo
   char* base = static_cast<char*>(workspace);
   Workspace& w = s->ws;
   w.tri_rect = reinterpret_cast<int4*>(base + L.tri_rect);
-  w.tri_margin = reinterpret_cast<int*>(base + L.tri_margin);
+  w.tri_rec = reinterpret_cast<int4*>(base + L.tri_rec);
   w.tri_z = reinterpret_cast<float2*>(base + L.tri_z);
   w.pverts = reinterpret_cast<int4*>(base + L.pverts);
   w.vbits = reinterpret_cast<uint8_t*>(base + L.vbits);

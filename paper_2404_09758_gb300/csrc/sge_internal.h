@@ -88,7 +88,8 @@ struct ViewList {
 // Scratch carved out of the caller's workspace.
 struct Workspace {
   int4* tri_rect;        // [max_views][nt] tile rectangle (x0,y0,x1,y1) of each triangle's bin span
-  int* tri_margin;       // [max_views][nt] perturbation margin of each triangle, fixed-point units
+  int4* tri_rec;         // [max_views][nt][2] each triangle unperturbed, for the pruning: (X0, Y0, X1, Y1), (X2, Y2,
+                         // perturbation margin in fixed-point units, drawable); NULL: not written
   float2* tri_z;         // [max_views][nt] depth interval of each triangle under any perturbation
   int4* pverts;          // [max_views][max_pairs][nv][2] projected perturbed vertices (X, Y, z, iw), sides +/-
   uint8_t* vbits;        // [max_views][max_pairs][nv] bits 0-2: s = -1 for x,y,z; 3: side + drawable; 4: side -

@@ -34,8 +34,7 @@ constexpr long long kBinEntries = SGE_STATIC_BIN_ENTRIES;
 
 constexpr size_t al(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t kOffRect = 0;
-constexpr size_t kOffMargin = kOffRect + al(sizeof(int4) * kMaxTriangles);
-constexpr size_t kOffZ = kOffMargin + al(sizeof(int) * kMaxTriangles);
+constexpr size_t kOffZ = kOffRect + al(sizeof(int4) * kMaxTriangles);
 constexpr size_t kOffCount = kOffZ + al(sizeof(float2) * kMaxTriangles);
 constexpr size_t kOffTileOff = kOffCount + al(sizeof(uint32_t) * kMaxTiles);
 constexpr size_t kOffCur = kOffTileOff + al(sizeof(uint32_t) * (kMaxTiles + 1));
@@ -145,7 +144,6 @@ extern "C" int sge_render_idb_static(const sge_scene_desc* d, int32_t view, uint
   Workspace ws;
   memset(&ws, 0, sizeof(ws));
   ws.tri_rect = reinterpret_cast<int4*>(b + kOffRect);
-  ws.tri_margin = reinterpret_cast<int*>(b + kOffMargin);
   ws.tri_z = reinterpret_cast<float2*>(b + kOffZ);
   ws.tile_count = reinterpret_cast<uint32_t*>(b + kOffCount);
   ws.tile_off = reinterpret_cast<uint32_t*>(b + kOffTileOff);
