@@ -1424,8 +1424,8 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
 // credits go to the global sums directly, texel credits through the windows and cells as in the fast path.
 // Bound by instruction issue (R is 70 % of it).  Against the general kernel it replaces, which set every
 // live triangle up in shared memory per pair, tested up to all of them at each pixel and hashed vertices and
-// texels: 24.6 -> 9.6 ms (GGX, 1 M triangles, 6,175 dense tiles x 4 pairs), 4.82 -> 2.11 ms (a batch of 8 unlit
-// assets), 1.32 -> 0.28 ms (Lambert, 41 tiles x 16 pairs).
+// texels: 24.6 -> 7.6 ms (GGX, 1 M triangles, 6,175 dense tiles x 4 pairs), 4.82 -> 1.73 ms (a batch of 8 unlit
+// assets), 1.32 -> 0.26 ms (Lambert, 41 tiles x 16 pairs).
 template <int SH, bool GR>
 __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
                                             const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
@@ -1535,11 +1535,12 @@ __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& 
             q[2] = __ldg(p + 2ll * t.z);
           };
           if (tid < 2 * nb) fetch(tid);
-          for (int t2 = tid; t2 < 2 * nb; t2 += M::THREADS) {
+          for (int t2 = tid; t2 - lane < 2 * nb; t2 += M::THREADS) {
             const int4 v0 = q[0], v1 = q[1], v2 = q[2];
             const int id = t.w;
             if (t2 + M::THREADS < 2 * nb) fetch(t2 + M::THREADS);
-            raster_tri(v0, v1, v2, id, rx, ry, keys + (st * 2 + (t2 & 1)) * TILE_PX);
+            if (t2 < 2 * nb) raster_tri(v0, v1, v2, id, rx, ry, keys + (st * 2 + (t2 & 1)) * TILE_PX);
+            __syncwarp();  // (lanes left to themselves stay apart after one's box: 9.6 instead of 7.6 ms)
           }
         }
         __syncthreads();
@@ -1804,12 +1805,16 @@ cudaError_t launch_dense(const SceneDev& S, const Workspace& ws, const ViewList&
 // hide behind one another, and 4 threads to a triangle, so small boxes leave few lanes idle (8,192 triangles,
 // 512^2, 8 views / 1 M triangles, 2048^2, 4 views: 7 CTAs 135 us / 1.96 ms, 5 CTAs 169 us / 2.29 ms; 8 threads
 // to a triangle 127 us / 2.16 ms; one wave of 256 tiles: 21.1 us with 16 threads, 24.1 us with 4).
-constexpr int kPruneOneWave = 2 * 152;
+// Up to one wave of those the fullest tile still counts: a row per thread (soup of 10,240 triangles, 512^2, one view:
+// 55.6 us before all this, 39.1 us; 47.0 us with 4 threads to a triangle).
+constexpr int kPruneOneWave = 2 * 152, kPruneSevenWave = 7 * 152;
 
 cudaError_t launch_prune(const SceneDev& S, const Workspace& ws, const ViewList& vl, cudaStream_t st) {
   const dim3 grid(n_tiles(S), vl.n);
   if ((long long)grid.x * grid.y <= kPruneOneWave)
     k_bin_prune<16, 2><<<grid, TILE_PX, 0, st>>>(S, ws, vl);
+  else if ((long long)grid.x * grid.y <= kPruneSevenWave)
+    k_bin_prune<16, 7><<<grid, TILE_PX, 0, st>>>(S, ws, vl);
   else
     k_bin_prune<4, 7><<<grid, TILE_PX, 0, st>>>(S, ws, vl);
   return cudaGetLastError();

@@ -673,20 +673,27 @@ __device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const
       e0 = -e0, e1 = -e1, e2 = -e2, area = -area;
       a0 = -a0, a1 = -a1, a2 = -a2, b0 = -b0, b1 = -b1, b2 = -b2;
     }
+    // a pixel at an edge belongs to the triangle if the edge is top or left: the tests E_k >= 0 of the others
+    // become E_k >= 1
+    const int n0 = a0 > 0 || (a0 == 0 && b0 > 0) ? 0 : 1, n1 = a1 > 0 || (a1 == 0 && b1 > 0) ? 0 : 1,
+              n2 = a2 > 0 || (a2 == 0 && b2 > 0) ? 0 : 1;
     float inv = 0.0f;
-    for (int y = r0; y <= r1; ++y) {
-      int E0 = e0 + a0 * (c0 * 256) + b0 * (y * 256), E1 = e1 + a1 * (c0 * 256) + b1 * (y * 256);
-      for (int x = c0; x <= c1; ++x, E0 += a0 * 256, E1 += a1 * 256) {
-        const int E2 = area - E0 - E1, lo = min(min(E0, E1), E2);
-        if (lo < 0) continue;
-        if (lo == 0 && ((E0 == 0 && !(a0 > 0 || (a0 == 0 && b0 > 0))) || (E1 == 0 && !(a1 > 0 || (a1 == 0 && b1 > 0))) ||
-                        (E2 == 0 && !(a2 > 0 || (a2 == 0 && b2 > 0)))))
-          continue;
+    int E0 = e0 + (a0 * c0 + b0 * r0) * 256, E1 = e1 + (a1 * c0 + b1 * r0) * 256;
+    const int w = c1 - c0, d0 = (b0 - a0 * w) * 256, d1 = (b1 - a1 * w) * 256;
+    // one loop over the box (rows in turn), so that lanes with boxes of other shapes keep together
+    for (int x = c0, y = r0; y <= r1;) {
+      const int E2 = area - E0 - E1;
+      if (min(min(E0 - n0, E1 - n1), E2 - n2) >= 0) {
         if (inv == 0.0f) inv = __fdiv_rn(1.0f, __int2float_rn(area));
         const float l[3] = {__fmul_rn(__int2float_rn(E0), inv), __fmul_rn(__int2float_rn(E1), inv),
                             __fmul_rn(__int2float_rn(E2), inv)};
         put(x, y, l);
       }
+      const bool turn = x == c1;
+      x = turn ? c0 : x + 1;
+      y += turn ? 1 : 0;
+      E0 += turn ? d0 : a0 * 256;
+      E1 += turn ? d1 : a1 * 256;
     }
     return;
   }
