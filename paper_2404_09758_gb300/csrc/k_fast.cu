@@ -1539,7 +1539,9 @@ __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& 
             const int4 v0 = q[0], v1 = q[1], v2 = q[2];
             const int id = t.w;
             if (t2 + M::THREADS < 2 * nb) fetch(t2 + M::THREADS);
-            if (t2 < 2 * nb) raster_tri(v0, v1, v2, id, rx, ry, keys + (st * 2 + (t2 & 1)) * TILE_PX);
+            int c0, c1, r0, r1;
+            if (t2 < 2 * nb && tri_box(v0, v1, v2, rx, ry, c0, c1, r0, r1))
+              raster_tri(v0, v1, v2, id, rx, ry, c0, c1, r0, r1, keys + (st * 2 + (t2 & 1)) * TILE_PX);
             __syncwarp();  // (lanes left to themselves stay apart after one's box: 9.6 instead of 7.6 ms)
           }
         }

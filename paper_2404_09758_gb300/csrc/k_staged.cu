@@ -12,6 +12,8 @@ namespace sge {
 namespace {
 
 constexpr int RCHUNK = TILE_PX;  // binned triangles staged per pass, one per thread
+// Pixels of the largest box that one lane walks alone in a bin of more than one chunk.
+constexpr int kLaneBox = 32;
 
 template <int NS>
 struct RSmem {
@@ -37,10 +39,12 @@ __device__ __forceinline__ int pixel_dx() { return ((threadIdx.x >> 5) & 1) * 8 
 __device__ __forceinline__ int pixel_dy() { return (threadIdx.x >> 6) * 4 + ((threadIdx.x >> 3) & 3); }
 
 // Visible triangle of every pixel of a tile for NS sides.  A bin of one chunk is set up in shared memory
-// and each pixel tests the triangles whose box holds it (warps skip those that miss their block); a larger
-// one (dense meshes) goes triangle by triangle into the pixels of its box.  Bound by instruction issue;
+// and each pixel tests the triangles whose box holds it (warps skip those that miss their block); of a larger
+// one the triangles of small boxes (dense meshes) go into the pixels of their boxes, a triangle per lane, and only
+// the others are set up and tested as before (by lane alone, a render of 100 K triangles grown over a 512^2
+// image walks up to 256 pixels in a lane: 9.96 ms an iteration of 8 pairs, this 4.4 ms, testing all of them 6.3 ms).  Bound by instruction issue;
 // 64-bit tests of every binned triangle at every pixel, and a second set-up per pixel, took 190 us for a view
-// of 32,768 triangles at 1024^2 (Lambert) where this takes 101 us.
+// of 32,768 triangles at 1024^2 (Lambert) where this takes 84 us.
 template <int NS>
 __device__ __forceinline__ void raster_tile(const SceneDev& S, const Workspace& ws, RSmem<NS>& sm, int slot, int tile,
                                             uint64_t key, const int (&sides)[NS], Hit (&hit)[NS], int rx, int ry,
@@ -99,23 +103,51 @@ __device__ __forceinline__ void raster_tile(const SceneDev& S, const Workspace& 
   }
 #pragma unroll
   for (int s = 0; s < NS; ++s) sm.keys[s][tid] = ~0ull;
-  __syncthreads();
-  for (int j = tid; j < nb; j += TILE_PX) {
-    const int tri = (int)bin_at(S, ws, beg + j);
+  for (int c0 = 0; c0 < nb; c0 += RCHUNK) {
+    const int cnt = min(RCHUNK, nb - c0);
+    bool staged = false;
+    __syncthreads();  // the keys are empty, the last chunk's set-ups are done with
 #pragma unroll
     for (int s = 0; s < NS; ++s) {
-      PVert v[3];
-      project_side(tri, s, v);
-      int4 q[3];
+      uint32_t span = 0u;
+      if (tid < cnt) {
+        const int tri = (int)bin_at(S, ws, beg + c0 + tid);
+        PVert v[3];
+        project_side(tri, s, v);
+        int4 q[3];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) q[k] = make_int4(v[k].ok ? v[k].X : kNotDrawn, v[k].Y, __float_as_int(v[k].z), 0);
-      raster_tri(q[0], q[1], q[2], tri, rx, ry, sm.keys[s]);
+        for (int k = 0; k < 3; ++k) q[k] = make_int4(v[k].ok ? v[k].X : kNotDrawn, v[k].Y, __float_as_int(v[k].z), 0);
+        int xa, xb, ya, yb;
+        if (tri_box(q[0], q[1], q[2], rx, ry, xa, xb, ya, yb)) {
+          if ((xb - xa + 1) * (yb - ya + 1) <= kLaneBox) {
+            raster_tri(q[0], q[1], q[2], tri, rx, ry, xa, xb, ya, yb, sm.keys[s]);
+          } else {
+            set_up_side(sm.t[s][tid], v, rx, ry);
+            span = box_span(v, rx, ry, 0);
+            sm.tri[tid] = tri;
+            staged = true;
+          }
+        }
+      }
+      sm.span[tid][s] = span;
+      __syncwarp();
     }
+    if (!__syncthreads_or(staged)) continue;
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+      for_spans(sm.span, s, cnt, block, dx, dy, [&](int j) {
+        float l[3];
+        float4 z;
+        if (!cover_lambdas(sm.t[s][j], dx * 256, dy * 256, l, z)) return;
+        const float zz[3] = {z.x, z.y, z.z};
+        const unsigned long long k = ((unsigned long long)ordered_bits(interp_depth(l, zz)) << 32) | (uint32_t)sm.tri[j];
+        hit[s].key = min(hit[s].key, k);
+      });
   }
   __syncthreads();
 #pragma unroll
   for (int s = 0; s < NS; ++s) {
-    hit[s].key = sm.keys[s][dy * TILE + dx];
+    hit[s].key = min(hit[s].key, sm.keys[s][dy * TILE + dx]);
     if (hit[s].key == ~0ull) continue;
     PVert v[3];
     project_side((int)(uint32_t)hit[s].key, s, v);

@@ -647,23 +647,32 @@ __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, fl
   return true;
 }
 
+// The pixel centres of the tile in a projected triangle's vertex box; false: none, or the triangle is not drawn.
+__device__ __forceinline__ bool tri_box(const int4& q0, const int4& q1, const int4& q2, int rx, int ry, int& c0, int& c1,
+                                        int& r0, int& r1) {
+  if (q0.x == kNotDrawn || q1.x == kNotDrawn || q2.x == kNotDrawn) return false;
+  c0 = max((min(q0.x, min(q1.x, q2.x)) - rx + 255) >> 8, 0), c1 = min((max(q0.x, max(q1.x, q2.x)) - rx) >> 8, TILE - 1);
+  r0 = max((min(q0.y, min(q1.y, q2.y)) - ry + 255) >> 8, 0), r1 = min((max(q0.y, max(q1.y, q2.y)) - ry) >> 8, TILE - 1);
+  return c0 <= c1 && r0 <= r1;
+}
+
+// A key (depth, id) into a pixel's nearest.
+__device__ __forceinline__ void put_key(unsigned long long* out, const float (&l)[3], float z0, float z1, float z2, int id) {
+  const float z[3] = {z0, z1, z2};
+  const unsigned long long key = ((unsigned long long)ordered_bits(interp_depth(l, z)) << 32) | (uint32_t)id;
+  if (key < *(volatile unsigned long long*)out) atomicMin(out, key);
+}
+
 // A projected triangle (records as the vertex pass writes them) into the tile's keys: the nearest (depth bits << 32 |
-// id) of each pixel centre it covers.  The arithmetic of set_up_side, cover_lambdas and
-// interp_depth, with the division left until a pixel is covered (most triangles of a dense tile cover
+// id) of each pixel centre it covers, columns c0..c1 and rows r0..r1 of its box.  The arithmetic of set_up_side,
+// cover_lambdas and interp_depth, with the division left until a pixel is covered (most triangles of a dense tile cover
 // none or one).
-__device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const int4& q2, int id, int rx, int ry,
-                                           unsigned long long* keys) {
-  if (q0.x == kNotDrawn || q1.x == kNotDrawn || q2.x == kNotDrawn) return;
+__device__ __forceinline__ void raster_tri(const int4& q0, const int4& q1, const int4& q2, int id, int rx, int ry, int c0,
+                                           int c1, int r0, int r1, unsigned long long* keys) {
   const int x0 = q0.x - rx, x1 = q1.x - rx, x2 = q2.x - rx, y0 = q0.y - ry, y1 = q1.y - ry, y2 = q2.y - ry;
-  // pixel centres in the vertex box
   const int xl = min(x0, min(x1, x2)), xh = max(x0, max(x1, x2)), yl = min(y0, min(y1, y2)), yh = max(y0, max(y1, y2));
-  const int c0 = max((xl + 255) >> 8, 0), c1 = min(xh >> 8, TILE - 1), r0 = max((yl + 255) >> 8, 0), r1 = min(yh >> 8, TILE - 1);
-  if (c0 > c1 || r0 > r1) return;
   auto put = [&](int x, int y, const float (&l)[3]) {
-    const float z[3] = {__int_as_float(q0.z), __int_as_float(q1.z), __int_as_float(q2.z)};
-    const unsigned long long key = ((unsigned long long)ordered_bits(interp_depth(l, z)) << 32) | (uint32_t)id;
-    unsigned long long* out = keys + y * TILE + x;
-    if (key < *(volatile unsigned long long*)out) atomicMin(out, key);
+    put_key(keys + y * TILE + x, l, __int_as_float(q0.z), __int_as_float(q1.z), __int_as_float(q2.z), id);
   };
   if (max(max(xh, yh), -min(xl, yl)) < (1 << 14)) {
     int e0 = x1 * y2 - x2 * y1, e1 = x2 * y0 - x0 * y2, e2 = x0 * y1 - x1 * y0, area = e0 + e1 + e2;

@@ -164,7 +164,7 @@ cudaError_t launch_prune_batch(const BatchArgs& P, int max_tiles, int max_views,
 // (the estimators), k_bin_prune then drops from each bin the triangles no perturbation can
 // make visible in the tile, lists the items by their live counts and stores each pixel's
 // candidate triangles.
-// defer_prune: the caller prunes later (k_bin_prune_batch): the scan lists no items either.
+// defer_prune: the caller prunes later (k_bin_prune_batch).
 cudaError_t launch_binning(const SceneDev& S, const Workspace& ws, const ViewList& vl, cudaStream_t st,
                            bool prune = false, bool defer_prune = false);
 cudaError_t launch_prune(const SceneDev& S, const Workspace& ws, const ViewList& vl, cudaStream_t st);

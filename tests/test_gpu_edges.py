@@ -28,6 +28,15 @@ def _lambert_dense(sizes, n):
                                width=40, height=36)
 
 
+def _grown_soup(n, scale, render):
+    """Triangles of all sizes up to several tiles, hundreds in every tile."""
+    sc, _ = synth.triangle_soup(n, render=render)
+    p = sc.positions.reshape(-1, 3, 3).astype(np.float64)
+    c = p.mean(1, keepdims=True)
+    p[..., :2] = c[..., :2] + np.linspace(0.2, scale, n)[:, None, None] * (p - c)[..., :2]
+    return dataclasses.replace(sc, positions=p.reshape(-1, 3).astype(np.float32))
+
+
 ESTIMATES = {
     # bins of more than 256 triangles of which a light tile's worth stays: marked, then listed
     "prune_chunks": (lambda: _sphere(52, 40, 30, 64, 64), 3),
@@ -38,6 +47,7 @@ ESTIMATES = {
     # dense tiles: more live triangles than are kept in shared memory, one to nine pairs
     "dense_pairs_1": (lambda: _sphere(96, 40, 30, 32, 30), 1),
     "dense_pairs_9": (lambda: _sphere(96, 40, 30, 32, 30), 9),
+    "dense_grown_soup": (lambda: _grown_soup(6000, 3.0, 72), 2),
     "dense_texture_1x1": (lambda: _sphere(72, 1, 1, 32, 30, 1), 3),
     "dense_hash": (lambda: _sphere(72, 900, 700, 32, 30), 3),
     "dense_lambert_group": (lambda: _lambert_dense([(40, 40)] * 2, 72), 3),
@@ -68,6 +78,8 @@ RENDERS = {
     "bins_of_thousands_ggx": lambda: dataclasses.replace(_lit(synth.config_scale, [(40, 30)] * 4, n_lon=96, n_lat=72),
                                                          width=40, height=36),
     "big_triangles_1672_tiles": lambda: _quads(700, 600),
+    # bins of several chunks with boxes on both sides of a lane's limit
+    "grown_soup": lambda: _grown_soup(3000, 6.0, 72),
 }
 
 
