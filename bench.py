@@ -51,12 +51,12 @@ OPS_VISIBLE, OPS_UV, OPS_FOOT, OPS_WEIGHTS, OPS_PER_TEXEL_CHANNEL = 20, 17, 14, 
 OPS_SHADE = {0: 0, 1: 55, 2: 125}  # unlit; Lambert with a normal map; GGX + Lambert (per side)
 OPS_LOSS_DIFF = 12  # per pixel pair: sum_c (I+ - I-)(I+ + I- - 2I)
 OPS_CREDIT = 2      # per contribution: one add to the parameter's sum, one to its count
-# One ncu --set full capture of this build's k_estimate_fast<unlit> on this workload (one launch =
-# one estimate call, 134.2 M pixel pairs): smsp__inst_executed.sum 5.158 G x 22.74 active lanes =
-# 874 thread instructions per pixel pair; dram__bytes_read.sum + dram__bytes_write.sum =
-# 164.16 MB + 6.58 MB per launch.  Set to None when the kernel changes until it is captured again.
-NCU_INSTR_PER_PIXEL_PAIR = 874.0
-NCU_DRAM_BYTES_PER_LAUNCH = 170.74e6
+# One ncu capture of this build's k_estimate_fast<unlit> on this workload (one launch = one estimate
+# call, 134.2 M pixel pairs): smsp__thread_inst_executed.sum 101.10 G = 753 thread instructions per
+# pixel pair; dram__bytes_read.sum + dram__bytes_write.sum = 212.69 MB + 8.57 MB per launch.  Set to
+# None when the kernel changes until it is captured again.
+NCU_INSTR_PER_PIXEL_PAIR = 753.2
+NCU_DRAM_BYTES_PER_LAUNCH = 221.26e6
 
 
 def method_ops(shading: int, read_channels, covered_sides: float, covered_pairs: float, contributions: float):
