@@ -33,6 +33,7 @@ __global__ void k_bin_rect_count(SceneDev S, Workspace ws, ViewList vl) {
   int view = vl.id[slot];
   // the call's counters: items and their work counters, bin entries (the status word stays)
   if (blockIdx.x == 0 && slot == 0 && threadIdx.x < 7 && threadIdx.x != 3) ws.counters[threadIdx.x] = 0u;
+  if (blockIdx.x == 0 && slot == 0 && threadIdx.x == 7) *bin_total(ws) = 0ull;
   if (threadIdx.x < 16) m[threadIdx.x] = S.mvp[16 * view + threadIdx.x];
   __syncthreads();
   int tri = blockIdx.x * blockDim.x + threadIdx.x;
@@ -118,39 +119,39 @@ __global__ void k_bin_rect_count(SceneDev S, Workspace ws, ViewList vl) {
 }
 
 // Each (slot, tile)'s place in the bins: a CTA's 1,024 counts are scanned and the CTA takes its range
-// from the running total (counters[2]), in whatever order the CTAs come; then the fill cursors.  Nothing
+// from the running total, in whatever order the CTAs come; then the fill cursors.  Nothing
 // needs the tiles in order, and one CTA scanning every count of a call serially took 12.5 us for
 // 8,192 counts and 160 us for 65,536 (both 3 us here).
-__global__ void __launch_bounds__(1024) k_bin_place(Workspace ws, int n) {
-  __shared__ uint32_t wsum[32], base;
+__global__ void __launch_bounds__(1024) k_bin_place(Workspace ws, int n, int n_triangles) {
+  __shared__ unsigned long long wsum[32], base;
   const int i = blockIdx.x * blockDim.x + threadIdx.x, lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const uint32_t c = i < n ? ws.tile_count[i] : 0u;
-  uint32_t x = c;
+  unsigned long long x = c;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+    const unsigned long long y = __shfl_up_sync(0xffffffffu, x, o);
     if (lane >= o) x += y;
   }
   if (lane == 31) wsum[wid] = x;
   __syncthreads();
   if (wid == 0) {
-    uint32_t w = wsum[lane];
+    unsigned long long w = wsum[lane];
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t y = __shfl_up_sync(0xffffffffu, w, o);
+      const unsigned long long y = __shfl_up_sync(0xffffffffu, w, o);
       if (lane >= o) w += y;
     }
     wsum[lane] = w;
     if (lane == 31) {
-      base = atomicAdd(ws.counters + 2, w);
-      if ((long long)base + w > ws.bin_capacity) atomicCAS(ws.counters + 3, 0u, (uint32_t)SGE_ERR_BIN_OVERFLOW);
+      base = atomicAdd(bin_total(ws), w);
+      if (base + w > (unsigned long long)ws.bin_capacity) atomicCAS(ws.counters + 3, 0u, (uint32_t)SGE_ERR_BIN_OVERFLOW);
     }
   }
   __syncthreads();
   if (i >= n) return;
-  const uint32_t off = base + (wid ? wsum[wid - 1] : 0u) + x - c;
+  const uint32_t off = bin_start(base + (wid ? wsum[wid - 1] : 0ull) + x - c, c, ws.bin_capacity);
   ws.tile_off[i] = off;
-  ws.tile_cur[i] = off;
+  ws.tile_cur[i] = bin_cursor(off, n_triangles);
 }
 
 __global__ void k_bin_fill(SceneDev S, Workspace ws) {
@@ -161,8 +162,9 @@ __global__ void k_bin_fill(SceneDev S, Workspace ws) {
   int nt = n_tiles(S);
   for (int ty = rect.y; ty <= rect.w; ++ty)
     for (int tx = rect.x; tx <= rect.z; ++tx) {
-      uint32_t pos = atomicAdd(ws.tile_cur + (long long)slot * nt + ty * S.tiles_x + tx, 1u);
-      if ((long long)pos < ws.bin_capacity && CHK(S, pos, S.chk.bins)) ws.bins[pos] = (uint32_t)tri;
+      const long long t = (long long)slot * nt + ty * S.tiles_x + tx;
+      const uint32_t pos = atomicAdd(ws.tile_cur + t, 1u);
+      if (bin_stores(pos, ws.tile_off + t, ws.bin_capacity, S.nt) && CHK(S, pos, S.chk.bins)) ws.bins[pos] = (uint32_t)tri;
     }
 }
 
@@ -175,7 +177,7 @@ cudaError_t launch_binning(const SceneDev& S, const Workspace& ws, const ViewLis
   if (e != cudaSuccess) return e;
   dim3 grid((S.nt + 255) / 256, vl.n);
   k_bin_rect_count<<<grid, 256, 0, st>>>(S, ws, vl);
-  k_bin_place<<<(vl.n * nt + 1023) / 1024, 1024, 0, st>>>(ws, vl.n * nt);
+  k_bin_place<<<(vl.n * nt + 1023) / 1024, 1024, 0, st>>>(ws, vl.n * nt, S.nt);
   k_bin_fill<<<grid, 256, 0, st>>>(S, ws);
   e = cudaGetLastError();
   if (e == cudaSuccess && prune && !defer_prune) e = launch_prune(S, ws, vl, st);

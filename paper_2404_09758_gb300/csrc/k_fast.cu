@@ -278,7 +278,7 @@ __device__ __forceinline__ void prune_tile(const SceneDev& S, const Workspace& w
                                            int light_bin, PruneSmem& sm) {
   const int tid = threadIdx.x;
   const int ntl = n_tiles(S), n_all = n_views * ntl;
-  if ((long long)ws.counters[2] > ws.bin_capacity) return;  // overflow: the bins were not stored
+  if (*bin_total(ws) > (unsigned long long)ws.bin_capacity) return;  // overflow: the bins were not stored
   const uint32_t beg = ws.tile_off[slot * ntl + tile];
   const int nb = (int)ws.tile_count[slot * ntl + tile];
   if (nb == 0) return;

@@ -974,14 +974,14 @@ int sge_kernel_time(sge_scene* s, float* total_ms, float* heavy_ms, int32_t* lau
 int sge_bin_stats(sge_scene* s, sge_stream_t stream, int64_t* light_items, int64_t* heavy_items,
                   int64_t* bin_entries) {
   if (!s || !light_items || !heavy_items || !bin_entries) return fail(SGE_ERR_INVALID_ARG, "NULL argument");
-  uint32_t c[7] = {};
+  uint32_t c[16] = {};
   cudaStream_t st = (cudaStream_t)stream;
   cudaError_t e = cudaMemcpyAsync(c, s->ws.counters, sizeof(c), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return cuda_fail(e, "sge_bin_stats");
   *light_items = (int64_t)c[0] + c[6];
   *heavy_items = c[4];
-  *bin_entries = c[2];
+  *bin_entries = (int64_t)((uint64_t)c[13] << 32 | c[12]);
   return SGE_OK;
 }
 

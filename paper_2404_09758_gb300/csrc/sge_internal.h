@@ -103,8 +103,8 @@ struct Workspace {
   int4* cand;            // [max_views][n_tiles][kCandWords][256] candidate triangles of each pixel of a light
                          // tile: 8-bit live indices in ascending order of their smallest depth
   uint8_t* ncand;        // [max_views][n_tiles][256] their number (more than fit: test every live triangle)
-  uint32_t* counters;    // [0] light items of at most kBigBin live triangles, [6] of more, [1] their work counter, [2] total bin entries, [3] status,
-                         // [4] heavy items, [5] their work counter
+  uint32_t* counters;    // [0] light items of at most kBigBin live triangles, [6] of more, [1] their work counter,
+                         // [3] status, [4] heavy items, [5] their work counter, [12..13] total bin entries
   unsigned long long* keys;  // [2][H*W] staged depth|ID buffers (both sides)
   float2* uvbuf;             // [2][H*W] staged UV buffers
   float* dfbuf;              // [H*W] staged loss differences
@@ -122,6 +122,27 @@ struct Workspace {
   int max_pairs;
   int light_bin;  // bins of at most this many triangles are light items (fast kernel)
 };
+
+// Running total of a call's bin entries.  64 bits: triangles that may cross the near limit are binned into
+// every tile, so 16,384 of them in 16 views of 2048^2 are 2^32 entries.
+__host__ __device__ inline unsigned long long* bin_total(const Workspace& ws) {
+  return reinterpret_cast<unsigned long long*>(ws.counters + 12);
+}
+// Where the bin of a tile of `count` entries starts when `before` entries come before it: kNoBin when it does
+// not fit the capacity (< 2^32), so that start + count is above the capacity for every reader.
+constexpr uint32_t kNoBin = 0xFFFFFFFFu;
+__host__ __device__ inline uint32_t bin_start(unsigned long long before, uint32_t count, long long capacity) {
+  return before + count <= (unsigned long long)capacity ? (uint32_t)before : kNoBin;
+}
+// Its fill cursor: that of a bin left out counts up to `n_triangles` entries without wrapping.
+__host__ __device__ inline uint32_t bin_cursor(uint32_t start, int n_triangles) {
+  return start == kNoBin ? kNoBin - (uint32_t)n_triangles : start;
+}
+// May the fill store at position pos of the bin that starts at *start?  (The start is read only where a
+// capacity close to 2^32 reaches the cursors of bins left out.)
+__host__ __device__ inline bool bin_stores(uint32_t pos, const uint32_t* start, long long capacity, int n_triangles) {
+  return (long long)pos < capacity && (capacity <= (long long)(kNoBin - (uint32_t)n_triangles) || *start != kNoBin);
+}
 
 // What a batched launch needs of one scene, kept in the scene's workspace (written on the
 // stream by launch_put_desc) so that the launch's parameter holds one pointer per asset.
