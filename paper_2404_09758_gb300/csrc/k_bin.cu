@@ -60,7 +60,14 @@ __global__ void k_bin_rect_count(SceneDev S, Workspace ws, ViewList vl) {
     clip_interval(m + 8, x, y, z, S.eps_pos, zl, zh);
     const float cw = clip_interval(m + 12, x, y, z, S.eps_pos, wl, wh);
     if (wh <= S.near_w) { skip = true; break; }  // always behind the near limit: triangle never drawn
-    if (wl <= S.near_w) { full = true; continue; }  // may or may not be drawn: bin everywhere
+    if (wl <= S.near_w) {
+      // may or may not be drawn: bin everywhere, at any depth (a bound without this vertex would rank the triangle
+      // behind ones it hides, and the search for the nearest would end before it)
+      full = true;
+      zlo = -3.4e38f;
+      zhi = 3.4e38f;
+      continue;
+    }
     float nx0 = fminf(fminf(xl / wl, xl / wh), fminf(xh / wl, xh / wh));
     float nx1 = fmaxf(fmaxf(xl / wl, xl / wh), fmaxf(xh / wl, xh / wh));
     float ny0 = fminf(fminf(yl / wl, yl / wh), fminf(yh / wl, yh / wh));
