@@ -3,6 +3,7 @@
 // are zeroed for the next iteration.  Memory bound.
 #include <cuda_runtime.h>
 
+#include <cfloat>
 #include <cmath>
 
 #include "sge_device.cuh"
@@ -46,9 +47,15 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
     c1 = -expm1f(t * logf(b1));
     c2 = -expm1f(t * logf(b2));
   }
-  const float tail = c1 > 0.0f && c2 > 0.0f ? 1.07374182e9f / (c1 * aeps) : INFINITY;  // 2^30 / (c1 adam_eps)
+  // group g's |lr| 2^30 / (c1 adam_eps): |m| times it below |theta| means a step below 2^-30 |theta| (no bound, infinity,
+  // where a factor is not positive or the product leaves the normal range)
+  auto bound = [&](int g) {
+    const float lr = fabsf(G.lr[g]);
+    const float k = lr * (aeps > 0.0f && c1 > 0.0f && c2 > 0.0f ? 1.07374182e9f / (c1 * aeps) : INFINITY);
+    return lr == 0.0f || k >= FLT_MIN ? k : INFINITY;
+  };
   // one parameter of group g: theta, m, v updated
-  auto update = [&](int g, float s, uint32_t cn, float& th, float& mm, float& vv) {
+  auto update = [&](int g, float kg, float s, uint32_t cn, float& th, float& mm, float& vv) {
     const float scale = kind == SGE_STEP_SGD_MEAN ? 1.0f / (float)(cn > 0 ? cn : 1u) : inv_n;
     const float gr = s * scale / (2.0f * G.eps[g]);
     if (kind == SGE_STEP_ADAM) {
@@ -57,7 +64,7 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
       // the step is at most lr |m| / (c1 adam_eps): below theta's rounding by 2^-30 it leaves theta as it
       // is, and the divisions, which take a slow path for the denormal moments of parameters that nothing
       // touches any more, are left out (52 M such parameters: 460 -> 305 us)
-      if (vv >= 0.0f && fabsf(mm) * fabsf(G.lr[g]) * tail < fabsf(th)) return;
+      if (vv >= 0.0f && fabsf(mm) * kg < fabsf(th)) return;
       th -= G.lr[g] * (mm / c1) / (sqrtf(vv / c2) + aeps);
     } else {
       th -= G.lr[g] * gr;
@@ -83,10 +90,11 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
 #pragma unroll
       for (int k = 0; k < 4; ++k) th[k] = theta[k];
     }
-    update(g, s4.x, n4.x, th[0], m4.x, v4.x);
-    update(g, s4.y, n4.y, th[1], m4.y, v4.y);
-    update(g, s4.z, n4.z, th[2], m4.z, v4.z);
-    update(g, s4.w, n4.w, th[3], m4.w, v4.w);
+    const float kg = bound(g);
+    update(g, kg, s4.x, n4.x, th[0], m4.x, v4.x);
+    update(g, kg, s4.y, n4.y, th[1], m4.y, v4.y);
+    update(g, kg, s4.z, n4.z, th[2], m4.z, v4.z);
+    update(g, kg, s4.w, n4.w, th[3], m4.w, v4.w);
     if (moments) {
       __stcs(reinterpret_cast<float4*>(m + i0), m4);
       __stcs(reinterpret_cast<float4*>(v + i0), v4);
@@ -106,7 +114,7 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
     const int gi = group_of(G, i);
     float* theta = G.theta[gi] + (i - G.begin[gi]);
     float th = *theta, mm = moments ? m[i] : 0.0f, vv = moments ? v[i] : 0.0f;
-    update(gi, grad[i], counts[i], th, mm, vv);
+    update(gi, bound(gi), grad[i], counts[i], th, mm, vv);
     if (moments) {
       m[i] = mm;
       v[i] = vv;
