@@ -1438,7 +1438,10 @@ __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& 
   unsigned long long* keys = reinterpret_cast<unsigned long long*>(&sm.side[0][0]);
   static_assert(sizeof(sm.side) >= 2 * P * TILE_PX * sizeof(unsigned long long), "keys");
   const int ntl = n_tiles(S), n_heavy = (int)ws.counters[4];
-  const int run = a.pairs_per_item > 0 ? max(1, a.pairs_per_item / 4) : run_of(a, n_heavy, P, kRun);
+  // (the P pairs at a time need P pairs an item: one, a quarter of pairs_per_item = 1..7, leaves half the warps
+  // without a pair.  100 K triangles at 256^2, 2 views x 8 pairs, pairs_per_item = 4: 857 us with one, 754 us with two)
+  const int ppi = a.pairs_per_item > 0 ? a.pairs_per_item : kRun;
+  const int run = run_of(a, n_heavy, max(P, ppi / 4), max(P, ppi));
   const int chunks = (a.pair_count + run - 1) / run;
   const long long n_work = (long long)n_heavy * chunks;
   if (n_work == 0 || (own_first && blockIdx.x >= n_work)) return;  // (uniform over the CTA)
