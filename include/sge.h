@@ -120,9 +120,9 @@ typedef struct {
 typedef struct {
     int32_t max_views_per_call; /* views per estimate call the workspace is sized for (default n_views, <= 64) */
     int64_t bin_capacity;       /* triangle-tile bin entries over those views (default (6 n_triangles + 8 tiles) * views) */
-    int32_t pairs_per_item;     /* antithetic pairs one CTA runs per (view, tile) item (<= 64; default: 8 to 32,
-                                   by how many items the call has; dense tiles run a quarter
-                                   of it, at least two, and up to it where there are many) */
+    int32_t pairs_per_item;     /* antithetic pairs one CTA runs per (view, tile) item (<= 64, 1 counts as 2;
+                                   default: 8 to 32, by how many items the call has; tiles of many
+                                   triangles run from a quarter of it, at least two, up to it) */
     int32_t blocks_per_sm;      /* persistent CTAs per SM (default: as many as fit) */
     int32_t max_pairs_per_call; /* pairs per view projected at once (default 64); more run in blocks */
     int32_t footprint;          /* texels a pixel credits (SGE_FOOT_*; default bilinear)           */

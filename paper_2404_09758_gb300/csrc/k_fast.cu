@@ -1131,8 +1131,11 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
   // would leave the other CTAs idle (4 views x 16 pairs at 501 x 397: CTAs busy 0.55 of 1.06 ms without
   // this, the kernel 0.63 ms with it; 8 views x 64 pairs at 512^2: 7.2 -> 5.9 ms with the longer runs).
   const int n_small = (int)ws.counters[0], n_big = (int)ws.counters[6];
-  const int ppi = a.pairs_per_item > 0 ? a.pairs_per_item : kRun;
-  const int run = a.pairs_per_item > 0 ? ppi : run_of(a, n_small, ppi, 4 * kRun), run_big = run_of(a, n_big, max(1, ppi / 4), ppi);
+  // No run is of one pair where the call has more: its units would be half as many as the CTA's warps, and
+  // a window would be found, filled and read for it alone (8,192 triangles, 512^2, 8 views x 64 pairs, pairs_per_item = 1: 21.3 ms
+  // in runs of one pair, 12.1 ms of two; a batch of 8 uneven assets 22.1 and 16.7 ms).
+  const int ppi = a.pairs_per_item > 0 ? max(2, a.pairs_per_item) : kRun;
+  const int run = a.pairs_per_item > 0 ? ppi : run_of(a, n_small, ppi, 4 * kRun), run_big = run_of(a, n_big, max(2, ppi / 4), ppi);
   const int chunks = (a.pair_count + run - 1) / run, chunks_big = (a.pair_count + run_big - 1) / run_big;
   const long long work_big = (long long)n_big * chunks_big, n_work = work_big + (long long)n_small * chunks;
   reset_smem<SH, GR>(sm);

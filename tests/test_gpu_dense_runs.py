@@ -17,3 +17,13 @@ def test_explicit_runs_of_dense_tiles_match_oracle(ppi, pairs):
     r = run_both(sc, tg, seed=13, it=2, views=[0], pairs=pairs, gpu_kwargs={"pairs_per_item": ppi})
     assert r["bins"][1] > 0
     assert_parity(sc, r)
+
+
+@pytest.mark.parametrize("pairs", [1, 2, 5])
+@pytest.mark.parametrize("ppi", [1, 2, 3, 7])
+def test_short_explicit_runs_of_light_tiles_match_oracle(ppi, pairs):
+    sc = _sphere(40, 40, 30, 61, 45)  # tiles on both sides of the line between small and large light ones
+    tg = np.random.default_rng(2).uniform(size=(1, sc.height, sc.width, 3)).astype(np.float32)
+    r = run_both(sc, tg, seed=13, it=2, views=[0], pairs=pairs, gpu_kwargs={"pairs_per_item": ppi})
+    assert r["bins"][0] > 0
+    assert_parity(sc, r)
