@@ -1205,10 +1205,12 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
     const int nact = (int)sm.nact;
     // pairs of a group: as many as the set-ups, the sign words and (below) the sums hold
     int Gcap = min(GMAX, M::SLOTS / max(nb, 1)), par = 0, G = 0, nh = 0;
-    // unlit calls of one or two pairs take no window: finding its bounds costs half a pair, and the
-    // footprints all go through hashed cells (one 256^2 estimate: the kernel 37.0 -> 29.5 us; lit items
-    // lose, 11.2 -> 20.1 ms)
-    const bool windowed = M::LIT || a.pair_count > 2;
+    // unlit calls of one or two pairs and few items take no window: finding its bounds costs half a pair and lengthens each
+    // CTA's chain, and the footprints all go through hashed cells (one 256^2 estimate: the kernel 37.0 -> 29.5 us; lit items
+    // lose, 11.2 -> 20.1 ms).  With many items the pixels' own work counts, which a window makes less (whole calls,
+    // 8,192 triangles, one pair a view, without / with: 512^2 1 view 145 / 147 us, 640^2 4 views 419 / 408 us, 1024^2 4 views
+    // 963 / 905 us; two pairs: 512^2 1 view 202 / 200 us, 8 views 608 / 562 us; the line lies where the two meet)
+    const bool windowed = M::LIT || a.pair_count > 2 || n_work * a.pair_count > 6ll * gridDim.x;
     if (!windowed) {
       nh = kHashNoWindow;
       Gcap = min(Gcap, M::ACAP / nh);
