@@ -406,14 +406,15 @@ __global__ void __launch_bounds__(TILE_PX, kCtas) k_bin_prune(SceneDev S, Worksp
 
 // Batched form: every (tile, view slot, asset) of a batched call in one launch; each CTA reads
 // its asset's scene and workspace from the asset's launch descriptor in device memory.
-__global__ void __launch_bounds__(TILE_PX, 7) k_bin_prune_batch(const BatchArgs P) {
+template <int kStep, int kCtas>
+__global__ void __launch_bounds__(TILE_PX, kCtas) k_bin_prune_batch(const BatchArgs P) {
   __shared__ PruneSmem sm;
   const BatchAsset& A = P.as[blockIdx.z];
   const int slot = blockIdx.y;
   if (slot >= A.n_views) return;
   const AssetDesc& D = *A.desc;
   if ((int)blockIdx.x >= D.S.tiles_x * D.S.tiles_y) return;
-  prune_tile<4>(D.S, D.ws, A.n_views, slot, blockIdx.x, P.light_bin, sm);
+  prune_tile<kStep>(D.S, D.ws, A.n_views, slot, blockIdx.x, P.light_bin, sm);
 }
 
 // ---------------------------------------------------------------- the estimator
@@ -1053,7 +1054,7 @@ __device__ __forceinline__ void credit_texels(const SceneDev& S, const Workspace
   }
 }
 
-// An empty start of a CTA's loop over items.
+// An empty start of a CTA's loop over items (every item, and the end of each asset's, leaves it empty again).
 template <int SH, bool GR>
 __device__ __forceinline__ void reset_smem(FastSmem<SH, GR>& sm) {
   using M = Model<SH, GR>;
@@ -1103,7 +1104,10 @@ __device__ __forceinline__ void add_losses(const EstimateArgs& a, FastSmem<SH, G
   // of the pixels' own sums
   if (a.loss)
     for (int s = threadIdx.x; s < n_slots; s += Model<SH, GR>::THREADS)
-      if (sm.loss[s] != 0.0) atomicAdd(a.loss + s, (float)(sm.loss[s] / (double)a.pairs));
+      if (sm.loss[s] != 0.0) {
+        atomicAdd(a.loss + s, (float)(sm.loss[s] / (double)a.pairs));
+        sm.loss[s] = 0.0;
+      }
 }
 
 // Pairs per item: `lo` doubled up to `hi` while every CTA still gets at least 16 items (a longer run
@@ -1115,11 +1119,13 @@ __device__ __forceinline__ int run_of(const EstimateArgs& a, int n_items, int lo
 }
 
 // Every light work item of one scene's call, taken one at a time from the scene's work
-// counter until none is left.  own_first: a CTA's first item is its own index, without a round trip to
+// counter until none is left.  clean: sm is as reset_smem leaves it.  alone: no other
+// scene shares the launch.  own_first: a CTA's first item is its own index, without a round trip to
 // the counter (a launch's first asset, which every CTA starts at the same time).
 template <int SH, bool GR>
 __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
-                                           const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
+                                           const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first, bool& clean,
+                                           bool alone) {
   using M = Model<SH, GR>;
   constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1138,7 +1144,8 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
   const int run = a.pairs_per_item > 0 ? ppi : run_of(a, n_small, ppi, 4 * kRun), run_big = run_of(a, n_big, max(2, ppi / 4), ppi);
   const int chunks = (a.pair_count + run - 1) / run, chunks_big = (a.pair_count + run_big - 1) / run_big;
   const long long work_big = (long long)n_big * chunks_big, n_work = work_big + (long long)n_small * chunks;
-  reset_smem<SH, GR>(sm);
+  if (!clean) reset_smem<SH, GR>(sm);
+  clean = true;
   const uint32_t first_of = own_first ? gridDim.x : 0u;
   if (tid == 0) sm.item = own_first ? blockIdx.x : atomicAdd(ws.counters + 1, 1u);
   __syncthreads();
@@ -1209,8 +1216,9 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
     // CTA's chain, and the footprints all go through hashed cells (one 256^2 estimate: the kernel 37.0 -> 29.5 us; lit items
     // lose, 11.2 -> 20.1 ms).  With many items the pixels' own work counts, which a window makes less (whole calls,
     // 8,192 triangles, one pair a view, without / with: 512^2 1 view 145 / 147 us, 640^2 4 views 419 / 408 us, 1024^2 4 views
-    // 963 / 905 us; two pairs: 512^2 1 view 202 / 200 us, 8 views 608 / 562 us; the line lies where the two meet)
-    const bool windowed = M::LIT || a.pair_count > 2 || n_work * a.pair_count > 6ll * gridDim.x;
+    // 963 / 905 us; two pairs: 512^2 1 view 202 / 200 us, 8 views 608 / 562 us; the line lies where the two meet), and so it does beside other assets
+    // (!alone: batches of 4 assets of 8,192 triangles, 512^2, 2 views, one pair 907 / 782 us, two 1,096 / 887 us)
+    const bool windowed = M::LIT || a.pair_count > 2 || !alone || n_work * a.pair_count > 6ll * gridDim.x;
     if (!windowed) {
       nh = kHashNoWindow;
       Gcap = min(Gcap, M::ACAP / nh);
@@ -1433,7 +1441,7 @@ __device__ __forceinline__ void fast_items(const SceneDev& S, const Workspace& w
 // assets), 1.32 -> 0.26 ms (Lambert, 41 tiles x 16 pairs).
 template <int SH, bool GR>
 __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& ws, const ViewList& vl,
-                                            const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first) {
+                                            const EstimateArgs& a, FastSmem<SH, GR>& sm, bool own_first, bool& clean) {
   using M = Model<SH, GR>;
   constexpr int NREAD = M::NREAD, NFOOT = M::NFOOT, BLOCKS = TILE_PX / 32;
   constexpr int P = M::WARPS / BLOCKS;  // pairs at a time
@@ -1450,7 +1458,8 @@ __device__ __forceinline__ void dense_items(const SceneDev& S, const Workspace& 
   const int chunks = (a.pair_count + run - 1) / run;
   const long long n_work = (long long)n_heavy * chunks;
   if (n_work == 0 || (own_first && blockIdx.x >= n_work)) return;  // (uniform over the CTA)
-  reset_smem<SH, GR>(sm);
+  if (!clean) reset_smem<SH, GR>(sm);
+  clean = true;
   const uint32_t first_of = own_first ? gridDim.x : 0u;
   if (tid == 0) sm.item = own_first ? blockIdx.x : atomicAdd(ws.counters + 5, 1u);
   __syncthreads();
@@ -1677,14 +1686,16 @@ template <int SH, bool GR>
 __global__ void __launch_bounds__(Model<SH, GR>::THREADS, Model<SH, GR>::CTAS)
     k_estimate_fast(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  fast_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true);
+  bool clean = false;
+  fast_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true, clean, true);
 }
 
 template <int SH, bool GR>
 __global__ void __launch_bounds__(Model<SH, GR>::THREADS, 1)
     k_estimate_dense(SceneDev S, Workspace ws, ViewList vl, EstimateArgs a) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  dense_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true);
+  bool clean = false;
+  dense_items<SH, GR>(S, ws, vl, a, *reinterpret_cast<FastSmem<SH, GR>*>(smem_raw), true, clean);
 }
 
 // The batched kernel keeps its asset after FastSmem, 16-byte aligned.  (Batched calls use the
@@ -1700,11 +1711,12 @@ __global__ void __launch_bounds__(Model<SH>::THREADS, Model<SH>::CTAS) k_estimat
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<FastSmem<SH, false>*>(smem_raw);
   BatchSmem& b = *reinterpret_cast<BatchSmem*>(smem_raw + fast_batch_off<SH>());
+  bool clean = false;
   for (int ai = 0; ai < P.n; ++ai) {
     __syncthreads();
     load_asset(P, ai, b);
     __syncthreads();
-    fast_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0);
+    fast_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0, clean, P.n == 1);
   }
 }
 
@@ -1714,11 +1726,12 @@ __global__ void __launch_bounds__(Model<SH>::THREADS, 1) k_estimate_dense_batch(
   extern __shared__ __align__(16) unsigned char smem_raw[];
   auto& sm = *reinterpret_cast<FastSmem<SH, false>*>(smem_raw);
   BatchSmem& b = *reinterpret_cast<BatchSmem*>(smem_raw + fast_batch_off<SH>());
+  bool clean = false;
   for (int ai = 0; ai < P.n; ++ai) {
     __syncthreads();
     load_asset(P, ai, b);
     __syncthreads();
-    dense_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0);
+    dense_items<SH, false>(b.d.S, b.d.ws, b.vl, b.a, sm, ai == 0, clean);
   }
 }
 
@@ -1831,7 +1844,14 @@ cudaError_t launch_prune(const SceneDev& S, const Workspace& ws, const ViewList&
 }
 
 cudaError_t launch_prune_batch(const BatchArgs& P, int max_tiles, int max_views, cudaStream_t st) {
-  k_bin_prune_batch<<<dim3(max_tiles, max_views, P.n), TILE_PX, 0, st>>>(P);
+  const dim3 grid(max_tiles, max_views, P.n);
+  const long long ctas = (long long)grid.x * grid.y * grid.z;
+  if (ctas <= kPruneOneWave)
+    k_bin_prune_batch<16, 2><<<grid, TILE_PX, 0, st>>>(P);
+  else if (ctas <= kPruneSevenWave)
+    k_bin_prune_batch<16, 7><<<grid, TILE_PX, 0, st>>>(P);
+  else
+    k_bin_prune_batch<4, 7><<<grid, TILE_PX, 0, st>>>(P);
   return cudaGetLastError();
 }
 
