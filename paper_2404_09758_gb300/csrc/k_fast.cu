@@ -593,16 +593,18 @@ __device__ __forceinline__ void fold(const SceneDev& S, const Workspace& ws, con
       }
     }
   }
-  // hashed footprints: their texels one by one
+  // hashed footprints: their texels, whose sign words are fetched together (one after another a window-less item's fold took
+  // 8 us on average, and 15 us in the fullest tile of a 256^2 call; soup of 10,240 triangles, one pair 150 -> 143 us)
   for (int h = threadIdx.x; h < nh; h += M::THREADS) {
     const uint32_t code = sm.hkey[h];
     if (code == EMPTY) continue;
     const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
     const int tw = S.rtex[r].w;
     const Quad Q(code, tw);
-#pragma unroll 1
-    for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q) {
-      if (Q.repeats(q)) continue;
+    const int nq = S.foot_nearest ? 1 : 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= nq || Q.repeats(q)) continue;
       const int texel = Q.texel(q, tw);
 #pragma unroll 1
       for (int k = 0; k < (GR ? M::NREAD : 1); ++k) {
@@ -698,9 +700,10 @@ __device__ __forceinline__ void flush_counts(const SceneDev& S, const EstimateAr
     const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
     const int tw = S.rtex[r].w;
     const Quad Q(code, tw);
-#pragma unroll 1
-    for (int q = 0; q < (S.foot_nearest ? 1 : 4); ++q) {
-      if (Q.repeats(q)) continue;
+    const int nq = S.foot_nearest ? 1 : 4;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      if (q >= nq || Q.repeats(q)) continue;
       const int texel = Q.texel(q, tw);
 #pragma unroll 1
       for (int k = 0; k < (GR ? M::NREAD : 1); ++k) {
