@@ -167,12 +167,19 @@ __global__ void k_bin_fill(SceneDev S, Workspace ws) {
   if (tri >= S.nt) return;
   int4 rect = ws.tri_rect[(long long)slot * S.nt + tri];
   int nt = n_tiles(S);
-  for (int ty = rect.y; ty <= rect.w; ++ty)
-    for (int tx = rect.x; tx <= rect.z; ++tx) {
-      const long long t = (long long)slot * nt + ty * S.tiles_x + tx;
-      const uint32_t pos = atomicAdd(ws.tile_cur + t, 1u);
-      if (bin_stores(pos, ws.tile_off + t, ws.bin_capacity, S.nt) && CHK(S, pos, S.chk.bins)) ws.bins[pos] = (uint32_t)tri;
-    }
+  auto fill = [&](auto stores) {
+    for (int ty = rect.y; ty <= rect.w; ++ty)
+      for (int tx = rect.x; tx <= rect.z; ++tx) {
+        const long long t = (long long)slot * nt + ty * S.tiles_x + tx;
+        const uint32_t pos = atomicAdd(ws.tile_cur + t, 1u);
+        if (stores(pos, t) && CHK(S, pos, S.chk.bins)) ws.bins[pos] = (uint32_t)tri;
+      }
+  };
+  // (apart, so that the usual loop reads nothing: a large triangle's is a chain of atomics)
+  if (cursors_above(ws.bin_capacity, S.nt))
+    fill([&](uint32_t pos, long long) { return (long long)pos < ws.bin_capacity; });
+  else
+    fill([&](uint32_t pos, long long t) { return (long long)pos < ws.bin_capacity && ws.tile_off[t] != kNoBin; });
 }
 
 }  // namespace

@@ -138,10 +138,9 @@ __host__ __device__ inline uint32_t bin_start(unsigned long long before, uint32_
 __host__ __device__ inline uint32_t bin_cursor(uint32_t start, int n_triangles) {
   return start == kNoBin ? kNoBin - (uint32_t)n_triangles : start;
 }
-// May the fill store at position pos of the bin that starts at *start?  (The start is read only where a
-// capacity close to 2^32 reaches the cursors of bins left out.)
-__host__ __device__ inline bool bin_stores(uint32_t pos, const uint32_t* start, long long capacity, int n_triangles) {
-  return (long long)pos < capacity && (capacity <= (long long)(kNoBin - (uint32_t)n_triangles) || *start != kNoBin);
+// Are the cursors of bins left out above every position below the capacity?  (If not, the fill asks for the start.)
+__host__ __device__ inline bool cursors_above(long long capacity, int n_triangles) {
+  return capacity <= (long long)(kNoBin - (uint32_t)n_triangles);
 }
 
 // What a batched launch needs of one scene, kept in the scene's workspace (written on the

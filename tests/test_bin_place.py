@@ -26,7 +26,9 @@ int main(int argc, char** argv) {
       const uint32_t off = sge::bin_start(total, c, cap), cur = sge::bin_cursor(off, nt);
       const uint32_t last = cur + c - 1;             // the last entry's position as the fill forms it: 32 bits
       if (last < cur) return 3;                      // wrapped
-      const bool first_in = sge::bin_stores(cur, &off, cap, nt), last_in = sge::bin_stores(last, &off, cap, nt);
+      // the fill's test of a position
+      auto stores = [&](uint32_t pos) { return (long long)pos < cap && (sge::cursors_above(cap, nt) || off != sge::kNoBin); };
+      const bool first_in = stores(cur), last_in = stores(last);
       if ((long long)off + c <= cap) {               // stored, by the readers' test
         if (off != total || off < end || cur != off || !first_in || !last_in) return 4;
         end = (unsigned long long)off + c;
