@@ -549,15 +549,17 @@ __device__ __forceinline__ bool in_span(uint32_t span, int dx, int dy) {
 // Small (every edge function over the tile fits 32 bits: |a|, |b| < 2^16, |e0| < 2^29, so
 // |e| < 2^30 at the offsets 0..15 * 256): e = (E_0, E_1, area, flags) with E_k at the tile's first
 // pixel centre and area = E_0 + E_1 + E_2, which is the same everywhere, so edge 2 follows from the
-// other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig): the vertices relative to the first pixel
-// centre, e = (X0, Y0, X1, flags), ab = (Y1, X2, Y2, -).  Not drawn: E_0 = -1 everywhere.
+// other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig) the same with 64-bit edge functions: e = (E_0 low, E_0 high,
+// E_1 low, flags), iw.w the bits of E_1 high; the area is |a_0 b_1 - a_1 b_0|.  (Kept as vertices and multiplied out at
+// each test, a full-image call of 8 pairs of 2,048 triangles of half a 512^2 image took 20.4 ms, this 17.4 ms.)  Not drawn: E_0 = -1
+// everywhere.
 struct __align__(16) SideTri {
   int4 e, ab;
   float4 z;   // z_0..2, 1 / area
-  float4 iw;  // 1 / w_0..2
+  float4 iw;  // 1 / w_0..2, -
 };
 static_assert(sizeof(SideTri) == 64, "SideTri layout");
-constexpr int kBig = 8, kFlip = 16;  // flags; bits 0-2: edge k is not a top/left edge
+constexpr int kBig = 8;  // flag; bits 0-2: edge k is not a top/left edge
 
 // Set up one side of a triangle from its projected vertices (rx, ry: the tile's first pixel centre).
 __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int rx, int ry) {
@@ -569,6 +571,7 @@ __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int
   const int x0 = v[0].X - rx, x1 = v[1].X - rx, x2 = v[2].X - rx, y0 = v[0].Y - ry, y1 = v[1].Y - ry, y2 = v[2].Y - ry;
   const int far = max(max(max(abs(x0), abs(x1)), abs(x2)), max(max(abs(y0), abs(y1)), abs(y2)));
   float inv;
+  int e1_high = 0;
   if (far < (1 << 14)) {
     // vertices within 64 pixels of the tile's corner: E_k = x_a y_b - x_b y_a there, all in 32 bits
     // (|E_k| < 2^29, |a|, |b| < 2^15)
@@ -606,19 +609,18 @@ __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int
     }
     if (small) {
       d.e = make_int4((int)t.e0[0], (int)t.e0[1], (int)(t.e0[0] + t.e0[1] + t.e0[2]), flags);
-      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
     } else {
-      const bool flip = (long long)(x1 - x0) * (y2 - y0) < (long long)(y1 - y0) * (x2 - x0);
-      d.e = make_int4(x0, y0, x1, flags | kBig | (flip ? kFlip : 0));
-      d.ab = make_int4(y1, x2, y2, 0);
+      d.e = make_int4((int)t.e0[0], (int)(t.e0[0] >> 32), (int)t.e0[1], flags | kBig);
+      e1_high = (int)(t.e0[1] >> 32);
     }
+    d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
     inv = t.inv_area;
   }
   d.z = make_float4(v[0].z, v[1].z, v[2].z, inv);
-  d.iw = make_float4(v[0].iw, v[1].iw, v[2].iw, 0.0f);
+  d.iw = make_float4(v[0].iw, v[1].iw, v[2].iw, __int_as_float(e1_high));
 }
 
-// Coverage of the pixel whose centre lies (X, Y) fixed-point units from the tile's first one, and
+// Coverage of the tile's pixel whose centre lies (X, Y) fixed-point units (whole pixels) from its first one, and
 // (covered) the barycentric weights E_k / area there as lambdas() forms them.
 __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, float l[3], float4& z) {
   const int4 e = t.e, ab = t.ab;
@@ -633,15 +635,16 @@ __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, fl
     l[2] = __fmul_rn(__int2float_rn(e2), z.w);
     return true;
   }
-  const int vx[3] = {e.x, e.z, ab.y}, vy[3] = {e.y, ab.x, ab.z};
+  // steps in whole pixels: |a|, |b| <= 2^24 (vertices lie within 2^15 pixels), so 15 of each fit 32 bits
+  const int dx = X >> 8, dy = Y >> 8;
+  auto wide = [](int lo, int hi) { return (long long)((unsigned long long)(uint32_t)hi << 32 | (uint32_t)lo); };
   long long E[3];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    const int a = (k + 1) % 3, b = (k + 2) % 3;
-    E[k] = edge_at(vx[a], vy[a], vx[b], vy[b], X, Y);
-    if (e.w & kFlip) E[k] = -E[k];
-    if (E[k] - ((e.w >> k) & 1) < 0) return false;
-  }
+  E[0] = wide(e.x, e.y) + 256ll * (ab.x * dx + ab.z * dy);
+  E[1] = wide(e.z, __float_as_int(t.iw.w)) + 256ll * (ab.y * dx + ab.w * dy);
+  const long long area = (long long)ab.x * ab.w - (long long)ab.y * ab.z;  // (a and b are both turned: its sign is not)
+  E[2] = (area < 0 ? -area : area) - E[0] - E[1];
+  if ((E[0] | E[1] | E[2]) < 0) return false;
+  if ((e.w & 7) && (((e.w & 1) && E[0] == 0) || ((e.w & 2) && E[1] == 0) || ((e.w & 4) && E[2] == 0))) return false;
   z = t.z;
   lambdas(E, z.w, l);
   return true;
