@@ -512,7 +512,7 @@ __device__ __forceinline__ int window_texel(const int4& win, int t, int w) {
 }
 
 // Credit code of a pixel's side in footprint r: the window cell (the slot of the footprint's first
-// texel), or with kOut a footprint code (Quad) and r above it.
+// texel), or with kOut a footprint code (Quad) and r above it.  In the hash a code without kOut is one texel.
 constexpr uint32_t kOut = 1u << 31, EMPTY = 0xFFFFFFFFu;
 constexpr int kFootShift = 29;
 
@@ -601,7 +601,7 @@ __device__ __forceinline__ void fold(const SceneDev& S, const Workspace& ws, con
     const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
     const int tw = S.rtex[r].w;
     const Quad Q(code, tw);
-    const int nq = S.foot_nearest ? 1 : 4;
+    const int nq = S.foot_nearest || (!M::LIT && !(code & kOut)) ? 1 : 4;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (q >= nq || Q.repeats(q)) continue;
@@ -700,7 +700,7 @@ __device__ __forceinline__ void flush_counts(const SceneDev& S, const EstimateAr
     const int r = GR ? 0 : (int)((code >> kFootShift) & 3u);
     const int tw = S.rtex[r].w;
     const Quad Q(code, tw);
-    const int nq = S.foot_nearest ? 1 : 4;
+    const int nq = S.foot_nearest || (!M::LIT && !(code & kOut)) ? 1 : 4;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       if (q >= nq || Q.repeats(q)) continue;
@@ -1051,8 +1051,21 @@ __device__ __forceinline__ void credit_texels(const SceneDev& S, const Workspace
     if (mine == all) {
       credit_cell(B);
     } else {
+      // One texel each, straight to the global sums; unlit, of footprints of one row through the hash: a flat triangle's colour is a texel
+      // of such a texture, footprints at its centre differ by rounding, and one that covers the image would send every pixel's
+      // to the same place (64 of them, 512^2, 8 pairs: 1.60 -> 0.92 ms).  Of other footprints few pixels share a texel, and hashed it costs
+      // more to find, fold and count than it saves (3 views of 413 x 311, Lambert, 5 pairs: 356 us, 413 us with all hashed).
 #pragma unroll 1
-      for (; mine; mine &= mine - 1) credit_id(QB.texel(__ffs((int)mine) - 1, T.w));
+      for (; mine; mine &= mine - 1) {
+        const int id = QB.texel(__ffs((int)mine) - 1, T.w);
+        const int h = !M::LIT && (B & kOneRow) ? hash_slot(sm.hkey, (uint32_t)id, nh) : -1;
+        if (h >= 0) {
+          atomicAdd(sums + n_win + h, df);
+          atomicAdd(sm.hcnt + h, 1u);
+        } else {
+          credit_id(id);
+        }
+      }
     }
   }
 }

@@ -82,3 +82,15 @@ def test_transparent_estimates_match_oracle(n, reach, grid):
     r = run_both(sc, tg, seed=3, it=1, views=[0], pairs=2, gpu_kwargs={"bin_capacity": n * 16 + 64})
     assert r["C"][: sc.n_pos_params].sum() > 0
     assert_parity(sc, r)
+
+
+@pytest.mark.parametrize("n,pairs", [(6, 1), (40, 9), (400, 3)])
+def test_flat_colours_match_oracle(n, pairs):
+    """A triangle's colour is one texel of a one-row texture, whose footprints at the texel's centre differ by rounding
+    between the sides: the texels left over on side - go through the hash."""
+    sc, tg = _scene(n, 200, False)
+    soup = synth.triangle_soup(n, render=R, seed=3)[0]
+    sc = dataclasses.replace(sc, uvs=soup.uvs, textures=soup.textures)
+    r = run_both(sc, tg, seed=13, it=2, views=[0], pairs=pairs, gpu_kwargs={"bin_capacity": n * 16 + 64})
+    assert r["C"][sc.n_pos_params:].sum() > 0
+    assert_parity(sc, r)
