@@ -33,11 +33,14 @@ __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_c
 // Four consecutive parameters per thread: HBM bound, 20 B read and 20 B written per parameter (Adam), each
 // flat array (sums, counts, m, v) as one 16-byte access and theta as one where its group starts on a
 // multiple of four parameters (else four 4-byte ones).  One parameter per thread and grid-stride
-// iteration reached 5.2 TB/s on 52 M parameters (394 us); this 6.6 TB/s (313 us).
+// iteration reached 5.2 TB/s on 52 M parameters (394 us); this 6.6 TB/s (313 us).  Steps of few parameters last as long as a
+// thread's chain, which four make longer (2,214 parameters 2.2 us with one a thread, 4.6 us with four; 198 K 3.6 and 5.1, 556 K 5.7 and 5.8,
+// 1.08 M 8.3 and 8.0): they keep one parameter a thread and iteration (kPer = 1).
+template <int kPer>
 __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* grad, uint32_t* counts, float inv_n,
                                               float b1, float b2, int t_host, float aeps, float* m, float* v,
                                               const int32_t* t_dev) {
-  const long long d = G.begin[G.n], i0 = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+  const long long d = G.begin[G.n], i0 = kPer * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (i0 >= d) return;
   // Adam's bias corrections 1 - beta^t for the step number t (from device memory in a replayed
   // graph's step), formed as -expm1(t log beta): no cancellation when beta^t is close to 1
@@ -72,7 +75,7 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
   };
   const int g = group_of(G, i0);
   const bool moments = kind == SGE_STEP_ADAM;
-  if (i0 + 4 <= G.begin[g + 1] && aligned16(grad) && aligned16(counts) && (!moments || (aligned16(m) && aligned16(v)))) {
+  if (kPer == 4 && i0 + 4 <= G.begin[g + 1] && aligned16(grad) && aligned16(counts) && (!moments || (aligned16(m) && aligned16(v)))) {
     const float4 s4 = __ldcs(reinterpret_cast<const float4*>(grad + i0));
     const uint4 n4 = __ldcs(reinterpret_cast<const uint4*>(counts + i0));
     float4 m4 = make_float4(0.f, 0.f, 0.f, 0.f), v4 = m4;
@@ -109,8 +112,9 @@ __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* gra
     __stcs(reinterpret_cast<uint4*>(counts + i0), make_uint4(0u, 0u, 0u, 0u));
     return;
   }
-  // a quad across two groups, the last parameters, or arrays that do not start on 16 bytes
-  for (long long i = i0; i < i0 + 4 && i < d; ++i) {
+  // a quad across two groups, the last parameters, or arrays that do not start on 16 bytes; with one a thread, all
+  const long long end = kPer == 4 && i0 + 4 < d ? i0 + 4 : d, by = kPer == 4 ? 1 : (long long)gridDim.x * blockDim.x;
+  for (long long i = i0; i < end; i += by) {
     const int gi = group_of(G, i);
     float* theta = G.theta[gi] + (i - G.begin[gi]);
     float th = *theta, mm = moments ? m[i] : 0.0f, vv = moments ? v[i] : 0.0f;
@@ -165,6 +169,10 @@ StepGroups groups_of(const SceneDev& S) {
   G.begin[G.n] = S.n_params;
   return G;
 }
+
+// Steps of at most so many parameters take one a thread (k_step), in at most eight CTAs per SM.
+constexpr long long kStepOne = 900000;
+constexpr unsigned kStepOneCtas = 8 * 152;
 
 // CTAs of 256 threads, four parameters each.
 unsigned grid_for(long long n) { return (unsigned)((n + 1023) / 1024); }
@@ -240,8 +248,13 @@ cudaError_t launch_step(const SceneDev& S, const sge_opt& o, float* grad, uint32
     G.lr[k + 1] = o.lr_tex[k];
   }
   G.begin[G.n] = S.n_params;
-  k_step<<<grid_for(S.n_params), 256, 0, st>>>(G, o.kind, grad, counts, (float)(1.0 / (double)n_total), o.beta1,
-                                           o.beta2, o.t, o.adam_eps, m, v, t_dev);
+  const float inv_n = (float)(1.0 / (double)n_total);
+  if (S.n_params <= kStepOne)
+    k_step<1><<<min((unsigned)((S.n_params + 255) / 256), kStepOneCtas), 256, 0, st>>>(
+        G, o.kind, grad, counts, inv_n, o.beta1, o.beta2, o.t, o.adam_eps, m, v, t_dev);
+  else
+    k_step<4><<<grid_for(S.n_params), 256, 0, st>>>(G, o.kind, grad, counts, inv_n, o.beta1, o.beta2, o.t, o.adam_eps, m, v,
+                                                    t_dev);
   return cudaGetLastError();
 }
 
