@@ -34,8 +34,8 @@ __device__ __forceinline__ bool aligned16(const void* p) { return (reinterpret_c
 // flat array (sums, counts, m, v) as one 16-byte access and theta as one where its group starts on a
 // multiple of four parameters (else four 4-byte ones).  One parameter per thread and grid-stride
 // iteration reached 5.2 TB/s on 52 M parameters (394 us); this 6.6 TB/s (313 us).  Steps of few parameters last as long as a
-// thread's chain, which four make longer (2,214 parameters 2.2 us with one a thread, 4.6 us with four; 198 K 3.6 and 5.1, 556 K 5.7 and 5.8,
-// 1.08 M 8.3 and 8.0): they keep one parameter a thread and iteration (kPer = 1).
+// thread's chain, which four make longer (2,214 parameters 2.0 us with one a thread, 4.6 us with four; 198 K 3.8 and 5.1, 395 K 5.1
+// and 5.4, 556 K 6.2 and 5.8): they keep one parameter a thread and iteration (kPer = 1).
 template <int kPer>
 __global__ void __launch_bounds__(256) k_step(StepGroups G, int kind, float* grad, uint32_t* counts, float inv_n,
                                               float b1, float b2, int t_host, float aeps, float* m, float* v,
@@ -136,21 +136,23 @@ __global__ void k_iter_advance(uint32_t* state, int d_iter, int d_t) {
 }
 
 // g_i = scale * grad_i / (2 eps_i n_total): the estimate of Eq. 9 (scale: device scalar or NULL).
-// Four parameters per thread, as k_step.
+// Four parameters per thread or one, as k_step (2,214 parameters 1.4 us with one, 2.1 us with four; 395 K 2.3 and 2.4).
+template <int kPer>
 __global__ void __launch_bounds__(256) k_gradient(StepGroups G, const float* grad, float inv_n, const float* scale,
                                                   float* out) {
-  const long long d = G.begin[G.n], i0 = 4 * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
+  const long long d = G.begin[G.n], i0 = kPer * ((long long)blockIdx.x * blockDim.x + threadIdx.x);
   if (i0 >= d) return;
   const float sc = scale ? *scale : 1.0f;
   const int g = group_of(G, i0);
-  if (i0 + 4 <= G.begin[g + 1] && aligned16(grad) && aligned16(out)) {
+  if (kPer == 4 && i0 + 4 <= G.begin[g + 1] && aligned16(grad) && aligned16(out)) {
     const float4 s = *reinterpret_cast<const float4*>(grad + i0);
     const float e = 2.0f * G.eps[g];
     *reinterpret_cast<float4*>(out + i0) =
         make_float4(sc * (s.x * inv_n / e), sc * (s.y * inv_n / e), sc * (s.z * inv_n / e), sc * (s.w * inv_n / e));
     return;
   }
-  for (long long i = i0; i < i0 + 4 && i < d; ++i) out[i] = sc * (grad[i] * inv_n / (2.0f * G.eps[group_of(G, i)]));
+  const long long end = kPer == 4 && i0 + 4 < d ? i0 + 4 : d, by = kPer == 4 ? 1 : (long long)gridDim.x * blockDim.x;
+  for (long long i = i0; i < end; i += by) out[i] = sc * (grad[i] * inv_n / (2.0f * G.eps[group_of(G, i)]));
 }
 
 StepGroups groups_of(const SceneDev& S) {
@@ -170,9 +172,9 @@ StepGroups groups_of(const SceneDev& S) {
   return G;
 }
 
-// Steps of at most so many parameters take one a thread (k_step), in at most eight CTAs per SM.
-constexpr long long kStepOne = 900000;
-constexpr unsigned kStepOneCtas = 8 * 152;
+// Steps and gradients of at most so many parameters take one a thread, in at most eight CTAs per SM.
+constexpr long long kStepOne = 450000;
+unsigned grid_one(long long n) { return (unsigned)(n > 256ll * 8 * 152 ? 8 * 152 : (n + 255) / 256); }
 
 // CTAs of 256 threads, four parameters each.
 unsigned grid_for(long long n) { return (unsigned)((n + 1023) / 1024); }
@@ -229,7 +231,11 @@ __global__ void k_csr_vec3(const int32_t* ptr, const int32_t* col, const float* 
 
 cudaError_t launch_gradient(const SceneDev& S, const float* grad, long long n_total, const float* scale, float* out,
                             cudaStream_t st) {
-  k_gradient<<<grid_for(S.n_params), 256, 0, st>>>(groups_of(S), grad, (float)(1.0 / (double)n_total), scale, out);
+  const float inv_n = (float)(1.0 / (double)n_total);
+  if (S.n_params <= kStepOne)
+    k_gradient<1><<<grid_one(S.n_params), 256, 0, st>>>(groups_of(S), grad, inv_n, scale, out);
+  else
+    k_gradient<4><<<grid_for(S.n_params), 256, 0, st>>>(groups_of(S), grad, inv_n, scale, out);
   return cudaGetLastError();
 }
 
@@ -250,8 +256,8 @@ cudaError_t launch_step(const SceneDev& S, const sge_opt& o, float* grad, uint32
   G.begin[G.n] = S.n_params;
   const float inv_n = (float)(1.0 / (double)n_total);
   if (S.n_params <= kStepOne)
-    k_step<1><<<min((unsigned)((S.n_params + 255) / 256), kStepOneCtas), 256, 0, st>>>(
-        G, o.kind, grad, counts, inv_n, o.beta1, o.beta2, o.t, o.adam_eps, m, v, t_dev);
+    k_step<1><<<grid_one(S.n_params), 256, 0, st>>>(G, o.kind, grad, counts, inv_n, o.beta1, o.beta2, o.t, o.adam_eps, m, v,
+                                                    t_dev);
   else
     k_step<4><<<grid_for(S.n_params), 256, 0, st>>>(G, o.kind, grad, counts, inv_n, o.beta1, o.beta2, o.t, o.adam_eps, m, v,
                                                     t_dev);
