@@ -365,8 +365,8 @@ int sge_estimate_grad_batch_state(const sge_batch_entry *entries, int32_t n_entr
 
 /* Autotuner of sge_estimate_grad_batch's launch shape (no counterpart in the paper,
  * which runs one asset at a time) for these entries: times
- * candidate shapes (pairs per item 1..64, 1 or 2 CTAs per SM, light-bin limit
- * 64/128/256; a coordinate search from the defaults), each as one untimed call then
+ * candidate shapes (the default, pairs per item 2..64, 1 or 2 CTAs per SM, light-bin
+ * limit 64/128/256; a coordinate search from the defaults, which it may return), each as one untimed call then
  * the mean of `repeats` calls (CUDA events on `stream`), and returns the fastest in
  * *out and its time in *best_ms (may be NULL).  Runs real estimates into the
  * entries' buffers and zeroes grad_sums, counts and loss_out before returning.

@@ -590,12 +590,16 @@ class Batch:
         return float(ms.value)
 
 
+TUNED_KERNELS = "groups"  # renamed when the estimators change so that shapes timed before no longer fit
+
+
 def tuning_key(gpu: str, assets, pairs_per_view: int) -> str:
-    """Key of a batch's launch shape in the tuning cache: the GPU's name, each asset's render
+    """Key of a batch's launch shape in the tuning cache: the GPU's name, the kernels the shapes were
+    timed for (TUNED_KERNELS), each asset's render
     size and triangle count rounded up to a power of two (in the batch's order), and the pairs per
     view.  assets: [(width, height, n_triangles), ...]."""
     parts = [f"{int(w)}x{int(h)}:T{1 << max(0, int(t) - 1).bit_length()}" for w, h, t in assets]
-    return f"{gpu}|{int(pairs_per_view)}|" + ",".join(parts)
+    return f"{gpu}|{TUNED_KERNELS}|{int(pairs_per_view)}|" + ",".join(parts)
 
 
 def tuning_cache_load(path: str, key: str):

@@ -873,35 +873,9 @@ int sge_autotune_batch(const sge_batch_entry* entries, int32_t n, int32_t pairs_
     ms /= (float)repeats;
     return SGE_OK;
   };
-  sge_batch_tuning best{8, 0, kLightBin};
-  if (best.pairs_per_item > pairs_per_view) best.pairs_per_item = pairs_per_view;
+  sge_batch_tuning best{};
   float best_t = 0.0f;
-  rc = time_of(best, best_t);
-  // coordinate search: pairs per item, then CTAs per SM, then the light-bin limit
-  const int ppi[] = {1, 2, 4, 8, 16, 32, 64};
-  for (int k = 0; k < 7 && !rc; ++k) {
-    if (ppi[k] > pairs_per_view || ppi[k] == best.pairs_per_item) continue;
-    sge_batch_tuning t = best;
-    t.pairs_per_item = ppi[k];
-    float ms = 0.0f;
-    rc = time_of(t, ms);
-    if (!rc && ms < best_t) best = t, best_t = ms;
-  }
-  for (int bps = 1; bps <= 2 && !rc; ++bps) {
-    sge_batch_tuning t = best;
-    t.blocks_per_sm = bps;
-    float ms = 0.0f;
-    rc = time_of(t, ms);
-    if (!rc && ms < best_t) best = t, best_t = ms;
-  }
-  const int lb[] = {64, 128};
-  for (int k = 0; k < 2 && !rc; ++k) {
-    sge_batch_tuning t = best;
-    t.light_bin = lb[k];
-    float ms = 0.0f;
-    rc = time_of(t, ms);
-    if (!rc && ms < best_t) best = t, best_t = ms;
-  }
+  rc = search_batch_shape(pairs_per_view, time_of, best, best_t);
   cudaEventDestroy(ev[0]);
   cudaEventDestroy(ev[1]);
   if (rc) return rc;

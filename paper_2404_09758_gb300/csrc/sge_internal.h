@@ -143,6 +143,25 @@ __host__ __device__ inline bool cursors_above(long long capacity, int n_triangle
   return capacity <= (long long)(kNoBin - (uint32_t)n_triangles);
 }
 
+// The autotuner's search: the default shape first, so that the shape it returns is never slower than that, then by
+// coordinate pairs per item (1 counts as 2), CTAs per SM and the light-bin limit.  time_of(shape, ms): 0 or an error.  Where every
+// pair fits 8 an item, 8 is the default's shape (k_fast.cu, run_of) and names it; else 0 does.
+template <typename F>
+int search_batch_shape(int pairs_per_view, F&& time_of, sge_batch_tuning& best, float& best_t) {
+  best = sge_batch_tuning{pairs_per_view > 8 ? 0 : 8, 0, kLightBin};
+  int rc = time_of(best, best_t);
+  auto consider = [&](const sge_batch_tuning& t) {
+    float ms = 0.0f;
+    rc = time_of(t, ms);
+    if (!rc && ms < best_t) best = t, best_t = ms;
+  };
+  for (int ppi = 2; ppi <= 64 && !rc; ppi *= 2)
+    if (ppi <= pairs_per_view && !(ppi == 8 && pairs_per_view == 8)) consider({ppi, best.blocks_per_sm, best.light_bin});
+  for (int bps = 1; bps <= 2 && !rc; ++bps) consider({best.pairs_per_item, bps, best.light_bin});
+  for (int lb = 64; lb <= 128 && !rc; lb *= 2) consider({best.pairs_per_item, best.blocks_per_sm, lb});
+  return rc;
+}
+
 // What a batched launch needs of one scene, kept in the scene's workspace (written on the
 // stream by launch_put_desc) so that the launch's parameter holds one pointer per asset.
 struct __align__(16) AssetDesc {
