@@ -190,7 +190,10 @@ cudaError_t launch_binning(const SceneDev& S, const Workspace& ws, const ViewLis
   cudaError_t e = cudaMemsetAsync(ws.tile_count, 0, sizeof(uint32_t) * (size_t)vl.n * nt, st);
   if (e != cudaSuccess) return e;
   dim3 grid((S.nt + 255) / 256, vl.n);
-  k_bin_rect_count<<<grid, 256, 0, st>>>(S, ws, vl);
+  // (only the pruning reads the records: three projections and 32 B a triangle and view less without it)
+  Workspace counted = ws;
+  if (!prune) counted.tri_rec = nullptr;
+  k_bin_rect_count<<<grid, 256, 0, st>>>(S, counted, vl);
   k_bin_place<<<(vl.n * nt + 1023) / 1024, 1024, 0, st>>>(ws, vl.n * nt, S.nt);
   k_bin_fill<<<grid, 256, 0, st>>>(S, ws);
   e = cudaGetLastError();
