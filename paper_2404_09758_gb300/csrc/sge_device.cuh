@@ -640,11 +640,12 @@ __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, fl
   auto wide = [](int lo, int hi) { return (long long)((unsigned long long)(uint32_t)hi << 32 | (uint32_t)lo); };
   long long E[3];
   E[0] = wide(e.x, e.y) + 256ll * (ab.x * dx + ab.z * dy);
+  if (E[0] - (e.w & 1) < 0) return false;
   E[1] = wide(e.z, __float_as_int(t.iw.w)) + 256ll * (ab.y * dx + ab.w * dy);
+  if (E[1] - ((e.w >> 1) & 1) < 0) return false;
   const long long area = (long long)ab.x * ab.w - (long long)ab.y * ab.z;  // (a and b are both turned: its sign is not)
   E[2] = (area < 0 ? -area : area) - E[0] - E[1];
-  if ((E[0] | E[1] | E[2]) < 0) return false;
-  if ((e.w & 7) && (((e.w & 1) && E[0] == 0) || ((e.w & 2) && E[1] == 0) || ((e.w & 4) && E[2] == 0))) return false;
+  if (E[2] - ((e.w >> 2) & 1) < 0) return false;
   z = t.z;
   lambdas(E, z.w, l);
   return true;
