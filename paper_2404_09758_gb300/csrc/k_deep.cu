@@ -127,7 +127,7 @@ __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& w
         sm.tri[j] = tri;
         load_uvs(S, tri, sm.uv[j]);
       }
-      set_up_side(sm.t[s][j], v, rx, ry);
+      set_up_side<true>(sm.t[s][j], v, rx, ry);
       // a covered pixel centre lies in the triangle's vertex box
       sm.span[j][s] = v[0].ok && v[1].ok && v[2].ok ? box_span(v, rx, ry, 0) : 0u;
     }
@@ -140,7 +140,7 @@ __device__ __forceinline__ int deep_raster(const SceneDev& S, const Workspace& w
       for_spans(sm.span, s, cnt, block, dx, dy, [&](int j) {
         float l[3];
         float4 z;
-        if (!cover_lambdas(sm.t[s][j], dx * 256, dy * 256, l, z)) return;
+        if (!cover_lambdas<true>(sm.t[s][j], dx * 256, dy * 256, l, z)) return;
         const float zz[3] = {z.x, z.y, z.z};
         deep_insert(M, Q, ((unsigned long long)ordered_bits(interp_depth(l, zz)) << 32) | (uint32_t)sm.tri[j], j);
       });
@@ -183,7 +183,7 @@ __device__ __forceinline__ float3 deep_composite(const SceneDev& S, const float*
     float4 z;
     if (staged) {
       const SideTri& t = staged[P[j]];
-      cover_lambdas(t, dx * 256, dy * 256, l, z);
+      cover_lambdas<true>(t, dx * 256, dy * 256, l, z);
       iw[0] = t.iw.x, iw[1] = t.iw.y, iw[2] = t.iw.z;
 #pragma unroll
       for (int k = 0; k < 6; ++k) uv[k] = uvs[P[j]][k];
@@ -206,8 +206,8 @@ __device__ __forceinline__ float3 deep_composite(const SceneDev& S, const float*
         iw[k] = v[k].iw;
       }
       SideTri own;
-      set_up_side(own, v, rx, ry);
-      cover_lambdas(own, dx * 256, dy * 256, l, z);
+      set_up_side<true>(own, v, rx, ry);
+      cover_lambdas<true>(own, dx * 256, dy * 256, l, z);
       load_uvs(S, tri, uv);
     }
     const PerspW pw = persp(l, iw);

@@ -552,16 +552,18 @@ __device__ __forceinline__ bool in_span(uint32_t span, int dx, int dy) {
 // other two; ab = (a_0, a_1, b_0, b_1).  Otherwise (kBig) the same with 64-bit edge functions: e = (E_0 low, E_0 high,
 // E_1 low, flags), iw.w the bits of E_1 high; the area is |a_0 b_1 - a_1 b_0|.  (Kept as vertices and multiplied out at
 // each test, a full-image call of 8 pairs of 2,048 triangles of half a 512^2 image took 20.4 ms, this 17.4 ms.)  Not drawn: E_0 = -1
-// everywhere.
+// everywhere.  kVerts: big ones as vertices relative to the first pixel centre all the same, e = (X0, Y0, X1, flags), ab =
+// (Y1, X2, Y2, -), which leaves the transparent kernel, bound by registers, fewer spills (8 views x 16 pairs 5,490 us, 5,566 us otherwise).
 struct __align__(16) SideTri {
   int4 e, ab;
   float4 z;   // z_0..2, 1 / area
   float4 iw;  // 1 / w_0..2, -
 };
 static_assert(sizeof(SideTri) == 64, "SideTri layout");
-constexpr int kBig = 8;  // flag; bits 0-2: edge k is not a top/left edge
+constexpr int kBig = 8, kFlip = 16;  // flags; bits 0-2: edge k is not a top/left edge
 
 // Set up one side of a triangle from its projected vertices (rx, ry: the tile's first pixel centre).
+template <bool kVerts = false>
 __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int rx, int ry) {
   if (!(v[0].ok && v[1].ok && v[2].ok)) {
     d.e = make_int4(-1, 0, 0, 0);
@@ -609,11 +611,16 @@ __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int
     }
     if (small) {
       d.e = make_int4((int)t.e0[0], (int)t.e0[1], (int)(t.e0[0] + t.e0[1] + t.e0[2]), flags);
+      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
+    } else if constexpr (kVerts) {
+      const bool flip = (long long)(x1 - x0) * (y2 - y0) < (long long)(y1 - y0) * (x2 - x0);
+      d.e = make_int4(x0, y0, x1, flags | kBig | (flip ? kFlip : 0));
+      d.ab = make_int4(y1, x2, y2, 0);
     } else {
       d.e = make_int4((int)t.e0[0], (int)(t.e0[0] >> 32), (int)t.e0[1], flags | kBig);
+      d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
       e1_high = (int)(t.e0[1] >> 32);
     }
-    d.ab = make_int4(t.a[0], t.a[1], t.b[0], t.b[1]);
     inv = t.inv_area;
   }
   d.z = make_float4(v[0].z, v[1].z, v[2].z, inv);
@@ -622,6 +629,7 @@ __device__ __forceinline__ void set_up_side(SideTri& d, const PVert (&v)[3], int
 
 // Coverage of the tile's pixel whose centre lies (X, Y) fixed-point units (whole pixels) from its first one, and
 // (covered) the barycentric weights E_k / area there as lambdas() forms them.
+template <bool kVerts = false>
 __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, float l[3], float4& z) {
   const int4 e = t.e, ab = t.ab;
   if (!(e.w & kBig)) {
@@ -633,6 +641,20 @@ __device__ __forceinline__ bool cover_lambdas(const SideTri& t, int X, int Y, fl
     l[0] = __fmul_rn(__int2float_rn(e0), z.w);
     l[1] = __fmul_rn(__int2float_rn(e1), z.w);
     l[2] = __fmul_rn(__int2float_rn(e2), z.w);
+    return true;
+  }
+  if constexpr (kVerts) {
+    const int vx[3] = {e.x, e.z, ab.y}, vy[3] = {e.y, ab.x, ab.z};
+    long long E[3];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const int a = (k + 1) % 3, b = (k + 2) % 3;
+      E[k] = edge_at(vx[a], vy[a], vx[b], vy[b], X, Y);
+      if (e.w & kFlip) E[k] = -E[k];
+      if (E[k] - ((e.w >> k) & 1) < 0) return false;
+    }
+    z = t.z;
+    lambdas(E, z.w, l);
     return true;
   }
   // steps in whole pixels: |a|, |b| <= 2^24 (vertices lie within 2^15 pixels), so 15 of each fit 32 bits
