@@ -464,7 +464,8 @@ int sge_kernel_time(sge_scene *scene, float *total_ms, float *heavy_ms, int32_t 
 /* Work list of the scene's last estimate call (after its binning and pruning; a
  * diagnostic with no counterpart in the paper):
  * tiles x views taken by the fast kernel (light_items), by the heavy-bin kernel
- * (heavy_items) and the triangle-tile bin entries before pruning.  Synchronises
+ * (heavy_items) and the triangle-tile bin entries before pruning.  Renders, losses, and plain,
+ * full-image and transparent calls do not prune: they leave 0 items.  Synchronises
  * `stream`.  For tuning sge_batch_tuning.light_bin and for diagnostics. */
 int sge_bin_stats(sge_scene *scene, sge_stream_t stream, int64_t *light_items, int64_t *heavy_items,
                   int64_t *bin_entries);

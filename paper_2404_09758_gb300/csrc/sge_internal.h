@@ -199,7 +199,7 @@ cudaError_t launch_prune_batch(const BatchArgs& P, int max_tiles, int max_views,
 
 // ---- kernels launchers (all asynchronous on `st`)
 // Tile binning of every triangle for each view of `vl`, conservative for any
-// perturbation of at most eps_pos per coordinate.  Fills ws bins / items.  With `prune`
+// perturbation of at most eps_pos per coordinate.  Fills ws bins.  With `prune`
 // (the estimators), k_bin_prune then drops from each bin the triangles no perturbation can
 // make visible in the tile, lists the items by their live counts and stores each pixel's
 // candidate triangles.
